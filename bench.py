@@ -254,12 +254,11 @@ def run_reference(args) -> None:
 
 
 def _fp64_ops(J: int) -> float:
-    """FP64 FMA-pipe operations per element of the padded tile region for one solve
-    of J iterations, as the pass kernels are written: row pass 3 (first iteration) or
-    11.39 (rebuild of the loaded 68 x 72 tile for a 64 x 64 core: 2.39; D: 1;
-    column and row stencils: 6; sweeps: 2), column pass 5 (rebuild 2, pivot scale 1,
-    sweeps 2)."""
-    return 3.0 + 11.39 * (J - 1) + 5.0 * J
+    """FP64 FMA-pipe operations per element of the padded region for one solve of J
+    iterations, as the pass kernels are written: row pass 5 (two sweeps, the sum
+    a = u + s v, two summary products), column pass 6 (two sweeps, u, D, two summary
+    products; 4 in the last iteration)."""
+    return 11.0 * J - 2.0
 
 
 def _time_solves(api, plan, F, X, steps, stream, flush=None):
@@ -515,8 +514,8 @@ def main() -> None:
 
     hbm, peak_kind = _peaks()
     n_pass = kt["count"]
-    col_bytes = 2 * 4.0 * N * N * (n_pass // 2)  # column pass: one FP32 read, one write per element
-    row_bytes = kt["alg_bytes"] - col_bytes
+    row_bytes = 2 * 4.0 * N * N * (n_pass // 2)  # row pass: one FP32 read, one write per element
+    col_bytes = kt["alg_bytes"] - row_bytes
     achieved = kt["alg_bytes"] / (kt["total_ms"] * 1e-3) / 1e9 if kt["total_ms"] > 0 else None
     tr = _recorded_traffic("sweep.cu")
     traffic = None
@@ -551,8 +550,8 @@ def main() -> None:
             "frac_survey": (achieved / hbm) if achieved else None, "traffic": traffic,
             "kernel": "ADI pass kernels (row pass + column pass of every inner iteration)",
             "bytes_per_launch": "12 B per element: the 6 FP32 words per element and iteration of the "
-                                "residual-form ADI (row pass: c, D read; D, result written; column pass: "
-                                "result read, c written), the survey's 3 words per half-step",
+                                "residual-form ADI (row pass: u read, a written; column pass: a, D read, u, D "
+                                "written), the survey's 3 words per half-step on average",
             "launches_timed": n_pass, "peak_kind": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)",
             "row_pass": {"ms": kt["row_ms"], "gbs": row_bytes / (kt["row_ms"] * 1e-3) / 1e9 if kt["row_ms"] else None,
                          "frac": row_bytes / (kt["row_ms"] * 1e-3) / 1e9 / hbm if kt["row_ms"] else None},
@@ -600,7 +599,7 @@ def main() -> None:
         J64t = api.plan_info(plan64t)["J"]
         api.plan_destroy(plan64t)
         fma_rate = api.probe_fma_rate("fp64")
-        Np = 64 * ((N + 63) // 64)
+        Np = 64 * ((N + 63) // 64)  # blocks of 32 unknowns per parity
         ops = _fp64_ops(info64["J"]) * Np * Np
         alg_ops = 12.0 * info64["J"] * N * N
         line["fp64"] = {

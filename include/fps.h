@@ -83,14 +83,15 @@ typedef struct {
     double tol;             /* requested tolerance */
     int64_t device_bytes;   /* device memory owned by the plan */
     int64_t kernel_launches; /* kernels of this library launched by the last solve */
-    int seg_len;            /* square plans: segment length of the partitioned sweeps (rows of a
-                               column-pass tile, columns of a row-pass tile); FP32_REFINE: picked
-                               by the autotuner unless FPS_AUTOTUNE=0 */
+    int seg_len;            /* square plans: segment length of the partitioned sweeps, counted in
+                               unknowns of both parities (64 or 128); FP32_REFINE: picked by the
+                               autotuner unless FPS_AUTOTUNE=0 */
     int64_t inner_iterations; /* cube: inner (slice Stein) ADI iterations over full
                                  tensors in the last solve, all levels and rounds */
     int chain_mode;         /* square plans: load batching of the segment-coupling kernel
                                (1 short, 2 long batches; FP32_REFINE: picked by the autotuner
-                               with seg_len, 0 = chosen by grid size when it did not run) */
+                               with seg_len, 0 = short when it did not run; plans of at most 16
+                               segments per line launch no such kernel) */
 } fps_plan_info_t;
 
 /*
@@ -215,10 +216,9 @@ int fps_plan_set_instrument(fps_plan *plan, int on);
  * timed launches of the ADI pass kernels (*count, two per iteration), their summed
  * duration in ms (*total_ms) and the algorithmic bytes they move (*alg_bytes: per
  * element and iteration the residual-form ADI reads and writes six n x n words --
- * the row pass reads c and D and writes D and its result, the column pass reads
- * that result and writes c -- four in the first iteration, five in the second;
- * 8 bytes per FP64 and 4 per FP32 word; no padding, halo, segment-summary or
- * re-read traffic).  Synchronises the plan's stream.
+ * the row pass reads u and writes a, the column pass reads a and D and writes u and
+ * D -- five in the first and in the last iteration; 8 bytes per FP64 and 4 per FP32
+ * word; no padding, segment-summary or re-read traffic).  Synchronises the plan's stream.
  * Errors: INVALID_ARG (not instrumented), TIMEOUT (a bounded device wait gave up), CUDA.
  */
 int fps_plan_kernel_times(fps_plan *plan, int *count, double *total_ms, double *alg_bytes);

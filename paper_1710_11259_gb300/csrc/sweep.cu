@@ -1,12 +1,10 @@
 // ADI pass kernels of the square solve (see sweep.cuh for the scheme and layout).
 //
-// Tiles travel through shared memory by bulk asynchronous copies (cp.async.bulk,
-// one copy per tile row, completion on an mbarrier; results leave by bulk stores),
-// so no thread spends registers or issue slots on address streams.  Inside a tile
-// every thread owns one line (a row in the row pass, a column in the column pass)
-// and keeps the whole segment of that line in registers: two interleaved
-// recurrences (even and odd positions, App. B) per thread, no shared-memory
-// traffic during the sweeps.
+// Tiles travel through shared memory by bulk asynchronous copies (cp.async.bulk, one
+// copy per S x S block, completion on an mbarrier; results leave by bulk stores), so no
+// thread spends registers or issue slots on address streams.  Inside a tile every
+// thread owns one line (a row in the row pass, a column in the column pass) and keeps
+// the forward values of its segment in registers.
 #include <cuda_runtime.h>
 
 #include "bulk.cuh"
@@ -17,18 +15,9 @@ namespace fps {
 
 namespace {
 
-constexpr int kR = 64;    // rows per row-pass tile
-constexpr int kC = 64;    // columns per column-pass tile
-constexpr int kRT = 128;  // row-pass threads: one per (row, parity of the column index)
-constexpr int kCT = 128;  // column-pass threads: one per (column, parity of the row index)
-constexpr int kChainLines = 64;
+constexpr int kL = kPassLines;  // lines of a tile = threads of a pass CTA
 
 // 16-byte chunks of T
-template <typename T>
-struct Ch {
-    static constexpr int V = 16 / sizeof(T);
-};
-
 template <typename T>
 __device__ __forceinline__ void ld16(const T *p, T (&v)[16 / sizeof(T)]);
 template <>
@@ -59,24 +48,6 @@ __device__ __forceinline__ void st16<double>(double *p, const double (&v)[2])
 {
     *reinterpret_cast<double2 *>(p) = make_double2(v[0], v[1]);
 }
-// four consecutive words (16-byte aligned) as one or two vector loads
-__device__ __forceinline__ void ld4(const float *p, float &a, float &b, float &c, float &d)
-{
-    const float4 f = *reinterpret_cast<const float4 *>(p);
-    a = f.x;
-    b = f.y;
-    c = f.z;
-    d = f.w;
-}
-__device__ __forceinline__ void ld4(const double *p, double &a, double &b, double &c, double &d)
-{
-    const double2 f = *reinterpret_cast<const double2 *>(p);
-    const double2 h = *reinterpret_cast<const double2 *>(p + 2);
-    a = f.x;
-    b = f.y;
-    c = h.x;
-    d = h.y;
-}
 
 template <typename T>
 __device__ __forceinline__ typename Vec2<T>::type mk2(T x, T y);
@@ -91,36 +62,30 @@ __device__ __forceinline__ double2 mk2<double>(double x, double y)
     return make_double2(x, y);
 }
 
-// Shared-memory row stride of the row-pass tile: S + 8 loaded columns plus padding
-// that makes the stride an odd number of 16-byte chunks (conflict-free 16-byte
-// accesses by threads that own consecutive rows).
-template <typename T, int S>
-struct RowGeom {
-    static constexpr int V = Ch<T>::V;
-    static constexpr int SW = S + 8 + V;
-    static_assert((SW * sizeof(T) / 16) % 2 == 1, "row stride must be an odd number of 16-byte chunks");
-    static constexpr size_t off_ct = 16;
-    static constexpr size_t off_zx = off_ct + sizeof(T) * (kR + 4) * SW;
-    static constexpr size_t off_frow = off_zx + sizeof(typename Vec2<T>::type) * 6 * (S + 8);
-    static constexpr size_t off_fcol = off_frow + sizeof(Fac<T>) * (kR + 4);
-    static constexpr size_t off_cf = off_fcol + sizeof(Fac<T>) * S;  // {cA, cB, cC, g} per column
-    static constexpr size_t bytes = off_cf + sizeof(T) * 4 * S;
-    static_assert(off_zx % 16 == 0 && off_frow % 16 == 0 && off_fcol % 16 == 0 && off_cf % 16 == 0, "alignment");
-};
+__host__ __device__ __forceinline__ int round4(int n) { return (n + 3) & ~3; }
 
+// Shared memory of a pass CTA: tile (and the tile of D), the solve tables of the
+// segment, the summary tables of the kL lines, and (fused recurrences) the segment
+// coefficients.
 template <typename T, int S>
-struct ColGeom {
-    static constexpr int ZS = S + 2;  // padded stride of the two parity rows of zx
-    static constexpr size_t off_tile = 16;
-    static constexpr size_t off_fac = off_tile + sizeof(T) * S * kC;
-    static constexpr size_t off_zx = off_fac + sizeof(Fac<T>) * S;
-    static constexpr size_t bytes = off_zx + sizeof(typename Vec2<T>::type) * 2 * ZS;
-    static_assert(off_fac % 16 == 0 && off_zx % 16 == 0, "alignment");
+struct Geo {
+    static constexpr int V = 16 / (int)sizeof(T);
+    static constexpr int B = S * S;       // elements of a block
+    static constexpr int CH = S / V;      // chunks of a row
+    static constexpr size_t off_tile = 128;
+    static constexpr size_t tile_bytes = sizeof(T) * kL * S;
+    static constexpr size_t tab_elems = 3 * S + 2 * kL + 3 * kMaxFused;
+    static constexpr size_t row_bytes = off_tile + tile_bytes + sizeof(T) * tab_elems;
+    static constexpr size_t col_bytes = off_tile + 2 * tile_bytes + sizeof(T) * tab_elems;
+    static constexpr size_t sum_bytes = row_bytes;
+    static_assert(CH >= 8, "the XOR permutation needs eight chunks per row");
 };
 
 // ---------------------------------------------------------------------------
 // Shift tables: one thread per (job, parity), FP64 arithmetic.
 // ---------------------------------------------------------------------------
+constexpr int kMaxS = 64;
+
 template <typename T>
 __global__ void fac_tables_kernel(const FacJob<T> *__restrict__ jobs, int njobs)
 {
@@ -128,44 +93,60 @@ __global__ void fac_tables_kernel(const FacJob<T> *__restrict__ jobs, int njobs)
     if (tid >= 2 * njobs) return;
     const FacJob<T> &jb = jobs[tid >> 1];
     const int p = tid & 1;
-    const int n = jb.n, N = jb.N, S = jb.S;
-    Fac<T> *out = jb.out + 2;  // position i at out[i]
-    // forward: pivots of the parity-p tridiagonal of A~ - qI, and phi within segments
-    double piv_prev = 1.0, phi = 1.0;
-    for (int i = p; i < N; i += 2) {
-        double ip = 0.0, g = 0.0, uf = 0.0;
-        if (i < n) {
-            const double em2 = (i >= 2) ? jb.e[i - 2] : 0.0;
-            double piv = jb.d[i] - jb.q;
-            if (i >= 2) piv -= em2 * em2 / piv_prev;
-            ip = 1.0 / piv;
-            g = em2 * ip;
-            uf = jb.e[i] * ip;
-            piv_prev = piv;
+    const int S = jb.S, nb = jb.nb, Mp = nb * S, m = (jb.n - p + 1) / 2, nbp = round4(nb);
+    const int64_t to = (int64_t)p * kTabs * Mp;
+    const double *d = jb.d + p, *e = jb.e + p;  // position i of this parity: index 2 i
+    // l_i = e_{i-1} ip_{i-1} and m_i = e_i ip_{i+1}; ip runs one position ahead
+    double ip = 0.0, ip_next = m > 0 ? 1.0 / (d[0] - jb.q) : 0.0;
+    double l_next = 0.0;
+    double lv[kMaxS], mv[kMaxS], v[kMaxS];
+    for (int s = 0; s < nb; ++s) {
+        for (int u = 0; u < S; ++u) {
+            const int i = s * S + u;
+            double l = 0.0, mm = 0.0;
+            ip = 0.0;
+            if (i < m) {
+                ip = ip_next;
+                l = l_next;
+                if (i + 1 < m) {
+                    const double ei = e[2 * i];
+                    l_next = ei * ip;
+                    ip_next = 1.0 / (d[2 * (i + 1)] - jb.q - ei * l_next);
+                    mm = ei * ip_next;
+                }
+            }
+            lv[u] = l;
+            mv[u] = mm;
+            v[u] = u == 0 ? 1.0 : v[u - 1] * -mv[u - 1];  // weight of w_i in y at the segment's start
+            for (int t = 0; t < 2; ++t) {
+                T *out = t == 0 ? jb.out1 : jb.out2;
+                if (!out) continue;
+                out[to + i] = (T)l;
+                out[to + Mp + i] = (T)mm;
+                out[to + 2 * Mp + i] = (T)((t == 0 ? jb.sc1 : jb.sc2) * ip);
+            }
         }
-        if ((i - p) % S == 0) phi = 1.0;  // first parity-p position of a segment
-        phi *= -g;
-        Fac<T> f;
-        f.ip = (T)ip;
-        f.g = (T)g;
-        f.uf = (T)uf;
-        f.phi = (T)phi;
-        f.Bv = 0;
-        f.Psi = 0;
-        out[i] = f;
-    }
-    // backward within each segment: Bv_i = phi_i - uf_i Bv_{i+2}, Psi_i = -uf_i Psi_{i+2}
-    double Bv = 0.0, Psi = 1.0;
-    for (int i = N - 2 + p; i >= p; i -= 2) {
-        if (i + 2 >= N || ((i + 2 - p) % S) == 0) {  // last parity-p position of its segment
-            Bv = 0.0;
-            Psi = 1.0;
+        double psi = 1.0, chi = 0.0;
+        for (int u = S - 1; u >= 0; --u) {
+            const int i = s * S + u;
+            if (u + 1 < S) psi *= -lv[u + 1];
+            chi = u + 1 < S ? v[u] - lv[u + 1] * chi : v[u];
+            const bool live = i < m;
+            for (int t = 0; t < 2; ++t) {
+                T *out = t == 0 ? jb.out1 : jb.out2;
+                if (!out) continue;
+                out[to + 3 * Mp + i] = live ? (T)psi : T(0);
+                out[to + 4 * Mp + i] = live ? (T)chi : T(0);
+            }
         }
-        const double uf = (double)out[i].uf;
-        Bv = (double)out[i].phi - uf * Bv;
-        Psi = -uf * Psi;
-        out[i].Bv = (T)Bv;
-        out[i].Psi = (T)Psi;
+        for (int t = 0; t < 2; ++t) {
+            T *ch = t == 0 ? jb.ch1 : jb.ch2;
+            if (!ch) continue;
+            ch += (int64_t)p * 3 * nbp;
+            ch[s] = (T)(-lv[0] * psi);
+            ch[nbp + s] = (T)(-lv[0] * chi);
+            ch[2 * nbp + s] = (T)(v[S - 1] * -mv[S - 1]);
+        }
     }
 }
 
@@ -179,383 +160,434 @@ __device__ __forceinline__ bool tile_ready(uint64_t *bar, int *err)
     return false;
 }
 
-// ---------------------------------------------------------------------------
-// Row pass.  Item {problem, rhs, row block (64 rows), column segment}.
-// MODE 0: j = 0, input rho_0.  MODE 1: j = 1, D = -2 q_0 c_0.  MODE 2: D -= 2 q_{j-1} c_{j-1}.
-// W: columns of this tile's segment (S, or 64 for a short last segment).
-// ---------------------------------------------------------------------------
-template <typename T, int S, int MODE, int W>
-__device__ __forceinline__ void row_pass_tile(const SwArgs<T> &a, int j, const int4 it, const SwProb<T> &pr,
-                                              unsigned char *smem)
+// The launches of a solve form one dependent chain; programmatic dependent launch lets
+// the next kernel's CTAs start while the last CTAs of this one run.  pdl_wait() returns
+// when every earlier kernel has completed; nothing that those write is read before it.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
+// Start of a pass CTA: the item, and whether there is work (mask of active problems, J,
+// an error anywhere).  Initialises `nbar` barriers; ends with a CTA barrier.
+template <typename T>
+__device__ __forceinline__ bool pass_begin(const SwArgs<T> &a, const SwItem<T> &it, int j, uint64_t *bar, int nbar)
 {
-    using G = RowGeom<T, S>;
-    using T2 = typename Vec2<T>::type;
-    constexpr int V = G::V, SW = G::SW;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
-    T *ct = reinterpret_cast<T *>(smem + G::off_ct);
-    T2 *zx = reinterpret_cast<T2 *>(smem + G::off_zx);
-    Fac<T> *frow = reinterpret_cast<Fac<T> *>(smem + G::off_frow);
-    Fac<T> *fcol = reinterpret_cast<Fac<T> *>(smem + G::off_fcol);
-    T *cf = reinterpret_cast<T *>(smem + G::off_cf);
-
-    const int tid = threadIdx.x;
-    const int N = pr.N, ldp = pr.ldp;
-    const int i0 = it.z * kR, cs = it.w, k0 = cs * S;
-    const int64_t base = pr.off + (int64_t)it.y * pr.rhs;
-    const T *src = (MODE == 0 ? a.rho0 : a.cl) + base;
-    T *Dp = a.D + base;
-    T *alp = a.al + base;
-    const int64_t sbase = pr.soff + (int64_t)it.y * pr.srhs;
-    const Fac<T> *facj = pr.facR + (int64_t)j * (N + 4);                      // this row solve
-    const Fac<T> *facp = pr.facC + (int64_t)(MODE > 0 ? j - 1 : 0) * (N + 4);  // previous column solve
-    const T sL = MODE > 0 ? pr.sh[3 * (j - 1)] : T(0);      // column-stencil shift of iteration j-1
-    const T sR = MODE > 0 ? pr.sh[3 * (j - 1) + 1] : T(0);  // row-stencil shift
-    const T fD = MODE > 0 ? pr.sh[3 * (j - 1) + 2] : T(0);  // correction factor
-
-    // column segments of the halo rows (row systems of the previous column pass)
-    const int sc = i0 / S, segstart = sc * S, segend = min(segstart + S, N);
-    const int s_above = (MODE > 0 && i0 == segstart && i0 > 0) ? sc - 1 : -1;
-    const int s_below = (MODE > 0 && i0 + kR == segend && segend < N) ? sc + 1 : -1;
-    constexpr int rows_ld = MODE == 0 ? kR : kR + 4;
-    constexpr int cw = MODE == 0 ? W : W + 8;  // loaded columns
-    const int row0 = MODE == 0 ? i0 : i0 - 2;  // first global row loaded
-    constexpr int smr0 = MODE == 0 ? 2 : 0;    // its shared-memory row
-    const int kc0 = MODE == 0 ? k0 : k0 - 4;   // first loaded column
-    constexpr int scc0 = MODE == 0 ? 4 : 0;    // its shared-memory column
-
-    if (tid == 0) {
-        bulk::mbar_init(bar, 1);
+    const bool in_range = j < it.J;
+    pdl_wait();
+    const int masked = *a.masked;
+    const bool act = in_range && (!masked || a.active[it.prob]);
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < nbar; ++b) bulk::mbar_init(bar + b, 1);
         bulk::fence_mbar_init();
     }
-    __syncthreads();
-    if (tid == 0) {
-        unsigned bytes = (unsigned)(rows_ld * cw * sizeof(T) + W * sizeof(Fac<T>));
-        if (MODE > 0)
-            bytes += (unsigned)((kR + 4) * sizeof(Fac<T>) +
-                                2 * cw * sizeof(T2) * (1 + (s_above >= 0) + (s_below >= 0)));
-        bulk::mbar_arrive_expect_tx(bar, bytes);
-    }
-    __syncthreads();
-    for (int r = tid; r < rows_ld; r += kRT)
-        bulk::g2s(ct + (smr0 + r) * SW + scc0, src + (int64_t)(row0 + r + 2) * ldp + (kc0 + 4),
-                  (unsigned)(cw * sizeof(T)), bar);
-    if (tid == kRT - 1) bulk::g2s(fcol, facj + k0 + 2, (unsigned)(W * sizeof(Fac<T>)), bar);
-    if (MODE > 0) {
-        if (tid == kRT - 2) bulk::g2s(frow, facp + i0, (unsigned)((kR + 4) * sizeof(Fac<T>)), bar);
-        if (tid >= kRT - 8 && tid < kRT - 2) {
-            const int k = tid - (kRT - 8), slot = k >> 1, par = k & 1;
-            const int sg = slot == 0 ? s_above : (slot == 1 ? sc : s_below);
-            if (sg >= 0)
-                bulk::g2s(zx + (slot * 2 + par) * (S + 8), a.zxC + sbase + ((int64_t)sg * 2 + par) * (N + 8) + k0,
-                          (unsigned)(cw * sizeof(T2)), bar);
-        }
-    }
-    // D of the tile's core into registers while the tile is in flight: thread t owns
-    // chunk t % CPR of rows t / CPR + m * (kRT / CPR) (coalesced 16-byte loads)
-    constexpr int CPR = W / V;
-    constexpr int DSTEP = kRT / CPR;
-    constexpr int NDC = kR / DSTEP;  // chunks per thread
-    const int dr0 = tid / CPR, dc = tid % CPR;
-    T dreg[NDC][V];
-    if (MODE == 2) {
-#pragma unroll
-        for (int m = 0; m < NDC; ++m)
-            ld16(Dp + (int64_t)(i0 + dr0 + m * DSTEP + 2) * ldp + (k0 + 4 + dc * V), dreg[m]);
-    }
-    if (!tile_ready(bar, a.err)) return;
-
-    // per-column records {ip e_{k-2}, ip (d_k + q), ip e_k, g} of the ip-scaled row stencil
-    for (int c = tid; c < W; c += kRT) {
-        const int k = k0 + c;
-        const T ipk = fcol[c].ip;
-        if (MODE > 0) {
-            cf[4 * c + 0] = ipk * pr.e[k];
-            cf[4 * c + 1] = ipk * (pr.d[k + 2] + sR);
-            cf[4 * c + 2] = ipk * pr.e[k + 2];
-        } else {
-            cf[4 * c + 0] = T(0);
-            cf[4 * c + 1] = ipk;
-            cf[4 * c + 2] = T(0);
-        }
-        cf[4 * c + 3] = fcol[c].g;
-    }
-    if (MODE > 0) {
-        // rebuild c_{j-1} = cl + Bv zin + Psi xout on the whole loaded tile
-        constexpr int cpr = cw / V;
-        constexpr int total = (kR + 4) * cpr;
-        for (int idx = tid; idx < total; idx += kRT) {
-            const int r = idx / cpr, cc = (idx - r * cpr) * V;
-            const int i = i0 - 2 + r;
-            if (i >= 0 && i < N) {
-                T *cp = ct + r * SW + cc;
-                T v[V];
-                ld16(cp, v);
-                const int slot = i < segstart ? 0 : (i >= segend ? 2 : 1);
-                const T2 *z = zx + (slot * 2 + (i & 1)) * (S + 8) + cc;
-                const T bv = frow[r].Bv, ps = frow[r].Psi;
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    const T2 zz = z[e];
-                    v[e] = fma(bv, zz.x, fma(ps, zz.y, v[e]));
-                }
-                st16(cp, v);
-            }
-        }
-        __syncthreads();
-        // D -= 2 q_{j-1} c_{j-1} on the core (D = -2 q_0 c_0 at j = 1)
-
-#pragma unroll
-        for (int m = 0; m < NDC; ++m) {
-            const int rr = dr0 + m * DSTEP;
-            T v[V], dv[V];
-            ld16(ct + (rr + 2) * SW + 4 + dc * V, v);
-#pragma unroll
-            for (int e = 0; e < V; ++e) dv[e] = MODE == 1 ? fD * v[e] : fma(fD, v[e], dreg[m][e]);
-            st16(Dp + (int64_t)(i0 + rr + 2) * ldp + (k0 + 4 + dc * V), dv);
-        }
-    }
-    __syncthreads();
-
-    // one thread per (row, parity of the column index): a warp holds 16 rows x 2 parities
-    const int lane = tid & 31;
-    const int rr = (tid >> 5) * 16 + (lane & 15), p = lane >> 4;
-    const int r = rr + 2, i = i0 + rr;
-    T wr[W / 2];
-    T we;
-    {
-        T w = 0;
-        if (MODE == 0) {
-#pragma unroll
-            for (int t = 0; t < W / 2; ++t) {
-                const int c = 2 * t + p;
-                const T rho = cf[4 * c + 1] * ct[r * SW + 4 + c];
-                w = fma(-cf[4 * c + 3], w, rho);
-                wr[t] = w;
-            }
-        } else {
-            // rho = ip (R + q)(L + q) c: column stencil u = (L + q) c, then the row stencil
-            const T eu = pr.e[i], dq = pr.d[i + 2] + sL, ed = pr.e[i + 2];
-            const T *r0 = ct + (r - 2) * SW + 4, *r1 = ct + r * SW + 4, *r2 = ct + (r + 2) * SW + 4;
-            auto u = [&](int x) { return fma(eu, r0[x], fma(dq, r1[x], ed * r2[x])); };
-            T um = u(p - 2), u0 = u(p);
-#pragma unroll
-            for (int t = 0; t < W / 2; ++t) {
-                const int c = 2 * t + p;
-                const T up = u(c + 2);
-                T cA, cB, cC, g;
-                ld4(cf + 4 * c, cA, cB, cC, g);
-                const T rho = fma(cA, um, fma(cB, u0, cC * up));
-                w = fma(-g, w, rho);
-                wr[t] = w;
-                um = u0;
-                u0 = up;
-            }
-        }
-        we = w;
-    }
-    {
-        T x = 0;  // local back substitution: zero beyond the segment
-#pragma unroll
-        for (int t = W / 2 - 1; t >= 0; --t) {
-            x = fma(-fcol[2 * t + p].uf, x, wr[t]);
-            wr[t] = x;
-        }
-    }
-    const bool live = i < pr.n;
-    __syncthreads();  // every thread is done reading the tile
-#pragma unroll
-    for (int t = 0; t < W / 2; ++t) ct[r * SW + 4 + 2 * t + p] = live ? wr[t] : T(0);
-    a.sumR[sbase + ((int64_t)cs * 2 + p) * (N + 8) + i + 4] = mk2<T>(live ? we : T(0), live ? wr[0] : T(0));
-    bulk::fence_proxy_async_shared();
-    __syncthreads();
-    if (tid < kR)
-        bulk::s2g(alp + (int64_t)(i0 + tid + 2) * ldp + (k0 + 4), ct + (tid + 2) * SW + 4, (unsigned)(W * sizeof(T)));
-    bulk::commit();
-    bulk::wait_read_all();
-}
-
-template <typename T, int S, int MODE>
-__global__ void __launch_bounds__(kRT, 3) row_pass_kernel(SwArgs<T> a, int j)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int4 it = a.items[blockIdx.x];
-    const SwProb<T> &pr = a.probs[it.x];
-    if (!a.active[it.x] || j >= pr.J) return;
     // after a timeout anywhere, leave at once (one read, agreed on by the whole CTA)
-    if (__syncthreads_or(threadIdx.x == 0 ? *(volatile int *)a.err : 0)) return;
-    if (S == kR || pr.N - it.w * S >= S) row_pass_tile<T, S, MODE, S>(a, j, it, pr, smem);
-    else row_pass_tile<T, S, MODE, kR>(a, j, it, pr, smem);
+    const int stop = __syncthreads_or(threadIdx.x == 0 ? *(volatile int *)a.err : 0);
+    return act && !stop;
 }
 
+// zin and yout of segment s of one line from the summaries of all its segments
+// (sum: segment 0 of the line, `step` apart); co: phi, Bv, Psi of nbp entries each.
+template <typename T>
+struct LineSums {
+    typename Vec2<T>::type v[kMaxFused];
+    __device__ __forceinline__ void load(const typename Vec2<T>::type *__restrict__ sum, int64_t step, int P)
+    {
+#pragma unroll
+        for (int s = 0; s < kMaxFused; ++s)
+            if (s < P) v[s] = sum[s * step];
+    }
+    __device__ __forceinline__ void run(const T *co, int nbp, int P, int seg, T &zin, T &yout) const
+    {
+        T z[kMaxFused];
+        T W = 0;
+#pragma unroll
+        for (int s = 0; s < kMaxFused; ++s)
+            if (s < P) {
+                z[s] = W;
+                if (s == seg) zin = W;
+                W = fma(co[s], W, v[s].x);
+            }
+        T Y = 0;
+#pragma unroll
+        for (int s = kMaxFused - 1; s >= 0; --s)
+            if (s < P) {
+                if (s == seg) yout = Y;
+                Y = fma(co[nbp + s], z[s], fma(co[2 * nbp + s], Y, v[s].y));
+            }
+    }
+};
+
 // ---------------------------------------------------------------------------
-// Column pass.  Item {problem, rhs, column block (64 columns), row segment}.
-// H: rows of this tile's segment (S, or 64 for a short last segment).
+// Row pass.  A tile is n_blk blocks of one block column: up to 128 rows x S columns.
+// FIRST: j = 0 (a = v).
 // ---------------------------------------------------------------------------
-template <typename T, int S, int H>
-__device__ __forceinline__ void col_pass_tile(const SwArgs<T> &a, int j, const int4 it, const SwProb<T> &pr,
-                                              unsigned char *smem)
+template <typename T, int S, bool FIRST, bool FUSED>
+__global__ void __launch_bounds__(kL, sizeof(T) == 4 ? 4 : 3) row_pass_kernel(SwArgs<T> A, int j)
 {
-    using G = ColGeom<T, S>;
+    using G = Geo<T, S>;
     using T2 = typename Vec2<T>::type;
+    constexpr int V = G::V;
+    extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
     T *tile = reinterpret_cast<T *>(smem + G::off_tile);
-    Fac<T> *fac = reinterpret_cast<Fac<T> *>(smem + G::off_fac);
-    T2 *zx = reinterpret_cast<T2 *>(smem + G::off_zx);
-
+    T *tl = tile + kL * S, *tm = tl + S, *ts = tm + S, *psi = ts + S, *chi = psi + kL, *co = chi + kL;
     const int tid = threadIdx.x;
-    const int N = pr.N, ldp = pr.ldp;
-    const int k0 = it.z * kC, rs = it.w, i0 = rs * S;
-    const int cs = k0 / S;  // row-system segment holding these columns
-    const int64_t base = pr.off + (int64_t)it.y * pr.rhs;
-    const int64_t sbase = pr.soff + (int64_t)it.y * pr.srhs;
-    const Fac<T> *facj = pr.facC + (int64_t)j * (N + 4);  // this column solve
-    const Fac<T> *facr = pr.facR + (int64_t)j * (N + 4);  // the row solve whose result is rebuilt
-
+    pdl_launch();
+    const SwItem<T> it = A.items[blockIdx.x];
+    if (!pass_begin(A, it, j, bar, 1)) return;
+    const int nb = it.nb, bi0 = it.b0, bk = it.b1, nblk = it.n_blk, Mp = nb * S, nbp = round4(nb);
+    T *X = A.X + it.xoff;
+    const int64_t bstride = (int64_t)nb * G::B;  // blocks of the tile are one block row apart
     if (tid == 0) {
-        bulk::mbar_init(bar, 1);
-        bulk::fence_mbar_init();
+        const T *tR = it.tabR + (int64_t)j * (2 * kTabs) * Mp + bk * S;
+        const T *tC = it.tabC + (int64_t)j * (2 * kTabs) * Mp + bi0 * S;
+        const unsigned tb = (unsigned)(S * sizeof(T)), pb = (unsigned)(nblk * S * sizeof(T));
+        unsigned total = (unsigned)(nblk * G::B * sizeof(T)) + 3 * tb + 2 * pb;
+        if (FUSED) total += (unsigned)(3 * nbp * sizeof(T));
+        bulk::mbar_arrive_expect_tx(bar, total);
+        for (int b = 0; b < nblk; ++b)
+            bulk::g2s(tile + b * G::B, X + b * bstride, (unsigned)(G::B * sizeof(T)), bar);
+        bulk::g2s(tl, tR, tb, bar);
+        bulk::g2s(tm, tR + Mp, tb, bar);
+        bulk::g2s(ts, tR + 2 * Mp, tb, bar);
+        bulk::g2s(psi, tC + 3 * Mp, pb, bar);
+        bulk::g2s(chi, tC + 4 * Mp, pb, bar);
+        if (FUSED) bulk::g2s(co, it.chR + (int64_t)j * 6 * nbp, (unsigned)(3 * nbp * sizeof(T)), bar);
     }
-    __syncthreads();
-    if (tid == 0)
-        bulk::mbar_arrive_expect_tx(bar, (unsigned)(H * kC * sizeof(T) + H * sizeof(Fac<T>) + 2 * H * sizeof(T2)));
-    __syncthreads();
-    for (int r = tid; r < H; r += kCT)
-        bulk::g2s(tile + r * kC, a.al + base + (int64_t)(i0 + r + 2) * ldp + (k0 + 4), (unsigned)(kC * sizeof(T)), bar);
-    if (tid == kCT - 1) bulk::g2s(fac, facj + i0 + 2, (unsigned)(H * sizeof(Fac<T>)), bar);
-    if (tid == kCT - 2 || tid == kCT - 3) {
-        const int par = kCT - 2 - tid;
-        bulk::g2s(zx + par * G::ZS, a.zxR + sbase + ((int64_t)cs * 2 + par) * (N + 8) + i0 + 4,
-                  (unsigned)(H * sizeof(T2)), bar);
-    }
-    // one thread per (column, parity of the row index)
-    const int kk = tid % kC, p = tid / kC;
-    const int k = k0 + kk;
-    const T bv = facr[k + 2].Bv, ps = facr[k + 2].Psi;
-    const T2 *zp = zx + (k & 1) * G::ZS;
-    if (!tile_ready(bar, a.err)) return;
-
-    // forward sweep and back substitution in place in the tile (own column, own parity)
-    const bool live = k < pr.n;
-    T we, x = 0;
-    {
-        T w = 0;
-#pragma unroll 8
-        for (int t = 0; t < H / 2; ++t) {
-            const int r = 2 * t + p;
-            const T2 z = zp[r];
-            const T av = fma(bv, z.x, fma(ps, z.y, tile[r * kC + kk]));
-            T ip, g, uf, phi;
-            ld4(&fac[r].ip, ip, g, uf, phi);
-            w = fma(-g, w, ip * av);
-            tile[r * kC + kk] = w;
+    const int b = tid / S, r = tid % S;
+    const bool on = b < nblk;
+    const int64_t line = it.soff + bi0 * S + tid;
+    T zin = 0, yout = 0;
+    LineSums<T> sums;
+    if (on) {
+        if (FUSED) {
+            sums.load(A.sumR + line, Mp, nb);
+        } else {
+            const T2 z = A.zxR[line + (int64_t)bk * Mp];
+            zin = z.x;
+            yout = z.y;
         }
-        we = w;
     }
-#pragma unroll 8
-    for (int t = H / 2 - 1; t >= 0; --t) {
-        const int r = 2 * t + p;
-        x = fma(-fac[r].uf, x, tile[r * kC + kk]);
-        tile[r * kC + kk] = live ? x : T(0);
+    if (!tile_ready(bar, A.err)) return;
+    if (on) {
+        if (FUSED) sums.run(co, nbp, nb, bk, zin, yout);
+        T *row = tile + b * G::B + r * S;
+        int sw[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) sw[q] = (q ^ (r & 7)) * V;
+        T w[S];
+        T z = zin;
+#pragma unroll
+        for (int c = 0; c < G::CH; ++c) {
+            T u[V], l[V];
+            ld16(row + (c / 8) * 8 * V + sw[c % 8], u);
+            ld16(tl + c * V, l);
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                z = fma(-l[e], z, u[e]);
+                w[c * V + e] = z;
+            }
+        }
+        T y = yout;
+#pragma unroll
+        for (int c = G::CH - 1; c >= 0; --c) {
+            T u[V], m[V], s[V];
+            T *pc = row + (c / 8) * 8 * V + sw[c % 8];
+            if (!FIRST) ld16(pc, u);
+            ld16(tm + c * V, m);
+            ld16(ts + c * V, s);
+#pragma unroll
+            for (int e = V - 1; e >= 0; --e) {
+                y = fma(-m[e], y, w[c * V + e]);
+                u[e] = FIRST ? s[e] * y : fma(s[e], y, u[e]);
+            }
+            st16(pc, u);
+        }
     }
-    a.sumC[sbase + ((int64_t)rs * 2 + p) * (N + 8) + k + 4] = mk2<T>(live ? we : T(0), live ? x : T(0));
     bulk::fence_proxy_async_shared();
     __syncthreads();
-    for (int r = tid; r < H; r += kCT)
-        bulk::s2g(a.cl + base + (int64_t)(i0 + r + 2) * ldp + (k0 + 4), tile + r * kC, (unsigned)(kC * sizeof(T)));
-    bulk::commit();
-    bulk::wait_read_all();
+    if (tid == 0) {
+        for (int q = 0; q < nblk; ++q)
+            bulk::s2g(X + q * bstride, tile + q * G::B, (unsigned)(G::B * sizeof(T)));
+        bulk::commit();
+    }
+    // summaries of the column solve: thread = (column c, block g)
+    {
+        const int g = tid / S, c = tid % S;
+        if (g < nblk) {
+            const T *col = tile + g * G::B + c % V;
+            int sw[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) sw[q] = ((c / V) ^ q) * V + q * S;
+            T wl[2] = {0, 0}, yl[2] = {0, 0};
+#pragma unroll
+            for (int r0 = 0; r0 < S; r0 += V) {
+                T ps[V], ch[V];
+                ld16(psi + g * S + r0, ps);
+                ld16(chi + g * S + r0, ch);
+#pragma unroll
+                for (int e = 0; e < V; ++e) {
+                    const int rr = r0 + e;
+                    const T x = col[(rr / 8) * 8 * S + sw[rr % 8]];
+                    wl[e & 1] = fma(ps[e], x, wl[e & 1]);
+                    yl[e & 1] = fma(ch[e], x, yl[e & 1]);
+                }
+            }
+            A.sumC[it.soff + (int64_t)(bi0 + g) * Mp + bk * S + c] = mk2<T>(wl[0] + wl[1], yl[0] + yl[1]);
+        }
+    }
+    if (tid == 0) bulk::wait_read_all();
 }
 
+// Summaries of the row solve with tables tR (psi, chi staged in shared memory for the
+// tile's columns): thread = (row r, block g).
 template <typename T, int S>
-__global__ void __launch_bounds__(kCT) col_pass_kernel(SwArgs<T> a, int j)
+__device__ __forceinline__ void row_summaries(const SwArgs<T> &A, const SwItem<T> &it, const T *tile, const T *psi,
+                                              const T *chi)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int4 it = a.items[blockIdx.x];
-    const SwProb<T> &pr = a.probs[it.x];
-    if (!a.active[it.x] || j >= pr.J) return;
-    if (__syncthreads_or(threadIdx.x == 0 ? *(volatile int *)a.err : 0)) return;
-    if (S == kC || pr.N - it.w * S >= S) col_pass_tile<T, S, S>(a, j, it, pr, smem);
-    else col_pass_tile<T, S, kC>(a, j, it, pr, smem);
+    using G = Geo<T, S>;
+    constexpr int V = G::V;
+    const int g = threadIdx.x / S, r = threadIdx.x % S;
+    if (g >= it.n_blk) return;
+    const T *row = tile + g * G::B + r * S;
+    int sw[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sw[q] = (q ^ (r & 7)) * V;
+    T wl[2] = {0, 0}, yl[2] = {0, 0};
+#pragma unroll
+    for (int c = 0; c < G::CH; ++c) {
+        T x[V], ps[V], ch[V];
+        ld16(row + (c / 8) * 8 * V + sw[c % 8], x);
+        ld16(psi + g * S + c * V, ps);
+        ld16(chi + g * S + c * V, ch);
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            wl[e & 1] = fma(ps[e], x[e], wl[e & 1]);
+            yl[e & 1] = fma(ch[e], x[e], yl[e & 1]);
+        }
+    }
+    const int Mp = it.nb * S;
+    A.sumR[it.soff + (int64_t)(it.b1 + g) * Mp + it.b0 * S + r] = mk2<T>(wl[0] + wl[1], yl[0] + yl[1]);
 }
 
 // ---------------------------------------------------------------------------
-// Chains: true forward value entering and true solution leaving every segment.
-// Item {problem, rhs, block of 64 lines}; thread = (line, parity).
-//   W_s = wl_end(s) + phi_end(s) W_{s-1},           zin(s)  = W_{s-1}
-//   X_s = xl_start(s) + Bv_start(s) zin(s) + Psi_start(s) X_{s+1},   xout(s) = X_{s+1}
+// Column pass.  A tile is n_blk blocks of one block row: S rows x up to 128 columns.
+// FIRST: j = 0 (D written, not read).  In the last iteration of a problem u and the
+// summaries are not needed.
 // ---------------------------------------------------------------------------
-// BIG: long load batches (fewer dependent round trips to L2, more registers) for
-// grids of a few CTAs per SM, where latency is all; short ones keep occupancy when
-// the grid fills the GPU (batches of many problems).
-template <typename T, bool BIG>
-__global__ void __launch_bounds__(2 * kChainLines) chain_kernel(SwArgs<T> a, int dir, int j)
+template <typename T, int S, bool FIRST, bool FUSED>
+__global__ void __launch_bounds__(kL, 3) col_pass_kernel(SwArgs<T> A, int j)
+{
+    using G = Geo<T, S>;
+    using T2 = typename Vec2<T>::type;
+    constexpr int V = G::V;
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
+    T *tile = reinterpret_cast<T *>(smem + G::off_tile), *dt = tile + kL * S;
+    T *tl = dt + kL * S, *tm = tl + S, *ts = tm + S, *psi = ts + S, *chi = psi + kL, *co = chi + kL;
+    const int tid = threadIdx.x;
+    pdl_launch();
+    // tiles in the reverse order of the row pass: those it wrote last are still in L2
+    const SwItem<T> it = A.items[gridDim.x - 1 - blockIdx.x];
+    if (!pass_begin(A, it, j, bar, 2)) return;
+    const int nb = it.nb, bi = it.b0, bk0 = it.b1, nblk = it.n_blk, Mp = nb * S, nbp = round4(nb);
+    const bool last = j + 1 == it.J;
+    T *X = A.X + it.xoff, *D = A.D + it.xoff;
+    const unsigned xb = (unsigned)(nblk * G::B * sizeof(T));  // the blocks of the tile are adjacent
+    if (tid == 0) {
+        const T *tC = it.tabC + (int64_t)j * (2 * kTabs) * Mp + bi * S;
+        const unsigned tb = (unsigned)(S * sizeof(T)), pb = (unsigned)(nblk * S * sizeof(T));
+        bulk::mbar_arrive_expect_tx(bar, xb + 3 * tb + (FUSED ? (unsigned)(3 * nbp * sizeof(T)) : 0u));
+        bulk::g2s(tile, X, xb, bar);
+        bulk::g2s(tl, tC, tb, bar);
+        bulk::g2s(tm, tC + Mp, tb, bar);
+        bulk::g2s(ts, tC + 2 * Mp, tb, bar);
+        if (FUSED) bulk::g2s(co, it.chC + (int64_t)j * 6 * nbp, (unsigned)(3 * nbp * sizeof(T)), bar);
+        const unsigned second = (FIRST ? 0u : xb) + (last ? 0u : 2 * pb);
+        if (second) bulk::mbar_arrive_expect_tx(bar + 1, second);
+        if (!FIRST) bulk::g2s(dt, D, xb, bar + 1);
+        if (!last) {
+            const T *tR = it.tabR + (int64_t)(j + 1) * (2 * kTabs) * Mp + bk0 * S;
+            bulk::g2s(psi, tR + 3 * Mp, pb, bar + 1);
+            bulk::g2s(chi, tR + 4 * Mp, pb, bar + 1);
+        }
+    }
+    const int b = tid / S, c = tid % S;
+    const bool on = b < nblk;
+    const int64_t line = it.soff + bk0 * S + tid;
+    T zin = 0, yout = 0;
+    LineSums<T> sums;
+    if (on) {
+        if (FUSED) {
+            sums.load(A.sumC + line, Mp, nb);
+        } else {
+            const T2 z = A.zxC[line + (int64_t)bi * Mp];
+            zin = z.x;
+            yout = z.y;
+        }
+    }
+    if (!tile_ready(bar, A.err)) {
+        if (!FIRST || !last) bulk::mbar_wait_bounded(bar + 1, 0);
+        return;
+    }
+    if (FUSED && on) sums.run(co, nbp, nb, bi, zin, yout);
+    int sw[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) sw[q] = ((c / V) ^ q) * V + q * S + c % V;
+    T w[S];
+    if (on) {
+        const T *col = tile + b * G::B;
+        T z = zin;
+#pragma unroll
+        for (int r0 = 0; r0 < S; r0 += V) {
+            T l[V];
+            ld16(tl + r0, l);
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                const int r = r0 + e;
+                z = fma(-l[e], z, col[(r / 8) * 8 * S + sw[r % 8]]);
+                w[r] = z;
+            }
+        }
+    }
+    if (!FIRST || !last) {
+        if (!tile_ready(bar + 1, A.err)) return;
+    }
+    if (on) {
+        T *col = tile + b * G::B, *dcol = dt + b * G::B;
+        T y = yout;
+#pragma unroll
+        for (int r0 = S - V; r0 >= 0; r0 -= V) {
+            T m[V], s[V];
+            ld16(tm + r0, m);
+            ld16(ts + r0, s);
+#pragma unroll
+            for (int e = V - 1; e >= 0; --e) {
+                const int r = r0 + e, o = (r / 8) * 8 * S + sw[r % 8];
+                y = fma(-m[e], y, w[r]);
+                col[o] = fma(s[e], y, col[o]);
+                dcol[o] = FIRST ? s[e] * y : fma(s[e], y, dcol[o]);
+            }
+        }
+    }
+    bulk::fence_proxy_async_shared();
+    __syncthreads();
+    if (tid == 0) {
+        if (!last) bulk::s2g(X, tile, xb);
+        bulk::s2g(D, dt, xb);
+        bulk::commit();
+    }
+    if (!last) row_summaries<T, S>(A, it, tile, psi, chi);
+    if (tid == 0) bulk::wait_read_all();
+}
+
+// Summaries of the row solve of iteration 0 (items of the column pass).
+template <typename T, int S>
+__global__ void __launch_bounds__(kL) row_sums_kernel(SwArgs<T> A)
+{
+    using G = Geo<T, S>;
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
+    T *tile = reinterpret_cast<T *>(smem + G::off_tile);
+    T *psi = tile + kL * S, *chi = psi + kL;
+    pdl_launch();
+    const SwItem<T> it = A.items[blockIdx.x];
+    if (!pass_begin(A, it, 0, bar, 1)) return;
+    const int Mp = it.nb * S;
+    if (threadIdx.x == 0) {
+        const T *tR = it.tabR + it.b1 * S;
+        const unsigned xb = (unsigned)(it.n_blk * G::B * sizeof(T)), pb = (unsigned)(it.n_blk * S * sizeof(T));
+        bulk::mbar_arrive_expect_tx(bar, xb + 2 * pb);
+        bulk::g2s(tile, A.X + it.xoff, xb, bar);
+        bulk::g2s(psi, tR + 3 * Mp, pb, bar);
+        bulk::g2s(chi, tR + 4 * Mp, pb, bar);
+    }
+    if (!tile_ready(bar, A.err)) return;
+    row_summaries<T, S>(A, it, tile, psi, chi);
+}
+
+// ---------------------------------------------------------------------------
+// Segment recurrences of 32 lines, latency bound.  Warp g owns LEN consecutive segments of every line
+// (lane = line): it composes their affine maps W -> alpha W + beta from the summaries in
+// registers, the warps' maps are composed through shared memory, and the true values
+// follow from one more walk; then the same backwards.  The summaries are read once
+// (n = 10^4, FP32: 10 us a launch; one thread walking all segments of a line took 16).
+// Lines of at most kMaxFused segments have no launch at all: every pass CTA walks its
+// lines' summaries while its tile is in flight (n = 1000: 72 + 72 launches of 7 us less).
+// ---------------------------------------------------------------------------
+template <typename T, int LEN>
+__global__ void chain_kernel(SwArgs<T> A, int dir, int j)
 {
     using T2 = typename Vec2<T>::type;
-    // segments whose loads are issued together (forward: 2 values, backward: 4 values
-    // per segment); each batch is one dependent round trip to L2
-    constexpr int B = BIG ? (sizeof(T) == 4 ? 40 : 20) : 16, B2 = BIG ? (sizeof(T) == 4 ? 24 : 12) : 16;
-    const int4 it = a.items[blockIdx.x];
-    const SwProb<T> &pr = a.probs[it.x];
-    if (!a.active[it.x] || j >= pr.J) return;
-    const int p = threadIdx.x / kChainLines;
-    const int l = it.z * kChainLines + (threadIdx.x % kChainLines);
-    const int N = pr.N, S = pr.S, P = pr.P;
-    if (l >= N) return;
-    const int64_t sbase = pr.soff + (int64_t)it.y * pr.srhs;
-    const T2 *__restrict__ sum = (dir == 0 ? a.sumR : a.sumC) + sbase + p * (N + 8) + l + 4;
-    T2 *__restrict__ zx = (dir == 0 ? a.zxR : a.zxC) + sbase + p * (N + 8) + l + 4;
-    T *__restrict__ zs = a.zin + sbase + p * (N + 8) + l + 4;
-    const int64_t step = 2 * (int64_t)(N + 8);  // next segment, same parity and line
-    const Fac<T> *__restrict__ facj = (dir == 0 ? pr.facR : pr.facC) + (int64_t)j * (N + 4) + 2;
+    __shared__ T beta[2][32][32];
+    __shared__ T alpha[2][32];
+    pdl_launch();
+    const SwItem<T> it = A.items[blockIdx.x];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, G = blockDim.x >> 5;
+    const int P = it.nb, nbp = round4(P), Mp = P * A.S;
+    const T *co = (dir == 0 ? it.chR : it.chC) + (int64_t)j * 6 * nbp;
+    const int s0 = g * LEN;
+    const bool in_range = j < it.J;
+    T phi[LEN], bv[LEN], ps[LEN];
+#pragma unroll
+    for (int b = 0; b < LEN; ++b) {  // tables of the plan: no launch of this solve writes them
+        const bool ok = in_range && s0 + b < P;
+        phi[b] = ok ? co[s0 + b] : T(0);
+        bv[b] = ok ? co[nbp + s0 + b] : T(0);
+        ps[b] = ok ? co[2 * nbp + s0 + b] : T(0);
+    }
+    pdl_wait();
+    if (!in_range || (*A.masked && !A.active[it.prob])) return;
+    const int64_t line = it.soff + it.b1 * 32 + lane;
+    const T2 *__restrict__ sum = (dir == 0 ? A.sumR : A.sumC) + line;
+    T2 *__restrict__ zx = (dir == 0 ? A.zxR : A.zxC) + line;
+    T2 v[LEN];
+#pragma unroll
+    for (int b = 0; b < LEN; ++b) v[b] = s0 + b < P ? sum[(int64_t)(s0 + b) * Mp] : mk2<T>(T(0), T(0));
+    T al = 1, be = 0;
+#pragma unroll
+    for (int b = 0; b < LEN; ++b) {
+        be = fma(phi[b], be, v[b].x);
+        al *= phi[b];
+    }
+    beta[0][g][lane] = be;
+    if (lane == 0) alpha[0][g] = al;
+    __syncthreads();
     T W = 0;
-    for (int s0 = 0; s0 < P; s0 += B) {
-        T sx[B], ph[B];
+    for (int h = 0; h < g; ++h) W = fma(alpha[0][h], W, beta[0][h][lane]);
+    T z[LEN];
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const int s = s0 + b;
-            if (s < P) {
-                sx[b] = sum[s * step].x;
-                ph[b] = facj[min(s * S + S, N) - 2 + p].phi;
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const int s = s0 + b;
-            if (s < P) {
-                zs[s * step] = W;
-                W = fma(ph[b], W, sx[b]);
-            }
-        }
+    for (int b = 0; b < LEN; ++b) {
+        z[b] = W;
+        W = fma(phi[b], W, v[b].x);
+        v[b].y = fma(bv[b], z[b], v[b].y);
     }
-    T X = 0;
-    for (int s1 = P - 1; s1 >= 0; s1 -= B2) {
-        T sy[B2], zi[B2], bv[B2], ps[B2];
+    al = 1;
+    be = 0;
 #pragma unroll
-        for (int b = 0; b < B2; ++b) {
-            const int s = s1 - b;
-            if (s >= 0) {
-                sy[b] = sum[s * step].y;
-                zi[b] = zs[s * step];
-                bv[b] = facj[s * S + p].Bv;
-                ps[b] = facj[s * S + p].Psi;
-            }
+    for (int b = LEN - 1; b >= 0; --b)
+        if (s0 + b < P) {
+            be = fma(ps[b], be, v[b].y);
+            al *= ps[b];
         }
+    beta[1][g][lane] = be;
+    if (lane == 0) alpha[1][g] = al;
+    __syncthreads();
+    T Y = 0;
+    for (int h = G - 1; h > g; --h) Y = fma(alpha[1][h], Y, beta[1][h][lane]);
 #pragma unroll
-        for (int b = 0; b < B2; ++b) {
-            const int s = s1 - b;
-            if (s >= 0) {
-                zx[s * step] = mk2<T>(zi[b], X);
-                X = fma(bv[b], zi[b], fma(ps[b], X, sy[b]));
-            }
+    for (int b = LEN - 1; b >= 0; --b)
+        if (s0 + b < P) {
+            zx[(int64_t)(s0 + b) * Mp] = mk2<T>(z[b], Y);
+            Y = fma(ps[b], Y, v[b].y);
         }
-    }
 }
 
 // ---------------------------------------------------------------------------
-// Elementwise kernels over 32 x 32 tiles of the n x n region.
+// Elementwise kernels over 32 x 32 tiles of the n x n region (caller layout); the
+// quarter-block arrays are addressed element by element.
 // ---------------------------------------------------------------------------
 struct TileView {
-    int n, ldp, prob, rhs, pair;
+    int n, nb, log_s, prob, rhs, pair;
     int64_t off64, offT;
     const double *d, *e, *s;
     double kx, ky;
@@ -569,7 +601,8 @@ __device__ __forceinline__ TileView tile_view(const TileArgs &t, int64_t idx = -
     v.prob = q.x >> 8;
     v.rhs = q.x & 255;
     v.n = p.n;
-    v.ldp = p.ldp;
+    v.nb = p.nb;
+    v.log_s = t.log_s;
     v.off64 = p.off64 + (int64_t)v.rhs * p.n * p.n;
     v.offT = p.off + (int64_t)v.rhs * p.rhs;
     v.d = p.d;
@@ -593,52 +626,24 @@ __device__ __forceinline__ void tile_run(int64_t ntiles, int64_t &t0, int64_t &t
     t1 = t0 + per < ntiles ? t0 + per : ntiles;
 }
 
-// c_{J-1} at (i, k) rebuilt from the column pass's local result and its chain.
+// Offset of element (i, k) of the n x n matrix in the quarter-block arrays.
 template <typename T>
-__device__ __forceinline__ T rebuilt_c(const SwArgs<T> &a, const SwProb<T> &pr, int64_t offT, int64_t sbase,
-                                       const Fac<T> &fi, int i, int k)
+__device__ __forceinline__ int64_t quarter_pos(const TileView &v, int i, int k)
 {
-    const T cl = a.cl[offT + (int64_t)(i + 2) * pr.ldp + k + 4];
-    const typename Vec2<T>::type z = a.zxC[sbase + ((int64_t)(i / pr.S) * 2 + (i & 1)) * (pr.N + 8) + k + 4];
-    return fma(fi.Bv, z.x, fma(fi.Psi, z.y, cl));
+    const int S = 1 << v.log_s, q = (i & 1) * 2 + (k & 1), a = i >> 1, b = k >> 1;
+    const int64_t blk = ((int64_t)q * v.nb + (a >> v.log_s)) * v.nb + (b >> v.log_s);
+    return v.offT + (blk << (2 * v.log_s)) + block_pos<T>(a & (S - 1), b & (S - 1), S);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) finalize_kernel(TileArgs t, SwArgs<T> a, const int *__restrict__ pair_active)
+__global__ void __launch_bounds__(256) finalize_out_kernel(TileArgs t, const double *__restrict__ D,
+                                                           double *__restrict__ X)
 {
     const TileView v = tile_view(t);
-    if (!pair_active[v.pair]) return;
-    const SwProb<T> &pr = a.probs[v.prob];
-    const int J = pr.J;
-    const T fD = pr.sh[3 * (J - 1) + 2];
-    const Fac<T> *fac = pr.facC + (int64_t)(J - 1) * (pr.N + 4) + 2;
-    const int64_t sbase = pr.soff + (int64_t)v.rhs * pr.srhs;
+    const double sc = -1.0 / v.ky;
     for (int r = threadIdx.y; r < 32; r += 8) {
         const int i = v.by + r, k = v.bx + threadIdx.x;
-        if (i < v.n && k < v.n) {
-            const T c = rebuilt_c(a, pr, v.offT, sbase, fac[i], i, k);
-            T *dp = a.D + v.offT + (int64_t)(i + 2) * pr.ldp + k + 4;
-            *dp = (J >= 2) ? fma(fD, c, *dp) : fD * c;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(256) finalize_out_kernel(TileArgs t, SwArgs<double> a, double *__restrict__ X)
-{
-    const TileView v = tile_view(t);
-    const SwProb<double> &pr = a.probs[v.prob];
-    if (!a.active[v.prob]) return;
-    const int J = pr.J;
-    const double fD = pr.sh[3 * (J - 1) + 2];
-    const Fac<double> *fac = pr.facC + (int64_t)(J - 1) * (pr.N + 4) + 2;
-    const int64_t sbase = pr.soff + (int64_t)v.rhs * pr.srhs;
-    for (int r = threadIdx.y; r < 32; r += 8) {
-        const int i = v.by + r, k = v.bx + threadIdx.x;
-        if (i < v.n && k < v.n) {
-            const double c = rebuilt_c(a, pr, v.offT, sbase, fac[i], i, k);
-            const double y = (J >= 2) ? fma(fD, c, a.D[v.offT + (int64_t)(i + 2) * pr.ldp + k + 4]) : fD * c;
-            X[v.off64 + (int64_t)i * v.n + k] = y * v.s[i] * v.s[k];
-        }
+        if (i < v.n && k < v.n)
+            X[v.off64 + (int64_t)i * v.n + k] = sc * D[quarter_pos<double>(v, i, k)] * v.s[i] * v.s[k];
     }
 }
 
@@ -697,15 +702,16 @@ __global__ void __launch_bounds__(256) scale_in_kernel(TileArgs t, const double 
     }
     for (int r = threadIdx.y; r < 32; r += 8) {
         const int i = v.by + r, k = v.bx + threadIdx.x;
+        double val = 0.0;
         if (i < v.n && k < v.n) {
-            const double val = F[v.off64 + (int64_t)i * v.n + k] * v.s[i] * v.s[k];
+            val = F[v.off64 + (int64_t)i * v.n + k] * v.s[i] * v.s[k];
             if (Ft) Ft[v.off64 + (int64_t)i * v.n + k] = val;
-            rho0[v.offT + (int64_t)(i + 2) * v.ldp + k + 4] = (T)(val * inv);
         }
+        rho0[quarter_pos<T>(v, i, k)] = (T)(val * inv);  // unused positions: zero
     }
 }
 
-// Yout = Y + s D; R = F~ - A~ Yout - Yout A~; rho0 = R / s; rmax = max |R|.
+// Yout = Y - s D / ky; R = F~ - A~ Yout - Yout A~; rho0 = R / s; rmax = max |R|.
 // Y and Yout are distinct buffers, so every CTA sees the same not-yet-updated halo.
 __global__ void __launch_bounds__(256) residual_kernel(TileArgs t, const double *__restrict__ Y,
                                                        double *__restrict__ Yout, const float *__restrict__ D,
@@ -739,7 +745,7 @@ __global__ void __launch_bounds__(256) residual_kernel(TileArgs t, const double 
             continue;
         }
         const double sF = __longlong_as_double((long long)smax[v.pair]);
-        const double inv = sF > 0.0 ? 1.0 / sF : 0.0;
+        const double inv = sF > 0.0 ? 1.0 / sF : 0.0, sD = -sF / v.ky;
         for (int r = ty; r < 36; r += 8) {
             const int i = v.by - 2 + r;
             for (int cc = tx; cc < 36; cc += 32) {
@@ -747,7 +753,7 @@ __global__ void __launch_bounds__(256) residual_kernel(TileArgs t, const double 
                 double val = 0.0;
                 if (i >= 0 && i < n && k >= 0 && k < n) {
                     val = y_zero ? 0.0 : Y[v.off64 + (int64_t)i * n + k];
-                    val = fma(sF, (double)D[v.offT + (int64_t)(i + 2) * v.ldp + k + 4], val);
+                    val = fma(sD, (double)D[quarter_pos<float>(v, i, k)], val);
                 }
                 Ys[r][cc] = val;
             }
@@ -782,7 +788,7 @@ __global__ void __launch_bounds__(256) residual_kernel(TileArgs t, const double 
                 acc = fma(cc[2][tx], Ys[r + 2][tx + 4], acc);
                 Yout[v.off64 + (int64_t)i * n + k] = y;
                 local = flag_nonfinite(fabs(acc), local);
-                rho0[v.offT + (int64_t)(i + 2) * v.ldp + k + 4] = (float)(acc * inv);
+                rho0[quarter_pos<float>(v, i, k)] = (float)(acc * inv);
             }
         }
         __syncthreads();  // Ys is refilled by the next tile
@@ -800,21 +806,46 @@ __global__ void __launch_bounds__(256) scale_out_kernel(TileArgs t, const double
     }
 }
 
-template <typename T, int S>
-cudaError_t row_pass_S(const SwArgs<T> &a, int j, int mode, cudaStream_t st)
+// Launch on `st` as a dependent of the launch before it (see pdl_wait).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args... args)
 {
-    const size_t sm = RowGeom<T, S>::bytes;
-    const dim3 grid((unsigned)a.nitems);
-    if (mode == 0) row_pass_kernel<T, S, 0><<<grid, kRT, sm, st>>>(a, j);
-    else if (mode == 1) row_pass_kernel<T, S, 1><<<grid, kRT, sm, st>>>(a, j);
-    else row_pass_kernel<T, S, 2><<<grid, kRT, sm, st>>>(a, j);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
+template <typename T, int S>
+cudaError_t row_pass_S(const SwArgs<T> &a, int j, cudaStream_t st)
+{
+    const size_t sm = Geo<T, S>::row_bytes;
+    const unsigned grid = (unsigned)a.nitems;
+    if (a.fused) {
+        if (j == 0) return launch_pdl(row_pass_kernel<T, S, true, true>, grid, kL, sm, st, a, j);
+        return launch_pdl(row_pass_kernel<T, S, false, true>, grid, kL, sm, st, a, j);
+    }
+    if (j == 0) return launch_pdl(row_pass_kernel<T, S, true, false>, grid, kL, sm, st, a, j);
+    return launch_pdl(row_pass_kernel<T, S, false, false>, grid, kL, sm, st, a, j);
 }
 template <typename T, int S>
 cudaError_t col_pass_S(const SwArgs<T> &a, int j, cudaStream_t st)
 {
-    col_pass_kernel<T, S><<<(unsigned)a.nitems, kCT, ColGeom<T, S>::bytes, st>>>(a, j);
-    return cudaGetLastError();
+    const size_t sm = Geo<T, S>::col_bytes;
+    const unsigned grid = (unsigned)a.nitems;
+    if (a.fused) {
+        if (j == 0) return launch_pdl(col_pass_kernel<T, S, true, true>, grid, kL, sm, st, a, j);
+        return launch_pdl(col_pass_kernel<T, S, false, true>, grid, kL, sm, st, a, j);
+    }
+    if (j == 0) return launch_pdl(col_pass_kernel<T, S, true, false>, grid, kL, sm, st, a, j);
+    return launch_pdl(col_pass_kernel<T, S, false, false>, grid, kL, sm, st, a, j);
 }
 
 // CTAs of a reduction kernel: 8 per SM (all resident), at most one per tile.
@@ -824,48 +855,68 @@ unsigned reduction_grid(int64_t ntiles)
     return (unsigned)(ntiles < g ? (ntiles > 0 ? ntiles : 1) : g);
 }
 
+template <typename T, int S>
+cudaError_t setup_S()
+{
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto *k, size_t bytes) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    set(row_pass_kernel<T, S, true, true>, Geo<T, S>::row_bytes);
+    set(row_pass_kernel<T, S, true, false>, Geo<T, S>::row_bytes);
+    set(row_pass_kernel<T, S, false, true>, Geo<T, S>::row_bytes);
+    set(row_pass_kernel<T, S, false, false>, Geo<T, S>::row_bytes);
+    set(col_pass_kernel<T, S, true, true>, Geo<T, S>::col_bytes);
+    set(col_pass_kernel<T, S, true, false>, Geo<T, S>::col_bytes);
+    set(col_pass_kernel<T, S, false, true>, Geo<T, S>::col_bytes);
+    set(col_pass_kernel<T, S, false, false>, Geo<T, S>::col_bytes);
+    set(row_sums_kernel<T, S>, Geo<T, S>::sum_bytes);
+    return e;
+}
+
 }  // namespace
 
-bool sweep_segment_supported(bool fp64, int S) { return S == 64 || (!fp64 && S == 128); }
+bool sweep_segment_supported(bool fp64, int seg) { return seg == 64 || (!fp64 && seg == 128); }
 
 cudaError_t sweep_setup_kernels()
 {
-    cudaError_t e;
-#define SETSM(kern, bytes)                                                                                \
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bytes))) !=    \
-        cudaSuccess)                                                                                      \
-        return e;
-    SETSM((row_pass_kernel<float, 128, 0>), (RowGeom<float, 128>::bytes));
-    SETSM((row_pass_kernel<float, 128, 1>), (RowGeom<float, 128>::bytes));
-    SETSM((row_pass_kernel<float, 128, 2>), (RowGeom<float, 128>::bytes));
-    SETSM((row_pass_kernel<float, 64, 0>), (RowGeom<float, 64>::bytes));
-    SETSM((row_pass_kernel<float, 64, 1>), (RowGeom<float, 64>::bytes));
-    SETSM((row_pass_kernel<float, 64, 2>), (RowGeom<float, 64>::bytes));
-    SETSM((row_pass_kernel<double, 64, 0>), (RowGeom<double, 64>::bytes));
-    SETSM((row_pass_kernel<double, 64, 1>), (RowGeom<double, 64>::bytes));
-    SETSM((row_pass_kernel<double, 64, 2>), (RowGeom<double, 64>::bytes));
-    SETSM((col_pass_kernel<float, 128>), (ColGeom<float, 128>::bytes));
-    SETSM((col_pass_kernel<float, 64>), (ColGeom<float, 64>::bytes));
-    SETSM((col_pass_kernel<double, 64>), (ColGeom<double, 64>::bytes));
-#undef SETSM
-    return cudaSuccess;
+    cudaError_t e = setup_S<float, 32>();
+    if (e == cudaSuccess) e = setup_S<float, 64>();
+    if (e == cudaSuccess) e = setup_S<double, 32>();
+    return e;
 }
 
 template <typename T>
 cudaError_t launch_fac_tables(const FacJob<T> *jobs, int njobs, cudaStream_t st)
 {
     const int threads = 2 * njobs;
-    fac_tables_kernel<T><<<(threads + 127) / 128, 128, 0, st>>>(jobs, njobs);
+    fac_tables_kernel<T><<<(threads + 31) / 32, 32, 0, st>>>(jobs, njobs);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_row_pass(const SwArgs<T> &a, int j, int mode, cudaStream_t st)
+cudaError_t launch_row_sums(const SwArgs<T> &a, cudaStream_t st)
+{
+    // the first kernel of a graph: an ordinary launch
+    if constexpr (sizeof(T) == 4) {
+        if (a.S == 64) {
+            row_sums_kernel<T, 64><<<(unsigned)a.nitems, kL, Geo<T, 64>::sum_bytes, st>>>(a);
+            return cudaGetLastError();
+        }
+    }
+    if (a.S != 32) return cudaErrorInvalidValue;
+    row_sums_kernel<T, 32><<<(unsigned)a.nitems, kL, Geo<T, 32>::sum_bytes, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_row_pass(const SwArgs<T> &a, int j, cudaStream_t st)
 {
     if constexpr (sizeof(T) == 4) {
-        if (a.S == 128) return row_pass_S<T, 128>(a, j, mode, st);
+        if (a.S == 64) return row_pass_S<T, 64>(a, j, st);
     }
-    if (a.S == 64) return row_pass_S<T, 64>(a, j, mode, st);
+    if (a.S == 32) return row_pass_S<T, 32>(a, j, st);
     return cudaErrorInvalidValue;
 }
 
@@ -873,33 +924,26 @@ template <typename T>
 cudaError_t launch_col_pass(const SwArgs<T> &a, int j, cudaStream_t st)
 {
     if constexpr (sizeof(T) == 4) {
-        if (a.S == 128) return col_pass_S<T, 128>(a, j, st);
+        if (a.S == 64) return col_pass_S<T, 64>(a, j, st);
     }
-    if (a.S == 64) return col_pass_S<T, 64>(a, j, st);
+    if (a.S == 32) return col_pass_S<T, 32>(a, j, st);
     return cudaErrorInvalidValue;
 }
 
 template <typename T>
 cudaError_t launch_chain(const SwArgs<T> &a, int dir, int j, cudaStream_t st)
 {
-    const bool big = a.chain_mode == 2 || (a.chain_mode == 0 && a.nitems <= 2 * (int64_t)current_sm_count());
-    if (big)
-        chain_kernel<T, true><<<(unsigned)a.nitems, 2 * kChainLines, 0, st>>>(a, dir, j);
-    else
-        chain_kernel<T, false><<<(unsigned)a.nitems, 2 * kChainLines, 0, st>>>(a, dir, j);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_finalize(const TileArgs &t, const SwArgs<T> &a, const int *pair_active, cudaStream_t st)
-{
-    finalize_kernel<T><<<(unsigned)t.ntiles, dim3(32, 8), 0, st>>>(t, a, pair_active);
-    return cudaGetLastError();
+    const unsigned warps = (unsigned)((a.max_nb + a.chain_len - 1) / a.chain_len), grid = (unsigned)a.nitems;
+    if (warps > 32) return cudaErrorInvalidValue;
+    if (a.chain_len == 8) return launch_pdl(chain_kernel<T, 8>, grid, 32 * warps, 0, st, a, dir, j);
+    if (a.chain_len == 16) return launch_pdl(chain_kernel<T, 16>, grid, 32 * warps, 0, st, a, dir, j);
+    if (a.chain_len == 24) return launch_pdl(chain_kernel<T, 24>, grid, 32 * warps, 0, st, a, dir, j);
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_finalize_out(const TileArgs &t, const SwArgs<double> &a, double *X, cudaStream_t st)
 {
-    finalize_out_kernel<<<(unsigned)t.ntiles, dim3(32, 8), 0, st>>>(t, a, X);
+    finalize_out_kernel<<<(unsigned)t.ntiles, dim3(32, 8), 0, st>>>(t, a.D, X);
     return cudaGetLastError();
 }
 
@@ -934,14 +978,14 @@ cudaError_t launch_scale_out(const TileArgs &t, const double *Y, double *X, cuda
 
 template cudaError_t launch_fac_tables<float>(const FacJob<float> *, int, cudaStream_t);
 template cudaError_t launch_fac_tables<double>(const FacJob<double> *, int, cudaStream_t);
-template cudaError_t launch_row_pass<float>(const SwArgs<float> &, int, int, cudaStream_t);
-template cudaError_t launch_row_pass<double>(const SwArgs<double> &, int, int, cudaStream_t);
+template cudaError_t launch_row_sums<float>(const SwArgs<float> &, cudaStream_t);
+template cudaError_t launch_row_sums<double>(const SwArgs<double> &, cudaStream_t);
+template cudaError_t launch_row_pass<float>(const SwArgs<float> &, int, cudaStream_t);
+template cudaError_t launch_row_pass<double>(const SwArgs<double> &, int, cudaStream_t);
 template cudaError_t launch_col_pass<float>(const SwArgs<float> &, int, cudaStream_t);
 template cudaError_t launch_col_pass<double>(const SwArgs<double> &, int, cudaStream_t);
 template cudaError_t launch_chain<float>(const SwArgs<float> &, int, int, cudaStream_t);
 template cudaError_t launch_chain<double>(const SwArgs<double> &, int, int, cudaStream_t);
-template cudaError_t launch_finalize<float>(const TileArgs &, const SwArgs<float> &, const int *, cudaStream_t);
-template cudaError_t launch_finalize<double>(const TileArgs &, const SwArgs<double> &, const int *, cudaStream_t);
 template cudaError_t launch_scale_in<float>(const TileArgs &, const double *, double *, float *,
                                             const unsigned long long *, cudaStream_t);
 template cudaError_t launch_scale_in<double>(const TileArgs &, const double *, double *, double *,

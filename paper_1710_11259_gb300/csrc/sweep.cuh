@@ -7,38 +7,56 @@
 // with L(Y) = A~ Y (along columns) and R(Y) = Y A~ (along rows); D after J
 // iterations is the ADI iterate Y_J of the paper's form started from Y_0 = 0 with
 // right-hand side rho_0 (the two forms agree term by term in exact arithmetic).
+// The products with A~ + q are never formed.  With a_j = (R - q_j)^{-1} rho_j and
+// u_j = (L + q_j) c_j,
+//     u_j = a_j + 2 q_j c_j                                (L + q = (L - q) + 2q),
+//     a_{j+1} = (R - q_{j+1})^{-1} (R + q_j) u_j
+//             = u_j + (q_j + q_{j+1}) (R - q_{j+1})^{-1} u_j,
+// so an iteration is two solves, two multiply-adds per element and the update of D:
+//     row pass:     a = u + s v,  v = (R - q_j)^{-1} u,  s = q_{j-1} + q_j  (a = v at j = 0)
+//     column pass:  t = 2 q_j c,  c = (L - q_j)^{-1} a,  u = a + t,  D <- D + t
+// and Y_J = -D.  The shifts fall with j, so neither sum cancels: on an eigenvector
+// with R -> 0 the row factor 1 - s/q_j is -q_{j-1}/q_j, the column factor -1.
 // On a rectangle the equation is kx A~ Y + ky Y A~ = F~ with shifts p_j (row side)
-// and q_j (column side) of App. A's general intervals; the same steps then read
-//     c_j = (L - q_j/kx)^{-1} (R + p_j/ky)^{-1} rho_j,
-//     D  <- D - (q_j - p_j)/(kx ky) c_j,    rho_{j+1} = (L - p_j/kx)(R + q_j/ky) c_j,
-// (the scalars kx, ky of the solves and the stencils cancel), so the kernels only
-// see two solve shifts, two stencil shifts and one correction factor per iteration.
+// and q_j (column side) of App. A's general intervals; the row solves then have the
+// shift -p_j/ky and s = (q_{j-1} - p_j)/ky, the column solves q_j/kx and
+// t = (q_j - p_j)/kx c, and Y_J = -D/ky.
 //
-// Each banded solve is split into the two tridiagonals of App. B (even and odd
-// indices) and every tridiagonal into segments of S positions.  A pass solves its
-// segments independently ("local" solutions: forward sweep started from zero,
-// back substitution ended at zero).  With the pivots of A~ - qI and
-//     w_i = ip_i r_i - g_i w_{i-2}        (forward, g_i = e_{i-2} ip_i)
-//     x_i = w_i - uf_i x_{i+2}            (back substitution, uf_i = e_i ip_i)
-// the true solution in a segment is
-//     x_i = xl_i + Bv_i zin + Psi_i xout,
-// where zin is the true forward value just before the segment, xout the true
-// solution just after it, and Bv, Psi depend only on the shift (tables below).
-// zin and xout of every segment follow from a two-sweep recurrence over the
-// segment summaries (wl at the segment end, xl at its start): the chain kernels.
-// The correction is applied lazily by the NEXT pass when it loads the data, so
-// every pass reads its input once and writes its output once:
-//   row pass j     reads cl_{j-1} (+ halo), rebuilds c_{j-1}, D -= 2q_{j-1} c_{j-1},
-//                  rho_j = (L+q_{j-1})(R+q_{j-1}) c_{j-1}, row-local solve -> al_j
-//   row chain j    zin/xout of the row segments
-//   column pass j  reads al_j, rebuilds a_j, column-local solve -> cl_j
-//   column chain j zin/xout of the column segments
-// (j = 0: the row pass reads rho_0 itself).  A finalize kernel adds the last c.
+// Even and odd indices decouple in both directions (App. B), so the n x n problem is
+// four independent problems ("quarters": row parity x column parity) of tridiagonal
+// systems of about n/2 unknowns, stored apart.
 //
-// Storage (type T = float or double): every n x n array of a (problem, rhs) is
-// padded to N = 64 * ceil(n/64) positions per side plus a halo of 2 rows and 4
-// columns on each side, row-major with leading dimension ldp = N + 8; element
-// (i, k) sits at (i + 2) * ldp + (k + 4).  Padding is zero and stays zero.
+// A tridiagonal A~ - qI of one parity, pivots piv_i, ip_i = 1/piv_i, is solved as
+//     w_i = r_i - l_i w_{i-1},     l_i = e_{i-1} ip_{i-1},
+//     y_i = w_i - m_i y_{i+1},     m_i = e_i ip_{i+1},       x_i = ip_i y_i
+// (the pivot of w is left in place and ip_i is folded into the scalars s and 2q that
+// x is multiplied with: one multiply-add per sweep and element).  Systems are cut into
+// segments of S unknowns.  A pass needs, per segment and line, w just before (zin) and
+// y just after it (yout); they follow from a recurrence over the segments of the two
+// segment summaries that the pass before left:
+//     wl = sum_i psi_i r_i  (w at the segment's end started from zero),
+//     yl = sum_i chi_i r_i  (y at its start, started from and ended at zero),
+//     W_s = wl(s) + phi(s) W_{s-1},                    zin(s)  = W_{s-1},
+//     Y_s = yl(s) + Bv(s) zin(s) + Psi(s) Y_{s+1},     yout(s) = Y_{s+1}
+// (psi, chi, phi, Bv, Psi depend on the shift only and are tabulated in FP64
+// arithmetic).  So every pass reads true values, writes true values, and forms on the
+// finished tile the summaries of the next solve, which runs across it:
+//   row pass j     reads u, writes a in place;  summaries of column solve j
+//   column pass j  reads a, D, writes u, D in place;  summaries of row solve j + 1
+// Every element is read and written once per pass by the same CTA: no halo, no second
+// array, 8 + 16 bytes per element and iteration in FP32, 11 FP64 operations in FP64.
+// Bound: HBM in FP32 where the arrays exceed L2, the FP64 rate in FP64.  Measured on
+// GB300: FP32 n = 10^4 row pass 128 us, column pass 237 us (6.1 and 6.7 TB/s of DRAM
+// traffic; a copy reaches 6.7), FP64 n = 4096 154 and 183 us; passes that formed the
+// products with A~ + q on tiles with halos and rebuilt the solve before them while
+// loading took 341 + 158 us and 393 + 174 us.
+//
+// Storage (type T = float or double) of a (problem, rhs): four quarters of nb x nb
+// blocks of S x S elements, nb = ceil(ceil(n/2)/S), block (bi, bk) of a quarter at
+// ((quarter * nb + bi) * nb + bk) * S * S, rows of S elements.  A tile is whole blocks,
+// so one bulk copy per block moves it.  The 16-byte chunks of row r are permuted by
+// XOR with r mod 8, which makes the row-wise 16-byte accesses of the sweeps along rows
+// free of bank conflicts.  Unused positions (>= the parity's size) are zero.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -57,52 +75,58 @@ struct Vec2<double> {
     using type = double2;
 };
 
-// Per-position coefficients of one shift (position i at index i + 2 of a table of
-// N + 4 records; the two records on each side and positions >= n are zero).
-template <typename T>
-struct alignas(16) Fac {
-    T ip, g, uf;   // pivot reciprocal, forward multiplier, back-substitution multiplier
-    T phi;         // prod of -g from the segment start to i (forward propagation of zin)
-    T Bv, Psi;     // coefficients of zin and xout in the true solution at i
-    T pad0, pad1;  // 8-word records: the first four words load as 16-byte vectors
-};
+constexpr int kPassLines = 128;  // rows of a row-pass tile, columns of a column-pass tile
+constexpr int kTabs = 5;         // per position and shift: l, m, solution scale, psi, chi
+constexpr int kMaxFused = 16;    // segments per line up to which a pass runs the recurrence itself
 
-// One problem at one tolerance level (device table entry).
+// Offset of element (r, c) inside an S x S block (V elements per 16-byte chunk).
 template <typename T>
-struct SwProb {
-    int n, S, P, N, ldp, J;
-    int64_t off, rhs;      // element offset of rhs 0 / stride between right-hand sides (T arrays)
-    int64_t soff, srhs;    // the same for the segment arrays ([P][2][N + 8] entries)
-    const Fac<T> *facR;    // [J][N + 4] tables of the row solves (shift -p_j / ky)
-    const Fac<T> *facC;    // [J][N + 4] tables of the column solves (shift q_j / kx); == facR on a square
-    const T *sh;           // [J][3]: {column-stencil shift -p_j/kx, row-stencil shift q_j/ky,
-                           //          correction factor -(q_j - p_j)/(kx ky)}; square: {q, q, -2q}
-    const T *d, *e;        // bands of A~ at index i + 2, zero outside [0, n)
+__host__ __device__ __forceinline__ int block_pos(int r, int c, int S)
+{
+    constexpr int V = 16 / (int)sizeof(T);
+    return r * S + (((c / V) ^ (r & 7)) * V) + c % V;
+}
+
+// One work item of a pass or chain launch at one tolerance level: everything a CTA
+// needs before it can issue its copies, in one 64-byte record (one round trip).
+template <typename T>
+struct alignas(16) SwItem {
+    int64_t xoff;          // passes: element offset of the tile's first block in X and D
+    int64_t soff;          // offset of the quarter in the segment arrays
+    const T *tabR, *tabC;  // [J][2][kTabs][nb * S] tables of the row / column solves of this quarter's parities
+                           // (offset to the parity: iteration j at + j * 2 * kTabs * nb * S)
+    const T *chR, *chC;    // [J][2][3][nbp] segment coefficients phi, Bv, Psi (nbp = nb rounded up to 4), likewise
+    int prob;              // problem index (mask of active problems)
+    int J;                 // iterations of the problem at this level
+    unsigned short nb, b0; // blocks per side; passes: first block along the lines (row pass: block row)
+    unsigned short b1, n_blk;  // passes: block along the solve; blocks of the tile.  Chains: first line / 32, -
 };
+static_assert(sizeof(SwItem<float>) == 64, "one 64-byte record per item");
 
 template <typename T>
 struct SwArgs {
     using T2 = typename Vec2<T>::type;
-    const SwProb<T> *probs;
-    const int4 *items;     // row/column pass: {problem, rhs, block of 64 rows/columns, segment}
-                           // chain: {problem, rhs, block of 64 lines, 0}
+    const SwItem<T> *items;
     int64_t nitems;
     const int *active;     // per problem
-    T *rho0, *cl, *al, *D;
-    T2 *sumR, *sumC;       // segment summaries {wl_end, xl_start}
-    T2 *zxR, *zxC;         // chain results {zin, xout}
-    T *zin;                // chain scratch ([P][2][N + 8] per rhs)
+    const int *masked;     // != 0 if any problem is inactive
+    T *X, *D;              // X: u / a in place; D: sum of t
+    T2 *sumR, *sumC;       // segment summaries {wl, yl}: [quarter][segment][line]
+    T2 *zxR, *zxC;         // recurrence results {zin, yout}, same layout (plans that run it in its own kernel)
     int *err;              // device error word: bit 0 = a bounded wait gave up
-    int S;                 // segment length of every problem (sweep_segment_supported)
-    int chain_mode;        // chain kernel loads: 0 = by grid size, 1 = short batches, 2 = long batches
+    int S;                 // block and segment size of every problem (sweep_segment_supported(., 2 S))
+    int fused;             // passes run the segment recurrence themselves (nb <= kMaxFused)
+    int chain_len;         // chain kernel: segments per thread
+    int max_nb;
 };
 
 // Elementwise tile kernels of the solve around the ADI loop.  A tile item is
-// {problem * 256 + rhs, tile column, tile row, 0} over the n x n region in 32 x 32 tiles.
+// {problem * 256 + rhs, tile column, tile row, 0}, 32 x 32 tiles of the n x n region
+// (scale-in: of the padded region).
 struct TileProb {
-    int n, ldp;
+    int n, nb;
     int64_t off64;          // FP64 packing of the caller's arrays: offset of rhs 0 (rhs stride n*n)
-    int64_t off, rhs;       // padded T arrays (as SwProb)
+    int64_t off, rhs;       // quarter-block arrays: offset of rhs 0, stride between right-hand sides
     const double *d, *e, *s;  // FP64 bands of A~ (d, e zero-padded to length n) and 1/sqrt(E)
     int pair0;              // index of (problem, rhs 0) among all pairs
     double kx, ky;          // scales of the two second derivatives (1, 1 on [-1,1]^2)
@@ -112,48 +136,51 @@ struct TileArgs {
     const TileProb *probs;
     const int4 *tiles;
     int64_t ntiles;
+    int log_s;              // log2 of the block size of the quarter-block arrays
 };
 
 // Shift tables of a list of (problem, shift) jobs, computed in FP64.
 template <typename T>
 struct FacJob {
     double q;
-    int n, N, S;
+    double sc1, sc2;       // factors of ip in the solution scales of out1 and out2
+    int n, nb, S;
     const double *d, *e;   // FP64 bands, e zero-padded to length n
-    Fac<T> *out;           // N + 4 records
+    T *out1, *out2;        // [2][kTabs][nb * S]; out2 may be null
+    T *ch1, *ch2;          // [2][3][nbp]; ch2 null with out2
 };
 
 cudaError_t sweep_setup_kernels();
-// Segment lengths with compiled pass kernels: 64 (FP32, FP64) and 128 (FP32).
-bool sweep_segment_supported(bool fp64, int S);
+// Segment lengths (unknowns of both parities) with compiled pass kernels: 64 (FP32, FP64)
+// and 128 (FP32), i.e. blocks of 32 and 64.
+bool sweep_segment_supported(bool fp64, int seg);
 
 template <typename T>
 cudaError_t launch_fac_tables(const FacJob<T> *jobs, int njobs, cudaStream_t st);
 
-// Row pass of iteration j over the items (mode 0: j = 0 reads rho0; mode 1: j = 1,
-// D = -2q c; mode 2: D -= 2q c).
+// Summaries of the row solve of iteration 0 of the right-hand sides in X (items of the
+// column pass).
 template <typename T>
-cudaError_t launch_row_pass(const SwArgs<T> &a, int j, int mode, cudaStream_t st);
+cudaError_t launch_row_sums(const SwArgs<T> &a, cudaStream_t st);
+template <typename T>
+cudaError_t launch_row_pass(const SwArgs<T> &a, int j, cudaStream_t st);
 template <typename T>
 cudaError_t launch_col_pass(const SwArgs<T> &a, int j, cudaStream_t st);
-// Chains of the row (dir 0) or column (dir 1) segments of iteration j.
+// Segment recurrences of the row (dir 0) or column (dir 1) solve of iteration j.
 template <typename T>
 cudaError_t launch_chain(const SwArgs<T> &a, int dir, int j, cudaStream_t st);
 
-// D <- D - 2 q_{J-1} c_{J-1} (or D = -2q c when J = 1) over the n x n region of every
-// (problem, rhs) pair with pair_active set.
-template <typename T>
-cudaError_t launch_finalize(const TileArgs &t, const SwArgs<T> &a, const int *pair_active, cudaStream_t st);
-// X = D_s (D - 2 q_{J-1} c_{J-1}) D_s straight into the caller's FP64 X.
+// X = -D_s D D_s / ky straight into the caller's FP64 X.
 cudaError_t launch_finalize_out(const TileArgs &t, const SwArgs<double> &a, double *X, cudaStream_t st);
 
 // Per (problem, rhs): smax = max |D_s F D_s| (bit patterns; must start at 0).
 cudaError_t launch_absmax(const TileArgs &t, const double *F, unsigned long long *smax, cudaStream_t st);
-// F~ = D_s F D_s (FP64, if Ft != nullptr) and rho0 = F~ / smax (T, padded; smax == nullptr: no scaling).
+// F~ = D_s F D_s (FP64, if Ft != nullptr) and rho0 = F~ / smax (T, quarter blocks, unused
+// positions set to zero; smax == nullptr: no scaling).  Tiles cover the padded region.
 template <typename T>
 cudaError_t launch_scale_in(const TileArgs &t, const double *F, double *Ft, T *rho0, const unsigned long long *smax,
                             cudaStream_t st);
-// Yout = Y + smax D (Y read as zero if y_zero), R = F~ - A~ Yout - Yout A~, rho0 = R / smax,
+// Yout = Y - smax D / ky (Y read as zero if y_zero), R = F~ - A~ Yout - Yout A~, rho0 = R / smax,
 // rmax = max |R| per pair (bit patterns; must start at 0); inactive pairs copy Y.
 cudaError_t launch_residual(const TileArgs &t, const double *Y, double *Yout, const float *D, const double *Ft,
                             float *rho0, const unsigned long long *smax, unsigned long long *rmax,

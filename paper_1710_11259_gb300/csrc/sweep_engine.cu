@@ -4,8 +4,8 @@
 // FP32 (refinement), per solve:
 //   smax = max |F~| per (problem, rhs) pair; F~ = D_s F D_s; rho_0 = F~ / smax
 //   round r: inner ADI in FP32 (one CUDA graph per tolerance level: every pass
-//            launch covers every problem; a finalize kernel adds the last c) gives
-//            the correction D; the FP64 residual kernel applies Y += smax D, forms
+//            launch covers every problem) gives the correction -D/ky; the FP64
+//            residual kernel applies Y -= smax D/ky, forms
 //            R~ = F~ - A~Y - YA~ and the next rho_0; pairs with max|R~| <= tol smax
 //            stop (their iterate is carried unchanged).
 //   X = D_s Y D_s.
@@ -15,7 +15,7 @@
 // finest level, 1e-7, is about what one FP32 inner solve can deliver).  Inner shifts come from the
 // tight spectral interval of A~ (the refinement is judged by the FP64 residual).
 // FP64 (plain method): rho_0 = F~, one graph of J iterations of (2.9), then
-// X = D_s Y_J D_s fused with the last correction.
+// X = D_s Y_J D_s.
 #include "sweep_engine.h"
 #include "trace.h"
 
@@ -41,8 +41,6 @@ double bits_to_double(unsigned long long b)
     return d;
 }
 const double kLevelTols[] = {1e-7, 1e-6, 1e-5, 1e-4, 1e-3, 1e-2};
-constexpr int kTileW = 64;       // rows of a row-pass tile / columns of a column-pass tile
-constexpr int kChainLines = 64;
 }  // namespace
 
 template <typename T>
@@ -85,8 +83,8 @@ void SweepEngine<T>::release()
     } while (0)
 
 // ---------------------------------------------------------------------------
-// Autotuner of the segment length (the tile height of the column pass and width of
-// the row pass; it also fixes the number of segments a chain walks).  Every
+// Autotuner of the segment length (unknowns of both parities: twice the block size of
+// sweep.cuh; it also fixes the number of segments a recurrence walks).  Every
 // candidate gets a complete engine of its own on the same sizes; the graph of the
 // coarsest tolerance level is timed with CUDA events and the fastest candidate
 // kept.  Results are cached per (GPU name, nrhs, size list) in $FPS_AUTOTUNE_CACHE
@@ -110,7 +108,7 @@ std::string tune_key(const std::vector<int64_t> &ns, int nrhs)
         }
     }
     std::ostringstream os;
-    os << "seg|" << name << "|" << nrhs << "|" << ns.size() << "|" << std::hex << h;
+    os << "blk|" << name << "|" << nrhs << "|" << ns.size() << "|" << std::hex << h;
     return os.str();
 }
 
@@ -122,6 +120,42 @@ std::string tune_cache_path()
     return std::string(home ? home : "/tmp") + "/.cache/fps_gb300_autotune.txt";
 }
 }  // namespace
+
+// Entries per segment-coefficient array: 16-byte multiples for the bulk copies.
+static int nbp_of(int nb) { return (nb + 3) & ~3; }
+
+// Segments per thread of the chain kernel: short or long runs (the autotuner's choice),
+// longer where a line has more segments than 32 warps of short runs cover.
+static int chain_len_of(int mode, int max_nb)
+{
+    int len = mode == 2 ? 16 : 8;
+    while (len < 24 && (max_nb + len - 1) / len > 32) len += 8;
+    return len;
+}
+
+template <typename T>
+TileArgs SweepEngine<T>::tiles(bool padded) const
+{
+    TileArgs t;
+    t.probs = d_tp_;
+    t.tiles = padded ? d_in_tiles_ : d_tiles_;
+    t.ntiles = padded ? nin_tiles_ : ntiles_;
+    t.log_s = seg_len == 128 ? 6 : 5;
+    return t;
+}
+
+// Problems with an active pair, and whether any problem is inactive.
+template <typename T>
+void SweepEngine<T>::set_active()
+{
+    const int np = (int)ns_.size();
+    h_active_[np] = 0;
+    for (int p = 0; p < np; ++p) {
+        h_active_[p] = 0;
+        for (int r = 0; r < nrhs_; ++r) h_active_[p] |= h_pair_active_[p * nrhs_ + r];
+        if (!h_active_[p]) h_active_[np] = 1;
+    }
+}
 
 template <typename T>
 int SweepEngine<T>::time_level(size_t li, int reps, float &ms, std::string &err)
@@ -142,12 +176,15 @@ int SweepEngine<T>::time_level(size_t li, int reps, float &ms, std::string &err)
 }
 
 // Mean time of a chain launch (both directions alternately) with the given load
-// batching, on this engine's arrays (the values do not change the time).
+// batching, on this engine's arrays (the values do not change the time); 0 where the
+// passes run the recurrences themselves.
 template <typename T>
 int SweepEngine<T>::time_chain(int mode, float &ms, std::string &err)
 {
     SwArgs<T> a = args(levels_.back(), 2);
-    a.chain_mode = mode;
+    ms = 0.f;
+    if (a.fused) return FPS_OK;
+    a.chain_len = chain_len_of(mode, max_nb_);
     cudaEvent_t e0, e1;
     ENG_CK(cudaEventCreate(&e0));
     ENG_CK(cudaEventCreate(&e1));
@@ -250,28 +287,28 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
         }
         seg_len = seg;
     }
-    const int S = seg_len;
-    N_.resize(np);
-    P_.resize(np);
+    const int S = seg_len / 2;  // block size: unknowns of one parity
+    nb_.resize(np);
     off64_.resize(np);
     offT_.resize(np);
     offS_.resize(np);
     tot64_ = totT_ = totS_ = 0;
-    int64_t totBT = 0, totB64 = 0;
+    max_nb_ = 0;
+    int64_t totB64 = 0;
     for (int p = 0; p < np; ++p) {
         const int64_t n = ns[p];
-        const int N = (int)((n + kTileW - 1) / kTileW * kTileW);
-        N_[p] = N;
-        P_[p] = (N + S - 1) / S;
+        const int64_t nb = ((n + 1) / 2 + S - 1) / S;
+        nb_[p] = (int)nb;
+        max_nb_ = std::max(max_nb_, (int)nb);
         off64_[p] = tot64_;
         offT_[p] = totT_;
         offS_[p] = totS_;
         tot64_ += (int64_t)nrhs * n * n;
-        totT_ += (int64_t)nrhs * (N + 4) * (N + 8);
-        totS_ += (int64_t)nrhs * P_[p] * 2 * (N + 8);
-        totBT += 2 * (int64_t)(N + 4);
+        totT_ += (int64_t)nrhs * 4 * nb * nb * S * S;
+        totS_ += (int64_t)nrhs * 4 * nb * nb * S;
         totB64 += 3 * n;
     }
+    fused_ = max_nb_ <= kMaxFused;
     npairs_ = np * nrhs;
 
     ENG_CK(sweep_setup_kernels());
@@ -281,66 +318,54 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
         ENG_CK(dalloc(&Y1_, (size_t)tot64_));
     }
     ENG_CK(dalloc(&bands64_, (size_t)totB64));
-    ENG_CK(dalloc(&bandsT_, (size_t)totBT));
-    ENG_CK(dalloc(&rho0_, (size_t)totT_));
-    ENG_CK(dalloc(&cl_, (size_t)totT_));
-    ENG_CK(dalloc(&al_, (size_t)totT_));
+    ENG_CK(dalloc(&X_, (size_t)totT_));
     ENG_CK(dalloc(&D_, (size_t)totT_));
-    ENG_CK(dalloc(&zin_, (size_t)totS_));
     ENG_CK(dalloc(&sumR_, (size_t)totS_));
     ENG_CK(dalloc(&sumC_, (size_t)totS_));
-    ENG_CK(dalloc(&zxR_, (size_t)totS_));
-    ENG_CK(dalloc(&zxC_, (size_t)totS_));
+    if (!fused_) {
+        ENG_CK(dalloc(&zxR_, (size_t)totS_));
+        ENG_CK(dalloc(&zxC_, (size_t)totS_));
+    }
     ENG_CK(dalloc(&err_, 1));
-    ENG_CK(dalloc(&d_active_, (size_t)np));
+    ENG_CK(dalloc(&d_active_, (size_t)np + 1));
     ENG_CK(dalloc(&d_pair_active_, (size_t)npairs_));
     ENG_CK(dalloc(&d_smax_, (size_t)npairs_));
     ENG_CK(dalloc(&d_rmax_, (size_t)npairs_));
-    ENG_CK(cudaMallocHost((void **)&h_active_, sizeof(int) * np));
+    ENG_CK(cudaMallocHost((void **)&h_active_, sizeof(int) * (np + 1)));  // last: any problem inactive
     ENG_CK(cudaMallocHost((void **)&h_pair_active_, sizeof(int) * npairs_));
     ENG_CK(cudaMallocHost((void **)&h_smax_, sizeof(unsigned long long) * npairs_));
     ENG_CK(cudaMallocHost((void **)&h_rmax_, sizeof(unsigned long long) * npairs_));
     ENG_CK(cudaMallocHost((void **)&h_err_, sizeof(int)));
     *h_err_ = 0;
-    // padding must be zero and stays zero
-    {
-        T *tb[] = {rho0_, cl_, al_, D_};
-        for (T *b : tb) ENG_CK(cudaMemsetAsync(b, 0, sizeof(T) * (size_t)totT_, cap_));
-        ENG_CK(cudaMemsetAsync(zin_, 0, sizeof(T) * (size_t)totS_, cap_));
-        T2 *sb[] = {sumR_, sumC_, zxR_, zxC_};
-        for (T2 *b : sb) ENG_CK(cudaMemsetAsync(b, 0, sizeof(T2) * (size_t)totS_, cap_));
-        ENG_CK(cudaMemsetAsync(err_, 0, sizeof(int), cap_));
-    }
+    // unused positions must be zero and stay zero
+    ENG_CK(cudaMemsetAsync(X_, 0, sizeof(T) * (size_t)totT_, cap_));
+    ENG_CK(cudaMemsetAsync(D_, 0, sizeof(T) * (size_t)totT_, cap_));
+    ENG_CK(cudaMemsetAsync(sumR_, 0, sizeof(T2) * (size_t)totS_, cap_));
+    ENG_CK(cudaMemsetAsync(sumC_, 0, sizeof(T2) * (size_t)totS_, cap_));
+    ENG_CK(cudaMemsetAsync(err_, 0, sizeof(int), cap_));
 
-    // bands: FP64 (d, e zero-padded, 1/sqrt(E)) and padded T copies (index i + 2)
+    // bands: FP64 (d, e zero-padded, 1/sqrt(E))
     std::vector<double> hb64((size_t)totB64);
-    std::vector<T> hbT((size_t)totBT, T(0));
     std::vector<TileProb> tp(np);
-    std::vector<int4> tiles;
-    std::vector<int64_t> ob64(np), obT(np);
+    std::vector<int4> tiles, in_tiles;  // 32 x 32 tiles of the n x n and of the padded region
+    std::vector<int64_t> ob64(np);
     {
-        int64_t o64 = 0, oT = 0;
+        int64_t o64 = 0;
         std::vector<double> d, e, s;
         for (int p = 0; p < np; ++p) {
             const int64_t n = ns[p];
-            const int N = N_[p];
             square_bands(n, d, e);
             inv_sqrt_E(n, s);
             std::copy(d.begin(), d.end(), hb64.begin() + o64);
             std::copy(e.begin(), e.end(), hb64.begin() + o64 + n);
             std::copy(s.begin(), s.end(), hb64.begin() + o64 + 2 * n);
-            for (int64_t i = 0; i < n; ++i) {
-                hbT[oT + i + 2] = (T)d[i];
-                hbT[oT + (N + 4) + i + 2] = (T)e[i];
-            }
             ob64[p] = o64;
-            obT[p] = oT;
             TileProb &t = tp[p];
             t.n = (int)n;
-            t.ldp = N + 8;
+            t.nb = nb_[p];
             t.off64 = off64_[p];
             t.off = offT_[p];
-            t.rhs = (int64_t)(N + 4) * (N + 8);
+            t.rhs = 4 * (int64_t)nb_[p] * nb_[p] * S * S;
             t.d = bands64_ + o64;
             t.e = bands64_ + o64 + n;
             t.s = bands64_ + o64 + 2 * n;
@@ -348,47 +373,32 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
             t.kx = kx_;
             t.ky = ky_;
             o64 += 3 * n;
-            oT += 2 * (N + 4);
-            const int nt = (int)((n + 31) / 32);
-            for (int r = 0; r < nrhs; ++r)
+            const int nt = (int)((n + 31) / 32), ntp = 2 * nb_[p] * S / 32;
+            for (int r = 0; r < nrhs; ++r) {
                 for (int ty = 0; ty < nt; ++ty)
                     for (int tx = 0; tx < nt; ++tx) tiles.push_back(make_int4(p * 256 + r, tx, ty, 0));
+                for (int ty = 0; ty < ntp; ++ty)
+                    for (int tx = 0; tx < ntp; ++tx) in_tiles.push_back(make_int4(p * 256 + r, tx, ty, 0));
+            }
         }
     }
     ntiles_ = (int64_t)tiles.size();
+    nin_tiles_ = (int64_t)in_tiles.size();
     ENG_CK(dalloc(&d_tp_, (size_t)np));
     ENG_CK(dalloc(&d_tiles_, (size_t)ntiles_));
+    ENG_CK(dalloc(&d_in_tiles_, (size_t)nin_tiles_));
     ENG_CK(cudaMemcpyAsync(bands64_, hb64.data(), sizeof(double) * totB64, cudaMemcpyHostToDevice, cap_));
-    ENG_CK(cudaMemcpyAsync(bandsT_, hbT.data(), sizeof(T) * totBT, cudaMemcpyHostToDevice, cap_));
     ENG_CK(cudaMemcpyAsync(d_tp_, tp.data(), sizeof(TileProb) * np, cudaMemcpyHostToDevice, cap_));
     ENG_CK(cudaMemcpyAsync(d_tiles_, tiles.data(), sizeof(int4) * ntiles_, cudaMemcpyHostToDevice, cap_));
+    ENG_CK(cudaMemcpyAsync(d_in_tiles_, in_tiles.data(), sizeof(int4) * nin_tiles_, cudaMemcpyHostToDevice, cap_));
 
-    // work items, largest problems first; a row pass sweeps row blocks down each column segment
-    {
-        std::vector<int> order(np);
-        for (int p = 0; p < np; ++p) order[p] = p;
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return ns[a] > ns[b]; });
-        std::vector<int4> it[3];
-        for (int p : order) {
-            const int nb = N_[p] / kTileW, P = P_[p], nl = (N_[p] + kChainLines - 1) / kChainLines;
-            for (int r = 0; r < nrhs; ++r) {
-                for (int sg = 0; sg < P; ++sg)
-                    for (int b = 0; b < nb; ++b) {
-                        it[0].push_back(make_int4(p, r, b, sg));
-                        it[1].push_back(make_int4(p, r, b, sg));
-                    }
-                for (int b = 0; b < nl; ++b) it[2].push_back(make_int4(p, r, b, 0));
-            }
-        }
-        for (int w = 0; w < 3; ++w) {
-            nitems_[w] = (int64_t)it[w].size();
-            ENG_CK(dalloc(&d_items_[w], (size_t)nitems_[w]));
-            ENG_CK(cudaMemcpyAsync(d_items_[w], it[w].data(), sizeof(int4) * nitems_[w], cudaMemcpyHostToDevice, cap_));
-        }
-    }
+    std::vector<int> order(np);  // items: largest problems first
+    for (int p = 0; p < np; ++p) order[p] = p;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return ns[x] > ns[y]; });
     for (int p = 0; p < np; ++p) h_active_[p] = 1;
+    h_active_[np] = 0;
     for (int k = 0; k < npairs_; ++k) h_pair_active_[k] = 1;
-    ENG_CK(cudaMemcpyAsync(d_active_, h_active_, sizeof(int) * np, cudaMemcpyHostToDevice, cap_));
+    ENG_CK(cudaMemcpyAsync(d_active_, h_active_, sizeof(int) * (np + 1), cudaMemcpyHostToDevice, cap_));
     ENG_CK(cudaMemcpyAsync(d_pair_active_, h_pair_active_, sizeof(int) * npairs_, cudaMemcpyHostToDevice, cap_));
 
     // tolerance levels: shifts, per-shift tables (FP64 arithmetic on the device)
@@ -411,30 +421,26 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
         // intervals of kx A~ (row side) and -ky A~ (column side): [a, b] = -kx [hi, lo],
         // [c, d] = ky [lo, hi]; on a square (kx = ky) the symmetric route gives p = -q
         const bool sym = kx_ == ky_;
-        const int ntab = sym ? 1 : 2;  // one table serves rows and columns on a square
-        int64_t nfac = 0, nq = 0;
+        int64_t nfac = 0, nch = 0, nq = 0;  // elements of one direction's tables, shifts
         for (int p = 0; p < np; ++p) {
             L.J[p] = adi_iterations(-kx_ * hi[p], -kx_ * lo[p], ky_ * lo[p], ky_ * hi[p], L.tol);
             L.Jmax = std::max(L.Jmax, L.J[p]);
-            nfac += (int64_t)ntab * L.J[p] * (N_[p] + 4);
+            nfac += (int64_t)L.J[p] * 2 * kTabs * nb_[p] * S;
+            nch += (int64_t)L.J[p] * 2 * 3 * nbp_of(nb_[p]);
             nq += L.J[p];
         }
-        ENG_CK(dalloc(&L.fac, (size_t)nfac));
-        ENG_CK(dalloc(&L.sh, (size_t)(3 * nq)));
-        ENG_CK(dalloc(&L.d_probs, (size_t)np));
-        ENG_CK(cudaMemsetAsync(L.fac, 0, sizeof(Fac<T>) * (size_t)nfac, cap_));
+        ENG_CK(dalloc(&L.tab, (size_t)(2 * nfac)));
+        ENG_CK(dalloc(&L.ch, (size_t)(2 * nch)));
+        const int njobs = (int)(sym ? nq : 2 * nq);
         FacJob<T> *d_jobs = nullptr;
-        ENG_CK(cudaMalloc((void **)&d_jobs, sizeof(FacJob<T>) * (size_t)(ntab * nq)));
-        std::vector<SwProb<T>> probs(np);
+        ENG_CK(cudaMalloc((void **)&d_jobs, sizeof(FacJob<T>) * (size_t)njobs));
         std::vector<FacJob<T>> jobs;
-        std::vector<T> shh;
-        jobs.reserve(ntab * nq);
-        shh.reserve(3 * nq);
-        int64_t of = 0, oq = 0;
+        jobs.reserve(njobs);
+        std::vector<int64_t> otab(np), och(np);
+        int64_t of = 0, oc = 0;
         std::vector<double> q, pp;
         for (int p = 0; p < np; ++p) {
             const int64_t n = ns[p];
-            const int N = N_[p];
             const double a = -kx_ * hi[p], b = -kx_ * lo[p], c = ky_ * lo[p], d = ky_ * hi[p];
             if (sym) {
                 zolotarev_shifts_symmetric(lo[p], hi[p], L.J[p], q);
@@ -456,50 +462,96 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
                 return FPS_ERR_INVALID_ARG;
             }
             if (li == 0) shifts[p] = q;
-            SwProb<T> &sp = probs[p];
-            sp.n = (int)n;
-            sp.S = S;
-            sp.P = P_[p];
-            sp.N = N;
-            sp.ldp = N + 8;
-            sp.J = L.J[p];
-            sp.off = offT_[p];
-            sp.rhs = (int64_t)(N + 4) * (N + 8);
-            sp.soff = offS_[p];
-            sp.srhs = (int64_t)P_[p] * 2 * (N + 8);
-            sp.facR = L.fac + of;
-            sp.facC = L.fac + of + (sym ? 0 : (int64_t)L.J[p] * (N + 4));
-            sp.sh = L.sh + 3 * oq;
-            sp.d = bandsT_ + obT[p];
-            sp.e = bandsT_ + obT[p] + (N + 4);
-            for (int t = 0; t < ntab; ++t)
-                for (int j = 0; j < L.J[p]; ++j) {
-                    FacJob<T> jb;
-                    jb.q = t == 0 ? -pp[j] / ky_ : q[j] / kx_;  // row solve, then column solve
-                    jb.n = (int)n;
-                    jb.N = N;
-                    jb.S = S;
-                    jb.d = bands64_ + ob64[p];
-                    jb.e = bands64_ + ob64[p] + n;
-                    jb.out = L.fac + of + ((int64_t)t * L.J[p] + j) * (N + 4);
+            otab[p] = of;
+            och[p] = oc;
+            const int64_t ts = 2 * (int64_t)kTabs * nb_[p] * S, cs = 2 * 3 * (int64_t)nbp_of(nb_[p]);
+            for (int j = 0; j < L.J[p]; ++j) {
+                FacJob<T> jb;
+                jb.n = (int)n;
+                jb.nb = nb_[p];
+                jb.S = S;
+                jb.d = bands64_ + ob64[p];
+                jb.e = bands64_ + ob64[p] + n;
+                // row solve, shift -p_j/ky: a = u + (q_{j-1} - p_j)/ky v
+                jb.q = -pp[j] / ky_;
+                jb.sc1 = j == 0 ? 1.0 : (q[j - 1] - pp[j]) / ky_;
+                jb.out1 = L.tab + of + j * ts;
+                jb.ch1 = L.ch + oc + j * cs;
+                // column solve, shift q_j/kx: t = (q_j - p_j)/kx c
+                const double sc_col = (q[j] - pp[j]) / kx_;
+                T *out_col = L.tab + nfac + of + j * ts, *ch_col = L.ch + nch + oc + j * cs;
+                jb.sc2 = sc_col;
+                jb.out2 = sym ? out_col : nullptr;
+                jb.ch2 = sym ? ch_col : nullptr;
+                jobs.push_back(jb);
+                if (!sym) {
+                    jb.q = q[j] / kx_;
+                    jb.sc1 = sc_col;
+                    jb.out1 = out_col;
+                    jb.ch1 = ch_col;
                     jobs.push_back(jb);
                 }
-            for (int j = 0; j < L.J[p]; ++j) {
-                shh.push_back((T)(-pp[j] / kx_));                    // column-stencil shift
-                shh.push_back((T)(q[j] / ky_));                      // row-stencil shift
-                shh.push_back((T)(-(q[j] - pp[j]) / (kx_ * ky_)));  // correction factor
             }
-            of += (int64_t)ntab * L.J[p] * (N + 4);
-            oq += L.J[p];
+            of += L.J[p] * ts;
+            oc += L.J[p] * cs;
         }
-        cudaError_t e1 = cudaMemcpyAsync(L.d_probs, probs.data(), sizeof(SwProb<T>) * np, cudaMemcpyHostToDevice, cap_);
-        if (e1 == cudaSuccess)
-            e1 = cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(FacJob<T>) * jobs.size(), cudaMemcpyHostToDevice, cap_);
-        if (e1 == cudaSuccess)
-            e1 = cudaMemcpyAsync(L.sh, shh.data(), sizeof(T) * shh.size(), cudaMemcpyHostToDevice, cap_);
+        // work items of the row passes, the column passes and the recurrences
+        std::vector<SwItem<T>> it[3];
+        const int R = kPassLines / S;
+        for (int p : order) {
+            const int nb = nb_[p];
+            const int64_t quarter = (int64_t)nb * nb * S * S, squarter = (int64_t)nb * nb * S;
+            for (int r = 0; r < nrhs; ++r)
+                for (int qd = 0; qd < 4; ++qd) {
+                    const int rp = qd >> 1, cp = qd & 1;
+                    if (ns[p] <= std::max(rp, cp)) continue;  // n = 1: one quarter only
+                    SwItem<T> x;
+                    x.soff = offS_[p] + ((int64_t)r * 4 + qd) * squarter;
+                    x.tabR = L.tab + otab[p] + (int64_t)cp * kTabs * nb * S;
+                    x.tabC = L.tab + nfac + otab[p] + (int64_t)rp * kTabs * nb * S;
+                    x.chR = L.ch + och[p] + cp * 3 * nbp_of(nb);
+                    x.chC = L.ch + nch + och[p] + rp * 3 * nbp_of(nb);
+                    x.prob = p;
+                    x.J = L.J[p];
+                    x.nb = (unsigned short)nb;
+                    const int64_t x0 = offT_[p] + ((int64_t)r * 4 + qd) * quarter;
+                    for (int b0 = 0; b0 < nb; b0 += R)
+                        for (int b1 = 0; b1 < nb; ++b1) {
+                            x.b0 = (unsigned short)b0;
+                            x.b1 = (unsigned short)b1;
+                            x.n_blk = (unsigned short)std::min(R, nb - b0);
+                            x.xoff = x0 + ((int64_t)b0 * nb + b1) * S * S;
+                            it[0].push_back(x);
+                        }
+                    for (int b0 = 0; b0 < nb; ++b0)
+                        for (int b1 = 0; b1 < nb; b1 += R) {
+                            x.b0 = (unsigned short)b0;
+                            x.b1 = (unsigned short)b1;
+                            x.n_blk = (unsigned short)std::min(R, nb - b1);
+                            x.xoff = x0 + ((int64_t)b0 * nb + b1) * S * S;
+                            it[1].push_back(x);
+                        }
+                    if (!fused_)
+                        for (int b1 = 0; b1 < nb * S / 32; ++b1) {
+                            x.b0 = 0;
+                            x.b1 = (unsigned short)b1;
+                            x.n_blk = 0;
+                            x.xoff = x0;
+                            it[2].push_back(x);
+                        }
+                }
+        }
+        cudaError_t e1 = cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(FacJob<T>) * jobs.size(), cudaMemcpyHostToDevice, cap_);
+        for (int w = 0; w < 3 && e1 == cudaSuccess; ++w) {
+            L.nitems[w] = (int64_t)it[w].size();
+            e1 = dalloc(&L.items[w], it[w].size());
+            if (e1 == cudaSuccess)
+                e1 = cudaMemcpyAsync(L.items[w], it[w].data(), sizeof(SwItem<T>) * it[w].size(), cudaMemcpyHostToDevice, cap_);
+        }
         if (e1 == cudaSuccess) e1 = launch_fac_tables<T>(d_jobs, (int)jobs.size(), cap_);
         // the host vectors and the job table must outlive the asynchronous work
-        if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(cap_);
+        const cudaError_t e2 = cudaStreamSynchronize(cap_);
+        if (e1 == cudaSuccess) e1 = e2;
         cudaFree(d_jobs);
         levels_.push_back(std::move(L));
         ENG_CK(e1);
@@ -521,22 +573,21 @@ template <typename T>
 SwArgs<T> SweepEngine<T>::args(const Level &L, int which) const
 {
     SwArgs<T> a;
-    a.probs = L.d_probs;
-    a.items = d_items_[which];
-    a.nitems = nitems_[which];
+    a.items = L.items[which];
+    a.nitems = L.nitems[which];
     a.active = d_active_;
-    a.rho0 = rho0_;
-    a.cl = cl_;
-    a.al = al_;
+    a.masked = d_active_ + ns_.size();
+    a.X = X_;
     a.D = D_;
     a.sumR = sumR_;
     a.sumC = sumC_;
     a.zxR = zxR_;
     a.zxC = zxC_;
-    a.zin = zin_;
     a.err = err_;
-    a.S = seg_len;
-    a.chain_mode = chain_mode;
+    a.S = seg_len / 2;
+    a.fused = fused_ ? 1 : 0;
+    a.chain_len = chain_len_of(chain_mode, max_nb_);
+    a.max_nb = max_nb_;
     return a;
 }
 
@@ -548,27 +599,28 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
         L.graph = nullptr;
     }
     const SwArgs<T> ar = args(L, 0), ac = args(L, 1), ach = args(L, 2);
-    TileArgs ta;
-    ta.probs = d_tp_;
-    ta.tiles = d_tiles_;
-    ta.ntiles = ntiles_;
     ENG_CK(cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     const bool ins = instrument_ && (int)L.ev.size() == 4 * L.Jmax;
     auto rec = [&](int k) {
         if (ins && e == cudaSuccess) e = cudaEventRecordWithFlags(L.ev[k], cap_, cudaEventRecordExternal);
     };
+    L.launches = 0;
+    auto run = [&](cudaError_t r) {
+        if (e == cudaSuccess) e = r;
+        ++L.launches;
+    };
+    run(launch_row_sums<T>(ac, cap_));
     for (int j = 0; j < L.Jmax && e == cudaSuccess; ++j) {
+        if (!fused_) run(launch_chain<T>(ach, 0, j, cap_));
         rec(4 * j);
-        if (e == cudaSuccess) e = launch_row_pass<T>(ar, j, j == 0 ? 0 : (j == 1 ? 1 : 2), cap_);
+        run(launch_row_pass<T>(ar, j, cap_));
         rec(4 * j + 1);
-        if (e == cudaSuccess) e = launch_chain<T>(ach, 0, j, cap_);
+        if (!fused_) run(launch_chain<T>(ach, 1, j, cap_));
         rec(4 * j + 2);
-        if (e == cudaSuccess) e = launch_col_pass<T>(ac, j, cap_);
+        run(launch_col_pass<T>(ac, j, cap_));
         rec(4 * j + 3);
-        if (e == cudaSuccess) e = launch_chain<T>(ach, 1, j, cap_);
     }
-    if (e == cudaSuccess && sizeof(T) == 4) e = launch_finalize<T>(ta, ar, d_pair_active_, cap_);
     cudaGraph_t g = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(cap_, &g);
     if (e != cudaSuccess) {
@@ -595,16 +647,13 @@ template <typename T>
 int SweepEngine<T>::solve_plain(const double *F, double *X, cudaStream_t st, std::string &err)
 {
     if constexpr (sizeof(T) == 8) {
-        TileArgs ta;
-        ta.probs = d_tp_;
-        ta.tiles = d_tiles_;
-        ta.ntiles = ntiles_;
-        ENG_CK(launch_scale_in<double>(ta, F, nullptr, rho0_, nullptr, st));
+        const TileArgs ta = tiles(false);
+        ENG_CK(launch_scale_in<double>(tiles(true), F, nullptr, X_, nullptr, st));
         ENG_CK(cudaGraphLaunch(levels_[0].graph, st));
         ENG_CK(launch_finalize_out(ta, args(levels_[0], 0), X, st));
         ENG_CK(cudaMemcpyAsync(h_err_, err_, sizeof(int), cudaMemcpyDeviceToHost, st));
         levels_used_.push_back(0);
-        launches_last = 2 + 4LL * levels_[0].Jmax;
+        launches_last = 2 + levels_[0].launches;
         rounds_last = 1;
         return FPS_OK;
     } else {
@@ -621,10 +670,7 @@ int SweepEngine<T>::solve_refine(const double *F, double *X, cudaStream_t st, st
 {
     if constexpr (sizeof(T) == 4) {
         const int np = (int)ns_.size();
-        TileArgs ta;
-        ta.probs = d_tp_;
-        ta.tiles = d_tiles_;
-        ta.ntiles = ntiles_;
+        const TileArgs ta = tiles(false);
 
         ENG_CK(cudaMemsetAsync(d_smax_, 0, sizeof(unsigned long long) * npairs_, st));
         ENG_CK(launch_absmax(ta, F, d_smax_, st));
@@ -640,13 +686,10 @@ int SweepEngine<T>::solve_refine(const double *F, double *X, cudaStream_t st, st
             }
             h_pair_active_[k] = sF[k] > 0.0 ? 1 : 0;  // an all-zero right-hand side is already solved (X = 0)
         }
-        for (int p = 0; p < np; ++p) {
-            h_active_[p] = 0;
-            for (int r = 0; r < nrhs_; ++r) h_active_[p] |= h_pair_active_[p * nrhs_ + r];
-        }
-        ENG_CK(cudaMemcpyAsync(d_active_, h_active_, sizeof(int) * np, cudaMemcpyHostToDevice, st));
+        set_active();
+        ENG_CK(cudaMemcpyAsync(d_active_, h_active_, sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
         ENG_CK(cudaMemcpyAsync(d_pair_active_, h_pair_active_, sizeof(int) * npairs_, cudaMemcpyHostToDevice, st));
-        ENG_CK(launch_scale_in<float>(ta, F, Ft_, rho0_, d_smax_, st));
+        ENG_CK(launch_scale_in<float>(tiles(true), F, Ft_, X_, d_smax_, st));
         launches_last += 1;
 
         std::vector<double> rel(npairs_, 0.0);
@@ -675,9 +718,9 @@ int SweepEngine<T>::solve_refine(const double *F, double *X, cudaStream_t st, st
             }
             ENG_CK(cudaGraphLaunch(levels_[li].graph, st));
             levels_used_.push_back((int)li);
-            launches_last += 4LL * levels_[li].Jmax + 1;
+            launches_last += levels_[li].launches;
             ENG_CK(cudaMemsetAsync(d_rmax_, 0, sizeof(unsigned long long) * npairs_, st));
-            ENG_CK(launch_residual(ta, Ycur, Ynext, D_, Ft_, rho0_, d_smax_, d_rmax_, d_pair_active_, round == 0, st));
+            ENG_CK(launch_residual(ta, Ycur, Ynext, D_, Ft_, X_, d_smax_, d_rmax_, d_pair_active_, round == 0, st));
             launches_last += 1;
             ENG_CK(cudaMemcpyAsync(h_rmax_, d_rmax_, sizeof(unsigned long long) * npairs_, cudaMemcpyDeviceToHost, st));
             ENG_CK(cudaMemcpyAsync(h_err_, err_, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -699,11 +742,8 @@ int SweepEngine<T>::solve_refine(const double *F, double *X, cudaStream_t st, st
                 if (r <= tol_) h_pair_active_[k] = 0;
                 else converged = false;
             }
-            for (int p = 0; p < np; ++p) {
-                h_active_[p] = 0;
-                for (int r = 0; r < nrhs_; ++r) h_active_[p] |= h_pair_active_[p * nrhs_ + r];
-            }
-            ENG_CK(cudaMemcpyAsync(d_active_, h_active_, sizeof(int) * np, cudaMemcpyHostToDevice, st));
+            set_active();
+            ENG_CK(cudaMemcpyAsync(d_active_, h_active_, sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
             ENG_CK(cudaMemcpyAsync(d_pair_active_, h_pair_active_, sizeof(int) * npairs_, cudaMemcpyHostToDevice, st));
         }
         rounds_last = round;
@@ -769,13 +809,12 @@ int SweepEngine<T>::kernel_times(int *count, double *total_ms, double *alg_bytes
             rms += t0;
             cms += t1;
             c += 2;
-            double ej = 0.0;
+            // row pass: u read, a written; column pass: a read, u written (but for the last
+            // iteration of a problem), D written and, after the first iteration, read
             for (size_t p = 0; p < ns_.size(); ++p)
-                if (j < L.J[p]) ej += (double)nrhs_ * (double)ns_[p] * (double)ns_[p];
-            // row pass: rho (or c) read, al written, D read and written (j >= 2) or written (j = 1);
-            // column pass: al read, cl written
-            const double row_words = j == 0 ? 2.0 : (j == 1 ? 3.0 : 4.0);
-            by += (row_words + 2.0) * sizeof(T) * ej;
+                if (j < L.J[p])
+                    by += (4.0 + (j > 0 ? 1.0 : 0.0) + (j + 1 < L.J[p] ? 1.0 : 0.0)) * sizeof(T) * (double)nrhs_ *
+                          (double)ns_[p] * (double)ns_[p];
         }
     }
     *count = c;

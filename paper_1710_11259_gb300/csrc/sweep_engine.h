@@ -19,7 +19,8 @@ class SweepEngine {
 public:
     // `ns`: problem sizes (caller packing: problem after problem, each problem's nrhs
     // n x n matrices back to back).  `tight`: shifts from the Sturm-bisection interval
-    // of A~ instead of Lemma B.2's.  `seg`: segment length of the partitioned sweeps
+    // of A~ instead of Lemma B.2's.  `seg`: segment length of the partitioned sweeps,
+    // counted in unknowns of both parities
     // (64 or 128 for FP32, 64 for FP64); seg <= 0 lets the autotuner pick it (FP32).
     // Returns an fps_status; on error `err` holds a message.
     // kx, ky: scales of the second derivatives along x and y (a kx^{-1/2} x ky^{-1/2}
@@ -34,8 +35,8 @@ public:
 
     int set_instrument(bool on, std::string &err);
     // ADI pass kernels (row and column passes) of the last solve: launches, summed
-    // duration, and the bytes they must move (sweep.cuh's residual form: 6 words per
-    // element and iteration, 4 in the first two iterations).
+    // duration, and the bytes they must move (6 words per element and iteration: u, a and
+    // D read and written once; 5 in the first and the last).
     int kernel_times(int *count, double *total_ms, double *alg_bytes, double *row_ms, double *col_ms,
                      std::string &err);
 
@@ -57,9 +58,10 @@ private:
         double tol = 0;
         int Jmax = 0;
         std::vector<int> J;
-        SwProb<T> *d_probs = nullptr;
-        Fac<T> *fac = nullptr;  // row tables then (rectangle) column tables
-        T *sh = nullptr;        // per iteration: stencil shifts and correction factor
+        T *tab = nullptr, *ch = nullptr;  // solve and summary tables, segment coefficients: rows, then columns
+        SwItem<T> *items[3] = {nullptr, nullptr, nullptr};  // row passes, column passes, recurrences
+        int64_t nitems[3] = {0, 0, 0};
+        int64_t launches = 0;             // kernels of the graph
         cudaGraphExec_t graph = nullptr;
         std::vector<cudaEvent_t> ev;  // 4 per iteration when instrumented
     };
@@ -68,6 +70,8 @@ private:
     int time_level(size_t li, int reps, float &ms, std::string &err);
     int time_chain(int mode, float &ms, std::string &err);
     SwArgs<T> args(const Level &L, int which) const;
+    TileArgs tiles(bool padded) const;
+    void set_active();
     int solve_refine(const double *F, double *X, cudaStream_t st, std::string &err);
     int solve_plain(const double *F, double *X, cudaStream_t st, std::string &err);
 
@@ -76,19 +80,19 @@ private:
     double tol_ = 0;
     double kx_ = 1.0, ky_ = 1.0;
     cudaStream_t cap_ = nullptr;
-    std::vector<int> N_, P_;
+    std::vector<int> nb_;  // blocks per side of a quarter
+    int max_nb_ = 0;
+    bool fused_ = false;   // the passes run the segment recurrences
     std::vector<int64_t> off64_, offT_, offS_;
     int64_t tot64_ = 0, totT_ = 0, totS_ = 0;
     int npairs_ = 0;
     double *Ft_ = nullptr, *Y0_ = nullptr, *Y1_ = nullptr, *bands64_ = nullptr;
-    T *bandsT_ = nullptr, *rho0_ = nullptr, *cl_ = nullptr, *al_ = nullptr, *D_ = nullptr, *zin_ = nullptr;
+    T *X_ = nullptr, *D_ = nullptr;
     T2 *sumR_ = nullptr, *sumC_ = nullptr, *zxR_ = nullptr, *zxC_ = nullptr;
     int *err_ = nullptr;
     TileProb *d_tp_ = nullptr;
-    int4 *d_tiles_ = nullptr;
-    int64_t ntiles_ = 0;
-    int4 *d_items_[3] = {nullptr, nullptr, nullptr};  // row pass, column pass, chains
-    int64_t nitems_[3] = {0, 0, 0};
+    int4 *d_tiles_ = nullptr, *d_in_tiles_ = nullptr;
+    int64_t ntiles_ = 0, nin_tiles_ = 0;
     int *d_active_ = nullptr, *d_pair_active_ = nullptr;
     int *h_active_ = nullptr, *h_pair_active_ = nullptr;
     unsigned long long *d_smax_ = nullptr, *d_rmax_ = nullptr, *h_smax_ = nullptr, *h_rmax_ = nullptr;
