@@ -12,7 +12,6 @@
 #include "../../include/fps.h"
 #include "host_math.h"
 #include "sweep_engine.h"
-#include "small.cuh"
 #include "cube.h"
 #include "legendre.cuh"
 #include "dirichlet.cuh"
@@ -103,9 +102,8 @@ struct fps_plan {
     // square: the ADI pass engine (FP32 sweeps + FP64 refinement, or plain FP64)
     fps::SweepEngine<float> *eng32 = nullptr;
     fps::SweepEngine<double> *eng64 = nullptr;
-    // FP64 squares with n <= 64: whole ADI in one launch (cluster kernel, warp-shuffle PCR)
+    // FP64 squares with n <= 64 are never streamed: no segment length, no pass timing
     bool small = false;
-    double *sm_bands = nullptr, *sm_q = nullptr, *sm_pcr = nullptr;
     // dim = 3: the nested cube ADI
     fps::CubeEngine *cube = nullptr;
     std::vector<int64_t> batch_ns;   // sizes of a batched plan (empty otherwise)
@@ -130,9 +128,6 @@ void release(fps_plan *p)
     DeviceGuard g(p->device);
     if (p->stage_in) cudaFree(p->stage_in);
     if (p->stage_out) cudaFree(p->stage_out);
-    if (p->sm_bands) cudaFree(p->sm_bands);
-    if (p->sm_q) cudaFree(p->sm_q);
-    if (p->sm_pcr) cudaFree(p->sm_pcr);
     for (double *b : {p->dir_F, p->dir_X, p->dir_d2, p->dir_ts})
         if (b) cudaFree(b);
     if (p->eng32) {
@@ -186,44 +181,6 @@ int solve_engine(fps_plan *p, E *eng, const double *F, double *X, bool fdev, boo
     return FPS_OK;
 }
 
-// FP64, n <= 64: one launch of the cluster kernel for all right-hand sides.
-int solve_small(fps_plan *p, const double *F, double *X, bool fdev, bool xdev, const char *what)
-{
-    const size_t bytes = sizeof(double) * (size_t)p->total_elems;
-    const double *Fd = F;
-    double *Xd = X;
-    if (!fdev) {
-        if (!p->stage_in) FPS_CK(cudaMalloc((void **)&p->stage_in, bytes));
-        FPS_CK(cudaMemcpyAsync(p->stage_in, F, bytes, cudaMemcpyHostToDevice, p->stream));
-        Fd = p->stage_in;
-    }
-    if (!xdev) {
-        if (!p->stage_out) FPS_CK(cudaMalloc((void **)&p->stage_out, bytes));
-        Xd = p->stage_out;
-    }
-    fps::SmallArgs a;
-    a.n = (int)p->n;
-    a.J = p->J;
-    a.nrhs = p->nrhs;
-    a.F = Fd;
-    a.X = Xd;
-    a.d = p->sm_bands;
-    a.e = p->sm_bands + p->n;
-    a.s = p->sm_bands + 2 * p->n;
-    a.q = p->sm_q;
-    a.pcr = p->sm_pcr;
-    cudaError_t e = fps::launch_small_adi(a, p->stream);
-    if (e != cudaSuccess) return fail(FPS_ERR_CUDA, std::string(what) + ": small-n kernel: " + cudaGetErrorString(e));
-    p->launches_last = 1;
-    if (!xdev) {
-        FPS_CK(cudaMemcpyAsync(X, Xd, bytes, cudaMemcpyDeviceToHost, p->stream));
-        FPS_CK(cudaStreamSynchronize(p->stream));
-    } else if (!fdev) {
-        FPS_CK(cudaStreamSynchronize(p->stream));
-    }
-    return FPS_OK;
-}
-
 int solve_square(fps_plan *p, const double *F, double *X, const char *what)
 {
     fps::TraceRange tr(what);
@@ -239,7 +196,6 @@ int solve_square(fps_plan *p, const double *F, double *X, const char *what)
         return fail(FPS_ERR_INVALID_ARG, std::string(what) + ": F or X is device memory of another device");
     const bool fdev = fk == Mem::kDevice, xdev = xk == Mem::kDevice;
     p->launches_last = 0;
-    if (p->small) return solve_small(p, F, X, fdev, xdev, what);
     if (p->eng32) return solve_engine(p, p->eng32, F, X, fdev, xdev, what);
     return solve_engine(p, p->eng64, F, X, fdev, xdev, what);
 }
@@ -300,27 +256,8 @@ int create_square(fps_plan **out, int64_t n, double tol, int precision, bool tig
     PCK(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
     std::string err;
     int st;
-    if (precision == FPS_FP64 && n <= fps::kSmallMaxN && kx == 1.0 && ky == 1.0) {
-        // whole ADI in one launch: bands, shifts and reduction coefficients on the device
-        std::vector<double> d, e, s, pcr;
-        fps::square_bands(n, d, e);
-        fps::inv_sqrt_E(n, s);
-        fps::small_pcr_coefficients(n, d, e, p->q, pcr);
-        std::vector<double> bands(3 * n);
-        std::copy(d.begin(), d.end(), bands.begin());
-        std::copy(e.begin(), e.end(), bands.begin() + n);
-        std::copy(s.begin(), s.end(), bands.begin() + 2 * n);
-        PCK(fps::small_setup_kernel());
-        PCK(cudaMalloc((void **)&p->sm_bands, sizeof(double) * 3 * n));
-        PCK(cudaMalloc((void **)&p->sm_q, sizeof(double) * p->J));
-        PCK(cudaMalloc((void **)&p->sm_pcr, sizeof(double) * pcr.size()));
-        PCK(cudaMemcpy(p->sm_bands, bands.data(), sizeof(double) * 3 * n, cudaMemcpyHostToDevice));
-        PCK(cudaMemcpy(p->sm_q, p->q.data(), sizeof(double) * p->J, cudaMemcpyHostToDevice));
-        PCK(cudaMemcpy(p->sm_pcr, pcr.data(), sizeof(double) * pcr.size(), cudaMemcpyHostToDevice));
-        p->bytes += (int64_t)sizeof(double) * (3 * n + p->J + (int64_t)pcr.size());
-        p->small = true;
-        st = FPS_OK;
-    } else if (precision == FPS_FP64) {
+    if (precision == FPS_FP64) {
+        p->small = n <= 64 && kx == 1.0 && ky == 1.0;
         p->eng64 = new fps::SweepEngine<double>();
         st = p->eng64->create(std::vector<int64_t>{n}, nrhs, tol, tight, p->cap_stream, err, 0, kx, ky);
         if (st == FPS_OK) p->bytes += p->eng64->bytes;
@@ -711,7 +648,7 @@ int fps_plan_info(const fps_plan *plan, fps_plan_info_t *info)
     info->tol = plan->tol;
     info->device_bytes = plan->bytes;
     info->kernel_launches = plan->launches_last;
-    info->seg_len = plan->eng32 ? plan->eng32->seg_len : (plan->eng64 ? plan->eng64->seg_len : 0);
+    info->seg_len = plan->eng32 ? plan->eng32->seg_len : (plan->eng64 && !plan->small ? plan->eng64->seg_len : 0);
     info->chain_mode = plan->eng32 ? plan->eng32->chain_mode : (plan->eng64 ? plan->eng64->chain_mode : 0);
     return FPS_OK;
 }
@@ -719,7 +656,7 @@ int fps_plan_info(const fps_plan *plan, fps_plan_info_t *info)
 int fps_plan_set_instrument(fps_plan *p, int on)
 {
     if (!p) return fail(FPS_ERR_INVALID_ARG, "fps_plan_set_instrument: plan is NULL");
-    if (!p->eng32 && !p->eng64)
+    if (!p->eng32 && (!p->eng64 || p->small))
         return fail(FPS_ERR_UNSUPPORTED, "fps_plan_set_instrument: square plans on the pass kernels only");
     DeviceGuard g(p->device);
     FPS_CK(cudaStreamSynchronize(p->cap_stream));

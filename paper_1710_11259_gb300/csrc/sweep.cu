@@ -602,7 +602,7 @@ __device__ __forceinline__ TileView tile_view(const TileArgs &t, int64_t idx = -
     v.rhs = q.x & 255;
     v.n = p.n;
     v.nb = p.nb;
-    v.log_s = t.log_s;
+    v.log_s = p.log_s;
     v.off64 = p.off64 + (int64_t)v.rhs * p.n * p.n;
     v.offT = p.off + (int64_t)v.rhs * p.rhs;
     v.d = p.d;
@@ -941,9 +941,9 @@ cudaError_t launch_chain(const SwArgs<T> &a, int dir, int j, cudaStream_t st)
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_finalize_out(const TileArgs &t, const SwArgs<double> &a, double *X, cudaStream_t st)
+cudaError_t launch_finalize_out(const TileArgs &t, const double *D, double *X, cudaStream_t st)
 {
-    finalize_out_kernel<<<(unsigned)t.ntiles, dim3(32, 8), 0, st>>>(t, a.D, X);
+    finalize_out_kernel<<<(unsigned)t.ntiles, dim3(32, 8), 0, st>>>(t, D, X);
     return cudaGetLastError();
 }
 

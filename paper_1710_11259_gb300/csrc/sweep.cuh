@@ -124,7 +124,7 @@ struct SwArgs {
 // {problem * 256 + rhs, tile column, tile row, 0}, 32 x 32 tiles of the n x n region
 // (scale-in: of the padded region).
 struct TileProb {
-    int n, nb;
+    int n, nb, log_s;       // nb: blocks of 2^log_s per side of a quarter
     int64_t off64;          // FP64 packing of the caller's arrays: offset of rhs 0 (rhs stride n*n)
     int64_t off, rhs;       // quarter-block arrays: offset of rhs 0, stride between right-hand sides
     const double *d, *e, *s;  // FP64 bands of A~ (d, e zero-padded to length n) and 1/sqrt(E)
@@ -136,7 +136,6 @@ struct TileArgs {
     const TileProb *probs;
     const int4 *tiles;
     int64_t ntiles;
-    int log_s;              // log2 of the block size of the quarter-block arrays
 };
 
 // Shift tables of a list of (problem, shift) jobs, computed in FP64.
@@ -171,7 +170,7 @@ template <typename T>
 cudaError_t launch_chain(const SwArgs<T> &a, int dir, int j, cudaStream_t st);
 
 // X = -D_s D D_s / ky straight into the caller's FP64 X.
-cudaError_t launch_finalize_out(const TileArgs &t, const SwArgs<double> &a, double *X, cudaStream_t st);
+cudaError_t launch_finalize_out(const TileArgs &t, const double *D, double *X, cudaStream_t st);
 
 // Per (problem, rhs): smax = max |D_s F D_s| (bit patterns; must start at 0).
 cudaError_t launch_absmax(const TileArgs &t, const double *F, unsigned long long *smax, cudaStream_t st);

@@ -14,6 +14,8 @@
 // level not above sqrt(0.1 tol), so that two rounds of equal gain reach tol (the
 // finest level, 1e-7, is about what one FP32 inner solve can deliver).  Inner shifts come from the
 // tight spectral interval of A~ (the refinement is judged by the FP64 residual).
+// Problems small enough for one cluster per quarter run all their iterations in one
+// launch (resident.cuh); the others are streamed by the passes.
 // FP64 (plain method): rho_0 = F~, one graph of J iterations of (2.9), then
 // X = D_s Y_J D_s.
 #include "sweep_engine.h"
@@ -140,7 +142,6 @@ TileArgs SweepEngine<T>::tiles(bool padded) const
     t.probs = d_tp_;
     t.tiles = padded ? d_in_tiles_ : d_tiles_;
     t.ntiles = padded ? nin_tiles_ : ntiles_;
-    t.log_s = seg_len == 128 ? 6 : 5;
     return t;
 }
 
@@ -225,6 +226,17 @@ int SweepEngine<T>::autotune(const std::vector<int64_t> &ns, int nrhs, double to
             }
         }
     }
+    auto remember = [&]() {
+        const size_t slash = path.find_last_of('/');
+        if (slash != std::string::npos && slash > 0) mkdir(path.substr(0, slash).c_str(), 0755);  // may exist
+        std::ofstream out(path, std::ios::app);
+        if (out) out << key << " " << seg_len << " " << chain_mode << "\n";
+    };
+    if (!streams_) {  // no pass runs: nothing to time
+        chain_mode = 1;
+        remember();
+        return FPS_OK;
+    }
     // tile shape: the segment length of the passes (a whole graph level timed per
     // candidate); then the chain kernel's load batching, timed on the winner's arrays
     const int cand[] = {64, 128};
@@ -250,10 +262,7 @@ int SweepEngine<T>::autotune(const std::vector<int64_t> &ns, int nrhs, double to
             chain_mode = c2 < c1 ? 2 : 1;
         }
     }
-    const size_t slash = path.find_last_of('/');
-    if (slash != std::string::npos && slash > 0) mkdir(path.substr(0, slash).c_str(), 0755);  // may exist
-    std::ofstream out(path, std::ios::app);
-    if (out) out << key << " " << seg_len << " " << chain_mode << "\n";
+    remember();
     return FPS_OK;
 }
 
@@ -272,6 +281,15 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     if (const char *mr = std::getenv("FPS_MAX_REFINE_ROUNDS")) {  // cap on refinement rounds (>= 1)
         const int v = std::atoi(mr);
         if (v >= 1) max_rounds = v;
+    }
+    res_s_.assign(np, 0);
+    streams_ = false;
+    for (int p = 0; p < np; ++p) {
+        const int m = (int)((ns[p] + 1) / 2), rs = resident_segment(kFP64, m);
+        bool fits = false;
+        if (rs > 0) ENG_CK(resident_setup<T>(rs, resident_cluster(m, rs), &fits));
+        if (fits) res_s_[p] = rs;
+        else streams_ = true;
     }
     if (seg <= 0) {
         if (kFP64) {
@@ -297,15 +315,18 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     int64_t totB64 = 0;
     for (int p = 0; p < np; ++p) {
         const int64_t n = ns[p];
-        const int64_t nb = ((n + 1) / 2 + S - 1) / S;
+        const int Sp = res_s_[p] ? 32 : S;
+        const int64_t nb = ((n + 1) / 2 + Sp - 1) / Sp;
         nb_[p] = (int)nb;
-        max_nb_ = std::max(max_nb_, (int)nb);
         off64_[p] = tot64_;
         offT_[p] = totT_;
         offS_[p] = totS_;
         tot64_ += (int64_t)nrhs * n * n;
-        totT_ += (int64_t)nrhs * 4 * nb * nb * S * S;
-        totS_ += (int64_t)nrhs * 4 * nb * nb * S;
+        totT_ += (int64_t)nrhs * 4 * nb * nb * Sp * Sp;
+        if (!res_s_[p]) {
+            max_nb_ = std::max(max_nb_, (int)nb);
+            totS_ += (int64_t)nrhs * 4 * nb * nb * S;
+        }
         totB64 += 3 * n;
     }
     fused_ = max_nb_ <= kMaxFused;
@@ -348,7 +369,7 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     std::vector<double> hb64((size_t)totB64);
     std::vector<TileProb> tp(np);
     std::vector<int4> tiles, in_tiles;  // 32 x 32 tiles of the n x n and of the padded region
-    std::vector<int64_t> ob64(np);
+    ob64_.resize(np);
     {
         int64_t o64 = 0;
         std::vector<double> d, e, s;
@@ -359,13 +380,14 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
             std::copy(d.begin(), d.end(), hb64.begin() + o64);
             std::copy(e.begin(), e.end(), hb64.begin() + o64 + n);
             std::copy(s.begin(), s.end(), hb64.begin() + o64 + 2 * n);
-            ob64[p] = o64;
+            ob64_[p] = o64;
             TileProb &t = tp[p];
             t.n = (int)n;
             t.nb = nb_[p];
+            t.log_s = res_s_[p] || S == 32 ? 5 : 6;
             t.off64 = off64_[p];
             t.off = offT_[p];
-            t.rhs = 4 * (int64_t)nb_[p] * nb_[p] * S * S;
+            t.rhs = 4 * (int64_t)nb_[p] * nb_[p] << (2 * t.log_s);
             t.d = bands64_ + o64;
             t.e = bands64_ + o64 + n;
             t.s = bands64_ + o64 + 2 * n;
@@ -373,7 +395,7 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
             t.kx = kx_;
             t.ky = ky_;
             o64 += 3 * n;
-            const int nt = (int)((n + 31) / 32), ntp = 2 * nb_[p] * S / 32;
+            const int nt = (int)((n + 31) / 32), ntp = 2 * (nb_[p] << t.log_s) / 32;
             for (int r = 0; r < nrhs; ++r) {
                 for (int ty = 0; ty < nt; ++ty)
                     for (int tx = 0; tx < nt; ++tx) tiles.push_back(make_int4(p * 256 + r, tx, ty, 0));
@@ -392,9 +414,9 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     ENG_CK(cudaMemcpyAsync(d_tiles_, tiles.data(), sizeof(int4) * ntiles_, cudaMemcpyHostToDevice, cap_));
     ENG_CK(cudaMemcpyAsync(d_in_tiles_, in_tiles.data(), sizeof(int4) * nin_tiles_, cudaMemcpyHostToDevice, cap_));
 
-    std::vector<int> order(np);  // items: largest problems first
-    for (int p = 0; p < np; ++p) order[p] = p;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return ns[x] > ns[y]; });
+    order_.resize(np);
+    for (int p = 0; p < np; ++p) order_[p] = p;
+    std::stable_sort(order_.begin(), order_.end(), [&](int x, int y) { return ns[x] > ns[y]; });
     for (int p = 0; p < np; ++p) h_active_[p] = 1;
     h_active_[np] = 0;
     for (int k = 0; k < npairs_; ++k) h_pair_active_[k] = 1;
@@ -415,146 +437,10 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     else tols.assign(std::begin(kLevelTols), std::end(kLevelTols));
     shifts.assign(np, {});
     for (size_t li = 0; li < tols.size(); ++li) {
-        Level L;
-        L.tol = tols[li];
-        L.J.resize(np);
-        // intervals of kx A~ (row side) and -ky A~ (column side): [a, b] = -kx [hi, lo],
-        // [c, d] = ky [lo, hi]; on a square (kx = ky) the symmetric route gives p = -q
-        const bool sym = kx_ == ky_;
-        int64_t nfac = 0, nch = 0, nq = 0;  // elements of one direction's tables, shifts
-        for (int p = 0; p < np; ++p) {
-            L.J[p] = adi_iterations(-kx_ * hi[p], -kx_ * lo[p], ky_ * lo[p], ky_ * hi[p], L.tol);
-            L.Jmax = std::max(L.Jmax, L.J[p]);
-            nfac += (int64_t)L.J[p] * 2 * kTabs * nb_[p] * S;
-            nch += (int64_t)L.J[p] * 2 * 3 * nbp_of(nb_[p]);
-            nq += L.J[p];
-        }
-        ENG_CK(dalloc(&L.tab, (size_t)(2 * nfac)));
-        ENG_CK(dalloc(&L.ch, (size_t)(2 * nch)));
-        const int njobs = (int)(sym ? nq : 2 * nq);
-        FacJob<T> *d_jobs = nullptr;
-        ENG_CK(cudaMalloc((void **)&d_jobs, sizeof(FacJob<T>) * (size_t)njobs));
-        std::vector<FacJob<T>> jobs;
-        jobs.reserve(njobs);
-        std::vector<int64_t> otab(np), och(np);
-        int64_t of = 0, oc = 0;
-        std::vector<double> q, pp;
-        for (int p = 0; p < np; ++p) {
-            const int64_t n = ns[p];
-            const double a = -kx_ * hi[p], b = -kx_ * lo[p], c = ky_ * lo[p], d = ky_ * hi[p];
-            if (sym) {
-                zolotarev_shifts_symmetric(lo[p], hi[p], L.J[p], q);
-                pp.resize(q.size());
-                for (size_t u = 0; u < q.size(); ++u) {
-                    q[u] *= kx_;
-                    pp[u] = -q[u];
-                }
-            } else {
-                zolotarev_shifts(a, b, c, d, L.J[p], pp, q);
-            }
-            inject_shift_fault(q);
-            std::vector<double> mp(pp.size());
-            for (size_t u = 0; u < pp.size(); ++u) mp[u] = -pp[u];
-            if (!shifts_valid(q, c, d) || !shifts_valid(mp, -b, -a)) {
-                cudaFree(d_jobs);
-                levels_.push_back(std::move(L));
-                err = "shift list failed validation (a shift is not finite or lies outside the spectral interval)";
-                return FPS_ERR_INVALID_ARG;
-            }
-            if (li == 0) shifts[p] = q;
-            otab[p] = of;
-            och[p] = oc;
-            const int64_t ts = 2 * (int64_t)kTabs * nb_[p] * S, cs = 2 * 3 * (int64_t)nbp_of(nb_[p]);
-            for (int j = 0; j < L.J[p]; ++j) {
-                FacJob<T> jb;
-                jb.n = (int)n;
-                jb.nb = nb_[p];
-                jb.S = S;
-                jb.d = bands64_ + ob64[p];
-                jb.e = bands64_ + ob64[p] + n;
-                // row solve, shift -p_j/ky: a = u + (q_{j-1} - p_j)/ky v
-                jb.q = -pp[j] / ky_;
-                jb.sc1 = j == 0 ? 1.0 : (q[j - 1] - pp[j]) / ky_;
-                jb.out1 = L.tab + of + j * ts;
-                jb.ch1 = L.ch + oc + j * cs;
-                // column solve, shift q_j/kx: t = (q_j - p_j)/kx c
-                const double sc_col = (q[j] - pp[j]) / kx_;
-                T *out_col = L.tab + nfac + of + j * ts, *ch_col = L.ch + nch + oc + j * cs;
-                jb.sc2 = sc_col;
-                jb.out2 = sym ? out_col : nullptr;
-                jb.ch2 = sym ? ch_col : nullptr;
-                jobs.push_back(jb);
-                if (!sym) {
-                    jb.q = q[j] / kx_;
-                    jb.sc1 = sc_col;
-                    jb.out1 = out_col;
-                    jb.ch1 = ch_col;
-                    jobs.push_back(jb);
-                }
-            }
-            of += L.J[p] * ts;
-            oc += L.J[p] * cs;
-        }
-        // work items of the row passes, the column passes and the recurrences
-        std::vector<SwItem<T>> it[3];
-        const int R = kPassLines / S;
-        for (int p : order) {
-            const int nb = nb_[p];
-            const int64_t quarter = (int64_t)nb * nb * S * S, squarter = (int64_t)nb * nb * S;
-            for (int r = 0; r < nrhs; ++r)
-                for (int qd = 0; qd < 4; ++qd) {
-                    const int rp = qd >> 1, cp = qd & 1;
-                    if (ns[p] <= std::max(rp, cp)) continue;  // n = 1: one quarter only
-                    SwItem<T> x;
-                    x.soff = offS_[p] + ((int64_t)r * 4 + qd) * squarter;
-                    x.tabR = L.tab + otab[p] + (int64_t)cp * kTabs * nb * S;
-                    x.tabC = L.tab + nfac + otab[p] + (int64_t)rp * kTabs * nb * S;
-                    x.chR = L.ch + och[p] + cp * 3 * nbp_of(nb);
-                    x.chC = L.ch + nch + och[p] + rp * 3 * nbp_of(nb);
-                    x.prob = p;
-                    x.J = L.J[p];
-                    x.nb = (unsigned short)nb;
-                    const int64_t x0 = offT_[p] + ((int64_t)r * 4 + qd) * quarter;
-                    for (int b0 = 0; b0 < nb; b0 += R)
-                        for (int b1 = 0; b1 < nb; ++b1) {
-                            x.b0 = (unsigned short)b0;
-                            x.b1 = (unsigned short)b1;
-                            x.n_blk = (unsigned short)std::min(R, nb - b0);
-                            x.xoff = x0 + ((int64_t)b0 * nb + b1) * S * S;
-                            it[0].push_back(x);
-                        }
-                    for (int b0 = 0; b0 < nb; ++b0)
-                        for (int b1 = 0; b1 < nb; b1 += R) {
-                            x.b0 = (unsigned short)b0;
-                            x.b1 = (unsigned short)b1;
-                            x.n_blk = (unsigned short)std::min(R, nb - b1);
-                            x.xoff = x0 + ((int64_t)b0 * nb + b1) * S * S;
-                            it[1].push_back(x);
-                        }
-                    if (!fused_)
-                        for (int b1 = 0; b1 < nb * S / 32; ++b1) {
-                            x.b0 = 0;
-                            x.b1 = (unsigned short)b1;
-                            x.n_blk = 0;
-                            x.xoff = x0;
-                            it[2].push_back(x);
-                        }
-                }
-        }
-        cudaError_t e1 = cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(FacJob<T>) * jobs.size(), cudaMemcpyHostToDevice, cap_);
-        for (int w = 0; w < 3 && e1 == cudaSuccess; ++w) {
-            L.nitems[w] = (int64_t)it[w].size();
-            e1 = dalloc(&L.items[w], it[w].size());
-            if (e1 == cudaSuccess)
-                e1 = cudaMemcpyAsync(L.items[w], it[w].data(), sizeof(SwItem<T>) * it[w].size(), cudaMemcpyHostToDevice, cap_);
-        }
-        if (e1 == cudaSuccess) e1 = launch_fac_tables<T>(d_jobs, (int)jobs.size(), cap_);
-        // the host vectors and the job table must outlive the asynchronous work
-        const cudaError_t e2 = cudaStreamSynchronize(cap_);
-        if (e1 == cudaSuccess) e1 = e2;
-        cudaFree(d_jobs);
-        levels_.push_back(std::move(L));
-        ENG_CK(e1);
+        levels_.emplace_back();
+        levels_.back().tol = tols[li];
+        const int st = build_tables(levels_.back(), (int)li, lo, hi, err);
+        if (st != FPS_OK) return st;
     }
     {
         int big = 0;
@@ -567,6 +453,240 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
         if (st != FPS_OK) return st;
     }
     return FPS_OK;
+}
+
+// Shifts, tables and work items of one tolerance level.
+template <typename T>
+int SweepEngine<T>::build_tables(Level &L, int level, const std::vector<double> &lo, const std::vector<double> &hi,
+                                 std::string &err)
+{
+    const int np = (int)ns_.size(), S = seg_len / 2;
+    // intervals of kx A~ (row side) and -ky A~ (column side): [a, b] = -kx [hi, lo],
+    // [c, d] = ky [lo, hi]; on a square (kx = ky) the symmetric route gives p = -q and one
+    // set of factors serves rows and columns
+    const bool sym = kx_ == ky_;
+    L.J.resize(np);
+    int64_t nfac = 0, nch = 0, nres = 0;  // elements of one direction's tables, coefficients, records
+    int nq = 0, nq_res = 0;               // shifts of the streamed and of the resident problems
+    for (int p = 0; p < np; ++p) {
+        L.J[p] = adi_iterations(-kx_ * hi[p], -kx_ * lo[p], ky_ * lo[p], ky_ * hi[p], L.tol);
+        L.Jmax = std::max(L.Jmax, L.J[p]);
+        if (res_s_[p]) {
+            nres += (int64_t)L.J[p] * 2 * res_record(res_s_[p]);
+            nq_res += L.J[p];
+        } else {
+            L.Jstream = std::max(L.Jstream, L.J[p]);
+            nfac += (int64_t)L.J[p] * 2 * kTabs * nb_[p] * S;
+            nch += (int64_t)L.J[p] * 2 * 3 * nbp_of(nb_[p]);
+            nq += L.J[p];
+        }
+    }
+    ENG_CK(dalloc(&L.tab, (size_t)(2 * nfac)));
+    ENG_CK(dalloc(&L.ch, (size_t)(2 * nch)));
+    ENG_CK(dalloc(&L.res_tab, (size_t)(2 * nres)));
+    struct Scratch {  // device copies of the job lists
+        void *p[2] = {nullptr, nullptr};
+        ~Scratch()
+        {
+            for (void *q : p)
+                if (q) cudaFree(q);
+        }
+    } scratch;
+    std::vector<FacJob<T>> jobs;
+    std::vector<ResTabJob<T>> rjobs;
+    jobs.reserve((size_t)nq * 2);
+    rjobs.reserve((size_t)nq_res * 2);
+    std::vector<int64_t> otab(np), och(np);  // offsets of a problem's tables (records) and coefficients
+    int64_t of = 0, oc = 0, ores = 0;
+    std::vector<double> q, pp;
+    for (int p = 0; p < np; ++p) {
+        const int64_t n = ns_[p];
+        const double a = -kx_ * hi[p], b = -kx_ * lo[p], c = ky_ * lo[p], d = ky_ * hi[p];
+        if (sym) {
+            zolotarev_shifts_symmetric(lo[p], hi[p], L.J[p], q);
+            pp.resize(q.size());
+            for (size_t u = 0; u < q.size(); ++u) {
+                q[u] *= kx_;
+                pp[u] = -q[u];
+            }
+        } else {
+            zolotarev_shifts(a, b, c, d, L.J[p], pp, q);
+        }
+        inject_shift_fault(q);
+        std::vector<double> mp(pp.size());
+        for (size_t u = 0; u < pp.size(); ++u) mp[u] = -pp[u];
+        if (!shifts_valid(q, c, d) || !shifts_valid(mp, -b, -a)) {
+            err = "shift list failed validation (a shift is not finite or lies outside the spectral interval)";
+            return FPS_ERR_INVALID_ARG;
+        }
+        if (level == 0) shifts[p] = q;
+        otab[p] = res_s_[p] ? ores : of;
+        och[p] = oc;
+        const double *bd = bands64_ + ob64_[p], *be = bd + n;
+        for (int j = 0; j < L.J[p]; ++j) {
+            // row solve, shift -p_j/ky: a = u + (q_{j-1} - p_j)/ky v;
+            // column solve, shift q_j/kx: t = (q_j - p_j)/kx c
+            const double q_row = -pp[j] / ky_, sc_row = j == 0 ? 1.0 : (q[j - 1] - pp[j]) / ky_;
+            const double q_col = q[j] / kx_, sc_col = (q[j] - pp[j]) / kx_;
+            if (res_s_[p]) {
+                const int64_t ts = 2 * (int64_t)res_record(res_s_[p]);
+                T *row = L.res_tab + ores + j * ts, *col = row + nres;
+                ResTabJob<T> jb{q_row, sc_row, sc_col, (int)n, res_s_[p], bd, be, row, sym ? col : nullptr};
+                rjobs.push_back(jb);
+                if (!sym) {
+                    jb.q = q_col;
+                    jb.row = nullptr;
+                    jb.col = col;
+                    rjobs.push_back(jb);
+                }
+                continue;
+            }
+            const int nb = nb_[p];
+            const int64_t ts = 2 * (int64_t)kTabs * nb * S, cs = 2 * 3 * (int64_t)nbp_of(nb);
+            T *row = L.tab + of + j * ts, *col = row + nfac, *ch_row = L.ch + oc + j * cs, *ch_col = ch_row + nch;
+            FacJob<T> jb{q_row, sc_row, sc_col, (int)n, nb, S, bd, be, row, sym ? col : nullptr,
+                         ch_row, sym ? ch_col : nullptr};
+            jobs.push_back(jb);
+            if (!sym) {
+                jb.q = q_col;
+                jb.sc1 = sc_col;
+                jb.out1 = col;
+                jb.ch1 = ch_col;
+                jobs.push_back(jb);
+            }
+        }
+        if (res_s_[p]) {
+            ores += L.J[p] * 2 * (int64_t)res_record(res_s_[p]);
+        } else {
+            of += L.J[p] * 2 * (int64_t)kTabs * nb_[p] * S;
+            oc += L.J[p] * 2 * 3 * (int64_t)nbp_of(nb_[p]);
+        }
+    }
+    // work items of the row passes, the column passes and the recurrences; resident items
+    std::vector<SwItem<T>> it[3];
+    std::vector<std::vector<ResItem<T>>> rit;
+    const int R = kPassLines / S;
+    for (int p : order_) {
+        const int nb = nb_[p], rs = res_s_[p], Sp = rs ? 32 : S;
+        const int64_t quarter = (int64_t)nb * nb * Sp * Sp, squarter = (int64_t)nb * nb * S;
+        size_t rc = 0;
+        if (rs) {
+            const int C = resident_cluster((int)((ns_[p] + 1) / 2), rs);
+            while (rc < L.res.size() && (L.res[rc].S != rs || L.res[rc].C != C)) ++rc;
+            if (rc == L.res.size()) {
+                ResClass c;
+                c.S = rs;
+                c.C = C;
+                L.res.push_back(c);
+                rit.emplace_back();
+            }
+        }
+        for (int r = 0; r < nrhs_; ++r)
+            for (int qd = 0; qd < 4; ++qd) {
+                const int rp = qd >> 1, cp = qd & 1;
+                if (ns_[p] <= std::max(rp, cp)) continue;  // n = 1: one quarter only
+                const int64_t x0 = offT_[p] + ((int64_t)r * 4 + qd) * quarter;
+                if (rs) {
+                    ResItem<T> x;
+                    x.xoff = x0;
+                    x.foff = off64_[p] + (int64_t)r * ns_[p] * ns_[p];
+                    x.tabR = L.res_tab + otab[p] + cp * res_record(rs);
+                    x.tabC = L.res_tab + nres + otab[p] + rp * res_record(rs);
+                    x.s = bands64_ + ob64_[p] + 2 * ns_[p];
+                    x.out_scale = -1.0 / ky_;
+                    x.prob = p;
+                    x.J = L.J[p];
+                    x.n = (int)ns_[p];
+                    x.lnb = nb;
+                    x.rp = rp;
+                    x.cp = cp;
+                    rit[rc].push_back(x);
+                    continue;
+                }
+                SwItem<T> x;
+                x.soff = offS_[p] + ((int64_t)r * 4 + qd) * squarter;
+                x.tabR = L.tab + otab[p] + (int64_t)cp * kTabs * nb * S;
+                x.tabC = L.tab + nfac + otab[p] + (int64_t)rp * kTabs * nb * S;
+                x.chR = L.ch + och[p] + cp * 3 * nbp_of(nb);
+                x.chC = L.ch + nch + och[p] + rp * 3 * nbp_of(nb);
+                x.prob = p;
+                x.J = L.J[p];
+                x.nb = (unsigned short)nb;
+                for (int b0 = 0; b0 < nb; b0 += R)
+                    for (int b1 = 0; b1 < nb; ++b1) {
+                        x.b0 = (unsigned short)b0;
+                        x.b1 = (unsigned short)b1;
+                        x.n_blk = (unsigned short)std::min(R, nb - b0);
+                        x.xoff = x0 + ((int64_t)b0 * nb + b1) * S * S;
+                        it[0].push_back(x);
+                    }
+                for (int b0 = 0; b0 < nb; ++b0)
+                    for (int b1 = 0; b1 < nb; b1 += R) {
+                        x.b0 = (unsigned short)b0;
+                        x.b1 = (unsigned short)b1;
+                        x.n_blk = (unsigned short)std::min(R, nb - b1);
+                        x.xoff = x0 + ((int64_t)b0 * nb + b1) * S * S;
+                        it[1].push_back(x);
+                    }
+                if (!fused_)
+                    for (int b1 = 0; b1 < nb * S / 32; ++b1) {
+                        x.b0 = 0;
+                        x.b1 = (unsigned short)b1;
+                        x.n_blk = 0;
+                        x.xoff = x0;
+                        it[2].push_back(x);
+                    }
+            }
+    }
+    cudaError_t e1 = cudaSuccess;
+    for (int w = 0; w < 3 && e1 == cudaSuccess; ++w) {
+        L.nitems[w] = (int64_t)it[w].size();
+        e1 = dalloc(&L.items[w], it[w].size());
+        if (e1 == cudaSuccess)
+            e1 = cudaMemcpyAsync(L.items[w], it[w].data(), sizeof(SwItem<T>) * it[w].size(), cudaMemcpyHostToDevice, cap_);
+    }
+    for (size_t c = 0; c < L.res.size() && e1 == cudaSuccess; ++c) {
+        L.res[c].nitems = (int64_t)rit[c].size();
+        e1 = dalloc(&L.res[c].items, rit[c].size());
+        if (e1 == cudaSuccess)
+            e1 = cudaMemcpyAsync(L.res[c].items, rit[c].data(), sizeof(ResItem<T>) * rit[c].size(), cudaMemcpyHostToDevice,
+                                 cap_);
+    }
+    auto upload = [&](int slot, const void *src, size_t bytes) -> void * {
+        if (e1 == cudaSuccess) e1 = cudaMalloc(&scratch.p[slot], bytes);
+        if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(scratch.p[slot], src, bytes, cudaMemcpyHostToDevice, cap_);
+        return scratch.p[slot];
+    };
+    if (!jobs.empty()) {
+        const FacJob<T> *d = (const FacJob<T> *)upload(0, jobs.data(), sizeof(FacJob<T>) * jobs.size());
+        if (e1 == cudaSuccess) e1 = launch_fac_tables<T>(d, (int)jobs.size(), cap_);
+    }
+    if (!rjobs.empty()) {
+        const ResTabJob<T> *d = (const ResTabJob<T> *)upload(1, rjobs.data(), sizeof(ResTabJob<T>) * rjobs.size());
+        if (e1 == cudaSuccess) e1 = launch_resident_tables<T>(d, (int)rjobs.size(), cap_);
+    }
+    // the host vectors and the scratch must outlive the asynchronous work
+    const cudaError_t e2 = cudaStreamSynchronize(cap_);
+    ENG_CK(e1);
+    ENG_CK(e2);
+    return FPS_OK;
+}
+
+template <typename T>
+ResArgs<T> SweepEngine<T>::res_args(const ResClass &c, const double *F, double *X) const
+{
+    ResArgs<T> a;
+    a.items = c.items;
+    a.nitems = c.nitems;
+    a.S = c.S;
+    a.C = c.C;
+    a.active = d_active_;
+    a.masked = d_active_ + ns_.size();
+    a.X = X_;
+    a.D = D_;
+    a.F = F;
+    a.out = X;
+    return a;
 }
 
 template <typename T>
@@ -601,7 +721,7 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
     const SwArgs<T> ar = args(L, 0), ac = args(L, 1), ach = args(L, 2);
     ENG_CK(cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    const bool ins = instrument_ && (int)L.ev.size() == 4 * L.Jmax;
+    const bool ins = instrument_ && (int)L.ev.size() == 4 * L.Jstream + 2;
     auto rec = [&](int k) {
         if (ins && e == cudaSuccess) e = cudaEventRecordWithFlags(L.ev[k], cap_, cudaEventRecordExternal);
     };
@@ -610,8 +730,11 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
         if (e == cudaSuccess) e = r;
         ++L.launches;
     };
-    run(launch_row_sums<T>(ac, cap_));
-    for (int j = 0; j < L.Jmax && e == cudaSuccess; ++j) {
+    rec(4 * L.Jstream);
+    for (const ResClass &c : L.res) run(launch_resident<T>(res_args(c, nullptr, nullptr), cap_));
+    rec(4 * L.Jstream + 1);
+    if (streams_) run(launch_row_sums<T>(ac, cap_));
+    for (int j = 0; j < L.Jstream && e == cudaSuccess; ++j) {
         if (!fused_) run(launch_chain<T>(ach, 0, j, cap_));
         rec(4 * j);
         run(launch_row_pass<T>(ar, j, cap_));
@@ -647,10 +770,18 @@ template <typename T>
 int SweepEngine<T>::solve_plain(const double *F, double *X, cudaStream_t st, std::string &err)
 {
     if constexpr (sizeof(T) == 8) {
-        const TileArgs ta = tiles(false);
+        if (!streams_ && !instrument_) {  // scale-in, all iterations and scale-out in one launch per class
+            for (const ResClass &c : levels_[0].res) {
+                ENG_CK(launch_resident<T>(res_args(c, F, X), st));
+                ++launches_last;
+            }
+            levels_used_.push_back(0);
+            rounds_last = 1;
+            return FPS_OK;
+        }
         ENG_CK(launch_scale_in<double>(tiles(true), F, nullptr, X_, nullptr, st));
         ENG_CK(cudaGraphLaunch(levels_[0].graph, st));
-        ENG_CK(launch_finalize_out(ta, args(levels_[0], 0), X, st));
+        ENG_CK(launch_finalize_out(tiles(false), D_, X, st));
         ENG_CK(cudaMemcpyAsync(h_err_, err_, sizeof(int), cudaMemcpyDeviceToHost, st));
         levels_used_.push_back(0);
         launches_last = 2 + levels_[0].launches;
@@ -777,7 +908,7 @@ int SweepEngine<T>::set_instrument(bool on, std::string &err)
         for (cudaEvent_t e : L.ev) cudaEventDestroy(e);
         L.ev.clear();
         if (on) {
-            L.ev.resize(4 * (size_t)L.Jmax);
+            L.ev.resize(4 * (size_t)L.Jstream + 2);
             for (auto &e : L.ev) ENG_CK(cudaEventCreate(&e));
         }
         int st = build_graph(L, err);
@@ -801,11 +932,19 @@ int SweepEngine<T>::kernel_times(int *count, double *total_ms, double *alg_bytes
         if (std::find(seen.begin(), seen.end(), li) != seen.end()) continue;
         seen.push_back(li);
         const Level &L = levels_[li];
-        if ((int)L.ev.size() != 4 * L.Jmax) continue;
+        if ((int)L.ev.size() != 4 * L.Jstream + 2) continue;
+        if (!L.res.empty()) {  // the resident launches alternate row and column solves
+            float t = 0.f;
+            ENG_CK(cudaEventElapsedTime(&t, L.ev[4 * L.Jstream], L.ev[4 * L.Jstream + 1]));
+            rms += 0.5 * t;
+            cms += 0.5 * t;
+        }
         for (int j = 0; j < L.Jmax; ++j) {
             float t0 = 0.f, t1 = 0.f;
+            if (j < L.Jstream) {
             ENG_CK(cudaEventElapsedTime(&t0, L.ev[4 * j], L.ev[4 * j + 1]));
             ENG_CK(cudaEventElapsedTime(&t1, L.ev[4 * j + 2], L.ev[4 * j + 3]));
+            }
             rms += t0;
             cms += t1;
             c += 2;

@@ -7,6 +7,7 @@
 #include <string>
 #include <vector>
 
+#include "resident.cuh"
 #include "sweep.cuh"
 
 namespace fps {
@@ -54,22 +55,34 @@ public:
 
 private:
     using T2 = typename Vec2<T>::type;
+    // Problems whose quarters stay in one cluster's shared memory (resident.cuh), by
+    // segment length and cluster size: one launch of all their iterations.
+    struct ResClass {
+        int S, C;
+        ResItem<T> *items = nullptr;
+        int64_t nitems = 0;
+    };
     struct Level {
         double tol = 0;
-        int Jmax = 0;
+        int Jmax = 0, Jstream = 0;  // largest J of all and of the streamed problems
         std::vector<int> J;
         T *tab = nullptr, *ch = nullptr;  // solve and summary tables, segment coefficients: rows, then columns
+        T *res_tab = nullptr;             // records of the resident problems, likewise
         SwItem<T> *items[3] = {nullptr, nullptr, nullptr};  // row passes, column passes, recurrences
         int64_t nitems[3] = {0, 0, 0};
+        std::vector<ResClass> res;
         int64_t launches = 0;             // kernels of the graph
         cudaGraphExec_t graph = nullptr;
-        std::vector<cudaEvent_t> ev;  // 4 per iteration when instrumented
+        std::vector<cudaEvent_t> ev;  // when instrumented: 4 per iteration, 2 around the resident launches
     };
     int build_graph(Level &L, std::string &err);
     int autotune(const std::vector<int64_t> &ns, int nrhs, double tol, bool tight, std::string &err);
     int time_level(size_t li, int reps, float &ms, std::string &err);
     int time_chain(int mode, float &ms, std::string &err);
     SwArgs<T> args(const Level &L, int which) const;
+    ResArgs<T> res_args(const ResClass &c, const double *F, double *X) const;
+    int build_tables(Level &L, int level, const std::vector<double> &lo, const std::vector<double> &hi,
+                     std::string &err);
     TileArgs tiles(bool padded) const;
     void set_active();
     int solve_refine(const double *F, double *X, cudaStream_t st, std::string &err);
@@ -80,7 +93,9 @@ private:
     double tol_ = 0;
     double kx_ = 1.0, ky_ = 1.0;
     cudaStream_t cap_ = nullptr;
-    std::vector<int> nb_;  // blocks per side of a quarter
+    std::vector<int> nb_;      // blocks per side of a quarter (of 32 for resident problems)
+    std::vector<int> res_s_;   // resident problems: segment length; 0: streamed by the passes
+    bool streams_ = false;     // any problem is streamed
     int max_nb_ = 0;
     bool fused_ = false;   // the passes run the segment recurrences
     std::vector<int64_t> off64_, offT_, offS_;
@@ -98,6 +113,8 @@ private:
     unsigned long long *d_smax_ = nullptr, *d_rmax_ = nullptr, *h_smax_ = nullptr, *h_rmax_ = nullptr;
     int *h_err_ = nullptr;
     std::vector<Level> levels_;
+    std::vector<int64_t> ob64_;  // offset of each problem's bands in bands64_
+    std::vector<int> order_;     // problems, largest first
     std::vector<int> levels_used_;
     bool instrument_ = false;
     std::vector<void *> allocs_;

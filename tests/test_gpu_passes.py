@@ -1,10 +1,11 @@
-"""Pass kernels of the square solve at the edges of their blocks, tiles and segment
-counts, against the CPU oracle through the C ABI.
+"""Square solves at the edges of their kernels' blocks, tiles and segment counts, against
+the CPU oracle through the C ABI.
 
-A quarter (one parity per direction) has ceil(n/2) unknowns per side in blocks of 32
-(FP64, FP32 segment length 64) or 64 (FP32 segment length 128) and tiles of 128 lines;
-up to 16 segments per line the passes run the segment recurrence themselves, beyond that
-the chain kernel does (FP64: n > 1024; FP32: n > 1024 or n > 2048).  Bars: the FP64 and
+One launch (resident kernel): quarters of m = ceil(n/2) <= 16 S unknowns for the compiled
+segment lengths S, FP64 up to n = 512, FP32 up to n = 1024.  Streamed: blocks of 32 (FP64,
+FP32 segment length 64) or 64 (FP32 segment length 128) unknowns, tiles of 128 lines; up
+to 16 segments per line the passes run the segment recurrence themselves, beyond that the
+chain kernel does (FP64: n > 1024; FP32: n > 1024 or n > 2048).  Bars: the FP64 and
 refinement bars of the workload definition."""
 import numpy as np
 import pytest
@@ -35,16 +36,38 @@ def _relmax(a, b):
     return float(np.abs(a - b).max() / np.abs(b).max())
 
 
-# one block and its neighbours, one tile of 128 lines, the last fused size and the first
-# size with the chain kernel (1024 / 1025), a last block of one unknown (1089)
-@pytest.mark.parametrize("n", [66, 127, 128, 129, 255, 256, 258, 1024, 1025, 1089])
-def test_fp64_block_edges(api, n):
+def _check_fp64(api, n):
     F = np.stack([inputs.square_rhs(n, 40 + n), inputs.square_rhs(n, 41 + n, power=1)])
     plan = api.plan_create(n, 2, 1e-13, "fp64", nrhs=2)
     X = api.poisson_square_solve(plan, torch.from_numpy(F).cuda()).cpu().numpy()
+    launches = api.plan_info(plan)["kernel_launches"]
     api.plan_destroy(plan)
     for r in range(2):
         assert _relmax(X[r], oracle.poisson_square(F[r], 1e-13)) <= TOL_FP64, r
+    return launches
+
+
+# full and just overfull segments of every compiled length: n = 32 S and 32 S + 1
+@pytest.mark.parametrize("S", [1, 2, 3, 4, 5, 6, 8, 10, 12, 14])
+def test_fp64_resident_edges(api, S):
+    for n in (32 * S - 1, 32 * S, 32 * S + 1):
+        assert _check_fp64(api, n) == 1, n
+
+
+# the last resident size; a last block of one unknown (513, 577, 1025, 1089); full blocks;
+# the last size without and the first with the chain kernel (1024, 1025)
+@pytest.mark.parametrize("n", [511, 512, 513, 514, 576, 577, 640, 1024, 1025, 1089])
+def test_fp64_block_edges(api, n):
+    assert (_check_fp64(api, n) == 1) == (n <= 512)
+
+
+@pytest.mark.parametrize("n", [512, 513, 640, 641, 768, 769, 896, 897, 1023, 1024, 1025])
+def test_refine_resident_edges(api, n):
+    F = inputs.square_rhs(n, 60 + n)
+    plan = api.plan_create(n, 2, 1e-10, "fp32_refine")
+    X = api.poisson_square_solve(plan, torch.from_numpy(F).cuda()).cpu().numpy()
+    api.plan_destroy(plan)
+    assert _relmax(X, oracle.poisson_square(F, 1e-13)) <= TOL_REFINE
 
 
 @pytest.mark.parametrize("seg,chain", [(64, 1), (64, 2), (128, 1), (128, 2)])
@@ -68,10 +91,10 @@ def test_refine_segment_counts(api, tmp_path, monkeypatch, seg, chain):
         o += n * n
 
 
-def test_nonfinite_input_leaves_no_trace(api):
-    """The passes work in place: a right-hand side with NaN and Inf must not reach the next
+@pytest.mark.parametrize("n", [101, 601])
+def test_nonfinite_input_leaves_no_trace(api, n):
+    """The kernels work in place: a right-hand side with NaN and Inf must not reach the next
     solve of the plan through the unused positions of the blocks."""
-    n = 101
     F = torch.from_numpy(inputs.square_rhs(n, 5)).cuda()
     plan = api.plan_create(n, 2, 1e-13, "fp64")
     X = api.poisson_square_solve(plan, F).clone()
