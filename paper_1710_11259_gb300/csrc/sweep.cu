@@ -583,37 +583,110 @@ __global__ void chain_kernel(SwArgs<T> A, int dir, int j)
 }
 
 // ---------------------------------------------------------------------------
-// Elementwise kernels over 32 x 32 tiles of the n x n region (caller layout); the
-// quarter-block arrays are addressed element by element.
+// Elementwise kernels.  GB300's FP64 pipe takes 64 cycles of an SM quadrant per warp
+// instruction, conversions and comparisons included (and 64-bit integer comparisons
+// measured the same), so these kernels convert between float and double, scale by powers
+// of two and compare magnitudes with 32-bit integer instructions, and keep the FP64
+// operations to the multiply-adds of the formulas.  A product alone is written as a
+// multiply-add with zero: multiplications measured 76 cycles.
 // ---------------------------------------------------------------------------
-struct TileView {
-    int n, nb, log_s, prob, rhs, pair;
-    int64_t off64, offT;
-    const double *d, *e, *s;
-    double kx, ky;
-    int bx, by;
+__device__ __forceinline__ double times(double a, double b) { return fma(a, b, 0.0); }
+
+// Largest magnitude as the bit pattern of |x| (NaN and Inf are above every finite value).
+struct MaxBits {
+    unsigned hi = 0, lo = 0;
+    __device__ __forceinline__ void add(unsigned h, unsigned l)
+    {
+        const bool gt = h > hi || (h == hi && l > lo);
+        hi = gt ? h : hi;
+        lo = gt ? l : lo;
+    }
+    __device__ __forceinline__ void add(double x)
+    {
+        add((unsigned)__double2hiint(x) & 0x7fffffffu, (unsigned)__double2loint(x));
+    }
+    __device__ __forceinline__ double value() const { return __hiloint2double((int)hi, (int)lo); }
 };
-__device__ __forceinline__ TileView tile_view(const TileArgs &t, int64_t idx = -1)
+
+// (double)f, subnormal floats read as zero.
+__device__ __forceinline__ double widen(float f)
 {
-    const int4 q = t.tiles[idx < 0 ? (int64_t)blockIdx.x : idx];
-    const TileProb &p = t.probs[q.x >> 8];
+    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+    unsigned hi = (a >> 3) + 0x38000000u;
+    if (a >= 0x7f800000u) hi |= 0x7ff00000u;  // Inf, NaN
+    if (a < 0x00800000u) hi = 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), a < 0x00800000u ? 0 : (int)(u << 29));
+}
+
+// x 2^54 where the scale is so small that subnormal doubles count (k is raised to match);
+// kept out of line, so that the product is not executed speculatively.
+__device__ __noinline__ double lift_subnormal(double x) { return x * 18014398509481984.0; }
+
+// (float)(x 2^-k), rounded to nearest even, -896 <= k; below the normal range zero, above
+// it Inf.
+__device__ __forceinline__ float narrow_scaled(double x, int k)
+{
+    const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
+    const unsigned sign = (unsigned)__double2hiint(x) & 0x80000000u;
+    const int e = (int)(h >> 20) - 896 - k;  // exponent field of the float
+    unsigned f = ((h - ((unsigned)(896 + k) << 20)) << 3) | (lo >> 29);
+    const unsigned rest = lo << 3;
+    f += rest > 0x80000000u || (rest == 0x80000000u && (f & 1u)) ? 1u : 0u;
+    if (e <= 0) f = 0u;
+    if (e >= 255) f = h >= 0x7ff00000u ? 0x7fc00000u : 0x7f800000u;  // the residual's NaN or Inf reaches the host
+    return __uint_as_float(sign | f);
+}
+
+// Scale of a pair's FP32 iteration: 2^k <= smax < 2^(k+1) (k >= -1022).
+__device__ __forceinline__ int scale_exponent(unsigned long long smax_bits)
+{
+    const int e = (int)(smax_bits >> 52);
+    return (e > 0 ? e : 1) - 1023;
+}
+__device__ __forceinline__ double power_of_two(int k)
+{
+    return __hiloint2double((k + 1023) << 20, 0);
+}
+
+// Tiles: q.x >> 8 problem, q.x & 255 right-hand side.
+struct TileView {
+    const TileProb *p;
+    int n, nb, ls, pair, by, bx;
+    int64_t off64, off;
+};
+__device__ __forceinline__ TileView tile_view(const TileArgs &t, int64_t idx)
+{
+    const int4 q = t.tiles[idx];
     TileView v;
-    v.prob = q.x >> 8;
-    v.rhs = q.x & 255;
-    v.n = p.n;
-    v.nb = p.nb;
-    v.log_s = p.log_s;
-    v.off64 = p.off64 + (int64_t)v.rhs * p.n * p.n;
-    v.offT = p.off + (int64_t)v.rhs * p.rhs;
-    v.d = p.d;
-    v.e = p.e;
-    v.s = p.s;
-    v.pair = p.pair0 + v.rhs;
-    v.kx = p.kx;
-    v.ky = p.ky;
-    v.bx = q.y * 32;
-    v.by = q.z * 32;
+    v.p = t.probs + (q.x >> 8);
+    const int rhs = q.x & 255;
+    v.n = v.p->n;
+    v.nb = v.p->nb;
+    v.ls = v.p->log_s;
+    v.pair = v.p->pair0 + rhs;
+    v.off64 = v.p->off64 + (int64_t)rhs * v.n * v.n;
+    v.off = v.p->off + (int64_t)rhs * v.p->rhs;
+    v.bx = q.y;
+    v.by = q.z;
     return v;
+}
+// Offset of element (a, b) of quarter q in the passes' arrays, and in the FP64 arrays of
+// the refinement (the same blocks, rows in natural order), from the pair's offset v.off:
+// below 2^31, n <= 40000.
+__device__ __forceinline__ unsigned block_base(const TileView &v, int q, int a, int b)
+{
+    return ((unsigned)(q * v.nb + (a >> v.ls)) * v.nb + (b >> v.ls)) << (2 * v.ls);
+}
+template <typename T>
+__device__ __forceinline__ unsigned quarter_pos(const TileView &v, int q, int a, int b)
+{
+    const int S = 1 << v.ls;
+    return block_base(v, q, a, b) + block_pos<T>(a & (S - 1), b & (S - 1), S);
+}
+__device__ __forceinline__ unsigned plain_pos(const TileView &v, int q, int a, int b)
+{
+    const int S = 1 << v.ls;
+    return block_base(v, q, a, b) + ((a & (S - 1)) << v.ls) + (b & (S - 1));
 }
 
 // The contiguous run of tiles of this CTA, for the reduction kernels (tiles are
@@ -626,184 +699,259 @@ __device__ __forceinline__ void tile_run(int64_t ntiles, int64_t &t0, int64_t &t
     t1 = t0 + per < ntiles ? t0 + per : ntiles;
 }
 
-// Offset of element (i, k) of the n x n matrix in the quarter-block arrays.
-template <typename T>
-__device__ __forceinline__ int64_t quarter_pos(const TileView &v, int i, int k)
+// Largest magnitude of the CTA.
+__device__ __forceinline__ void block_max_to(const MaxBits &m, unsigned long long *out)
 {
-    const int S = 1 << v.log_s, q = (i & 1) * 2 + (k & 1), a = i >> 1, b = k >> 1;
-    const int64_t blk = ((int64_t)q * v.nb + (a >> v.log_s)) * v.nb + (b >> v.log_s);
-    return v.offT + (blk << (2 * v.log_s)) + block_pos<T>(a & (S - 1), b & (S - 1), S);
-}
-
-__global__ void __launch_bounds__(256) finalize_out_kernel(TileArgs t, const double *__restrict__ D,
-                                                           double *__restrict__ X)
-{
-    const TileView v = tile_view(t);
-    const double sc = -1.0 / v.ky;
-    for (int r = threadIdx.y; r < 32; r += 8) {
-        const int i = v.by + r, k = v.bx + threadIdx.x;
-        if (i < v.n && k < v.n)
-            X[v.off64 + (int64_t)i * v.n + k] = sc * D[quarter_pos<double>(v, i, k)] * v.s[i] * v.s[k];
-    }
-}
-
-__device__ __forceinline__ double flag_nonfinite(double x, double local)
-{
-    // NaN and Inf both become +Inf so that the maximum flags them (fmax drops NaN)
-    return (x <= 1.7976931348623157e308) ? fmax(local, x) : __longlong_as_double(0x7ff0000000000000LL);
-}
-
-__device__ __forceinline__ void block_max_to(double local, unsigned long long *out)
-{
-    for (int off = 16; off > 0; off >>= 1) local = fmax(local, __shfl_xor_sync(0xffffffffu, local, off));
-    __shared__ double wmax[8];
+    unsigned long long local = ((unsigned long long)m.hi << 32) | m.lo;
+    for (int off = 16; off > 0; off >>= 1) local = max(local, __shfl_xor_sync(0xffffffffu, local, off));
+    __shared__ unsigned long long wmax[8];
     if (threadIdx.x == 0) wmax[threadIdx.y] = local;
     __syncthreads();
     if (threadIdx.x == 0 && threadIdx.y == 0) {
-        double bm = 0.0;
-        for (int q = 0; q < (int)blockDim.y; ++q) bm = fmax(bm, wmax[q]);
-        atomicMax(out, (unsigned long long)__double_as_longlong(bm));
+        unsigned long long bm = 0;
+        for (int q = 0; q < (int)blockDim.y; ++q) bm = max(bm, wmax[q]);
+        atomicMax(out, bm);
     }
     __syncthreads();  // wmax is reused by the next reduction
 }
 
+// Natural 64 x 64 tiles: one multiplication per element (|F| s_i, largest over the
+// thread's rows, then times s_k).
 __global__ void __launch_bounds__(256) absmax_kernel(TileArgs t, const double *__restrict__ F,
                                                      unsigned long long *__restrict__ smax)
 {
     int64_t t0, t1;
     tile_run(t.ntiles, t0, t1);
-    double local = 0.0;
+    MaxBits local;
     int cur = -1;
     for (int64_t tt = t0; tt < t1; ++tt) {
         const TileView v = tile_view(t, tt);
         if (v.pair != cur) {
             if (cur >= 0) block_max_to(local, smax + cur);
-            local = 0.0;
+            local = MaxBits();
             cur = v.pair;
         }
-        for (int r = threadIdx.y; r < 32; r += 8) {
-            const int i = v.by + r, k = v.bx + threadIdx.x;
-            if (i < v.n && k < v.n)
-                local = flag_nonfinite(fabs(F[v.off64 + (int64_t)i * v.n + k] * v.s[i] * v.s[k]), local);
+        const double *s = v.p->s;
+        double f[8][2], si[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int i = v.by * 64 + threadIdx.y + 8 * q;
+            const double *row = F + v.off64 + (int64_t)i * v.n;
+            si[q] = i < v.n ? s[i] : 0.0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = v.bx * 64 + 32 * h + threadIdx.x;
+                f[q][h] = i < v.n && k < v.n ? row[k] : 0.0;
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            MaxBits m;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) m.add(times(f[q][h], si[q]));
+            const int k = v.bx * 64 + 32 * h + threadIdx.x;
+            if (k < v.n) local.add(times(m.value(), s[k]));
         }
     }
     if (cur >= 0) block_max_to(local, smax + cur);
 }
 
+// Pairs and problems with something to solve: 0 < smax < Inf (masked: any problem without).
+__global__ void init_masks_kernel(const unsigned long long *__restrict__ smax, int np, int nrhs,
+                                  int *__restrict__ pair_active, int *__restrict__ active, int *__restrict__ masked)
+{
+    for (int p = threadIdx.x; p < np; p += blockDim.x) {
+        int any = 0;
+        for (int r = 0; r < nrhs; ++r) {
+            const unsigned long long b = smax[p * nrhs + r];
+            const int on = b > 0 && b < 0x7ff0000000000000ULL;
+            pair_active[p * nrhs + r] = on;
+            any |= on;
+        }
+        active[p] = any;
+        if (!any) *masked = 1;
+    }
+}
+
+// Tiles of 32 x 32 positions of all four quarters (64 x 64 natural), padded region: F~ in
+// the FP64 blocks (if Ft), rho0 = F~ 2^-k (float) or F~ (double) in the passes' blocks,
+// zero at unused positions.
 template <typename T>
 __global__ void __launch_bounds__(256) scale_in_kernel(TileArgs t, const double *__restrict__ F, double *__restrict__ Ft,
                                                        T *__restrict__ rho0, const unsigned long long *__restrict__ smax)
 {
-    const TileView v = tile_view(t);
-    double inv = 1.0;
-    if (smax) {
-        const double sF = __longlong_as_double((long long)smax[v.pair]);
-        inv = sF > 0.0 ? 1.0 / sF : 0.0;
+    const TileView v = tile_view(t, blockIdx.x);
+    const double *s = v.p->s;
+    const int k = smax ? scale_exponent(smax[v.pair]) : 0;
+    const int b = v.bx * 32 + threadIdx.x;
+    double sk[2], f[8][2], si[8];
+#pragma unroll
+    for (int cp = 0; cp < 2; ++cp) sk[cp] = 2 * b + cp < v.n ? s[2 * b + cp] : 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int i = v.by * 64 + threadIdx.y + 8 * q;
+        si[q] = i < v.n ? s[i] : 0.0;
+#pragma unroll
+        for (int cp = 0; cp < 2; ++cp)
+            f[q][cp] = i < v.n && 2 * b + cp < v.n ? F[v.off64 + (int64_t)i * v.n + 2 * b + cp] : 0.0;
     }
-    for (int r = threadIdx.y; r < 32; r += 8) {
-        const int i = v.by + r, k = v.bx + threadIdx.x;
-        double val = 0.0;
-        if (i < v.n && k < v.n) {
-            val = F[v.off64 + (int64_t)i * v.n + k] * v.s[i] * v.s[k];
-            if (Ft) Ft[v.off64 + (int64_t)i * v.n + k] = val;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int i = v.by * 64 + threadIdx.y + 8 * q, a = i >> 1, rp = i & 1;
+#pragma unroll
+        for (int cp = 0; cp < 2; ++cp) {
+            const int qd = rp * 2 + cp;
+            const double val = times(times(f[q][cp], si[q]), sk[cp]);
+            if (Ft && i < v.n && 2 * b + cp < v.n) Ft[v.off + plain_pos(v, qd, a, b)] = val;
+            T *out = rho0 + v.off + quarter_pos<T>(v, qd, a, b);
+            if constexpr (sizeof(T) == 4) *out = k < -896 ? narrow_scaled(lift_subnormal(val), k + 54) : narrow_scaled(val, k);
+            else *out = val;
         }
-        rho0[quarter_pos<T>(v, i, k)] = (T)(val * inv);  // unused positions: zero
     }
 }
 
-// Yout = Y - s D / ky; R = F~ - A~ Yout - Yout A~; rho0 = R / s; rmax = max |R|.
+// X[i][k] = sc Z s_i s_k, Z in the passes' blocks (FP64 solve) or in the FP64 blocks
+// (PLAIN, refinement).  Tiles as in scale_in_kernel; even and odd columns are put in
+// natural order by shuffles, so that every store is contiguous.
+template <bool PLAIN>
+__global__ void __launch_bounds__(256) scale_out_kernel(TileArgs t, const double *__restrict__ Z, double *__restrict__ X)
+{
+    const TileView v = tile_view(t, blockIdx.x);
+    const double *s = v.p->s;
+    const double sc = PLAIN ? 1.0 : -v.p->inv_ky;
+    const int lane = threadIdx.x, b = v.bx * 32 + lane, m0 = (v.n + 1) / 2;
+    double sk[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int kk = v.bx * 64 + 32 * h + lane;
+        sk[h] = kk < v.n ? (PLAIN ? s[kk] : sc * s[kk]) : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int rr = threadIdx.y + 8 * q, a = v.by * 32 + (rr >> 1), rp = rr & 1, i = 2 * a + rp;
+        if (i >= v.n) continue;  // the whole warp
+        double z[2];
+#pragma unroll
+        for (int cp = 0; cp < 2; ++cp) {
+            const unsigned pos = PLAIN ? plain_pos(v, rp * 2 + cp, a, b) : quarter_pos<double>(v, rp * 2 + cp, a, b);
+            z[cp] = b < m0 - (cp & v.n) ? Z[v.off + pos] : 0.0;
+        }
+        const double si = s[i];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int src = 16 * h + (lane >> 1);
+            const double e = __shfl_sync(0xffffffffu, z[0], src), o = __shfl_sync(0xffffffffu, z[1], src);
+            const int kk = v.bx * 64 + 32 * h + lane;
+            if (kk < v.n) X[v.off64 + (int64_t)i * v.n + kk] = times(times(lane & 1 ? o : e, si), sk[h]);
+        }
+    }
+}
+
+// Yout = Y - s D / ky; R = F~ - A~ Yout - Yout A~; rho0 = R / s; rmax = max |R|, with s the
+// power of two of the pair's scale.  In a quarter the products with A~ are 3-point
+// stencils with neighbours at distance one.  Tiles of 64 rows x 32 columns of a quarter;
 // Y and Yout are distinct buffers, so every CTA sees the same not-yet-updated halo.
-__global__ void __launch_bounds__(256) residual_kernel(TileArgs t, const double *__restrict__ Y,
+// Bound: the FP64 pipe, 7.1 operations per element (the update 1.1 with the halo, the
+// stencils 6).  n = 4096: 250 us (78 % of the pipe; 24 to 32 B per element of HBM would
+// take 80 us), 370 us with conversions left to the FP64 pipe and 64-bit comparisons;
+// n = 10^4: 1.5 ms, 3.5 ms on interleaved parities with a halo of two.
+constexpr int kResR = 64;
+__global__ void __launch_bounds__(256, 3) residual_kernel(TileArgs t, const double *__restrict__ Y,
                                                        double *__restrict__ Yout, const float *__restrict__ D,
                                                        const double *__restrict__ Ft, float *__restrict__ rho0,
                                                        const unsigned long long *__restrict__ smax,
                                                        unsigned long long *__restrict__ rmax,
                                                        const int *__restrict__ pair_active, int y_zero)
 {
-    __shared__ double Ys[36][37];
-    // stencil coefficients of the tile's rows and columns: -kx d_i, -kx e_{i-2}, -kx e_i
-    // and -ky d_k, -ky e_{k-2}, -ky e_k (formed once per tile, not per element)
-    __shared__ double cr[3][32], cc[3][32];
+    __shared__ double Ys[kResR + 2][35];
+    // stencil coefficients of the tile's rows and columns: -kx {d_i, e_{i-1}, e_i} and -ky
+    __shared__ double cr[3][kResR], cc[3][32];
     int64_t t0, t1;
     tile_run(t.ntiles, t0, t1);
-    double local = 0.0;
+    MaxBits local;
     int cur = -1;
-    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
     for (int64_t tt = t0; tt < t1; ++tt) {
         const TileView v = tile_view(t, tt);
-        const int n = v.n;
+        const int qd = v.bx & 3, bx = (v.bx >> 2) * 32, by = v.by * kResR, rp = qd >> 1, cp = qd & 1;
+        const int mr = (v.n - rp + 1) / 2, mc = (v.n - cp + 1) / 2;
         if (v.pair != cur) {
             if (cur >= 0) block_max_to(local, rmax + cur);
-            local = 0.0;
+            local = MaxBits();
             cur = v.pair;
         }
         if (!pair_active[v.pair]) {  // converged pair: carry its iterate over unchanged
-            for (int r = ty; r < 32; r += 8) {
-                const int i = v.by + r, k = v.bx + tx;
-                if (i < n && k < n) Yout[v.off64 + (int64_t)i * n + k] = y_zero ? 0.0 : Y[v.off64 + (int64_t)i * n + k];
-            }
+            for (int r = ty; r < kResR; r += 8)
+                if (by + r < mr && bx + tx < mc) {
+                    const int64_t pos = v.off + plain_pos(v, qd, by + r, bx + tx);
+                    Yout[pos] = y_zero ? 0.0 : Y[pos];
+                }
             continue;
         }
-        const double sF = __longlong_as_double((long long)smax[v.pair]);
-        const double inv = sF > 0.0 ? 1.0 / sF : 0.0, sD = -sF / v.ky;
-        for (int r = ty; r < 36; r += 8) {
-            const int i = v.by - 2 + r;
-            for (int cc = tx; cc < 36; cc += 32) {
-                const int k = v.bx - 2 + cc;
-                double val = 0.0;
-                if (i >= 0 && i < n && k >= 0 && k < n) {
-                    val = y_zero ? 0.0 : Y[v.off64 + (int64_t)i * n + k];
-                    val = fma(sD, (double)D[quarter_pos<float>(v, i, k)], val);
-                }
-                Ys[r][cc] = val;
-            }
+        const double *Yp = Y + v.off, *Fp = Ft + v.off;
+        double *Yo = Yout + v.off;
+        const float *Dp = D + v.off;
+        float *rho = rho0 + v.off;
+        const int k = scale_exponent(smax[v.pair]);
+        const double sD = -power_of_two(k) * v.p->inv_ky;
+        // all of the tile's loads in flight before the first is used
+        constexpr int kHalo = (kResR + 2) * 34, kIt = (kHalo + 255) / 256;
+        double yv[kIt], fv[kResR / 8];
+        float dv[kIt];
+#pragma unroll
+        for (int q = 0; q < kIt; ++q) {
+            const int idx = tid + 256 * q, r = idx / 34, c = idx - r * 34, a = by - 1 + r, b = bx - 1 + c;
+            const bool ok = a >= 0 && a < mr && b >= 0 && b < mc && idx < kHalo;
+            dv[q] = ok ? Dp[quarter_pos<float>(v, qd, a, b)] : 0.f;
+            yv[q] = ok && !y_zero ? Yp[plain_pos(v, qd, a, b)] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < kResR / 8; ++q) {
+            const int a = by + ty + 8 * q, b = bx + tx;
+            fv[q] = a < mr && b < mc ? Fp[plain_pos(v, qd, a, b)] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < kIt; ++q) {
+            const int idx = tid + 256 * q, r = idx / 34, c = idx - r * 34;
+            if (idx < kHalo) Ys[r][c] = fma(sD, widen(dv[q]), yv[q]);
         }
         {
-            const int q = ty * 32 + tx;  // 192 of the 256 threads form one coefficient each
-            if (q < 192) {
-                const int which = q >> 5, w = q & 31, set = which % 3;
-                const bool row = which < 3;
-                const int idx = (row ? v.by : v.bx) + w;
-                const double sc = row ? v.kx : v.ky;
+            const double *nd = v.p->nd, *ne = v.p->ne;  // -kx d, -kx e (rows), then -ky d, -ky e
+            for (int q = tid; q < 3 * (kResR + 32); q += 256) {
+                const bool row = q < 3 * kResR;
+                const int set = row ? q / kResR : (q - 3 * kResR) / 32, w = row ? q % kResR : (q - 3 * kResR) % 32;
+                const int a = (row ? by : bx) + w, full = 2 * a + (row ? rp : cp);
+                const double *dd = row ? nd : nd + v.n, *ee = row ? ne : ne + v.n;
                 double c = 0.0;
-                if (idx < n) {
-                    if (set == 0) c = -sc * v.d[idx];
-                    else if (set == 1) c = idx >= 2 ? -sc * v.e[idx - 2] : 0.0;
-                    else c = -sc * v.e[idx];  // e[idx] = 0 when idx + 2 >= n
-                }
-                (row ? cr : cc)[set][w] = c;
+                if (full < v.n) c = set == 0 ? dd[full] : (set == 1 ? (a >= 1 ? ee[full - 2] : 0.0) : ee[full]);
+                (row ? cr[set] : cc[set])[w] = c;  // e is zero where full + 2 >= n
             }
         }
         __syncthreads();
-        for (int r = ty; r < 32; r += 8) {
-            const int i = v.by + r, k = v.bx + tx;
-            if (i < n && k < n) {
-                const double y = Ys[r + 2][tx + 2];
-                double acc = Ft[v.off64 + (int64_t)i * n + k];
-                // halo entries outside [0, n) are zero in Ys, and so are their coefficients
-                acc = fma(cr[0][r] + cc[0][tx], y, acc);
-                acc = fma(cr[1][r], Ys[r][tx + 2], acc);
-                acc = fma(cr[2][r], Ys[r + 4][tx + 2], acc);
-                acc = fma(cc[1][tx], Ys[r + 2][tx], acc);
-                acc = fma(cc[2][tx], Ys[r + 2][tx + 4], acc);
-                Yout[v.off64 + (int64_t)i * n + k] = y;
-                local = flag_nonfinite(fabs(acc), local);
-                rho0[quarter_pos<float>(v, i, k)] = (float)(acc * inv);
+        const int b = bx + tx;
+        const double c0 = cc[0][tx], c1 = cc[1][tx], c2 = cc[2][tx];
+#pragma unroll
+        for (int q = 0; q < kResR / 8; ++q) {
+            const int r = ty + 8 * q, a = by + r;
+            if (a < mr && b < mc) {
+                const double y = Ys[r + 1][tx + 1];
+                const unsigned pos = plain_pos(v, qd, a, b);
+                double acc = fv[q];
+                acc = fma(cr[0][r], y, acc);
+                acc = fma(c0, y, acc);
+                acc = fma(cr[1][r], Ys[r][tx + 1], acc);
+                acc = fma(cr[2][r], Ys[r + 2][tx + 1], acc);
+                acc = fma(c1, Ys[r + 1][tx], acc);
+                acc = fma(c2, Ys[r + 1][tx + 2], acc);
+                Yo[pos] = y;
+                local.add(acc);
+                rho[quarter_pos<float>(v, qd, a, b)] =
+                    k < -896 ? narrow_scaled(lift_subnormal(acc), k + 54) : narrow_scaled(acc, k);
             }
         }
         __syncthreads();  // Ys is refilled by the next tile
     }
     if (cur >= 0) block_max_to(local, rmax + cur);
-}
-
-__global__ void __launch_bounds__(256) scale_out_kernel(TileArgs t, const double *__restrict__ Y, double *__restrict__ X)
-{
-    const TileView v = tile_view(t);
-    for (int r = threadIdx.y; r < 32; r += 8) {
-        const int i = v.by + r, k = v.bx + threadIdx.x;
-        if (i < v.n && k < v.n)
-            X[v.off64 + (int64_t)i * v.n + k] = Y[v.off64 + (int64_t)i * v.n + k] * v.s[i] * v.s[k];
-    }
 }
 
 // Launch on `st` as a dependent of the launch before it (see pdl_wait).
@@ -941,15 +1089,18 @@ cudaError_t launch_chain(const SwArgs<T> &a, int dir, int j, cudaStream_t st)
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_finalize_out(const TileArgs &t, const double *D, double *X, cudaStream_t st)
-{
-    finalize_out_kernel<<<(unsigned)t.ntiles, dim3(32, 8), 0, st>>>(t, D, X);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_absmax(const TileArgs &t, const double *F, unsigned long long *smax, cudaStream_t st)
 {
     absmax_kernel<<<reduction_grid(t.ntiles), dim3(32, 8), 0, st>>>(t, F, smax);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_init_masks(const unsigned long long *smax, int np, int nrhs, int *pair_active, int *active,
+                              int *masked, cudaStream_t st)
+{
+    const cudaError_t e = cudaMemsetAsync(masked, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    init_masks_kernel<<<1, 256, 0, st>>>(smax, np, nrhs, pair_active, active, masked);
     return cudaGetLastError();
 }
 
@@ -970,9 +1121,10 @@ cudaError_t launch_residual(const TileArgs &t, const double *Y, double *Yout, co
     return cudaGetLastError();
 }
 
-cudaError_t launch_scale_out(const TileArgs &t, const double *Y, double *X, cudaStream_t st)
+cudaError_t launch_scale_out(const TileArgs &t, const double *Z, bool plain, double *X, cudaStream_t st)
 {
-    scale_out_kernel<<<(unsigned)t.ntiles, dim3(32, 8), 0, st>>>(t, Y, X);
+    if (plain) scale_out_kernel<true><<<(unsigned)t.ntiles, dim3(32, 8), 0, st>>>(t, Z, X);
+    else scale_out_kernel<false><<<(unsigned)t.ntiles, dim3(32, 8), 0, st>>>(t, Z, X);
     return cudaGetLastError();
 }
 

@@ -121,15 +121,17 @@ struct SwArgs {
 };
 
 // Elementwise tile kernels of the solve around the ADI loop.  A tile item is
-// {problem * 256 + rhs, tile column, tile row, 0}, 32 x 32 tiles of the n x n region
-// (scale-in: of the padded region).
+// {problem * 256 + rhs, x, y, 0}: x, y in tiles of 64 x 64 elements (32 x 32 of every
+// quarter) of the live or of the padded region, or, for the residual, x = tile column * 4 +
+// quarter and y = tile row in tiles of 64 rows x 32 columns of a quarter.
 struct TileProb {
     int n, nb, log_s;       // nb: blocks of 2^log_s per side of a quarter
     int64_t off64;          // FP64 packing of the caller's arrays: offset of rhs 0 (rhs stride n*n)
     int64_t off, rhs;       // quarter-block arrays: offset of rhs 0, stride between right-hand sides
-    const double *d, *e, *s;  // FP64 bands of A~ (d, e zero-padded to length n) and 1/sqrt(E)
+    const double *s;        // 1/sqrt(E), n entries
+    const double *nd, *ne;  // {-kx d, -ky d} and {-kx e, -ky e}, n entries each (e zero-padded)
     int pair0;              // index of (problem, rhs 0) among all pairs
-    double kx, ky;          // scales of the two second derivatives (1, 1 on [-1,1]^2)
+    double inv_ky;          // 1 / scale of the second derivative along y
 };
 
 struct TileArgs {
@@ -169,22 +171,24 @@ cudaError_t launch_col_pass(const SwArgs<T> &a, int j, cudaStream_t st);
 template <typename T>
 cudaError_t launch_chain(const SwArgs<T> &a, int dir, int j, cudaStream_t st);
 
-// X = -D_s D D_s / ky straight into the caller's FP64 X.
-cudaError_t launch_finalize_out(const TileArgs &t, const double *D, double *X, cudaStream_t st);
-
 // Per (problem, rhs): smax = max |D_s F D_s| (bit patterns; must start at 0).
 cudaError_t launch_absmax(const TileArgs &t, const double *F, unsigned long long *smax, cudaStream_t st);
-// F~ = D_s F D_s (FP64, if Ft != nullptr) and rho0 = F~ / smax (T, quarter blocks, unused
-// positions set to zero; smax == nullptr: no scaling).  Tiles cover the padded region.
+// Masks of the pairs and problems with 0 < smax < Inf; *masked = any problem without one.
+cudaError_t launch_init_masks(const unsigned long long *smax, int np, int nrhs, int *pair_active, int *active,
+                              int *masked, cudaStream_t st);
+// F~ = D_s F D_s (FP64 blocks, if Ft != nullptr) and rho0 = F~ / s (passes' blocks, unused
+// positions set to zero), s the power of two below smax (smax == nullptr: s = 1).  Tiles
+// cover the padded region.
 template <typename T>
 cudaError_t launch_scale_in(const TileArgs &t, const double *F, double *Ft, T *rho0, const unsigned long long *smax,
                             cudaStream_t st);
-// Yout = Y - smax D / ky (Y read as zero if y_zero), R = F~ - A~ Yout - Yout A~, rho0 = R / smax,
+// Yout = Y - s D / ky (Y read as zero if y_zero), R = F~ - A~ Yout - Yout A~, rho0 = R / s,
 // rmax = max |R| per pair (bit patterns; must start at 0); inactive pairs copy Y.
 cudaError_t launch_residual(const TileArgs &t, const double *Y, double *Yout, const float *D, const double *Ft,
                             float *rho0, const unsigned long long *smax, unsigned long long *rmax,
                             const int *pair_active, bool y_zero, cudaStream_t st);
-// X = D_s Y D_s.
-cudaError_t launch_scale_out(const TileArgs &t, const double *Y, double *X, cudaStream_t st);
+// Caller layout: X = D_s Z D_s of the FP64 blocks (plain), or X = -D_s Z D_s / ky of the
+// passes' blocks.
+cudaError_t launch_scale_out(const TileArgs &t, const double *Z, bool plain, double *X, cudaStream_t st);
 
 }  // namespace fps

@@ -2,10 +2,11 @@
 // a batch.
 //
 // FP32 (refinement), per solve:
-//   smax = max |F~| per (problem, rhs) pair; F~ = D_s F D_s; rho_0 = F~ / smax
+//   smax = max |F~| per (problem, rhs) pair; F~ = D_s F D_s; s = 2^floor(log2 smax);
+//   rho_0 = F~ / s
 //   round r: inner ADI in FP32 (one CUDA graph per tolerance level: every pass
 //            launch covers every problem) gives the correction -D/ky; the FP64
-//            residual kernel applies Y -= smax D/ky, forms
+//            residual kernel applies Y -= s D/ky, forms
 //            R~ = F~ - A~Y - YA~ and the next rho_0; pairs with max|R~| <= tol smax
 //            stop (their iterate is carried unchanged).
 //   X = D_s Y D_s.
@@ -67,12 +68,11 @@ void SweepEngine<T>::release()
     levels_.clear();
     for (void *p : allocs_) cudaFree(p);
     allocs_.clear();
-    void *hp[] = {h_active_, h_pair_active_, h_smax_, h_rmax_, h_err_};
+    void *hp[] = {h_active_, h_pair_active_, h_stat_};
     for (void *p : hp)
         if (p) cudaFreeHost(p);
     h_active_ = h_pair_active_ = nullptr;
-    h_smax_ = h_rmax_ = nullptr;
-    h_err_ = nullptr;
+    h_stat_ = nullptr;
 }
 
 #define ENG_CK(call)                                                                                     \
@@ -136,12 +136,12 @@ static int chain_len_of(int mode, int max_nb)
 }
 
 template <typename T>
-TileArgs SweepEngine<T>::tiles(bool padded) const
+TileArgs SweepEngine<T>::tiles(int which) const
 {
     TileArgs t;
     t.probs = d_tp_;
-    t.tiles = padded ? d_in_tiles_ : d_tiles_;
-    t.ntiles = padded ? nin_tiles_ : ntiles_;
+    t.tiles = d_tiles_[which];
+    t.ntiles = ntiles_[which];
     return t;
 }
 
@@ -327,16 +327,16 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
             max_nb_ = std::max(max_nb_, (int)nb);
             totS_ += (int64_t)nrhs * 4 * nb * nb * S;
         }
-        totB64 += 3 * n;
+        totB64 += 7 * n;
     }
     fused_ = max_nb_ <= kMaxFused;
     npairs_ = np * nrhs;
 
     ENG_CK(sweep_setup_kernels());
     if (!kFP64) {
-        ENG_CK(dalloc(&Ft_, (size_t)tot64_));
-        ENG_CK(dalloc(&Y0_, (size_t)tot64_));
-        ENG_CK(dalloc(&Y1_, (size_t)tot64_));
+        ENG_CK(dalloc(&Ft_, (size_t)totT_));  // quarter blocks, as X and D
+        ENG_CK(dalloc(&Y0_, (size_t)totT_));
+        ENG_CK(dalloc(&Y1_, (size_t)totT_));
     }
     ENG_CK(dalloc(&bands64_, (size_t)totB64));
     ENG_CK(dalloc(&X_, (size_t)totT_));
@@ -347,28 +347,26 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
         ENG_CK(dalloc(&zxR_, (size_t)totS_));
         ENG_CK(dalloc(&zxC_, (size_t)totS_));
     }
-    ENG_CK(dalloc(&err_, 1));
     ENG_CK(dalloc(&d_active_, (size_t)np + 1));
     ENG_CK(dalloc(&d_pair_active_, (size_t)npairs_));
-    ENG_CK(dalloc(&d_smax_, (size_t)npairs_));
-    ENG_CK(dalloc(&d_rmax_, (size_t)npairs_));
+    // what a round reports, read back in one copy: rmax and smax per pair, the error word
+    ENG_CK(dalloc(&d_stat_, 2 * (size_t)npairs_ + 1));
+    err_ = (int *)(d_stat_ + 2 * npairs_);
     ENG_CK(cudaMallocHost((void **)&h_active_, sizeof(int) * (np + 1)));  // last: any problem inactive
     ENG_CK(cudaMallocHost((void **)&h_pair_active_, sizeof(int) * npairs_));
-    ENG_CK(cudaMallocHost((void **)&h_smax_, sizeof(unsigned long long) * npairs_));
-    ENG_CK(cudaMallocHost((void **)&h_rmax_, sizeof(unsigned long long) * npairs_));
-    ENG_CK(cudaMallocHost((void **)&h_err_, sizeof(int)));
-    *h_err_ = 0;
+    ENG_CK(cudaMallocHost((void **)&h_stat_, sizeof(unsigned long long) * (2 * (size_t)npairs_ + 1)));
+    h_stat_[2 * npairs_] = 0;
     // unused positions must be zero and stay zero
     ENG_CK(cudaMemsetAsync(X_, 0, sizeof(T) * (size_t)totT_, cap_));
     ENG_CK(cudaMemsetAsync(D_, 0, sizeof(T) * (size_t)totT_, cap_));
     ENG_CK(cudaMemsetAsync(sumR_, 0, sizeof(T2) * (size_t)totS_, cap_));
     ENG_CK(cudaMemsetAsync(sumC_, 0, sizeof(T2) * (size_t)totS_, cap_));
-    ENG_CK(cudaMemsetAsync(err_, 0, sizeof(int), cap_));
+    ENG_CK(cudaMemsetAsync(d_stat_, 0, sizeof(unsigned long long) * (2 * (size_t)npairs_ + 1), cap_));
 
-    // bands: FP64 (d, e zero-padded, 1/sqrt(E))
+    // bands: FP64 (d, e zero-padded, 1/sqrt(E), then {-kx d, -ky d} and {-kx e, -ky e})
     std::vector<double> hb64((size_t)totB64);
     std::vector<TileProb> tp(np);
-    std::vector<int4> tiles, in_tiles;  // 32 x 32 tiles of the n x n and of the padded region
+    std::vector<int4> tiles[3];  // live region, padded region, residual
     ob64_.resize(np);
     {
         int64_t o64 = 0;
@@ -380,6 +378,12 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
             std::copy(d.begin(), d.end(), hb64.begin() + o64);
             std::copy(e.begin(), e.end(), hb64.begin() + o64 + n);
             std::copy(s.begin(), s.end(), hb64.begin() + o64 + 2 * n);
+            for (int64_t i = 0; i < n; ++i) {
+                hb64[o64 + 3 * n + i] = -kx_ * d[i];
+                hb64[o64 + 4 * n + i] = -ky_ * d[i];
+                hb64[o64 + 5 * n + i] = -kx_ * e[i];
+                hb64[o64 + 6 * n + i] = -ky_ * e[i];
+            }
             ob64_[p] = o64;
             TileProb &t = tp[p];
             t.n = (int)n;
@@ -388,31 +392,34 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
             t.off64 = off64_[p];
             t.off = offT_[p];
             t.rhs = 4 * (int64_t)nb_[p] * nb_[p] << (2 * t.log_s);
-            t.d = bands64_ + o64;
-            t.e = bands64_ + o64 + n;
             t.s = bands64_ + o64 + 2 * n;
+            t.nd = bands64_ + o64 + 3 * n;
+            t.ne = bands64_ + o64 + 5 * n;
             t.pair0 = p * nrhs;
-            t.kx = kx_;
-            t.ky = ky_;
-            o64 += 3 * n;
-            const int nt = (int)((n + 31) / 32), ntp = 2 * (nb_[p] << t.log_s) / 32;
+            t.inv_ky = 1.0 / ky_;
+            o64 += 7 * n;
+            const int m = (int)((n + 1) / 2), nt = (m + 31) / 32, ntp = (nb_[p] << t.log_s) / 32;
             for (int r = 0; r < nrhs; ++r) {
+                const int id = p * 256 + r;
                 for (int ty = 0; ty < nt; ++ty)
-                    for (int tx = 0; tx < nt; ++tx) tiles.push_back(make_int4(p * 256 + r, tx, ty, 0));
+                    for (int tx = 0; tx < nt; ++tx) tiles[0].push_back(make_int4(id, tx, ty, 0));
                 for (int ty = 0; ty < ntp; ++ty)
-                    for (int tx = 0; tx < ntp; ++tx) in_tiles.push_back(make_int4(p * 256 + r, tx, ty, 0));
+                    for (int tx = 0; tx < ntp; ++tx) tiles[1].push_back(make_int4(id, tx, ty, 0));
+                if (!kFP64)
+                    for (int q = 0; q < 4; ++q)
+                        for (int ty = 0; ty < (m + 63) / 64; ++ty)
+                            for (int tx = 0; tx < nt; ++tx) tiles[2].push_back(make_int4(id, tx * 4 + q, ty, 0));
             }
         }
     }
-    ntiles_ = (int64_t)tiles.size();
-    nin_tiles_ = (int64_t)in_tiles.size();
     ENG_CK(dalloc(&d_tp_, (size_t)np));
-    ENG_CK(dalloc(&d_tiles_, (size_t)ntiles_));
-    ENG_CK(dalloc(&d_in_tiles_, (size_t)nin_tiles_));
+    for (int w = 0; w < 3; ++w) {
+        ntiles_[w] = (int64_t)tiles[w].size();
+        ENG_CK(dalloc(&d_tiles_[w], tiles[w].size()));
+        ENG_CK(cudaMemcpyAsync(d_tiles_[w], tiles[w].data(), sizeof(int4) * tiles[w].size(), cudaMemcpyHostToDevice, cap_));
+    }
     ENG_CK(cudaMemcpyAsync(bands64_, hb64.data(), sizeof(double) * totB64, cudaMemcpyHostToDevice, cap_));
     ENG_CK(cudaMemcpyAsync(d_tp_, tp.data(), sizeof(TileProb) * np, cudaMemcpyHostToDevice, cap_));
-    ENG_CK(cudaMemcpyAsync(d_tiles_, tiles.data(), sizeof(int4) * ntiles_, cudaMemcpyHostToDevice, cap_));
-    ENG_CK(cudaMemcpyAsync(d_in_tiles_, in_tiles.data(), sizeof(int4) * nin_tiles_, cudaMemcpyHostToDevice, cap_));
 
     order_.resize(np);
     for (int p = 0; p < np; ++p) order_[p] = p;
@@ -779,10 +786,10 @@ int SweepEngine<T>::solve_plain(const double *F, double *X, cudaStream_t st, std
             rounds_last = 1;
             return FPS_OK;
         }
-        ENG_CK(launch_scale_in<double>(tiles(true), F, nullptr, X_, nullptr, st));
+        ENG_CK(launch_scale_in<double>(tiles(kPadded), F, nullptr, X_, nullptr, st));
         ENG_CK(cudaGraphLaunch(levels_[0].graph, st));
-        ENG_CK(launch_finalize_out(tiles(false), D_, X, st));
-        ENG_CK(cudaMemcpyAsync(h_err_, err_, sizeof(int), cudaMemcpyDeviceToHost, st));
+        ENG_CK(launch_scale_out(tiles(kLive), D_, false, X, st));
+        ENG_CK(cudaMemcpyAsync(h_stat_ + 2 * npairs_, err_, sizeof(int), cudaMemcpyDeviceToHost, st));
         levels_used_.push_back(0);
         launches_last = 2 + levels_[0].launches;
         rounds_last = 1;
@@ -801,70 +808,68 @@ int SweepEngine<T>::solve_refine(const double *F, double *X, cudaStream_t st, st
 {
     if constexpr (sizeof(T) == 4) {
         const int np = (int)ns_.size();
-        const TileArgs ta = tiles(false);
 
-        ENG_CK(cudaMemsetAsync(d_smax_, 0, sizeof(unsigned long long) * npairs_, st));
-        ENG_CK(launch_absmax(ta, F, d_smax_, st));
-        ENG_CK(cudaMemcpyAsync(h_smax_, d_smax_, sizeof(unsigned long long) * npairs_, cudaMemcpyDeviceToHost, st));
-        ENG_CK(cudaStreamSynchronize(st));
-        launches_last += 1;
-        std::vector<double> sF(npairs_);
-        for (int k = 0; k < npairs_; ++k) {
-            sF[k] = bits_to_double(h_smax_[k]);
-            if (!std::isfinite(sF[k])) {
-                err = "F holds NaN or Inf";
-                return FPS_ERR_NONFINITE;
-            }
-            h_pair_active_[k] = sF[k] > 0.0 ? 1 : 0;  // an all-zero right-hand side is already solved (X = 0)
-        }
-        set_active();
-        ENG_CK(cudaMemcpyAsync(d_active_, h_active_, sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
-        ENG_CK(cudaMemcpyAsync(d_pair_active_, h_pair_active_, sizeof(int) * npairs_, cudaMemcpyHostToDevice, st));
-        ENG_CK(launch_scale_in<float>(tiles(true), F, Ft_, X_, d_smax_, st));
-        launches_last += 1;
+        // The first round is launched without waiting for smax: the device masks what has
+        // nothing to solve, and the host looks at smax together with the round's residuals.
+        unsigned long long *d_rmax = d_stat_, *d_smax = d_stat_ + npairs_;
+        const unsigned long long *h_rmax = h_stat_, *h_smax = h_stat_ + npairs_;
+        ENG_CK(cudaMemsetAsync(d_stat_, 0, sizeof(unsigned long long) * 2 * npairs_, st));
+        ENG_CK(launch_absmax(tiles(kLive), F, d_smax, st));
+        ENG_CK(launch_init_masks(d_smax, np, nrhs_, d_pair_active_, d_active_, d_active_ + np, st));
+        ENG_CK(launch_scale_in<float>(tiles(kPadded), F, Ft_, X_, d_smax, st));
+        launches_last += 3;
 
-        std::vector<double> rel(npairs_, 0.0);
-        for (int k = 0; k < npairs_; ++k) rel[k] = h_pair_active_[k] ? 1.0 : 0.0;
+        std::vector<double> rel(npairs_, 0.0), sF(npairs_, 0.0);
         double *Ycur = Y0_, *Ynext = Y1_;
-        bool any_active = false;
-        for (int k = 0; k < npairs_; ++k) any_active = any_active || h_pair_active_[k];
+        bool any_active = true;
         int round = 0;
-        bool converged = !any_active;
+        bool converged = false;
         for (; round < max_rounds && !converged; ++round) {
             TraceRange tr("fps refinement round");
-            double worst = 0.0;
-            for (int k = 0; k < npairs_; ++k)
-                if (h_pair_active_[k]) worst = std::max(worst, rel[k]);
-            const double want = 0.1 * tol_ / worst;
+            // two balanced rounds: the first stops near sqrt(0.1 tol), which leaves the
+            // second a gain of the same size (1e-6 then 1e-5 for tol = 1e-10)
+            double want = std::sqrt(0.1 * tol_);
+            if (round > 0) {
+                double worst = 0.0;
+                for (int k = 0; k < npairs_; ++k)
+                    if (h_pair_active_[k]) worst = std::max(worst, rel[k]);
+                want = 0.1 * tol_ / worst;
+            }
             size_t li = 0;
             for (size_t l = 0; l < levels_.size(); ++l)
                 if (levels_[l].tol <= want) li = l;
-            if (round == 0) {
-                // two balanced rounds: the first stops near sqrt(0.1 tol), which leaves the
-                // second a gain of the same size (1e-6 then 1e-5 for tol = 1e-10)
-                const double first = std::sqrt(0.1 * tol_);
-                li = 0;
-                for (size_t l = 0; l < levels_.size(); ++l)
-                    if (levels_[l].tol <= first) li = l;
-            }
             ENG_CK(cudaGraphLaunch(levels_[li].graph, st));
             levels_used_.push_back((int)li);
             launches_last += levels_[li].launches;
-            ENG_CK(cudaMemsetAsync(d_rmax_, 0, sizeof(unsigned long long) * npairs_, st));
-            ENG_CK(launch_residual(ta, Ycur, Ynext, D_, Ft_, X_, d_smax_, d_rmax_, d_pair_active_, round == 0, st));
+            if (round > 0) ENG_CK(cudaMemsetAsync(d_rmax, 0, sizeof(unsigned long long) * npairs_, st));
+            ENG_CK(launch_residual(tiles(kResidual), Ycur, Ynext, D_, Ft_, X_, d_smax, d_rmax, d_pair_active_, round == 0,
+                                   st));
             launches_last += 1;
-            ENG_CK(cudaMemcpyAsync(h_rmax_, d_rmax_, sizeof(unsigned long long) * npairs_, cudaMemcpyDeviceToHost, st));
-            ENG_CK(cudaMemcpyAsync(h_err_, err_, sizeof(int), cudaMemcpyDeviceToHost, st));
+            ENG_CK(cudaMemcpyAsync(h_stat_, d_stat_, sizeof(unsigned long long) * (2 * (size_t)npairs_ + 1),
+                                   cudaMemcpyDeviceToHost, st));
             ENG_CK(cudaStreamSynchronize(st));
-            if (*h_err_) {
+            if (timed_out()) {
                 err = "a bounded device wait gave up (tile copy not completed)";
                 return FPS_ERR_TIMEOUT;
+            }
+            if (round == 0) {
+                any_active = false;
+                for (int k = 0; k < npairs_; ++k) {
+                    sF[k] = bits_to_double(h_smax[k]);
+                    if (!std::isfinite(sF[k])) {
+                        err = "F holds NaN or Inf";
+                        return FPS_ERR_NONFINITE;
+                    }
+                    h_pair_active_[k] = sF[k] > 0.0 ? 1 : 0;  // an all-zero right-hand side is already solved (X = 0)
+                    any_active = any_active || h_pair_active_[k];
+                }
+                if (!any_active) break;
             }
             std::swap(Ycur, Ynext);
             converged = true;
             for (int k = 0; k < npairs_; ++k) {
                 if (!h_pair_active_[k]) continue;
-                const double r = bits_to_double(h_rmax_[k]) / sF[k];
+                const double r = bits_to_double(h_rmax[k]) / sF[k];
                 if (!std::isfinite(r)) {
                     err = "non-finite residual";
                     return FPS_ERR_NONFINITE;
@@ -873,6 +878,7 @@ int SweepEngine<T>::solve_refine(const double *F, double *X, cudaStream_t st, st
                 if (r <= tol_) h_pair_active_[k] = 0;
                 else converged = false;
             }
+            if (converged) continue;
             set_active();
             ENG_CK(cudaMemcpyAsync(d_active_, h_active_, sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
             ENG_CK(cudaMemcpyAsync(d_pair_active_, h_pair_active_, sizeof(int) * npairs_, cudaMemcpyHostToDevice, st));
@@ -880,11 +886,11 @@ int SweepEngine<T>::solve_refine(const double *F, double *X, cudaStream_t st, st
         rounds_last = round;
         resid_last = 0.0;
         for (int k = 0; k < npairs_; ++k) resid_last = std::max(resid_last, rel[k]);
-        if (round == 0) {
+        if (!any_active) {
             ENG_CK(cudaMemsetAsync(X, 0, sizeof(double) * tot64_, st));  // every right-hand side was zero
             return FPS_OK;
         }
-        ENG_CK(launch_scale_out(ta, Ycur, X, st));
+        ENG_CK(launch_scale_out(tiles(kLive), Ycur, true, X, st));
         launches_last += 1;
         if (!converged) {
             err = "refinement did not reach tol";
@@ -921,7 +927,7 @@ template <typename T>
 int SweepEngine<T>::kernel_times(int *count, double *total_ms, double *alg_bytes, double *row_ms, double *col_ms,
                                  std::string &err)
 {
-    if (h_err_ && *h_err_) {
+    if (timed_out()) {
         err = "a bounded device wait gave up (tile copy not completed)";
         return FPS_ERR_TIMEOUT;
     }

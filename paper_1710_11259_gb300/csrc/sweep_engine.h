@@ -83,7 +83,8 @@ private:
     ResArgs<T> res_args(const ResClass &c, const double *F, double *X) const;
     int build_tables(Level &L, int level, const std::vector<double> &lo, const std::vector<double> &hi,
                      std::string &err);
-    TileArgs tiles(bool padded) const;
+    enum { kLive, kPadded, kResidual };  // tile lists (sweep.cuh)
+    TileArgs tiles(int which) const;
     void set_active();
     int solve_refine(const double *F, double *X, cudaStream_t st, std::string &err);
     int solve_plain(const double *F, double *X, cudaStream_t st, std::string &err);
@@ -106,12 +107,12 @@ private:
     T2 *sumR_ = nullptr, *sumC_ = nullptr, *zxR_ = nullptr, *zxC_ = nullptr;
     int *err_ = nullptr;
     TileProb *d_tp_ = nullptr;
-    int4 *d_tiles_ = nullptr, *d_in_tiles_ = nullptr;
-    int64_t ntiles_ = 0, nin_tiles_ = 0;
+    int4 *d_tiles_[3] = {nullptr, nullptr, nullptr};
+    int64_t ntiles_[3] = {0, 0, 0};
     int *d_active_ = nullptr, *d_pair_active_ = nullptr;
     int *h_active_ = nullptr, *h_pair_active_ = nullptr;
-    unsigned long long *d_smax_ = nullptr, *d_rmax_ = nullptr, *h_smax_ = nullptr, *h_rmax_ = nullptr;
-    int *h_err_ = nullptr;
+    unsigned long long *d_stat_ = nullptr, *h_stat_ = nullptr;  // rmax, smax [npairs], error word
+    bool timed_out() const { return h_stat_ && (unsigned)h_stat_[2 * npairs_] != 0; }
     std::vector<Level> levels_;
     std::vector<int64_t> ob64_;  // offset of each problem's bands in bands64_
     std::vector<int> order_;     // problems, largest first

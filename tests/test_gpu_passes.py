@@ -105,3 +105,18 @@ def test_nonfinite_input_leaves_no_trace(api, n):
     torch.cuda.synchronize()
     api.plan_destroy(plan)
     assert torch.equal(X, again)
+
+
+@pytest.mark.parametrize("n", [65, 1100])
+@pytest.mark.parametrize("k", [900, -600, -1000])
+def test_refine_scales_with_powers_of_two(api, n, k):
+    """The FP32 iteration runs on the residual scaled by a power of two, converted with
+    integer instructions: right-hand sides near the ends of the FP64 range (at k = -1000
+    part of the scaled right-hand side is subnormal) give the scaled solution."""
+    F = inputs.square_rhs(n, 3)
+    plan = api.plan_create(n, 2, 1e-10, "fp32_refine")
+    X = api.poisson_square_solve(plan, torch.from_numpy(np.ldexp(F, k)).cuda()).cpu().numpy()
+    info = api.plan_info(plan)
+    api.plan_destroy(plan)
+    assert info["last_residual"] <= 1e-10
+    assert _relmax(np.ldexp(X, -k), oracle.poisson_square(F, 1e-13)) <= TOL_REFINE
