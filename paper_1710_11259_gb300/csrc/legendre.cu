@@ -8,200 +8,142 @@
 // u = (1-x^2)(1-y^2) sum X_ij C~_i(y) C~_j(x), is U = L X L^T with L ((n+2) x n)
 // L[j][j] = c_j, L[j+2][j] = -c_j, c_j = s_j (j+1)(j+2)/(2j+3): the product
 // B^{-1} M of the C~ -> Legendre conversion and the multiplication (3.7) by
-// (1 - x^2) collapses to two terms.  Algorithmic traffic is one FP64 read and one
-// write per element; at four FP64 operations per element GB300's FP64 rate, not
-// its HBM, bounds both maps.
+// (1 - x^2) collapses to two terms.
+//
+// Both maps and their transposes are one kernel: every row a is combined along the
+// columns,  q_a[k] = x_k in[a][k] + y_k in[a][k +- 2],  and two rows are combined,
+// out = X q_a + Y q_{a +- 2}.  A thread walks down LEN rows of one parity in one column
+// and forms every q once: four FP64 operations per element, the bound on GB300 (0.64 ms
+// at n = 10^4; one read and one write of HBM would take 0.24 ms).
 #include "legendre.cuh"
 
 namespace fps {
 
 namespace {
 
-constexpr int kTC = 32;  // output tile: kTC columns (one per lane) ...
-constexpr int kTR = 64;  // ... by kTR rows (output map); thread row ty takes parity ty & 1 and 8 rows of it
-constexpr int kRows = 8;
+enum Map { kIn, kOut, kInT, kOutT };
 
-__device__ __forceinline__ double snorm(int64_t k)
+constexpr int kCols = 32;  // a warp: 32 columns; two parities x kWarps / 2 column groups per CTA
+
+// sqrt((j+1)(j+2)/(j+3/2)) / d, i.e. 1/(s_j d)
+__device__ __forceinline__ double inv_snorm(int64_t j, double d)
 {
-    const double K = (double)k;
-    return sqrt((K + 1.5) / ((K + 1.0) * (K + 2.0)));
+    const double J = (double)j, A = (J + 1.0) * (J + 2.0);
+    return A * rsqrt(A * (J + 1.5) * (d * d));
+}
+__device__ __forceinline__ double b_diag(int64_t j) { return inv_snorm(j, 2.0 * (double)j + 1.0); }
+__device__ __forceinline__ double b_off(int64_t j) { return -inv_snorm(j, 2.0 * (double)j + 5.0); }
+// c_j = s_j (j+1)(j+2)/(2j+3) = (j+1)(j+2)/2 / sqrt((j+1)(j+2)(j+3/2)); 0 outside [0, n)
+__device__ __forceinline__ double c_val(int64_t j, int64_t n)
+{
+    if (j < 0 || j >= n) return 0.0;
+    const double J = (double)j, A = (J + 1.0) * (J + 2.0);
+    return 0.5 * A * rsqrt(A * (J + 1.5));
 }
 
-// F[j][k] = sum_{a in {j, j+2}} sum_{b in {k, k+2}} B[j][a] B[k][b] G[a][b]: one thread per
-// output element (this kernel runs faster with the extra FP64 products than with
-// fewer, longer-running threads that reuse row combinations).
-__global__ void __launch_bounds__(256) legendre_to_ctilde_kernel(const double *__restrict__ G,
-                                                                 double *__restrict__ F, int64_t n)
+// Coefficients of position i of the output: x on the near index, y on the one two away
+// (kIn, kOutT: i and i + 2; kOut, kInT: i and i - 2), zero where that one is outside.
+template <int MAP>
+__device__ __forceinline__ double2 coefficients(int64_t i, int64_t n)
 {
-    __shared__ double rd[kTC], ro[kTC], cd[kTC], co[kTC];  // B entries of the tile's rows and columns
-    const int64_t j0 = (int64_t)blockIdx.y * kTC, k0 = (int64_t)blockIdx.x * kTC;
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    if (tid < kTC) {
-        const int64_t j = j0 + tid;
-        const double s = snorm(j);
-        rd[tid] = 1.0 / ((2.0 * (double)j + 1.0) * s);
-        ro[tid] = -1.0 / ((2.0 * (double)j + 5.0) * s);
-    } else if (tid < 2 * kTC) {
-        const int64_t k = k0 + tid - kTC;
-        const double s = snorm(k);
-        cd[tid - kTC] = 1.0 / ((2.0 * (double)k + 1.0) * s);
-        co[tid - kTC] = -1.0 / ((2.0 * (double)k + 5.0) * s);
-    }
-    __syncthreads();
-    const int64_t k = k0 + threadIdx.x;
-    if (k >= n) return;
-    const bool k2 = k + 2 < n;
-    for (int r = threadIdx.y; r < kTC; r += blockDim.y) {
-        const int64_t j = j0 + r;
-        if (j >= n) break;
-        const double *g0 = G + j * n + k;
-        double row0 = cd[threadIdx.x] * g0[0];
-        if (k2) row0 = fma(co[threadIdx.x], g0[2], row0);
-        double v = rd[r] * row0;
-        if (j + 2 < n) {
-            const double *g2 = g0 + 2 * n;
-            double row2 = cd[threadIdx.x] * g2[0];
-            if (k2) row2 = fma(co[threadIdx.x], g2[2], row2);
-            v = fma(ro[r], row2, v);
-        }
-        F[j * n + k] = v;
-    }
+    if (MAP == kIn) return make_double2(b_diag(i), i + 2 < n ? b_off(i) : 0.0);
+    if (MAP == kOut) return make_double2(c_val(i, n), -c_val(i - 2, n));
+    if (MAP == kInT) return make_double2(b_diag(i), i >= 2 ? b_off(i - 2) : 0.0);
+    const double c = c_val(i, n);
+    return make_double2(c, -c);
 }
 
-//   U[i] = c_i w_i - c_{i-2} w_{i-2},  w_a = c_k X[a][k] - c_{k-2} X[a][k-2]  (a in [0, n)):
-// each thread walks a strip of same-parity rows and forms every w once (FP64
-// arithmetic, not HBM, bounds this map on GB300; measured 2.5 ms against 3.1 ms
-// for one thread per element at n = 10^4).
-__global__ void __launch_bounds__(256) solution_to_legendre_kernel(const double *__restrict__ X,
-                                                                   double *__restrict__ U, int64_t n)
+template <int MAP, int LEN, int kWarps>
+__global__ void __launch_bounds__(kCols *kWarps) legendre_kernel(const double *__restrict__ in, double *__restrict__ out,
+                                                                 int64_t n)
 {
-    __shared__ double rc[kTR + 2];  // c_a for a = i0 - 2 .. i0 + kTR - 1 (0 outside [0, n))
+    constexpr bool kForward = MAP == kIn || MAP == kOutT;
+    constexpr int kChunk = LEN < 8 ? LEN : 8;
+    __shared__ double2 rc[2 * LEN];  // row coefficients of the tile's rows
     const int64_t m = n + 2;
-    const int64_t i0 = (int64_t)blockIdx.y * kTR, k0 = (int64_t)blockIdx.x * kTC;
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    auto cval = [&](int64_t a) {
-        if (a < 0 || a >= n) return 0.0;
-        const double A = (double)a;
-        return snorm(a) * (A + 1.0) * (A + 2.0) / (2.0 * A + 3.0);
-    };
-    if (tid < kTR + 2) rc[tid] = cval(i0 - 2 + tid);
+    const int64_t rows_in = MAP == kOutT ? m : n, rows_out = MAP == kOut ? m : n;  // square matrices
+    const int64_t i0 = (int64_t)blockIdx.y * (2 * LEN);
+    for (int t = threadIdx.x; t < 2 * LEN; t += kCols * kWarps)
+        if (i0 + t < rows_out) rc[t] = coefficients<MAP>(i0 + t, n);
+    const int warp = threadIdx.x >> 5, par = warp & 1;
+    const int64_t k = (int64_t)blockIdx.x * (kCols * kWarps / 2) + (warp >> 1) * kCols + (threadIdx.x & 31);
+    const bool on = k < rows_out;
+    const double2 cx = on ? coefficients<MAP>(k, n) : make_double2(0.0, 0.0);
+    const int64_t k2 = kForward ? k + 2 : k - 2;
+    const bool near_in = on && k < rows_in, far_in = on && k2 >= 0 && k2 < rows_in;
     __syncthreads();
-    const int64_t k = k0 + threadIdx.x;
-    if (k >= m) return;
-    const bool kin = k < n, km2 = k >= 2;  // columns k and k - 2 present in X (k - 2 < n always)
-    const double ck = cval(k), ckm2 = cval(k - 2);
-    auto wrow = [&](int64_t a) {  // (X L^T)[a][k], zero outside [0, n)
-        if (a < 0 || a >= n) return 0.0;
-        const double *x = X + a * n;
-        double v = kin ? ck * x[k] : 0.0;
-        return km2 ? fma(-ckm2, x[k - 2], v) : v;
+    // q of row a; rows outside the input are zero
+    auto combine = [&](double u, double v) { return fma(cx.y, v, fma(cx.x, u, 0.0)); };
+    auto load = [&](int64_t a, double &u, double &v) {
+        const bool ok = a >= 0 && a < rows_in;
+        const double *row = in + a * rows_in;
+        u = ok && near_in ? row[k] : 0.0;
+        v = ok && far_in ? row[k2] : 0.0;
     };
-    const int par = threadIdx.y & 1, strip = threadIdx.y >> 1;
-    const int r_lo = par + 2 * kRows * strip;
-    const int r_hi = r_lo + 2 * (kRows - 1);
-    double prv = wrow(i0 + r_lo - 2);                   // w_{i-2} for the first row
-    for (int r = r_lo; r <= r_hi; r += 2) {
-        const int64_t i = i0 + r;
-        const double cur = wrow(i);
-        if (i < m) U[i * m + k] = fma(-rc[r], prv, rc[r + 2] * cur);
-        prv = cur;
-    }
-}
-
-// Transpose of the input map, Gbar = B^T Fbar B:
-//   Gbar[a][b] = sum_{i in {a, a-2}} sum_{j in {b, b-2}} B[i][a] B[j][b] Fbar[i][j],
-// with B[a][a] and B[a-2][a] the two entries of column a.  One thread per element.
-__global__ void __launch_bounds__(256) legendre_to_ctilde_adjoint_kernel(const double *__restrict__ Fb,
-                                                                         double *__restrict__ Gb, int64_t n)
-{
-    __shared__ double rd[kTC], ro[kTC], cd[kTC], co[kTC];  // column a of B: {B[a][a], B[a-2][a]} (0 if a < 2)
-    const int64_t a0 = (int64_t)blockIdx.y * kTC, b0 = (int64_t)blockIdx.x * kTC;
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    auto diag = [](int64_t j) { return 1.0 / ((2.0 * (double)j + 1.0) * snorm(j)); };
-    auto off = [](int64_t j) { return j < 2 ? 0.0 : -1.0 / ((2.0 * (double)(j - 2) + 5.0) * snorm(j - 2)); };
-    if (tid < kTC) {
-        rd[tid] = diag(a0 + tid);
-        ro[tid] = off(a0 + tid);
-    } else if (tid < 2 * kTC) {
-        cd[tid - kTC] = diag(b0 + tid - kTC);
-        co[tid - kTC] = off(b0 + tid - kTC);
-    }
-    __syncthreads();
-    const int64_t b = b0 + threadIdx.x;
-    if (b >= n) return;
-    const bool b2 = b >= 2;
-    for (int r = threadIdx.y; r < kTC; r += blockDim.y) {
-        const int64_t a = a0 + r;
-        if (a >= n) break;
-        const double *f0 = Fb + a * n + b;
-        double row0 = cd[threadIdx.x] * f0[0];
-        if (b2) row0 = fma(co[threadIdx.x], f0[-2], row0);
-        double v = rd[r] * row0;
-        if (a >= 2) {
-            const double *f2 = f0 - 2 * n;
-            double row2 = cd[threadIdx.x] * f2[0];
-            if (b2) row2 = fma(co[threadIdx.x], f2[-2], row2);
-            v = fma(ro[r], row2, v);
+    const int64_t first = i0 + par - (kForward ? 0 : 2);
+    double u, v;
+    load(first, u, v);
+    double q = combine(u, v);
+    for (int t0 = 0; t0 < LEN; t0 += kChunk) {
+        double us[kChunk], vs[kChunk];
+#pragma unroll
+        for (int t = 0; t < kChunk; ++t) load(first + 2 * (t0 + t + 1), us[t], vs[t]);
+#pragma unroll
+        for (int t = 0; t < kChunk; ++t) {
+            const int r = par + 2 * (t0 + t);
+            const double nxt = combine(us[t], vs[t]);
+            if (on && i0 + r < rows_out) {
+                const double2 c = rc[r];
+                out[(i0 + r) * rows_out + k] = kForward ? fma(c.x, q, fma(c.y, nxt, 0.0)) : fma(c.x, nxt, fma(c.y, q, 0.0));
+            }
+            q = nxt;
         }
-        Gb[a * n + b] = v;
     }
 }
 
-// Transpose of the output map, Xbar = L^T Ubar L with L[a][a] = c_a, L[a+2][a] = -c_a:
-//   Xbar[a][k] = c_a c_k (Ubar[a][k] - Ubar[a][k+2] - Ubar[a+2][k] + Ubar[a+2][k+2]).
-__global__ void __launch_bounds__(256) solution_to_legendre_adjoint_kernel(const double *__restrict__ Ub,
-                                                                           double *__restrict__ Xb, int64_t n)
+// Long walks amortise the coefficients (a reciprocal square root costs as much as four
+// elements); short ones give a small matrix enough CTAs.  Both maps together, walks of
+// 64 / 16 / 8 rows against one output element per thread with 6 and 4 operations:
+// n = 10^4 1.75 ms (3.93 ms), n = 2048 109 us (179 us), n = 777 31 us (42 us).
+template <int MAP, int LEN, int kWarps>
+void launch_len(const double *in, double *out, int64_t n, cudaStream_t st)
 {
-    __shared__ double rc[kTC], cc[kTC];
-    const int64_t m = n + 2;
-    const int64_t a0 = (int64_t)blockIdx.y * kTC, k0 = (int64_t)blockIdx.x * kTC;
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    auto cval = [](int64_t a) {
-        const double A = (double)a;
-        return snorm(a) * (A + 1.0) * (A + 2.0) / (2.0 * A + 3.0);
-    };
-    if (tid < kTC) rc[tid] = cval(a0 + tid);
-    else if (tid < 2 * kTC) cc[tid - kTC] = cval(k0 + tid - kTC);
-    __syncthreads();
-    const int64_t k = k0 + threadIdx.x;
-    if (k >= n) return;
-    for (int r = threadIdx.y; r < kTC; r += blockDim.y) {
-        const int64_t a = a0 + r;
-        if (a >= n) break;
-        const double *u0 = Ub + a * m + k, *u2 = u0 + 2 * m;
-        Xb[a * n + k] = rc[r] * cc[threadIdx.x] * ((u0[0] - u0[2]) - (u2[0] - u2[2]));
-    }
+    const int64_t rows = MAP == kOut ? n + 2 : n, cols = kCols * kWarps / 2;
+    const dim3 grid((unsigned)((rows + cols - 1) / cols), (unsigned)((rows + 2 * LEN - 1) / (2 * LEN)));
+    legendre_kernel<MAP, LEN, kWarps><<<grid, kCols * kWarps, 0, st>>>(in, out, n);
+}
+
+template <int MAP>
+cudaError_t launch_map(const double *in, double *out, int64_t n, cudaStream_t st)
+{
+    if (n >= 3072) launch_len<MAP, 64, 8>(in, out, n, st);
+    else if (n >= 900) launch_len<MAP, 16, 8>(in, out, n, st);
+    else launch_len<MAP, 8, 4>(in, out, n, st);
+    return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_legendre_to_ctilde(const double *G, double *F, int64_t n, cudaStream_t st)
 {
-    const dim3 block(kTC, 8), grid((unsigned)((n + kTC - 1) / kTC), (unsigned)((n + kTC - 1) / kTC));
-    legendre_to_ctilde_kernel<<<grid, block, 0, st>>>(G, F, n);
-    return cudaGetLastError();
+    return launch_map<kIn>(G, F, n, st);
 }
 
 cudaError_t launch_solution_to_legendre(const double *X, double *U, int64_t n, cudaStream_t st)
 {
-    const int64_t m = n + 2;
-    const dim3 block(kTC, 8), grid((unsigned)((m + kTC - 1) / kTC), (unsigned)((m + kTR - 1) / kTR));
-    solution_to_legendre_kernel<<<grid, block, 0, st>>>(X, U, n);
-    return cudaGetLastError();
+    return launch_map<kOut>(X, U, n, st);
 }
 
+// Transpose of the input map, Gbar = B^T Fbar B.
 cudaError_t launch_legendre_to_ctilde_adjoint(const double *Fbar, double *Gbar, int64_t n, cudaStream_t st)
 {
-    const dim3 block(kTC, 8), grid((unsigned)((n + kTC - 1) / kTC), (unsigned)((n + kTC - 1) / kTC));
-    legendre_to_ctilde_adjoint_kernel<<<grid, block, 0, st>>>(Fbar, Gbar, n);
-    return cudaGetLastError();
+    return launch_map<kInT>(Fbar, Gbar, n, st);
 }
 
+// Transpose of the output map, Xbar = L^T Ubar L.
 cudaError_t launch_solution_to_legendre_adjoint(const double *Ubar, double *Xbar, int64_t n, cudaStream_t st)
 {
-    const dim3 block(kTC, 8), grid((unsigned)((n + kTC - 1) / kTC), (unsigned)((n + kTC - 1) / kTC));
-    solution_to_legendre_adjoint_kernel<<<grid, block, 0, st>>>(Ubar, Xbar, n);
-    return cudaGetLastError();
+    return launch_map<kOutT>(Ubar, Xbar, n, st);
 }
 
 }  // namespace fps

@@ -120,3 +120,14 @@ def test_refine_scales_with_powers_of_two(api, n, k):
     api.plan_destroy(plan)
     assert info["last_residual"] <= 1e-10
     assert _relmax(np.ldexp(X, -k), oracle.poisson_square(F, 1e-13)) <= TOL_REFINE
+
+
+@pytest.mark.parametrize("n", [15, 17, 65, 127, 129, 899, 900, 3071, 3072, 3073])
+def test_legendre_walk_edges(api, n):
+    """Legendre maps at the edges of their tiles (16 rows x 64 columns, 32 and 128 x 128) and on
+    both sides of the sizes where the walk length changes."""
+    G, X = inputs.gaussian(n, (n, n)), inputs.square_rhs(n, n + 1)
+    F = api.legendre_to_ctilde(torch.from_numpy(G).cuda()).cpu().numpy()
+    U = api.solution_to_legendre(torch.from_numpy(X).cuda()).cpu().numpy()
+    assert _relmax(F, oracle.legendre_to_ctilde(G)) <= 1e-14
+    assert _relmax(U, oracle.solution_to_legendre(X)) <= 1e-13
