@@ -48,10 +48,9 @@ public:
 private:
     std::vector<void *> allocs_;
     double *G_ = nullptr, *R1_ = nullptr, *R2_ = nullptr;
-    double *bands_ = nullptr;       // [7][n + 4]: Md, Me, D, L1d, L1u (a = i - 2), L1l (a = i + 2), Q4
-    double2 *zfac_ = nullptr;       // [sum J][n] {1/den, u} of (M + p D)
-    double *rfac_ = nullptr;        // [sum J][n][6] LU of (Q - q P): {l1, l2, 1/u0, u1, u2, -}
-    double *shifts_ = nullptr;      // [modes][Jmax][2] {p_j, q_j}
+    double *zfac_ = nullptr, *rfac_ = nullptr;  // factor tables of every (mode, iteration)
+    void *units_ = nullptr;                     // n <= 256: the quarters, one CTA each
+    int nunits_ = 0, half_ = 0;                 // half line length of their kernel (0: streaming kernels)
     int *joff_ = nullptr;           // [modes] offset of the mode's first iteration in the tables
     int *jcount_ = nullptr;         // [modes] J
     template <typename U>

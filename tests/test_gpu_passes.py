@@ -131,3 +131,24 @@ def test_legendre_walk_edges(api, n):
     U = api.solution_to_legendre(torch.from_numpy(X).cuda()).cpu().numpy()
     assert _relmax(F, oracle.legendre_to_ctilde(G)) <= 1e-14
     assert _relmax(U, oracle.solution_to_legendre(X)) <= 1e-13
+
+
+# half lines of 2, 4, .., 64 unknowns per CTA, full and with unused places; 256 is the last
+# size that stays on chip, 257 and 300 stream.  Against the oracle's ADI at tol 1e-15 with
+# the bar of the n = 128 cylinder test, 10 tol kappa_k + 3e-11; its rounding floor grows
+# with the entries of P, k^2 + n^2, hence the factor above n = 128.
+@pytest.mark.parametrize("n,k", [(4, 2), (5, 3), (9, 2), (33, 2), (47, 5), (65, 17), (97, 2), (129, 3), (161, 2),
+                                 (193, 40), (224, 2), (255, 5), (256, 2), (257, 2), (300, 12)])
+def test_cylinder_line_lengths(api, n, k):
+    from oracle import cylinder as cyl
+
+    F = np.stack([inputs.square_rhs(n, n), inputs.square_rhs(n, n + 1)])
+    plan = api.plan_create_cylinder(n, k, k, 1e-13, 2)
+    Y = api.poisson_cylinder_solve(plan, torch.from_numpy(F[None].copy()).cuda()).cpu().numpy()[0]
+    api.plan_destroy(plan)
+    P, Q, _, _ = cyl.mode_operators(n, k)
+    kappa = np.linalg.cond(np.linalg.eig(np.linalg.solve(P, Q))[1])
+    bar = 10 * 1e-13 * kappa + 3e-11 * max(1.0, (n / 128.0) ** 2)
+    for r in range(2):
+        Yo, _ = cyl.mode_adi(F[r], k, 1e-15)
+        assert _relmax(Y[r], Yo) <= bar, (r, bar)
