@@ -8,13 +8,14 @@
 //   inner  (5.7)-(5.9): A~_a Z A~_b + c Z = R per slice, as A~_a Z - Z(-c A~_b^{-1}) = R A~_b^{-1}:
 //          Z_h = [R - (A~_a - p) Z A~_b] (c + p A~_b)^{-1}
 //          (A~_a - q) Z+ = (R - c Z_h) A~_b^{-1} - q Z_h
-// Every operation is a banded product or a banded (even/odd decoupled, App. B)
+// FP64: every operation is a banded product or a banded (even/odd decoupled, App. B)
 // solve along one mode of the whole tensor: all slices of a level are solved at
 // once.  The solves run one thread per (line, parity) over 32 lines per CTA with
-// coalesced global traffic.  The same kernels run in FP64 and in FP32.
+// coalesced global traffic.
 //
 // FP32 + refinement: the nested ADI (every level in residual-propagating form, see
-// run_residual, hsolve_res, stein_res; every level's shifts on the tight
+// CubeRounds::run and hsolve_res; the inner level runs all its iterations in one launch,
+// one CTA per parity quarter of a slice, cube_unit.cuh; every level's shifts on the tight
 // Sturm-bisection interval of A~, 2.5x fewer inner iterations than on Lemma B.2's
 // at n = 256) runs in FP32 at loose level tolerances on
 // the normalised residual rho = R / max|R|, R = G - (T_01 + T_02 + T_12) Y computed
@@ -32,12 +33,11 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
-#include <type_traits>
 #include <vector>
 
 #include "../../include/fps.h"
 #include "cube.h"
-#include "cube_slice.cuh"
+#include "cube_unit.cuh"
 #include "device_info.h"
 #include "host_math.h"
 #include "trace.h"
@@ -48,31 +48,17 @@ namespace {
 
 constexpr int kLines = 32;  // lines per CTA of the solve kernels
 constexpr int kLineThreads = 128;  // threads per CTA: all move the tiles, the first 2 kLines sweep
-constexpr int kU = 8;       // global loads in flight per thread in the solve output phase
-
-template <typename T>
-struct V2;
-template <>
-struct V2<double> {
-    using type = double2;
-    static __device__ __forceinline__ double2 make(double a, double b) { return make_double2(a, b); }
-};
-template <>
-struct V2<float> {
-    using type = float2;
-    static __device__ __forceinline__ float2 make(double a, double b) { return make_float2((float)a, (float)b); }
-};
 
 // Y = sop * ((alpha A~ + beta) X along `mode`) + sr * R   (R may be null; Y may alias R)
-template <typename T>
-__global__ void cube_band_kernel(const T *__restrict__ X, const T *R, T *Y, const T *__restrict__ d,
-                                 const T *__restrict__ e, int n, int mode, T alpha, T beta, T sop, T sr)
+__global__ void cube_band_kernel(const double *__restrict__ X, const double *R, double *Y, const double *__restrict__ d,
+                                 const double *__restrict__ e, int n, int mode, double alpha, double beta,
+                                 double sop, double sr)
 {
     const int N = n * n * n;
     const int st = (mode == 0) ? n * n : ((mode == 1) ? n : 1);
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += gridDim.x * blockDim.x) {
         const int t = (mode == 0) ? idx / (n * n) : ((mode == 1) ? (idx / n) % n : idx % n);
-        T v = (alpha * d[t] + beta) * X[idx];
+        double v = (alpha * d[t] + beta) * X[idx];
         if (t >= 2) v = fma(alpha * e[t - 2], X[idx - 2 * st], v);
         if (t + 2 < n) v = fma(alpha * e[t], X[idx + 2 * st], v);
         v *= sop;
@@ -82,27 +68,17 @@ __global__ void cube_band_kernel(const T *__restrict__ X, const T *R, T *Y, cons
 }
 
 // Z = a X + b Y (element-wise; Z may alias X or Y)
-template <typename T>
-__global__ void cube_axpby_kernel(const T *X, const T *Y, T *Z, int N, T a, T b)
+__global__ void cube_axpby_kernel(const double *X, const double *Y, double *Z, int N, double a, double b)
 {
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += gridDim.x * blockDim.x)
         Z[idx] = fma(a, X[idx], b * Y[idx]);
 }
 
-// V = a X + b Y + c W (element-wise; V may alias any input)
-template <typename T>
-__global__ void cube_axpy3_kernel(const T *X, const T *Y, const T *W, T *V, int N, T a, T b, T c)
-{
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += gridDim.x * blockDim.x)
-        V[idx] = fma(a, X[idx], fma(b, Y[idx], c * W[idx]));
-}
-
-// Thomas factors of (alpha A~ + beta I) for a list of (alpha, beta) pairs, computed
-// in FP64 and stored in T: one thread per (set, parity); fac[set * n + t] =
+// Thomas factors of (alpha A~ + beta I) for a list of (alpha, beta) pairs, one
+// thread per (set, parity); fac[set * n + t] =
 // {1/den_t, alpha e_t / den_t}.
-template <typename T>
 __global__ void cube_factor_kernel(const double *__restrict__ d, const double *__restrict__ e, int n,
-                                   const double2 *__restrict__ ab, int nsets, typename V2<T>::type *__restrict__ fac)
+                                   const double2 *__restrict__ ab, int nsets, double2 *__restrict__ fac)
 {
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     if (tid >= 2 * nsets) return;
@@ -114,21 +90,17 @@ __global__ void cube_factor_kernel(const double *__restrict__ d, const double *_
         if (t >= 2) den -= alpha * e[t - 2] * u_prev;
         const double ip = 1.0 / den;
         const double u = alpha * e[t] * ip;
-        fac[(int64_t)set * n + t] = V2<T>::make(ip, u);
+        fac[(int64_t)set * n + t] = make_double2(ip, u);
         u_prev = u;
     }
 }
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
-// Asynchronous copy of one element (4 or 8 bytes) from global to shared memory.
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T *dst, const T *src)
+// Asynchronous copy of one element from global to shared memory.
+__device__ __forceinline__ void cp_async8(double *dst, const double *src)
 {
-    if constexpr (sizeof(T) == 8)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
 
 // Shared-memory row pitch of a contiguous-mode tile: odd, so that the 32 lanes of a
@@ -142,10 +114,9 @@ __host__ __device__ __forceinline__ int line_tile_elems(int n, bool contig)
 }
 
 // Dynamic shared memory of the line solve: the factor set and one or two tiles.
-template <typename T>
 int line_smem_bytes(int n, bool contig, int ntiles)
 {
-    return n * (int)sizeof(typename V2<T>::type) + ntiles * line_tile_elems(n, contig) * (int)sizeof(T);
+    return n * (int)sizeof(double2) + ntiles * line_tile_elems(n, contig) * (int)sizeof(double);
 }
 
 // 16-byte asynchronous copy (both addresses 16-byte aligned).
@@ -155,31 +126,26 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 }
 
 // Banded solves along one mode for kLines lines per CTA:
-//   IN = s1 R1 + s2 R2            (preband: IN = s1 (A~ R1) along the mode, R2 unused)
-//   X  = oscale (alpha A~ + beta)^{-1} IN + oin IN + oacc X      (X read only if oacc != 0)
+//   X = (alpha A~ + beta)^{-1} (R1 + s2 R2)      (R2 may be null)
 // The whole tile of R1 (and R2) is fetched with asynchronous copies (16-byte ones
 // when the rows are aligned), so one CTA has all its bytes in flight at once.  The
-// forward sweep forms IN as it goes; both Thomas sweeps (App. B parity decoupling:
-// warp = parity, lane = line) run in shared memory in chunks whose operands are
-// read ahead of the dependent FMAs, and the output combination is written back
-// coalesced.  X may alias R1 or R2.  Tile A holds R1, then z and x; tile B (present
-// when R2, oin or preband is used) holds R2, then IN (oin) or z and x (preband, A
-// keeping R1 for the stencil).
+// forward sweep forms the right-hand side as it goes; both Thomas sweeps (App. B parity
+// decoupling: warp = parity, lane = line) run in shared memory in chunks whose operands
+// are read ahead of the dependent FMAs, and the solution is written back coalesced.  X
+// may alias R1 or R2.  Tile A holds R1, then z and x; tile B holds R2.
 // CONTIG (mode 2): kLines consecutive lines, tile [line][t].  Otherwise (modes 0,
 // 1): kLines lines adjacent in mode 2, one CTA per (index of the other strided mode,
 // block of kLines), tile [t][line].
-template <typename T, bool CONTIG>
-__global__ void __launch_bounds__(kLineThreads) cube_line_kernel(const typename V2<T>::type *__restrict__ fac, const T *R1,
-                                                       T s1, const T *R2, T s2, T *X, int n, int mode, T oscale,
-                                                       T oin, T oacc, bool preband, const T *__restrict__ d,
-                                                       const T *__restrict__ e)
+template <bool CONTIG>
+__global__ void __launch_bounds__(kLineThreads) cube_line_kernel(const double2 *__restrict__ fac, const double *R1,
+                                                                 const double *R2, double s2, double *X, int n,
+                                                                 int mode)
 {
-    using F2 = typename V2<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tsz = line_tile_elems(n, CONTIG);
-    F2 *fs = reinterpret_cast<F2 *>(smem_raw);  // the factor set, n entries
-    T *A = reinterpret_cast<T *>(fs + n);
-    T *B = A + tsz;
+    double2 *fs = reinterpret_cast<double2 *>(smem_raw);  // the factor set, n entries
+    double *A = reinterpret_cast<double *>(fs + n);
+    double *B = A + tsz;
     for (int t = threadIdx.x; t < n; t += blockDim.x) fs[t] = fac[t];
     const int pitch = CONTIG ? contig_pitch(n) : 0;
     // geometry: element (li, t) of the tile <-> global offset gbase + li * gl + t * gt
@@ -211,14 +177,12 @@ __global__ void __launch_bounds__(kLineThreads) cube_line_kernel(const typename 
             li = q & 31;
         }
     };
-    const bool has_r2 = R2 != nullptr && !preband;
+    const bool has_r2 = R2 != nullptr;
     // strided tiles whose rows are whole, 16-byte aligned rows of the tensor move in
     // 16-byte pieces (V elements)
-    constexpr int V = 16 / (int)sizeof(T);
-    const bool vec = !CONTIG && nl == kLines && ((gt * (int64_t)sizeof(T)) % 16 == 0) &&
-                     ((gbase * (int64_t)sizeof(T)) % 16 == 0) && (((uintptr_t)R1 & 15) == 0) &&
-                     (!has_r2 || ((uintptr_t)R2 & 15) == 0) && (((uintptr_t)X & 15) == 0) &&
-                     ((n * (int)sizeof(F2)) % 16 == 0);
+    constexpr int V = 2;
+    const bool vec = !CONTIG && nl == kLines && gt % V == 0 && gbase % V == 0 && ((uintptr_t)R1 & 15) == 0 &&
+                     (!has_r2 || ((uintptr_t)R2 & 15) == 0) && ((uintptr_t)X & 15) == 0;
     const int total = kLines * n;
     if (vec) {
         for (int q = threadIdx.x * V; q < total; q += blockDim.x * V) {
@@ -233,290 +197,68 @@ __global__ void __launch_bounds__(kLineThreads) cube_line_kernel(const typename 
             qmap(q, li, t);
             if (li < nl) {
                 const int64_t g = gbase + li * gl + t * gt;
-                cp_async_elem(&A[sidx(li, t)], R1 + g);
-                if (has_r2) cp_async_elem(&B[sidx(li, t)], R2 + g);
+                cp_async8(&A[sidx(li, t)], R1 + g);
+                if (has_r2) cp_async8(&B[sidx(li, t)], R2 + g);
             }
         }
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
-    T *Z = preband ? B : A;  // z, then x
     const int lane = threadIdx.x & 31, par = threadIdx.x >> 5;
     const int m = (n - par + 1) / 2;  // unknowns of this parity: t = par + 2 i, i < m
     if (threadIdx.x < 2 * kLines && lane < nl) {
         // Both sweeps in chunks of kC steps: the chunk's operands are read from shared
         // memory first, so only the kC dependent FMAs remain on the critical path.
         constexpr int kC = 8;
-        T z = 0, u_prev = 0;
+        double z = 0, u_prev = 0;
         for (int i0 = 0; i0 < m; i0 += kC) {
-            T in[kC], uf[kC];
+            double in[kC], uf[kC];
 #pragma unroll
             for (int u = 0; u < kC; ++u) {
                 const int t = par + 2 * min(i0 + u, m - 1);
-                T v;
-                if (preband) {
-                    v = d[t] * A[sidx(lane, t)];
-                    if (t >= 2) v = fma(e[t - 2], A[sidx(lane, t - 2)], v);
-                    if (t + 2 < n) v = fma(e[t], A[sidx(lane, t + 2)], v);
-                    v *= s1;
-                } else {
-                    v = s1 * A[sidx(lane, t)];
-                    if (has_r2) v = fma(s2, B[sidx(lane, t)], v);
-                }
+                double v = A[sidx(lane, t)];
+                if (has_r2) v = fma(s2, B[sidx(lane, t)], v);
                 in[u] = v;
                 uf[u] = fs[t].y;
             }
 #pragma unroll
             for (int u = 0; u < kC; ++u)
                 if (i0 + u < m) {
-                    const int k = sidx(lane, par + 2 * (i0 + u));
                     z = fma(-u_prev, z, in[u]);
-                    Z[k] = z;
-                    if (oin != T(0)) B[k] = in[u];
+                    A[sidx(lane, par + 2 * (i0 + u))] = z;
                     u_prev = uf[u];
                 }
         }
-        T x = 0;
+        double x = 0;
         for (int i0 = m - 1; i0 >= 0; i0 -= kC) {
-            T zz[kC];
-            F2 ff[kC];
+            double zz[kC];
+            double2 ff[kC];
 #pragma unroll
             for (int u = 0; u < kC; ++u) {
                 const int t = par + 2 * max(i0 - u, 0);
-                zz[u] = Z[sidx(lane, t)];
+                zz[u] = A[sidx(lane, t)];
                 ff[u] = fs[t];
             }
 #pragma unroll
             for (int u = 0; u < kC; ++u)
                 if (i0 - u >= 0) {
                     x = fma(-ff[u].y, x, ff[u].x * zz[u]);
-                    Z[sidx(lane, par + 2 * (i0 - u))] = x;
+                    A[sidx(lane, par + 2 * (i0 - u))] = x;
                 }
         }
     }
     __syncthreads();
-    if (vec) {
-        for (int q0 = threadIdx.x * V; q0 < total; q0 += kU * blockDim.x * V) {
-            T xo[kU][V];
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const int q = q0 + u * blockDim.x * V;
-#pragma unroll
-                for (int w = 0; w < V; ++w) xo[u][w] = 0;
-                if (oacc != T(0) && q < total) {
-                    const int t = q >> 5, li = q & 31;
-                    const T *src = X + gbase + li + t * gt;
-#pragma unroll
-                    for (int w = 0; w < V; ++w) xo[u][w] = src[w];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const int q = q0 + u * blockDim.x * V;
-                if (q < total) {
-                    const int t = q >> 5, li = q & 31;
-                    const int k = t * kLines + li;
-                    T v[V];
-#pragma unroll
-                    for (int w = 0; w < V; ++w) {
-                        T val = oscale * Z[k + w];
-                        if (oin != T(0)) val = fma(oin, B[k + w], val);
-                        if (oacc != T(0)) val = fma(oacc, xo[u][w], val);
-                        v[w] = val;
-                    }
-                    T *dst = X + gbase + li + t * gt;
-                    if constexpr (sizeof(T) == 4)
-                        *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
-                    else
-                        *reinterpret_cast<double2 *>(dst) = make_double2(v[0], v[1]);
-                }
-            }
-        }
-    } else {
-        for (int q0 = threadIdx.x; q0 < total; q0 += kU * blockDim.x) {
-            T xo[kU];
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const int q = q0 + u * blockDim.x;
-                xo[u] = 0;
-                if (oacc != T(0) && q < total) {
-                    int li, t;
-                    qmap(q, li, t);
-                    if (li < nl) xo[u] = X[gbase + li * gl + t * gt];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const int q = q0 + u * blockDim.x;
-                if (q < total) {
-                    int li, t;
-                    qmap(q, li, t);
-                    if (li < nl) {
-                        const int k = sidx(li, t);
-                        T v = oscale * Z[k];
-                        if (oin != T(0)) v = fma(oin, B[k], v);
-                        if (oacc != T(0)) v = fma(oacc, xo[u], v);
-                        X[gbase + li * gl + t * gt] = v;
-                    }
-                }
-            }
-        }
-    }
-}
-
-// The two solves along `ma` of one residual-form inner iteration (stein_res) in one
-// launch, both with the set (A~ - q): with w = rho + (p - q) a1,
-//   rho <- (q - p) (A~ - q)^{-1} w + w,     Z <- (q - p) (A~ - q)^{-1} a1 + zacc Z.
-// Strided modes only (ma is 0 or 1); tiles [t][line]: A holds rho, then the z of the
-// w chain, then the new rho; B holds a1, then the z and x of the a1 chain.  The back
-// sweep recovers w_t = z_t + u_{t-2} z_{t-2} from the forward values below t (not yet
-// overwritten), so no third tile is needed.  Each thread runs both dependency chains.
-template <typename T>
-__global__ void __launch_bounds__(kLineThreads) cube_dual_kernel(const typename V2<T>::type *__restrict__ fac, T *rho,
-                                                                 const T *a1, T *Z, int n, int mode, T pq, T qp,
-                                                                 T zacc)
-{
-    using F2 = typename V2<T>::type;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    F2 *fs = reinterpret_cast<F2 *>(smem_raw);
-    T *A = reinterpret_cast<T *>(fs + n);
-    T *B = A + kLines * n;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) fs[t] = fac[t];
-    const int nkb = (n + kLines - 1) / kLines;
-    const int other = blockIdx.x / nkb, k0 = (blockIdx.x % nkb) * kLines;
-    const int64_t nn = (int64_t)n * n;
-    const int nl = min(kLines, n - k0);
-    const int64_t gbase = ((mode == 0) ? (int64_t)other * n : (int64_t)other * nn) + k0;
-    const int64_t gt = (mode == 0) ? nn : (int64_t)n;
-    constexpr int V = 16 / (int)sizeof(T);
-    const bool vec = nl == kLines && ((gt * (int64_t)sizeof(T)) % 16 == 0) && ((gbase * (int64_t)sizeof(T)) % 16 == 0) &&
-                     (((uintptr_t)rho & 15) == 0) && (((uintptr_t)a1 & 15) == 0) && (((uintptr_t)Z & 15) == 0) &&
-                     ((n * (int)sizeof(F2)) % 16 == 0);
-    const int total = kLines * n;
     if (vec) {
         for (int q = threadIdx.x * V; q < total; q += blockDim.x * V) {
             const int t = q >> 5, li = q & 31;
-            const int64_t g = gbase + li + t * gt;
-            cp_async16(&A[t * kLines + li], rho + g);
-            cp_async16(&B[t * kLines + li], a1 + g);
+            *reinterpret_cast<double2 *>(X + gbase + li + t * gt) = *reinterpret_cast<double2 *>(&A[t * kLines + li]);
         }
     } else {
         for (int q = threadIdx.x; q < total; q += blockDim.x) {
-            const int t = q >> 5, li = q & 31;
-            if (li < nl) {
-                const int64_t g = gbase + li + t * gt;
-                cp_async_elem(&A[t * kLines + li], rho + g);
-                cp_async_elem(&B[t * kLines + li], a1 + g);
-            }
-        }
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    __syncthreads();
-    const int lane = threadIdx.x & 31, par = threadIdx.x >> 5;
-    const int m = (n - par + 1) / 2;
-    if (threadIdx.x < 2 * kLines && lane < nl) {
-        constexpr int kC = 8;
-        T z1 = 0, z2 = 0, up = 0;
-        for (int i0 = 0; i0 < m; i0 += kC) {
-            T r[kC], a[kC], uf[kC];
-#pragma unroll
-            for (int u = 0; u < kC; ++u) {
-                const int t = par + 2 * min(i0 + u, m - 1);
-                r[u] = A[t * kLines + lane];
-                a[u] = B[t * kLines + lane];
-                uf[u] = fs[t].y;
-            }
-#pragma unroll
-            for (int u = 0; u < kC; ++u)
-                if (i0 + u < m) {
-                    const int k = (par + 2 * (i0 + u)) * kLines + lane;
-                    z1 = fma(-up, z1, fma(pq, a[u], r[u]));
-                    z2 = fma(-up, z2, a[u]);
-                    A[k] = z1;
-                    B[k] = z2;
-                    up = uf[u];
-                }
-        }
-        T x1 = 0, x2 = 0;
-        for (int i0 = m - 1; i0 >= 0; i0 -= kC) {
-            T za[kC + 1], zb[kC], ub[kC];
-            F2 ff[kC];
-#pragma unroll
-            for (int u = 0; u <= kC; ++u) {
-                const int i = max(i0 - u, 0);
-                za[u] = A[(par + 2 * i) * kLines + lane];
-            }
-#pragma unroll
-            for (int u = 0; u < kC; ++u) {
-                const int i = max(i0 - u, 0);
-                zb[u] = B[(par + 2 * i) * kLines + lane];
-                ff[u] = fs[par + 2 * i];
-                ub[u] = i >= 1 ? fs[par + 2 * i - 2].y : T(0);
-            }
-#pragma unroll
-            for (int u = 0; u < kC; ++u)
-                if (i0 - u >= 0) {
-                    const int k = (par + 2 * (i0 - u)) * kLines + lane;
-                    x1 = fma(-ff[u].y, x1, ff[u].x * za[u]);
-                    x2 = fma(-ff[u].y, x2, ff[u].x * zb[u]);
-                    const T w = (i0 - u >= 1) ? fma(ub[u], za[u + 1], za[u]) : za[u];
-                    A[k] = fma(qp, x1, w);
-                    B[k] = x2;
-                }
-        }
-    }
-    __syncthreads();
-    // out: kU groups of V consecutive elements per thread, the old Z of all groups
-    // loaded before any store (as in cube_line_kernel)
-    const int vw = vec ? V : 1;
-    for (int q0 = threadIdx.x * vw; q0 < total; q0 += kU * blockDim.x * vw) {
-        T zo[kU][V];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int q = q0 + u * blockDim.x * vw;
-#pragma unroll
-            for (int w = 0; w < V; ++w) zo[u][w] = 0;
-            const int t = q >> 5, li = q & 31;
-            if (zacc != T(0) && q < total && (vec || li < nl)) {
-                const T *src = Z + gbase + li + t * gt;
-                if (vec) {
-                    if constexpr (sizeof(T) == 4) {
-                        const float4 v4 = *reinterpret_cast<const float4 *>(src);
-                        zo[u][0] = v4.x, zo[u][1] = v4.y, zo[u][2] = v4.z, zo[u][3] = v4.w;
-                    } else {
-                        const double2 v2 = *reinterpret_cast<const double2 *>(src);
-                        zo[u][0] = v2.x, zo[u][1] = v2.y;
-                    }
-                } else {
-                    zo[u][0] = src[0];
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int q = q0 + u * blockDim.x * vw;
-            const int t = q >> 5, li = q & 31;
-            if (q < total && (vec || li < nl)) {
-                const int k = t * kLines + li;
-                const int64_t g = gbase + li + t * gt;
-                if (vec) {
-                    T zr[V];
-#pragma unroll
-                    for (int w = 0; w < V; ++w) zr[w] = fma(qp, B[k + w], zacc * zo[u][w]);
-                    if constexpr (sizeof(T) == 4) {
-                        *reinterpret_cast<float4 *>(rho + g) = make_float4(A[k], A[k + 1], A[k + 2], A[k + 3]);
-                        *reinterpret_cast<float4 *>(Z + g) = make_float4(zr[0], zr[1], zr[2], zr[3]);
-                    } else {
-                        *reinterpret_cast<double2 *>(rho + g) = make_double2(A[k], A[k + 1]);
-                        *reinterpret_cast<double2 *>(Z + g) = make_double2(zr[0], zr[1]);
-                    }
-                } else {
-                    rho[g] = A[k];
-                    Z[g] = fma(qp, B[k], zacc * zo[u][0]);
-                }
-            }
+            int li, t;
+            qmap(q, li, t);
+            if (li < nl) X[gbase + li * gl + t * gt] = A[sidx(li, t)];
         }
     }
 }
@@ -596,22 +338,57 @@ __global__ void __launch_bounds__(256) cube_residual_kernel(const double *__rest
     block_max_bits(local, rmax);
 }
 
-// rho = R / max|R| in FP32
-__global__ void cube_to32_kernel(const double *__restrict__ R, float *__restrict__ rho, int N,
-                                 const unsigned long long *__restrict__ rmax)
+// The FP32 tensors have mode 0 fastest, (i, j, k) at (j n + k) n + i; the FP64 ones mode 2.
+// Tiles of 32 x 32 over (i, k) at fixed j go through shared memory.
+__device__ __forceinline__ bool cube_tile(int n, int &j, int &i0, int &k0)
 {
+    const int nt = (n + 31) / 32;
+    const int b = blockIdx.x;
+    j = b / (nt * nt);
+    i0 = (b / nt) % nt * 32;
+    k0 = b % nt * 32;
+    return j < n;
+}
+
+// rho = R / max|R| in FP32
+__global__ void __launch_bounds__(256) cube_to32_kernel(const double *__restrict__ R, float *__restrict__ rho, int n,
+                                                        const unsigned long long *__restrict__ rmax)
+{
+    __shared__ float t[32][33];
     const double inv = 1.0 / __longlong_as_double((long long)*rmax);
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += gridDim.x * blockDim.x)
-        rho[idx] = (float)(R[idx] * inv);
+    int j, i0, k0;
+    if (!cube_tile(n, j, i0, k0)) return;
+    const int x = threadIdx.x & 31;
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (i0 + y < n && k0 + x < n) t[y][x] = (float)(R[((int64_t)(i0 + y) * n + j) * n + k0 + x] * inv);
+    __syncthreads();
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (k0 + y < n && i0 + x < n) rho[((int64_t)j * n + k0 + y) * n + i0 + x] = t[x][y];
 }
 
 // Y = (first ? 0 : Y) + max|R| delta  in FP64
-__global__ void cube_update_kernel(double *__restrict__ Y, const float *__restrict__ delta, int N,
-                                   const unsigned long long *__restrict__ rmax, bool first)
+__global__ void __launch_bounds__(256) cube_update_kernel(double *__restrict__ Y, const float *__restrict__ delta, int n,
+                                                          const unsigned long long *__restrict__ rmax, bool first)
 {
+    __shared__ float t[32][33];
     const double sc = __longlong_as_double((long long)*rmax);
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += gridDim.x * blockDim.x)
-        Y[idx] = fma(sc, (double)delta[idx], first ? 0.0 : Y[idx]);
+    int j, i0, k0;
+    if (!cube_tile(n, j, i0, k0)) return;
+    const int x = threadIdx.x & 31;
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (k0 + y < n && i0 + x < n) t[y][x] = delta[((int64_t)j * n + k0 + y) * n + i0 + x];
+    __syncthreads();
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (i0 + y < n && k0 + x < n) {
+            double *p = Y + ((int64_t)(i0 + y) * n + j) * n + k0 + x;
+            *p = fma(sc, (double)t[x][y], first ? 0.0 : *p);
+        }
+}
+
+unsigned tiles_for(int n)
+{
+    const int nt = (n + 31) / 32;
+    return (unsigned)(n * nt * nt);
 }
 
 int grid_for(int64_t N) { return (int)std::min<int64_t>((N + 255) / 256, 16 * (int64_t)current_sm_count()); }
@@ -628,11 +405,10 @@ int grid_for(int64_t N) { return (int)std::min<int64_t>((N + 255) / 256, 16 * (i
     } while (0)
 
 // ===========================================================================
-// CubeNested<T>
+// CubeSchedule
 // ===========================================================================
 
-template <typename T>
-int CubeNested<T>::add_stein(double c)
+int CubeSchedule::add_stein(double c)
 {
     // A~_a Z - Z B = C with sigma(A~_a) in [-hi, -lo] and sigma(B) = sigma(-c A~_b^{-1})
     // in [c/hi, c/lo]
@@ -641,20 +417,13 @@ int CubeNested<T>::add_stein(double c)
     const double a = -hi_, b = -lo_, cl = c / hi_, d = c / lo_;
     s.J = adi_iterations(a, b, cl, d, tol_in_);
     zolotarev_shifts(a, b, cl, d, s.J, s.p, s.q);
-    s.ab_off = steins_.empty() ? 0 : steins_.back().ab_off + 2 * steins_.back().J + 1;
-    max_sets_ = std::max(max_sets_, 2 * s.J + 1);
     steins_.push_back(std::move(s));
     return (int)steins_.size() - 1;
 }
 
-template <typename T>
-int CubeNested<T>::create(int64_t n, double tol, double tol_mid, double tol_in, bool residual, bool tight,
-                          std::string &err)
+void CubeSchedule::schedule(int64_t n, double tol, double tol_mid, double tol_in, bool residual, bool tight)
 {
-    residual_ = residual;
     n_ = n;
-    tol_ = tol;
-    tol_mid_ = tol_mid;
     tol_in_ = tol_in;
     lo_ = square_eps(n);
     hi_ = 1.0;
@@ -663,7 +432,7 @@ int CubeNested<T>::create(int64_t n, double tol, double tol_mid, double tol_in, 
     // spectrum in [lo^2, hi^2], so sigma(H) is in [2 lo^2, 2 hi^2] and sigma(-V) in
     // [-hi^2, -lo^2]
     const double e2 = lo_ * lo_, h2 = hi_ * hi_;
-    J_outer = adi_iterations(-h2, -e2, 2 * e2, 2 * h2, tol_);
+    J_outer = adi_iterations(-h2, -e2, 2 * e2, 2 * h2, tol);
     std::vector<double> pp, qq;
     zolotarev_shifts(-h2, -e2, 2 * e2, 2 * h2, J_outer, pp, qq);
     inner_per_run = 0;
@@ -672,175 +441,154 @@ int CubeNested<T>::create(int64_t n, double tol, double tol_mid, double tol_in, 
         o.p = qq[j];  // in sigma(H)'s interval [2 lo^2, 2 hi^2]
         o.q = pp[j];  // in sigma(-V)'s interval [-hi^2, -lo^2]
         o.stein_v = add_stein(o.p);
-        inner_per_run += (residual_ ? 2 : 1) * steins_[o.stein_v].J;
+        inner_per_run += (residual && j + 1 < J_outer ? 2 : 1) * steins_[o.stein_v].J;
         const double s = -o.q, lo = e2 + s / 2, hi = h2 + s / 2;
-        const int Jm = adi_iterations(-hi, -lo, lo, hi, tol_mid_);
+        const int Jm = adi_iterations(-hi, -lo, lo, hi, tol_mid);
         std::vector<double> am;
         zolotarev_shifts_symmetric(lo, hi, Jm, am);
         for (int m = 0; m < Jm; ++m) {
             Middle mid;
             mid.a = am[m];
             mid.stein = add_stein(s / 2 + am[m]);
-            inner_per_run += (residual_ && m + 1 < Jm ? 3 : 2) * steins_[mid.stein].J;
+            inner_per_run += (residual && m + 1 < Jm ? 3 : 2) * steins_[mid.stein].J;
             o.mid.push_back(mid);
         }
         outer_.push_back(std::move(o));
     }
-    std::vector<double2> hab;
-    for (const Stein &s : steins_) {
-        hab.push_back(make_double2(1.0, 0.0));
-        for (int l = 0; l < s.J; ++l) {
-            hab.push_back(make_double2(s.p[l], s.c));
-            hab.push_back(make_double2(1.0, -s.q[l]));
-        }
-    }
-    std::vector<double> d, e;
-    square_bands(n, d, e);
-    std::vector<T> dT(d.begin(), d.end()), eT(e.begin(), e.end());
-    const size_t N = (size_t)n * n * n;
-    auto alloc = [&](void **p, size_t b) -> cudaError_t {
-        cudaError_t r = cudaMalloc(p, b ? b : 1);
-        if (r == cudaSuccess) {
-            allocs_.push_back(*p);
-            bytes += (int64_t)b;
-        }
-        return r;
-    };
-    CUBE_CK(alloc((void **)&bd64_, sizeof(double) * n));
-    CUBE_CK(alloc((void **)&be64_, sizeof(double) * n));
-    CUBE_CK(alloc((void **)&bd_, sizeof(T) * n));
-    CUBE_CK(alloc((void **)&be_, sizeof(T) * n));
-    const int nwork = residual_ ? 9 : 8;
-    for (int w = 0; w < nwork; ++w) CUBE_CK(alloc((void **)&work_[w], sizeof(T) * N));
-    CUBE_CK(alloc(&fac_, sizeof(typename V2<T>::type) * (size_t)max_sets_ * n));
-    CUBE_CK(alloc((void **)&ab_, sizeof(double2) * hab.size()));
-    CUBE_CK(cudaMemcpy(bd64_, d.data(), sizeof(double) * n, cudaMemcpyHostToDevice));
-    CUBE_CK(cudaMemcpy(be64_, e.data(), sizeof(double) * n, cudaMemcpyHostToDevice));
-    CUBE_CK(cudaMemcpy(bd_, dT.data(), sizeof(T) * n, cudaMemcpyHostToDevice));
-    CUBE_CK(cudaMemcpy(be_, eT.data(), sizeof(T) * n, cudaMemcpyHostToDevice));
-    CUBE_CK(cudaMemcpy(ab_, hab.data(), sizeof(double2) * hab.size(), cudaMemcpyHostToDevice));
-    CUBE_CK(cudaFuncSetAttribute(cube_line_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 line_smem_bytes<T>((int)n, true, 2)));
-    CUBE_CK(cudaFuncSetAttribute(cube_line_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 line_smem_bytes<T>((int)n, false, 2)));
-    CUBE_CK(cudaFuncSetAttribute(cube_dual_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 line_smem_bytes<T>((int)n, false, 2)));
-    fac_entry_ = -1;
-    slice_ = false;
-    if (std::is_same<T, float>::value && residual_ && std::getenv("FPS_CUBE_SLICE") != nullptr)
-        CUBE_CK(slice_setup((int)n, &slice_));
-    return FPS_OK;
 }
 
-template <typename T>
-void CubeNested<T>::release()
+cudaError_t CubeSchedule::alloc(void **p, size_t b)
+{
+    cudaError_t r = cudaMalloc(p, b ? b : 1);
+    if (r == cudaSuccess) {
+        allocs_.push_back(*p);
+        bytes += (int64_t)b;
+    }
+    return r;
+}
+
+cudaError_t CubeSchedule::copy(void **p, const void *src, size_t b)
+{
+    const cudaError_t r = alloc(p, b);
+    return r == cudaSuccess ? cudaMemcpy(*p, src, b, cudaMemcpyHostToDevice) : r;
+}
+
+void CubeSchedule::release()
 {
     for (void *p : allocs_) cudaFree(p);
     allocs_.clear();
 }
 
-template <typename T>
-cudaError_t CubeNested<T>::band(const T *X, const T *R, T *Y, int mode, double alpha, double beta, double sop,
-                                double sr)
-{
-    const int64_t N = n_ * n_ * n_;
-    cube_band_kernel<T><<<grid_for(N), 256, 0, st_>>>(X, R, Y, bd_, be_, (int)n_, mode, (T)alpha, (T)beta, (T)sop,
-                                                       (T)sr);
-    ++launches;
-    return cudaGetLastError();
-}
+// ===========================================================================
+// CubeNested
+// ===========================================================================
 
-template <typename T>
-cudaError_t CubeNested<T>::axpby(const T *X, const T *Y, T *Z, double a, double b)
+int CubeNested::create(int64_t n, double tol, double tol_level, std::string &err)
 {
-    const int64_t N = n_ * n_ * n_;
-    cube_axpby_kernel<T><<<grid_for(N), 256, 0, st_>>>(X, Y, Z, (int)N, (T)a, (T)b);
-    ++launches;
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t CubeNested<T>::axpy3(const T *X, const T *Y, const T *W, T *V, double a, double b, double c)
-{
-    const int64_t N = n_ * n_ * n_;
-    cube_axpy3_kernel<T><<<grid_for(N), 256, 0, st_>>>(X, Y, W, V, (int)N, (T)a, (T)b, (T)c);
-    ++launches;
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t CubeNested<T>::solve(int set, const T *R1, double s1, const T *R2, double s2, T *X, int mode,
-                                 double oscale, double oacc, double oin, bool preband)
-{
-    using F2 = typename V2<T>::type;
-    const F2 *fac = reinterpret_cast<const F2 *>(fac_) + (int64_t)set * n_;
-    const int n = (int)n_;
-    const int ntiles = (R2 != nullptr || oin != 0.0 || preband) ? 2 : 1;
-    if (mode == 2) {
-        const int blocks = (n * n + kLines - 1) / kLines;
-        const int smem = line_smem_bytes<T>(n, true, ntiles);
-        cube_line_kernel<T, true><<<blocks, kLineThreads, smem, st_>>>(fac, R1, (T)s1, R2, (T)s2, X, n, mode,
-                                                                     (T)oscale, (T)oin, (T)oacc, preband, bd_, be_);
-    } else {
-        const int nkb = (n + kLines - 1) / kLines;
-        const int smem = line_smem_bytes<T>(n, false, ntiles);
-        cube_line_kernel<T, false><<<n * nkb, kLineThreads, smem, st_>>>(fac, R1, (T)s1, R2, (T)s2, X, n, mode,
-                                                                       (T)oscale, (T)oin, (T)oacc, preband, bd_,
-                                                                       be_);
+    schedule(n, tol, tol_level, tol_level, false, false);
+    std::vector<double2> ab;
+    int64_t sets = 0;
+    for (Stein &s : steins_) {
+        s.off = (int64_t)ab.size();
+        sets = std::max(sets, 2 * (int64_t)s.J + 1);
+        ab.push_back(make_double2(1.0, 0.0));
+        for (int l = 0; l < s.J; ++l) {
+            ab.push_back(make_double2(s.p[l], s.c));
+            ab.push_back(make_double2(1.0, -s.q[l]));
+        }
     }
+    std::vector<double> d, e;
+    square_bands(n, d, e);
+    const size_t N = (size_t)n * n * n;
+    CUBE_CK(copy((void **)&bd_, d.data(), sizeof(double) * n));
+    CUBE_CK(copy((void **)&be_, e.data(), sizeof(double) * n));
+    for (double *&w : work_) CUBE_CK(alloc((void **)&w, sizeof(double) * N));
+    CUBE_CK(alloc((void **)&fac_, sizeof(double2) * (size_t)sets * n));
+    CUBE_CK(copy((void **)&ab_, ab.data(), sizeof(double2) * ab.size()));
+    CUBE_CK(cudaFuncSetAttribute(cube_line_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 line_smem_bytes((int)n, true, 2)));
+    CUBE_CK(cudaFuncSetAttribute(cube_line_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 line_smem_bytes((int)n, false, 2)));
+    entry_ = -1;
+    return FPS_OK;
+}
+
+cudaError_t CubeNested::band(const double *X, const double *R, double *Y, int mode, double alpha, double beta,
+                             double sop, double sr)
+{
+    const int64_t N = n_ * n_ * n_;
+    cube_band_kernel<<<grid_for(N), 256, 0, st_>>>(X, R, Y, bd_, be_, (int)n_, mode, alpha, beta, sop, sr);
     ++launches;
     return cudaGetLastError();
 }
 
-template <typename T>
-int CubeNested<T>::load_factors(int entry, std::string &err)
+cudaError_t CubeNested::axpby(const double *X, const double *Y, double *Z, double a, double b)
 {
-    if (fac_entry_ == entry) return FPS_OK;
+    const int64_t N = n_ * n_ * n_;
+    cube_axpby_kernel<<<grid_for(N), 256, 0, st_>>>(X, Y, Z, (int)N, a, b);
+    ++launches;
+    return cudaGetLastError();
+}
+
+cudaError_t CubeNested::solve(int set, const double *R1, const double *R2, double s2, double *X, int mode)
+{
+    const double2 *fac = fac_ + (int64_t)set * n_;
+    const int n = (int)n_;
+    const int smem = line_smem_bytes(n, mode == 2, R2 ? 2 : 1);
+    if (mode == 2)
+        cube_line_kernel<true><<<(n * n + kLines - 1) / kLines, kLineThreads, smem, st_>>>(fac, R1, R2, s2, X, n, mode);
+    else
+        cube_line_kernel<false>
+            <<<n * ((n + kLines - 1) / kLines), kLineThreads, smem, st_>>>(fac, R1, R2, s2, X, n, mode);
+    ++launches;
+    return cudaGetLastError();
+}
+
+int CubeNested::load_factors(int entry, std::string &err)
+{
+    if (entry_ == entry) return FPS_OK;
     const Stein &S = steins_[entry];
     const int nsets = 2 * S.J + 1;
     // factor sets: 0 = A~; 1 + 2l = c + p_l A~; 2 + 2l = A~ - q_l
-    cube_factor_kernel<T><<<(2 * nsets + 127) / 128, 128, 0, st_>>>(bd64_, be64_, (int)n_, ab_ + S.ab_off, nsets,
-                                                                     reinterpret_cast<typename V2<T>::type *>(fac_));
+    cube_factor_kernel<<<(2 * nsets + 127) / 128, 128, 0, st_>>>(bd_, be_, (int)n_, ab_ + S.off, nsets, fac_);
     ++launches;
     CUBE_CK(cudaGetLastError());
-    fac_entry_ = entry;
+    entry_ = entry;
     return FPS_OK;
 }
 
 // Z = (T_ab + c)^{-1} R, the inner level in the paper's form (entry = schedule
 // index).  Uses work_[0], work_[1].
-template <typename T>
-int CubeNested<T>::stein(int ma, int mb, int entry, const T *R, T *Z, std::string &err)
+int CubeNested::stein(int ma, int mb, int entry, const double *R, double *Z, std::string &err)
 {
     int st = load_factors(entry, err);
     if (st != FPS_OK) return st;
     const Stein &S = steins_[entry];
-    T *W1 = work_[0], *W2 = work_[1];
+    double *W1 = work_[0], *W2 = work_[1];
     const double c = S.c;
     for (int l = 0; l < S.J; ++l) {
-        const T *U = R;
+        const double *U = R;
         if (l > 0) {
             CUBE_CK(band(Z, nullptr, W1, mb, 1.0, 0.0, 1.0, 0.0));                // Z A~_b
             CUBE_CK(band(W1, R, W2, ma, 1.0, -S.p[l], -1.0, 1.0));                // R - (A~_a - p) ( . )
             U = W2;
         }
-        CUBE_CK(solve(1 + 2 * l, U, 1.0, nullptr, 0.0, W1, mb, 1.0, 0.0, 0.0, false));  // Z_h = ( . ) (c + p A~_b)^{-1}
-        CUBE_CK(solve(0, R, 1.0, W1, -c, W2, mb, 1.0, 0.0, 0.0, false));                 // (R - c Z_h) A~_b^{-1}
-        CUBE_CK(solve(2 + 2 * l, W2, 1.0, W1, -S.q[l], Z, ma, 1.0, 0.0, 0.0, false));    // (A~_a - q)^{-1} ( . - q Z_h)
+        CUBE_CK(solve(1 + 2 * l, U, nullptr, 0.0, W1, mb));    // Z_h = ( . ) (c + p A~_b)^{-1}
+        CUBE_CK(solve(0, R, W1, -c, W2, mb));              // (R - c Z_h) A~_b^{-1}
+        CUBE_CK(solve(2 + 2 * l, W2, W1, -S.q[l], Z, ma));  // (A~_a - q)^{-1} ( . - q Z_h)
     }
     return FPS_OK;
 }
 
 // Y = (T_01 + T_02 + s)^{-1} R with s = -o.q, the middle level in the paper's
 // form.  Uses work_[2..4].
-template <typename T>
-int CubeNested<T>::hsolve(const Outer &o, const T *R, T *Y, std::string &err)
+int CubeNested::hsolve(const Outer &o, const double *R, double *Y, std::string &err)
 {
     const double s = -o.q;
-    T *Wh = work_[2], *T1 = work_[3], *T2 = work_[4];
+    double *Wh = work_[2], *T1 = work_[3], *T2 = work_[4];
     for (size_t m = 0; m < o.mid.size(); ++m) {
         const double a = o.mid[m].a;
-        const T *U = R;  // R - (T_01 + s/2 - a) Y, with Y = 0 at m = 0
+        const double *U = R;  // R - (T_01 + s/2 - a) Y, with Y = 0 at m = 0
         if (m > 0) {
             CUBE_CK(band(Y, nullptr, T1, 0, 1.0, 0.0, 1.0, 0.0));
             CUBE_CK(band(T1, R, T2, 1, 1.0, 0.0, -1.0, 1.0));
@@ -859,134 +607,14 @@ int CubeNested<T>::hsolve(const Outer &o, const T *R, T *Y, std::string &err)
     return FPS_OK;
 }
 
-// The inner level with its residual carried.  The slice equation is the Sylvester
-// equation A Z - Z B = C with A = A~_a, B = -c A~_b^{-1}, C = R A~_b^{-1}; with
-// rho = C - A Z + Z B the two half-steps of Algorithm 2 become
-//   rho+ = (A - q)^{-1} (A - p) rho (B - p)^{-1} (B - q),
-//   Z+   = Z + (q - p) (A - q)^{-1} rho (B - p)^{-1},
-// and rho (B - p)^{-1} = -rho A~_b (c + p A~_b)^{-1}.  Per iteration two launches:
-// a1 = rho (B - p)^{-1} along b (the product with A~_b folded in), then one
-// cube_dual_kernel along a for rho+ = c1 + (q - p)(A - q)^{-1} c1 with
-// c1 = rho + (p - q) a1 (in place) and Z += (q - p)(A - q)^{-1} a1 (the last
-// iteration needs only the Z solve).  Solves Z = (T_ab + c)^{-1} (r1 R1 + r2 R2), or
-// adds it to Z when accumulate.  Uses work_[0], work_[1].
-template <typename T>
-int CubeNested<T>::stein_res(int ma, int mb, int entry, const T *R1, double r1, const T *R2, double r2, T *Z,
-                             bool accumulate, std::string &err)
-{
-    int st = load_factors(entry, err);
-    if (st != FPS_OK) return st;
-    const Stein &S = steins_[entry];
-    if constexpr (std::is_same<T, float>::value) {
-        if (slice_) {  // all J iterations with every slice on chip (cube_slice.cu)
-            SliceArgs sa;
-            sa.fac = reinterpret_cast<const float2 *>(fac_);
-            sa.ab = ab_ + S.ab_off;
-            sa.J = S.J;
-            sa.R1 = R1;
-            sa.R2 = R2;
-            sa.r1 = (float)r1;
-            sa.r2 = (float)r2;
-            sa.Z = Z;
-            sa.accumulate = accumulate;
-            sa.d = bd_;
-            sa.e = be_;
-            sa.n = (int)n_;
-            sa.ma = ma;
-            sa.mb = mb;
-            CUBE_CK(launch_stein_slice(sa, st_));
-            ++launches;
-            return FPS_OK;
-        }
-    }
-    T *rho = work_[0], *a1 = work_[1];
-    CUBE_CK(solve(0, R1, r1, R2, r2, rho, mb, 1.0, 0.0, 0.0, false));                  // rho = R A~_b^{-1}
-    for (int l = 0; l < S.J; ++l) {
-        const double p = S.p[l], q = S.q[l];
-        if (l == 0) CUBE_CK(solve(1, R1, -r1, R2, -r2, a1, mb, 1.0, 0.0, 0.0, false));    // rho A~_b = R
-        else CUBE_CK(solve(1 + 2 * l, rho, -1.0, nullptr, 0.0, a1, mb, 1.0, 0.0, 0.0, true));
-        const double zacc = (l > 0 || accumulate) ? 1.0 : 0.0;
-        if (l + 1 < S.J) {  // both solves along ma in one launch
-            using F2 = typename V2<T>::type;
-            const int n = (int)n_;
-            const int nkb = (n + kLines - 1) / kLines;
-            cube_dual_kernel<T><<<n * nkb, kLineThreads, line_smem_bytes<T>(n, false, 2), st_>>>(
-                reinterpret_cast<const F2 *>(fac_) + (int64_t)(2 + 2 * l) * n, rho, a1, Z, n, ma, (T)(p - q),
-                (T)(q - p), (T)zacc);
-            ++launches;
-            CUBE_CK(cudaGetLastError());
-        } else {
-            CUBE_CK(solve(2 + 2 * l, a1, 1.0, nullptr, 0.0, Z, ma, q - p, zacc, 0.0, false));
-        }
-    }
-    return FPS_OK;
-}
-
-// The middle level with its residual carried: for A' W + B' W = R (A' = T_01 + s/2,
-// B' = T_02 + s/2) and shifts +-a,
-//   rho+ = [I - 2a (A' + a)^{-1}] [I - 2a (B' + a)^{-1}] rho,
-//   W+   = W + (A' + a)^{-1} 2a (B' + a)^{-1} rho,
-// three slice Stein solves per iteration (two in the last).  Uses work_[3..5].
-template <typename T>
-int CubeNested<T>::hsolve_res(const Outer &o, const T *R, T *W, std::string &err)
-{
-    T *rho = work_[3], *v = work_[4], *g = work_[5];
-    const size_t J = o.mid.size();
-    for (size_t m = 0; m < J; ++m) {
-        const double a = o.mid[m].a;
-        const int entry = o.mid[m].stein;
-        const T *r = (m == 0) ? R : rho;
-        int st = stein_res(0, 2, entry, r, 1.0, nullptr, 0.0, v, false, err);        // v = (B' + a)^{-1} rho
-        if (st != FPS_OK) return st;
-        if (m + 1 < J) {
-            st = stein_res(0, 1, entry, r, 1.0, v, -2.0 * a, g, false, err);         // g = (A' + a)^{-1} (rho - 2a v)
-            if (st != FPS_OK) return st;
-            CUBE_CK(axpy3(r, v, g, rho, 1.0, -2.0 * a, -2.0 * a));                  // rho+ = rho - 2a v - 2a g
-        }
-        st = stein_res(0, 1, entry, v, 2.0 * a, nullptr, 0.0, W, m > 0, err);        // W += (A' + a)^{-1} 2a v
-        if (st != FPS_OK) return st;
-    }
-    return FPS_OK;
-}
-
-// The outer level with the residual rho = G - (H + V) Y carried instead of Y's
-// right-hand sides.  The two half-steps of (5.3)-(5.4) are Y_h = Y + (V + p)^{-1} rho
-// and Y+ = Y_h + (H - q)^{-1} rho_h, so that, the operators commuting,
-//   rho+ = [I + (q - p)(V + p)^{-1}] [I + (q - p)(H - q)^{-1}] rho,
-//   Y+   = Y + (V + p)^{-1} (p - q) (H - q)^{-1} rho:
-// only residuals are solved with and no product with H or V of a growing iterate
-// is formed, which keeps FP32 rounding relative to the residual (the paper's form
-// loses it to cancellation at small shifts).  Uses work_[6..8].
-template <typename T>
-int CubeNested<T>::run_residual(const T *G, T *Y, std::string &err)
-{
-    T *rho = work_[6], *w = work_[7], *u = work_[8];
-    for (int j = 0; j < J_outer; ++j) {
-        const Outer &o = outer_[j];
-        const T *r = (j == 0) ? G : rho;
-        int s = hsolve_res(o, r, w, err);                                         // w = (H - q)^{-1} rho
-        if (s != FPS_OK) return s;
-        s = stein_res(1, 2, o.stein_v, r, 1.0, w, o.q - o.p, u, false, err);      // u = (V + p)^{-1} c,
-        if (s != FPS_OK) return s;                                                //   c = rho + (q - p) w
-        CUBE_CK(axpy3(r, w, u, rho, 1.0, o.q - o.p, o.q - o.p));                  // rho+ = c + (q - p) u
-        // the scalar p - q enters with the right-hand side: w ~ rho / eps^2 and
-        // (V + p)^{-1} w ~ rho / eps^4 would leave the FP32 range for n >~ 100
-        s = stein_res(1, 2, o.stein_v, w, o.p - o.q, nullptr, 0.0, Y, j > 0, err); // Y += (V + p)^{-1} (p - q) w
-        if (s != FPS_OK) return s;
-    }
-    return FPS_OK;
-}
-
-template <typename T>
-int CubeNested<T>::run(const T *G, T *Y, cudaStream_t st, std::string &err)
+int CubeNested::run(const double *G, double *Y, cudaStream_t st, std::string &err)
 {
     st_ = st;
     launches = 0;
-    if (residual_) return run_residual(G, Y, err);
-    T *Yh = work_[5], *T1 = work_[6], *T2 = work_[7];
+    double *Yh = work_[5], *T1 = work_[6], *T2 = work_[7];
     for (int j = 0; j < J_outer; ++j) {
         const Outer &o = outer_[j];
-        const T *U = G;  // G - (H - p) Y, with Y = 0 at j = 0
+        const double *U = G;  // G - (H - p) Y, with Y = 0 at j = 0
         if (j > 0) {
             CUBE_CK(band(Y, nullptr, T2, 0, 1.0, 0.0, 1.0, 0.0));      // A~_0 Y
             CUBE_CK(band(T2, G, T1, 1, 1.0, 0.0, -1.0, 1.0));          // G - T_01 Y
@@ -1006,8 +634,123 @@ int CubeNested<T>::run(const T *G, T *Y, cudaStream_t st, std::string &err)
     return FPS_OK;
 }
 
-template class CubeNested<double>;
-template class CubeNested<float>;
+// ===========================================================================
+// CubeRounds
+// ===========================================================================
+
+int CubeRounds::create(int64_t n, double tol, double tol_mid, double tol_in, std::string &err)
+{
+    schedule(n, tol, tol_mid, tol_in, true, true);
+    unit_ = unit_half(n);
+    if (!unit_) {
+        err = "the cube supports n <= 320";
+        return FPS_ERR_UNSUPPORTED;
+    }
+    std::vector<double> d, e;
+    square_bands(n, d, e);
+    const size_t N = (size_t)n * n * n;
+    CUBE_CK(copy((void **)&bd_, d.data(), sizeof(double) * n));
+    CUBE_CK(copy((void **)&be_, e.data(), sizeof(double) * n));
+    for (float *&w : work_) CUBE_CK(alloc((void **)&w, sizeof(float) * N));
+    CUBE_CK(unit_setup(unit_));
+    // tables of every entry of the schedule
+    int64_t total = 0;
+    std::vector<UnitEntry> entries;
+    std::vector<double2> pq;
+    for (Stein &s : steins_) {
+        s.off = total;
+        entries.push_back(UnitEntry{s.c, total, (int)pq.size(), s.J});
+        for (int l = 0; l < s.J; ++l) pq.push_back(make_double2(s.p[l], s.q[l]));
+        total += (int64_t)s.J * 4 * unit_table(unit_);
+    }
+    CUBE_CK(alloc((void **)&tab_, sizeof(float) * (size_t)total));
+    CUBE_CK(alloc((void **)&bands_, sizeof(float) * 2 * unit_bands(unit_)));
+    CUBE_CK(copy((void **)&entries_, entries.data(), sizeof(UnitEntry) * entries.size()));
+    CUBE_CK(copy((void **)&pq_, pq.data(), sizeof(double2) * pq.size()));
+    CUBE_CK(launch_unit_bands(bd_, be_, (int)n, unit_, bands_, nullptr));
+    CUBE_CK(launch_unit_tables(entries_, (int)entries.size(), (int)pq.size(), pq_, bd_, be_, (int)n, unit_, tab_,
+                               nullptr));
+    CUBE_CK(cudaStreamSynchronize(nullptr));
+    return FPS_OK;
+}
+
+// One launch of the inner level: every job's out = kR R + kZ (T_ab + c)^{-1} R + kacc out
+// (R = r1 R1 + r2 R2), the jobs sharing the schedule entry.
+int CubeRounds::stein(int ma, int mb, int entry, const UnitJob *jobs, int njobs, std::string &err)
+{
+    const Stein &S = steins_[entry];
+    // mode 0 fastest: both slice kinds of the middle level contain it, so their elements are
+    // read and written in runs
+    const int64_t st[3] = {1, n_ * n_, n_};
+    UnitArgs a;
+    a.tab = tab_ + S.off;
+    a.bands = bands_;
+    a.J = S.J;
+    a.n = (int)n_;
+    a.njobs = njobs;
+    a.sa = st[ma];
+    a.sb = st[mb];
+    a.sc = st[3 - ma - mb];
+    for (int q = 0; q < njobs; ++q) a.job[q] = jobs[q];
+    CUBE_CK(launch_stein_units(a, unit_, st_));
+    ++launches;
+    return FPS_OK;
+}
+
+// The middle level with its residual carried: for A' W + B' W = R (A' = T_01 + s/2,
+// B' = T_02 + s/2) and shifts +-a,
+//   rho+ = [I - 2a (A' + a)^{-1}] [I - 2a (B' + a)^{-1}] rho,
+//   W+   = W + (A' + a)^{-1} 2a (B' + a)^{-1} rho,
+// with v = (B' + a)^{-1} rho in one launch and (A' + a)^{-1} of rho - 2a v (giving rho+)
+// and of 2a v (added to W) in a second.  Uses work_[0..1].
+int CubeRounds::hsolve_res(const Outer &o, const float *R, float *W, std::string &err)
+{
+    float *rho = work_[0], *v = work_[1];
+    const size_t J = o.mid.size();
+    for (size_t m = 0; m < J; ++m) {
+        const float a2 = (float)(2.0 * o.mid[m].a);
+        const int entry = o.mid[m].stein;
+        const float *r = (m == 0) ? R : rho;
+        const UnitJob first{r, nullptr, v, 1.0f, 0.0f, 0.0f, 1.0f, 0.0f};
+        int st = stein(0, 2, entry, &first, 1, err);
+        if (st != FPS_OK) return st;
+        const UnitJob jobs[2] = {{v, nullptr, W, a2, 0.0f, 0.0f, 1.0f, m > 0 ? 1.0f : 0.0f},
+                                 {r, v, rho, 1.0f, -a2, 1.0f, -a2, 0.0f}};
+        st = stein(0, 1, entry, jobs, m + 1 < J ? 2 : 1, err);
+        if (st != FPS_OK) return st;
+    }
+    return FPS_OK;
+}
+
+// The outer level with the residual rho = G - (H + V) Y carried instead of Y's
+// right-hand sides.  The two half-steps of (5.3)-(5.4) are Y_h = Y + (V + p)^{-1} rho
+// and Y+ = Y_h + (H - q)^{-1} rho_h, so that, the operators commuting,
+//   rho+ = [I + (q - p)(V + p)^{-1}] [I + (q - p)(H - q)^{-1}] rho,
+//   Y+   = Y + (V + p)^{-1} (p - q) (H - q)^{-1} rho:
+// only residuals are solved with and no product with H or V of a growing iterate
+// is formed, which keeps FP32 rounding relative to the residual (the paper's form
+// loses it to cancellation at small shifts).  Uses work_[2..3].
+int CubeRounds::run(const float *G, float *Y, cudaStream_t st, std::string &err)
+{
+    st_ = st;
+    launches = 0;
+    float *rho = work_[2], *w = work_[3];
+    for (int j = 0; j < J_outer; ++j) {
+        const Outer &o = outer_[j];
+        const float *r = (j == 0) ? G : rho;
+        int s = hsolve_res(o, r, w, err);  // w = (H - q)^{-1} rho
+        if (s != FPS_OK) return s;
+        // Y += (V + p)^{-1} (p - q) w and, with c = rho + (q - p) w, rho+ = c + (q - p) (V + p)^{-1} c.
+        // The scalar p - q enters with the right-hand side: w ~ rho / eps^2 and
+        // (V + p)^{-1} w ~ rho / eps^4 would leave the FP32 range for n >~ 100
+        const float qp = (float)(o.q - o.p);
+        const UnitJob jobs[2] = {{w, nullptr, Y, -qp, 0.0f, 0.0f, 1.0f, j > 0 ? 1.0f : 0.0f},
+                                 {r, w, rho, 1.0f, qp, 1.0f, qp, 0.0f}};
+        s = stein(1, 2, o.stein_v, jobs, j + 1 < J_outer ? 2 : 1, err);
+        if (s != FPS_OK) return s;
+    }
+    return FPS_OK;
+}
 
 // ===========================================================================
 // CubeEngine
@@ -1066,8 +809,8 @@ int CubeEngine::create(int64_t n, double tol, int precision, std::string &err)
     CUBE_CK(cudaMemcpy(bs_, s.data(), sizeof(double) * n, cudaMemcpyHostToDevice));
     int st;
     if (precision == FPS_FP64) {
-        n64_ = new CubeNested<double>();
-        st = n64_->create(n, tol, 1e-15, 1e-15, false, false, err);
+        n64_ = new CubeNested();
+        st = n64_->create(n, tol, 1e-15, err);
         if (st != FPS_OK) return st;
         J_outer = n64_->J_outer;
         bytes += n64_->bytes;
@@ -1077,9 +820,9 @@ int CubeEngine::create(int64_t n, double tol, int precision, std::string &err)
         CUBE_CK(alloc((void **)&delta_, sizeof(float) * N));
         CUBE_CK(alloc((void **)&d_max_, sizeof(unsigned long long)));
         CUBE_CK(cudaMallocHost((void **)&h_max_, sizeof(unsigned long long)));
-        n32_ = new CubeNested<float>();
+        n32_ = new CubeRounds();
         ref_tol_outer = refinement_outer_tol(n, tol);
-        st = n32_->create(n, ref_tol_outer, kRefTolMid, kRefTolIn, true, true, err);
+        st = n32_->create(n, ref_tol_outer, kRefTolMid, kRefTolIn, err);
         if (st != FPS_OK) return st;
         J_outer = J_outer_inner = n32_->J_outer;
         bytes += n32_->bytes;
@@ -1152,13 +895,13 @@ int CubeEngine::solve_cube(const double *F, double *X, cudaStream_t st, std::str
                 break;
             }
             if (r == max_rounds) break;
-            cube_to32_kernel<<<grid_for(N), 256, 0, st>>>(R_, rho_, (int)N, d_max_);
+            cube_to32_kernel<<<tiles_for((int)n_), 256, 0, st>>>(R_, rho_, (int)n_, d_max_);
             ++launches_last;
             CUBE_CK(cudaGetLastError());
             const int s = n32_->run(rho_, delta_, st, err);
             launches_last += n32_->launches;
             if (s != FPS_OK) return s;
-            cube_update_kernel<<<grid_for(N), 256, 0, st>>>(Y_, delta_, (int)N, d_max_, r == 0);
+            cube_update_kernel<<<tiles_for((int)n_), 256, 0, st>>>(Y_, delta_, (int)n_, d_max_, r == 0);
             ++launches_last;
             CUBE_CK(cudaGetLastError());
             inner_iters += n32_->inner_per_run;

@@ -1,12 +1,12 @@
 // Nested ADI for the cube (Sec. 5) (internal header).
 //
-// CubeNested<T> runs the three-level ADI of Sec. 5 in arithmetic T on the
-// symmetrised tensor equation (T_01 + T_02 + T_12) Y = G; its schedule (every
-// shift of every level) is fixed at plan time.  CubeEngine is the plan object:
-// FP64 runs the nested ADI once at the requested tolerance (inner and middle
-// levels to 1e-15); FP32 + refinement runs it in FP32 at loose tolerances, every
-// level in residual-propagating form, inside an FP64 defect-correction loop on
-// the residual G - (T_01 + T_02 + T_12) Y.
+// The nested ADI runs the three levels of Sec. 5 on the symmetrised tensor equation
+// (T_01 + T_02 + T_12) Y = G; its schedule (every shift of every level) is fixed at plan
+// time.  CubeEngine is the plan object: FP64 runs the nested ADI once at the requested
+// tolerance in the paper's form (CubeNested, inner and middle levels to 1e-15); FP32 +
+// refinement runs it in FP32 at loose tolerances, every level in residual-propagating form
+// (CubeRounds), inside an FP64 defect-correction loop on the residual
+// G - (T_01 + T_02 + T_12) Y.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -14,30 +14,25 @@
 #include <string>
 #include <vector>
 
+#include "cube_unit.cuh"
+
 namespace fps {
 
-template <typename T>
-class CubeNested {
+// Shifts of every level and the device memory of a nested ADI.
+class CubeSchedule {
 public:
-    // tol: outer tolerance of (2.9); tol_mid / tol_in: middle and inner levels;
-    // residual: run every level in residual-propagating form (the FP32 rounds);
-    // tight: every level's intervals from the Sturm-bisection interval of A~ instead
-    // of Lemma B.2's [-1, -1/(30 n^4)].
-    int create(int64_t n, double tol, double tol_mid, double tol_in, bool residual, bool tight, std::string &err);
     void release();
-    // Y = the nested-ADI approximation of (T_01 + T_02 + T_12)^{-1} G (device tensors).
-    int run(const T *G, T *Y, cudaStream_t st, std::string &err);
 
     int J_outer = 0;
     int64_t inner_per_run = 0;   // inner (slice Stein) iterations over full tensors per run
     int64_t launches = 0;        // kernel launches of the last run
     int64_t bytes = 0;
 
-private:
+protected:
     struct Stein {
         double c = 0;
         int J = 0;
-        int64_t ab_off = 0;          // first (alpha, beta) set of this entry in the device table
+        int64_t off = 0;         // of this entry in its class's device tables
         std::vector<double> p, q;
     };
     struct Middle {
@@ -49,38 +44,65 @@ private:
         int stein_v = 0;
         std::vector<Middle> mid;
     };
-    cudaError_t band(const T *X, const T *R, T *Y, int mode, double alpha, double beta, double sop, double sr);
-    cudaError_t axpby(const T *X, const T *Y, T *Z, double a, double b);
-    cudaError_t axpy3(const T *X, const T *Y, const T *W, T *V, double a, double b, double c);
-    // X = oscale * (alpha A~ + beta)^{-1} IN + oin * IN + oacc * X along `mode`, with
-    // IN = s1 R1 + s2 R2, or IN = s1 A~ R1 along `mode` when preband
-    cudaError_t solve(int set, const T *R1, double s1, const T *R2, double s2, T *X, int mode, double oscale,
-                      double oacc, double oin, bool preband);
-    int load_factors(int entry, std::string &err);
-    int stein(int ma, int mb, int entry, const T *R, T *Z, std::string &err);
-    int hsolve(const Outer &o, const T *R, T *Y, std::string &err);
-    int stein_res(int ma, int mb, int entry, const T *R1, double r1, const T *R2, double r2, T *Z, bool accumulate,
-                  std::string &err);
-    int hsolve_res(const Outer &o, const T *R, T *W, std::string &err);
-    int run_residual(const T *G, T *Y, std::string &err);
+    // tol: outer tolerance of (2.9); tol_mid / tol_in: middle and inner levels; residual:
+    // inner iterations counted for the residual-propagating form; tight: every level's
+    // intervals from the Sturm-bisection interval of A~ instead of Lemma B.2's
+    // [-1, -1/(30 n^4)].
+    void schedule(int64_t n, double tol, double tol_mid, double tol_in, bool residual, bool tight);
     int add_stein(double c);
+    cudaError_t alloc(void **p, size_t b);
+    cudaError_t copy(void **p, const void *src, size_t b);  // alloc and upload
 
     int64_t n_ = 0;
-    double tol_ = 0, tol_mid_ = 0, tol_in_ = 0;
+    double tol_in_ = 0;
     double lo_ = 0, hi_ = 1;     // sigma(A~) in [-hi_, -lo_]
-    bool residual_ = false;
     cudaStream_t st_ = nullptr;
-    double *bd64_ = nullptr, *be64_ = nullptr;
-    T *bd_ = nullptr, *be_ = nullptr;
-    T *work_[9] = {nullptr};
-    void *fac_ = nullptr;        // factor sets of the current Stein entry ({1/den, u} in T)
-    double2 *ab_ = nullptr;      // (alpha, beta) of every factor set of every Stein entry
-    int fac_entry_ = -1;         // entry whose factors fac_ holds (stream order makes reuse safe)
-    bool slice_ = false;         // FP32 inner solves by the slice-resident cluster kernel
-    int max_sets_ = 0;
+    double *bd_ = nullptr, *be_ = nullptr;
     std::vector<Stein> steins_;
     std::vector<Outer> outer_;
     std::vector<void *> allocs_;
+};
+
+// FP64, the paper's form: an error of one iteration is part of the next one's residual, so
+// the solution keeps FP64 accuracy without refinement.
+class CubeNested : public CubeSchedule {
+public:
+    int create(int64_t n, double tol, double tol_level, std::string &err);
+    // Y = the nested-ADI approximation of (T_01 + T_02 + T_12)^{-1} G (device tensors).
+    int run(const double *G, double *Y, cudaStream_t st, std::string &err);
+
+private:
+    cudaError_t band(const double *X, const double *R, double *Y, int mode, double alpha, double beta, double sop,
+                     double sr);
+    cudaError_t axpby(const double *X, const double *Y, double *Z, double a, double b);
+    // X = (alpha A~ + beta)^{-1} (R1 + s2 R2) along `mode` (R2 may be null)
+    cudaError_t solve(int set, const double *R1, const double *R2, double s2, double *X, int mode);
+    int load_factors(int entry, std::string &err);
+    int stein(int ma, int mb, int entry, const double *R, double *Z, std::string &err);
+    int hsolve(const Outer &o, const double *R, double *Y, std::string &err);
+
+    double *work_[8] = {nullptr};
+    double2 *fac_ = nullptr;     // factor sets of the current Stein entry ({1/den, u})
+    double2 *ab_ = nullptr;      // (alpha, beta) of every factor set of every Stein entry
+    int entry_ = -1;             // entry whose factors fac_ holds (stream order makes reuse safe)
+};
+
+// FP32, every level in residual-propagating form; tensors have mode 0 fastest, (i, j, k) at
+// (j n + k) n + i.
+class CubeRounds : public CubeSchedule {
+public:
+    int create(int64_t n, double tol, double tol_mid, double tol_in, std::string &err);
+    int run(const float *G, float *Y, cudaStream_t st, std::string &err);
+
+private:
+    int stein(int ma, int mb, int entry, const UnitJob *jobs, int njobs, std::string &err);
+    int hsolve_res(const Outer &o, const float *R, float *W, std::string &err);
+
+    float *work_[4] = {nullptr};
+    int unit_ = 0;               // half line length of the inner level's kernel
+    float *tab_ = nullptr, *bands_ = nullptr;  // its tables, every Stein entry
+    UnitEntry *entries_ = nullptr;
+    double2 *pq_ = nullptr;
 };
 
 class CubeEngine {
@@ -110,8 +132,8 @@ private:
     int64_t n_ = 0;
     double tol_ = 0;
     int precision_ = 0;
-    CubeNested<double> *n64_ = nullptr;
-    CubeNested<float> *n32_ = nullptr;
+    CubeNested *n64_ = nullptr;
+    CubeRounds *n32_ = nullptr;
     double *bd_ = nullptr, *be_ = nullptr, *bs_ = nullptr;
     double *G_ = nullptr, *Y_ = nullptr, *R_ = nullptr;
     float *rho_ = nullptr, *delta_ = nullptr;

@@ -152,3 +152,28 @@ def test_cylinder_line_lengths(api, n, k):
     for r in range(2):
         Yo, _ = cyl.mode_adi(F[r], k, 1e-15)
         assert _relmax(Y[r], Yo) <= bar, (r, bar)
+
+
+def _along(T, B):  # B on all three modes
+    for _ in range(3):
+        T = np.tensordot(T, B, axes=([0], [1]))
+    return T
+
+
+# the slice kernel's line lengths (2 H unknowns per parity), full and with unused places
+@pytest.mark.parametrize("n", [3, 4, 7, 9, 12, 13, 16, 24, 25, 33, 40, 41, 49, 65, 81, 97, 113, 129, 145])
+def test_cube_refine_line_lengths(api, n):
+    """Against the exact solution by diagonalisation, at the cube's refinement bar."""
+    F = inputs.cube_rhs(n, n)
+    plan = api.plan_create(n, 3, 1e-10, "fp32_refine")
+    X = api.poisson_cube_solve(plan, torch.from_numpy(F).cuda()).cpu().numpy()
+    api.plan_destroy(plan)
+    d, e = oracle.square_bands(n)
+    A = np.diag(d) + np.diag(e[: n - 2], 2) + np.diag(e[: n - 2], -2)
+    lam, V = np.linalg.eigh(A)
+    s = 1.0 / np.sqrt((np.arange(n) + 1.0) * (np.arange(n) + 2.0))
+    S = s[:, None, None] * s[None, :, None] * s[None, None, :]
+    L = lam[:, None, None] * lam[None, :, None] + lam[:, None, None] * lam[None, None, :] + \
+        lam[None, :, None] * lam[None, None, :]
+    Xd = _along(_along(-F * S, V.T) / L, V) * S
+    assert _relmax(X, Xd) <= TOL_REFINE
