@@ -16,15 +16,17 @@
 // a flat right-hand side at n = 32 would grow from 6e-11 to 7e-8).
 //
 // Slices are independent, and so are the four parity quarters of a slice: one CTA per
-// quarter keeps u and Z (about (n/2)^2 each) in shared memory for all iterations.  A line
-// of 2 H unknowns is eliminated from both ends by two threads (half-warps) that keep the
-// forward values of their half in registers and meet in the middle.
+// quarter keeps u in shared memory and Z in registers for all iterations.  A line of 2 H
+// unknowns is eliminated from both ends by two threads (half-warps) that keep the forward
+// values of their half in registers and meet in the middle.  Tables are read 16 bytes at a
+// time and in groups ahead of the dependent FMAs.
 //
-// What bounds it: at small n the chain of dependent operations of one line (about 4 H
-// FMAs, the table and line reads between them and two barriers per iteration) and the
-// number of launches that depend on one another; at large n the shared-memory accesses (17
-// words per unknown and iteration).  Against one launch per line solve and banded product
-// (5 per iteration): n = 32 635 -> 31 ms, n = 64 2.44 s -> 222 ms, n = 256 44.4 -> 10.3 s.
+// What bounds it: at small n the latency of the 260 instructions of an iteration on the one
+// or two warps of a CTA (n = 32: 0.4 us) and the launches that depend on one another; at
+// large n the shared-memory accesses.  Against one launch per line solve and banded product
+// (5 per iteration), and against this kernel with u and Z in shared memory and tables read
+// word by word: n = 32 635 -> 31 -> 21 ms, n = 64 2.44 s -> 222 -> 88 ms, n = 256 44.4 ->
+// 10.3 -> 7.0 s.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -32,12 +34,18 @@
 
 namespace fps {
 
-// Tables of one tridiagonal of N = 2 H unknowns, both halves from their outer end, [2][H]
-// each:  l, m, the solution scale; then the two coefficients per half of the middle solve.
-__host__ __device__ constexpr int unit_table(int H) { return 6 * H + 4; }
-// Bands of A~ of one parity: diagonal [2][H], coupling to the outer neighbour
-// [2][H], the coupling across the middle, padded.
-__host__ __device__ constexpr int unit_bands(int H) { return 4 * H + 4; }
+// Distance between the two halves of a table: whole 16-byte words, and not a multiple of 8
+// so that the two half-warps read from different banks.
+__host__ __device__ constexpr int unit_half_pitch(int H)
+{
+    return (H + 3) / 4 * 4 % 8 ? (H + 3) / 4 * 4 : (H + 3) / 4 * 4 + 4;
+}
+// Tables of one tridiagonal of N = 2 H unknowns, both halves from their outer end: l [2][H],
+// {m, the solution scale} [2][H], then the two coefficients per half of the middle solve.
+__host__ __device__ constexpr int unit_table(int H) { return 6 * unit_half_pitch(H) + 4; }
+// Bands of A~ of one parity: {diagonal, coupling to the outer neighbour} [2][H], then the
+// coupling across the middle, padded.
+__host__ __device__ constexpr int unit_bands(int H) { return 4 * unit_half_pitch(H) + 4; }
 
 // out = kR R + kZ Z + kacc out, Z = (T_ab + c)^{-1} R, R = r1 R1 + r2 R2 (R2 may be null; out
 // may be R1 or R2).
