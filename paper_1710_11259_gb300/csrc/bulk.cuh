@@ -61,6 +61,48 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, unsigned parity
     return false;
 }
 
+// As mbar_wait_bounded, for bytes that other CTAs of the cluster send (send_pair).
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, unsigned parity)
+{
+    for (int it = 0; it < (1 << 20); ++it) {
+        unsigned ok;
+        asm volatile(
+            "{\n"
+            " .reg .pred p;\n"
+            " mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n"
+            " selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(ok)
+            : "r"(smem_u32(bar)), "r"(parity), "r"(1000u)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+
+// Address of the same shared variable in CTA `rank` of the cluster.
+__device__ __forceinline__ unsigned peer_smem(const void *p, int rank)
+{
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+
+// Asynchronous store of a pair into a CTA of the cluster, counted by that CTA's barrier
+// (both addresses from peer_smem).
+__device__ __forceinline__ void send_pair(unsigned dst, unsigned bar, float2 v)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];\n" ::"r"(dst),
+                 "f"(v.x), "f"(v.y), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void send_pair(unsigned dst, unsigned bar, double2 v)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];\n" ::"r"(dst),
+                 "d"(v.x), "d"(v.y), "r"(bar)
+                 : "memory");
+}
+
 // global -> shared bulk copy completing on `bar` (complete_tx of `bytes`).
 __device__ __forceinline__ void g2s(void *dst_smem, const void *src_gmem, unsigned bytes, uint64_t *bar)
 {

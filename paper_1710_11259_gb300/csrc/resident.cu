@@ -2,6 +2,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include "bulk.cuh"
 #include "resident.cuh"
 #include "sweep.cuh"
 
@@ -42,7 +43,8 @@ struct ResGeo {
     static constexpr int off_tab = off_bd + up(2 * kG * S);
     // tables of one iteration: row record, column scan coefficients, column slice [5][S]
     static constexpr int tab = res_record(S) + kScan + up(kTabs * S);
-    static constexpr size_t bytes = sizeof(T) * (size_t)(off_tab + 2 * tab);
+    static constexpr int off_bar = off_tab + 2 * up(tab);  // two mbarriers
+    static constexpr size_t bytes = sizeof(T) * (size_t)off_bar + 16;
 };
 
 __device__ __forceinline__ void copy16_async(void *dst, const void *src)
@@ -92,6 +94,7 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
     T2 *cs = reinterpret_cast<T2 *>(reinterpret_cast<T *>(smem) + G::off_cs);
     T2 *bd = reinterpret_cast<T2 *>(reinterpret_cast<T *>(smem) + G::off_bd);
     T *tab = reinterpret_cast<T *>(smem) + G::off_tab;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(reinterpret_cast<T *>(smem) + G::off_bar);
     // global position of element (i, k) of the quarter
     auto qpos = [&](int i, int k) {
         return it.xoff + (((int64_t)(i >> 5) * it.lnb + (k >> 5)) << 10) + block_pos<T>(i & 31, k & 31, 32);
@@ -111,6 +114,11 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
     load_tables(0);
+    if (tid == 0) {
+        bulk::mbar_init(bar, 1);
+        bulk::mbar_init(bar + 1, 1);
+        bulk::fence_mbar_init();
+    }
     for (int q = tid; q < S * M; q += G::kThreads) {  // the slab: rows i0 .. i0 + S
         const int r = q / M, k = q - r * M, i = i0 + r;
         T v = 0;
@@ -134,10 +142,28 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
     const bool col_on = tid < M && gc < C;
     T *xr = X + r0 * G::pitch + g * G::SS;
     T *xc = X + gc * G::SS + cc;
+    // Exchange: each of the C S pairs of a step is an asynchronous store that the receiver's
+    // barrier counts.  A CTA sends a step's pairs only after it has received all of the step
+    // before, which its peers send after reading what the new pairs overwrite.
+    const unsigned bytes = (unsigned)(C * S * sizeof(T2));
+    const int pc = min(gc, C - 1), pr = min(g, C - 1);  // peers that own the column, that want its segment
+    const unsigned to_cs = bulk::peer_smem(cs + cc * G::cpitch + rank, pc), bar_cs = bulk::peer_smem(bar, pc);
+    const unsigned to_bd = bulk::peer_smem(bd + i0 + r0, pr), bar_bd = bulk::peer_smem(bar + 1, pr);
+    bool ok = true;  // false: a wait gave up; the thread runs on without waiting or sending
+    auto wait = [&](uint64_t *b, int j) {
+        if (ok && !bulk::mbar_wait_cluster(b, j & 1)) {
+            ok = false;
+            *(volatile int *)a.err = 1;
+        }
+    };
     for (int j = 0; j < J; ++j) {
         const T *tr = tab + (j & 1) * G::tab;
         const T2 *sums = reinterpret_cast<const T2 *>(tr) + g, *back = reinterpret_cast<const T2 *>(tr + 2 * M) + g;
         const T *fwd = tr + 4 * M + g, *kr = tr + 5 * M, *kc = tr + res_record(S), *tc = kc + kScan;
+        if (tid == 0) {
+            bulk::mbar_arrive_expect_tx(bar, bytes);
+            bulk::mbar_arrive_expect_tx(bar + 1, bytes);
+        }
         if (j + 1 < J) load_tables(j + 1);
         T v[S], w[S];
         {
@@ -176,16 +202,16 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
                 wl[i & 1] = fma(tc[3 * S + i], v[i], wl[i & 1]);
                 yl[i & 1] = fma(tc[4 * S + i], v[i], yl[i & 1]);
             }
-            if (col_on) *cl.map_shared_rank(cs + cc * G::cpitch + rank, gc) = pair_of<T>(wl[0] + wl[1], yl[0] + yl[1]);
+            if (col_on && ok) bulk::send_pair(to_cs, bar_cs, pair_of<T>(wl[0] + wl[1], yl[0] + yl[1]));
         }
-        cl.sync();
+        wait(bar, j);
         {  // the columns this CTA owns, rank * S + r0, all their segments
             const T2 s = cs[r0 * G::cpitch + g];
             T z, y;
             scan_segments<T>(s.x, s.y, kc, g, z, y);
-            if (row_on && g < C) *cl.map_shared_rank(bd + i0 + r0, g) = pair_of<T>(z, y);
+            if (row_on && g < C && ok) bulk::send_pair(to_bd, bar_bd, pair_of<T>(z, y));
         }
-        cl.sync();
+        wait(bar + 1, j);
         if (col_on) {
             const T2 b = bd[col];
             T z = b.x, y = b.y;
@@ -204,16 +230,20 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
     }
+    // no CTA leaves while a peer whose wait gave up may still have stores under way to it
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
     if (col_on && col < mc) {
 #pragma unroll
         for (int r = 0; r < S; ++r) {
             const int i = i0 + r;
+            if (!ok) D[r] = (T)NAN;
             if (i < mr) {
                 if (a.F) a.out[npos(i, col)] = it.out_scale * (double)D[r] * it.s[2 * i + it.rp] * it.s[2 * col + it.cp];
                 else a.D[qpos(i, col)] = D[r];
             }
         }
     }
+    asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");
 }
 
 // One thread per (job, parity), FP64 arithmetic; the recurrences of fac_tables_kernel.

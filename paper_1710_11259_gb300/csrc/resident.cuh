@@ -8,19 +8,22 @@
 //                 two summaries per thread, the recurrence over the segments as warp
 //                 scans, then the sweeps of the segment in registers;
 //   column solve  thread = column, the CTA's S rows are one segment: its summaries go to
-//                 the CTA that owns the column (distributed shared memory, cluster
-//                 barrier), which runs the same scans and returns zin and yout to every
-//                 CTA (cluster barrier), then the sweeps.
+//                 the CTA that owns the column, which runs the same scans and returns zin
+//                 and yout to every CTA, then the sweeps.  Both ways each pair is an
+//                 asynchronous store into the receiver's shared memory, counted by the
+//                 receiver's mbarrier.
 // Scans: with kf[t][s] = prod_{s-2^t < u <= s} phi(u) and kb[t][s] = prod_{s <= u < s+2^t}
 // Psi(u), four steps W_s += kf[t][s] W_{s-2^t} and four backwards.
 //
 // Bound: the FP64 pipe in FP64 (a warp-wide FP64 instruction takes 64 cycles of an SM
 // quadrant, so threads are laid out to do few of them: 16 segments per line, scans
-// instead of one long recurrence), latency of the two cluster barriers and the sweeps in
-// FP32.  Measured on GB300 per solve: n = 64 FP64, two right-hand sides, 247 us (801 us
-// with one cluster of 8 CTAs per right-hand side solving every line by cyclic reduction
-// and exchanging whole iterates), n = 301 FP64 0.69 ms (2.5 ms streamed by the passes),
-// n = 1000 FP32+refine 0.61 ms (1.18 ms streamed).
+// instead of one long recurrence), latency of the two exchanges and the sweeps in FP32.
+// Measured on GB300 per solve: n = 64 FP64, two right-hand sides, 202 us (801 us with one
+// cluster of 8 CTAs per right-hand side solving every line by cyclic reduction and
+// exchanging whole iterates; 250 us with remote stores between cluster barriers, whose
+// fences alone were a fifth of the time), n = 301 FP64 0.63 ms (2.5 ms streamed by the
+// passes, 0.69 with cluster barriers), n = 1000 FP32+refine 0.53 ms (1.18 streamed, 0.56
+// with cluster barriers).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -58,6 +61,7 @@ struct ResArgs {
     T *X, *D;                // quarter-block arrays (F == nullptr)
     const double *F;         // caller's right-hand sides and solution: scale-in and -out in the launch
     double *out;
+    int *err;                // set if a bounded wait gave up (device or pinned host memory)
 };
 
 template <typename T>

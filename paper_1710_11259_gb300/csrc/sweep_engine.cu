@@ -693,6 +693,8 @@ ResArgs<T> SweepEngine<T>::res_args(const ResClass &c, const double *F, double *
     a.D = D_;
     a.F = F;
     a.out = X;
+    // a launch outside the solve that copies err_ back reports to the host's copy itself
+    a.err = F ? (int *)(h_stat_ + 2 * npairs_) : err_;
     return a;
 }
 
