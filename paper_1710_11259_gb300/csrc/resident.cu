@@ -41,9 +41,10 @@ struct ResGeo {
     static constexpr int off_cs = off_x + up(S * pitch);       // column summaries of the owned columns
     static constexpr int off_bd = off_cs + up(2 * S * cpitch);  // zin, yout of this CTA's column segments
     static constexpr int off_tab = off_bd + up(2 * kG * S);
-    // tables of one iteration: row record, column scan coefficients, column slice [5][S]
-    static constexpr int tab = res_record(S) + kScan + up(kTabs * S);
-    static constexpr int off_bar = off_tab + 2 * up(tab);  // two mbarriers
+    // tables of one iteration: row record, column scan coefficients, column slice [5][SP]
+    static constexpr int SP = up(S);
+    static constexpr int tab = res_record(S) + kScan + kTabs * SP;
+    static constexpr int off_bar = off_tab + 2 * tab;  // two mbarriers
     static constexpr size_t bytes = sizeof(T) * (size_t)off_bar + 16;
 };
 
@@ -58,6 +59,18 @@ __device__ __forceinline__ void copy_async(T *dst, const T *src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
                  "n"(sizeof(T))
                  : "memory");
+}
+
+// A 16-byte word of a table.
+__device__ __forceinline__ void read16(float (&o)[4], const float *p)
+{
+    const float4 f = *reinterpret_cast<const float4 *>(p);
+    o[0] = f.x, o[1] = f.y, o[2] = f.z, o[3] = f.w;
+}
+__device__ __forceinline__ void read16(double (&o)[2], const double *p)
+{
+    const double2 f = *reinterpret_cast<const double2 *>(p);
+    o[0] = f.x, o[1] = f.y;
 }
 
 // zin and yout of segment g (lane g of a half-warp) of a line from the summaries that the
@@ -83,6 +96,10 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
     using G = ResGeo<T, S>;
     using T2 = typename Vec2<T>::type;
     constexpr int M = kG * S;
+    // partial sums of a summary: an FP64 instruction of a warp occupies its issue for as long as
+    // its latency, so a second chain only costs its addition
+    constexpr int kAcc = sizeof(T) == 8 ? 1 : 2;
+    auto total = [](const T(&x)[kAcc]) { return kAcc == 1 ? x[0] : x[0] + x[kAcc - 1]; };
     extern __shared__ __align__(16) unsigned char smem[];
     cg::cluster_group cl = cg::this_cluster();
     const int C = a.C, rank = (int)cl.block_rank(), tid = threadIdx.x;
@@ -106,11 +123,11 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
         const T *tR = it.tabR + j * rec, *tC = it.tabC + j * rec;
         for (int q = tid * G::A; q < res_record(S); q += G::kThreads * G::A) copy16_async(t + q, tR + q);
         t += res_record(S);
-        for (int q = tid * G::A; q < kScan; q += G::kThreads * G::A) copy16_async(t + q, tC + kTabs * M + q);
+        for (int q = tid * G::A; q < kScan; q += G::kThreads * G::A) copy16_async(t + q, tC + res_scan_col(S) + q);
         t += kScan;
         if (tid < S)
 #pragma unroll
-            for (int q = 0; q < kTabs; ++q) copy_async(t + q * S + tid, tC + q * M + i0 + tid);
+            for (int q = 0; q < kTabs; ++q) copy_async(t + q * G::SP + tid, tC + q * M + i0 + tid);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
     load_tables(0);
@@ -159,7 +176,8 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
     for (int j = 0; j < J; ++j) {
         const T *tr = tab + (j & 1) * G::tab;
         const T2 *sums = reinterpret_cast<const T2 *>(tr) + g, *back = reinterpret_cast<const T2 *>(tr + 2 * M) + g;
-        const T *fwd = tr + 4 * M + g, *kr = tr + 5 * M, *kc = tr + res_record(S), *tc = kc + kScan;
+        const T2 *fwd = reinterpret_cast<const T2 *>(tr + 4 * M) + g;
+        const T *kr = tr + res_scan_row(S), *kc = tr + res_record(S), *tc = kc + kScan;
         if (tid == 0) {
             bulk::mbar_arrive_expect_tx(bar, bytes);
             bulk::mbar_arrive_expect_tx(bar + 1, bytes);
@@ -167,20 +185,25 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
         if (j + 1 < J) load_tables(j + 1);
         T v[S], w[S];
         {
-            T wl[2] = {0, 0}, yl[2] = {0, 0};
+            T wl[kAcc] = {}, yl[kAcc] = {};
 #pragma unroll
             for (int i = 0; i < S; ++i) {
                 const T2 p = sums[i * kG];
                 v[i] = xr[i];
-                wl[i & 1] = fma(p.x, v[i], wl[i & 1]);
-                yl[i & 1] = fma(p.y, v[i], yl[i & 1]);
+                wl[i % kAcc] = fma(p.x, v[i], wl[i % kAcc]);
+                yl[i % kAcc] = fma(p.y, v[i], yl[i % kAcc]);
             }
             T z, y;
-            scan_segments<T>(wl[0] + wl[1], yl[0] + yl[1], kr, g, z, y);
+            scan_segments<T>(total(wl), total(yl), kr, g, z, y);
 #pragma unroll
-            for (int i = 0; i < S; ++i) {
-                z = fma(-fwd[i * kG], z, v[i]);
+            for (int i = 0; i < S; i += 2) {
+                const T2 l = fwd[i / 2 * kG];
+                z = fma(-l.x, z, v[i]);
                 w[i] = z;
+                if (i + 1 < S) {
+                    z = fma(-l.y, z, v[i + 1]);
+                    w[i + 1] = z;
+                }
             }
             const bool first = j == 0;
 #pragma unroll
@@ -195,14 +218,20 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
         }
         __syncthreads();
         {
-            T wl[2] = {0, 0}, yl[2] = {0, 0};
+            T wl[kAcc] = {}, yl[kAcc] = {};
 #pragma unroll
-            for (int i = 0; i < S; ++i) {
-                v[i] = xc[i * G::pitch];
-                wl[i & 1] = fma(tc[3 * S + i], v[i], wl[i & 1]);
-                yl[i & 1] = fma(tc[4 * S + i], v[i], yl[i & 1]);
+            for (int c = 0; c < S; c += G::A) {
+                T psi[G::A], chi[G::A];
+                read16(psi, tc + 3 * G::SP + c);
+                read16(chi, tc + 4 * G::SP + c);
+#pragma unroll
+                for (int i = c; i < min(c + G::A, S); ++i) {
+                    v[i] = xc[i * G::pitch];
+                    wl[i % kAcc] = fma(psi[i - c], v[i], wl[i % kAcc]);
+                    yl[i % kAcc] = fma(chi[i - c], v[i], yl[i % kAcc]);
+                }
             }
-            if (col_on && ok) bulk::send_pair(to_cs, bar_cs, pair_of<T>(wl[0] + wl[1], yl[0] + yl[1]));
+            if (col_on && ok) bulk::send_pair(to_cs, bar_cs, pair_of<T>(total(wl), total(yl)));
         }
         wait(bar, j);
         {  // the columns this CTA owns, rank * S + r0, all their segments
@@ -216,15 +245,26 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
             const T2 b = bd[col];
             T z = b.x, y = b.y;
 #pragma unroll
-            for (int i = 0; i < S; ++i) {
-                z = fma(-tc[i], z, v[i]);
-                w[i] = z;
+            for (int c = 0; c < S; c += G::A) {
+                T l[G::A];
+                read16(l, tc + c);
+#pragma unroll
+                for (int i = c; i < min(c + G::A, S); ++i) {
+                    z = fma(-l[i - c], z, v[i]);
+                    w[i] = z;
+                }
             }
 #pragma unroll
-            for (int i = S - 1; i >= 0; --i) {
-                y = fma(-tc[S + i], y, w[i]);
-                xc[i * G::pitch] = fma(tc[2 * S + i], y, v[i]);
-                D[i] = fma(tc[2 * S + i], y, D[i]);
+            for (int c = G::SP - G::A; c >= 0; c -= G::A) {
+                T mm[G::A], gg[G::A];
+                read16(mm, tc + G::SP + c);
+                read16(gg, tc + 2 * G::SP + c);
+#pragma unroll
+                for (int i = min(c + G::A, S) - 1; i >= c; --i) {
+                    y = fma(-mm[i - c], y, w[i]);
+                    xc[i * G::pitch] = fma(gg[i - c], y, v[i]);
+                    D[i] = fma(gg[i - c], y, D[i]);
+                }
             }
         }
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
@@ -256,6 +296,7 @@ __global__ void resident_tables_kernel(const ResTabJob<T> *__restrict__ jobs, in
     const int p = tid & 1, S = jb.S, M = kG * S, m = (jb.n - p + 1) / 2;
     T *row = jb.row ? jb.row + (int64_t)p * res_record(S) : nullptr;
     T *col = jb.col ? jb.col + (int64_t)p * res_record(S) : nullptr;
+    T *row_scan = row ? row + res_scan_row(S) : nullptr, *col_scan = col ? col + res_scan_col(S) : nullptr;
     const double *d = jb.d + p, *e = jb.e + p;  // position i of this parity: index 2 i
     double ip = 0.0, ip_next = m > 0 ? 1.0 / (d[0] - jb.q) : 0.0, l_next = 0.0;
     double lv[32], mv[32], v[32], phi[kG], bv[kG], ps[kG];
@@ -280,7 +321,7 @@ __global__ void resident_tables_kernel(const ResTabJob<T> *__restrict__ jobs, in
             if (row) {
                 row[2 * M + 2 * (u * kG + g)] = (T)mm;
                 row[2 * M + 2 * (u * kG + g) + 1] = (T)(jb.sc_row * ip);
-                row[4 * M + u * kG + g] = (T)l;
+                row[4 * M + (u / 2 * kG + g) * 2 + u % 2] = (T)l;
             }
             if (col) {
                 col[i] = (T)l;
@@ -318,14 +359,14 @@ __global__ void resident_tables_kernel(const ResTabJob<T> *__restrict__ jobs, in
                 kb = 1.0;
                 for (int u = s; u < s + (1 << t); ++u) kb *= ps[u];
             }
-            for (T *o : {row, col})
+            for (T *o : {row_scan, col_scan})
                 if (o) {
-                    o[5 * M + t * kG + s] = (T)kf;
-                    o[5 * M + (5 + t) * kG + s] = (T)kb;
+                    o[t * kG + s] = (T)kf;
+                    o[(5 + t) * kG + s] = (T)kb;
                 }
         }
-        for (T *o : {row, col})
-            if (o) o[5 * M + 4 * kG + s] = (T)bv[s];
+        for (T *o : {row_scan, col_scan})
+            if (o) o[4 * kG + s] = (T)bv[s];
     }
 }
 

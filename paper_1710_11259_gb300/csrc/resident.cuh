@@ -18,10 +18,10 @@
 // Bound: the FP64 pipe in FP64 (a warp-wide FP64 instruction takes 64 cycles of an SM
 // quadrant, so threads are laid out to do few of them: 16 segments per line, scans
 // instead of one long recurrence), latency of the two exchanges and the sweeps in FP32.
-// Measured on GB300 per solve: n = 64 FP64, two right-hand sides, 202 us (801 us with one
+// Measured on GB300 per solve: n = 64 FP64, two right-hand sides, 192 us (801 us with one
 // cluster of 8 CTAs per right-hand side solving every line by cyclic reduction and
 // exchanging whole iterates; 250 us with remote stores between cluster barriers, whose
-// fences alone were a fifth of the time), n = 301 FP64 0.63 ms (2.5 ms streamed by the
+// fences alone were a fifth of the time), n = 301 FP64 0.60 ms (2.5 ms streamed by the
 // passes, 0.69 with cluster barriers), n = 1000 FP32+refine 0.53 ms (1.18 streamed, 0.56
 // with cluster barriers).
 #pragma once
@@ -35,10 +35,12 @@ constexpr int kResSeg = 16;                    // segments per line, and the lar
 constexpr int kScan = 9 * kResSeg;             // kf[4], Bv, kb[4] of the segments
 
 // Tables of one (shift, parity), elements of T.
-// Row record: {psi, chi}[S][16], {m, scale}[S][16], l[S][16] (position i of segment g at
-// [i][g]), then the scan coefficients.  Column record: l, m, scale, psi, chi [5][16 S] in
-// natural order, then the scan coefficients.
-__host__ __device__ constexpr int res_record(int S) { return 5 * kResSeg * S + kScan; }
+// Row record: {psi, chi}[S][16], {m, scale}[S][16], l[(S + 1) / 2][16][2] (position i of
+// segment g at [i][g], l at [i / 2][g][i % 2]), then the scan coefficients.  Column record:
+// l, m, scale, psi, chi [5][16 S] in natural order, then the scan coefficients.
+__host__ __device__ constexpr int res_scan_row(int S) { return kResSeg * (5 * S + S % 2); }
+__host__ __device__ constexpr int res_scan_col(int S) { return kResSeg * 5 * S; }
+__host__ __device__ constexpr int res_record(int S) { return res_scan_row(S) + kScan; }
 
 // One quarter of one (problem, right-hand side).
 template <typename T>
