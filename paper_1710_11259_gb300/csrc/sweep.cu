@@ -62,11 +62,14 @@ __device__ __forceinline__ double2 mk2<double>(double x, double y)
     return make_double2(x, y);
 }
 
+// Segments per thread of the recurrences that the passes run.
+__host__ __device__ constexpr int chain_segments(bool fp64) { return fp64 ? 4 : 8; }
+
 __host__ __device__ __forceinline__ int round4(int n) { return (n + 3) & ~3; }
 
-// Shared memory of a pass CTA: tile (and the tile of D), the solve tables of the
-// segment, the summary tables of the kL lines, and (fused recurrences) the segment
-// coefficients.
+// Shared memory of a pass CTA: tile (and the tile of D), the solve tables of the tile's
+// positions, the summary tables of one segment, and the exchange of the segment recurrence
+// (zin and yout of the kL threads, partial values of the thread groups).
 template <typename T, int S>
 struct Geo {
     static constexpr int V = 16 / (int)sizeof(T);
@@ -74,10 +77,16 @@ struct Geo {
     static constexpr int CH = S / V;      // chunks of a row
     static constexpr size_t off_tile = 128;
     static constexpr size_t tile_bytes = sizeof(T) * kL * S;
-    static constexpr size_t tab_elems = 3 * S + 2 * kL + 3 * kMaxFused;
+    static constexpr int G = kL / S;      // blocks of a tile, thread groups of the segment recurrence
+    static constexpr size_t tab_elems = 3 * kL + 2 * S + 2 * kL + 2 * kL + 2 * G;
     static constexpr size_t row_bytes = off_tile + tile_bytes + sizeof(T) * tab_elems;
     static constexpr size_t col_bytes = off_tile + 2 * tile_bytes + sizeof(T) * tab_elems;
     static constexpr size_t sum_bytes = row_bytes;
+    // Resident CTAs per SM that the registers are limited for.  Blocks of 32 in FP32 serve
+    // n = 1025 .. 2048, about one wave of tiles: with 6 and 5 resident CTAs (no limit) a nearly
+    // empty second wave cost n = 2048 5 % of the solve.
+    static constexpr int row_ctas = sizeof(T) == 8 ? 3 : (S == 32 ? 7 : 4);
+    static constexpr int col_ctas = sizeof(T) == 4 && S == 32 ? 6 : 3;
     static_assert(CH >= 8, "the XOR permutation needs eight chunks per row");
 };
 
@@ -184,44 +193,95 @@ __device__ __forceinline__ bool pass_begin(const SwArgs<T> &a, const SwItem<T> &
     return act && !stop;
 }
 
-// zin and yout of segment s of one line from the summaries of all its segments
-// (sum: segment 0 of the line, `step` apart); co: phi, Bv, Psi of nbp entries each.
-template <typename T>
-struct LineSums {
-    typename Vec2<T>::type v[kMaxFused];
-    __device__ __forceinline__ void load(const typename Vec2<T>::type *__restrict__ sum, int64_t step, int P)
+// Segment recurrence of the S lines of a tile by the pass itself: the G groups of S
+// threads (lane = line) own LEN consecutive segments each; a group composes the affine maps
+// W -> alpha W + beta of its segments, the groups' maps are composed through shared memory
+// and the true values follow from one more walk; then the same backwards.  The result
+// {zin, yout} of the tile's segments is left in zx[block][line].  Runs while the tile is in
+// flight.  (A tile across the lines, every thread walking all segments of its own line, read
+// the summaries once per segment of the line and ended at 16 segments.)
+template <typename T, int S>
+struct LineChain {
+    using T2 = typename Vec2<T>::type;
+    static constexpr int LEN = chain_segments(sizeof(T) == 8);
+    static constexpr int G = kL / S;
+    T phi[LEN], bv[LEN], ps[LEN];
+    T2 v[LEN];
+    int s0, li, g;
+
+    // tables of the plan: may be read before the kernels before have finished
+    __device__ __forceinline__ void tables(const T *__restrict__ co, int P)
     {
+        li = threadIdx.x % S;
+        g = threadIdx.x / S;
+        s0 = g * LEN;
+        const int nbp = round4(P);
 #pragma unroll
-        for (int s = 0; s < kMaxFused; ++s)
-            if (s < P) v[s] = sum[s * step];
+        for (int b = 0; b < LEN; ++b) {
+            const bool ok = s0 + b < P;
+            phi[b] = ok ? co[s0 + b] : T(0);
+            bv[b] = ok ? co[nbp + s0 + b] : T(0);
+            ps[b] = ok ? co[2 * nbp + s0 + b] : T(0);
+        }
     }
-    __device__ __forceinline__ void run(const T *co, int nbp, int P, int seg, T &zin, T &yout) const
+    // sum: segment 0 of the tile's first line, segments `step` apart
+    __device__ __forceinline__ void load(const T2 *__restrict__ sum, int64_t step, int P)
     {
-        T z[kMaxFused];
+#pragma unroll
+        for (int b = 0; b < LEN; ++b) v[b] = s0 + b < P ? sum[li + (s0 + b) * step] : mk2<T>(T(0), T(0));
+    }
+    // part: 2 kL + 2 G elements; first, count: the tile's segments.  Ends with a CTA barrier.
+    __device__ __forceinline__ void run(T2 *zx, T *part, int first, int count)
+    {
+        T *beta = part, *alpha = part + 2 * kL;
+        T al = phi[0], be = v[0].x;
+#pragma unroll
+        for (int b = 1; b < LEN; ++b) {
+            be = fma(phi[b], be, v[b].x);
+            al *= phi[b];
+        }
+        beta[threadIdx.x] = be;
+        if (li == 0) alpha[g] = al;
+        __syncthreads();
         T W = 0;
+        for (int h = 0; h < g; ++h) W = fma(alpha[h], W, beta[h * S + li]);
+        T z[LEN];
 #pragma unroll
-        for (int s = 0; s < kMaxFused; ++s)
-            if (s < P) {
-                z[s] = W;
-                if (s == seg) zin = W;
-                W = fma(co[s], W, v[s].x);
-            }
+        for (int b = 0; b < LEN; ++b) {
+            z[b] = W;
+            if (b + 1 < LEN) W = fma(phi[b], W, v[b].x);
+            v[b].y = fma(bv[b], z[b], v[b].y);
+        }
+        // segments past the last have zero maps: what a group composes starts at its last segment
+        al = ps[LEN - 1];
+        be = v[LEN - 1].y;
+#pragma unroll
+        for (int b = LEN - 2; b >= 0; --b) {
+            be = fma(ps[b], be, v[b].y);
+            al *= ps[b];
+        }
+        beta[kL + threadIdx.x] = be;
+        if (li == 0) alpha[G + g] = al;
+        __syncthreads();
         T Y = 0;
+        for (int h = G - 1; h > g; --h) Y = fma(alpha[G + h], Y, beta[kL + h * S + li]);
 #pragma unroll
-        for (int s = kMaxFused - 1; s >= 0; --s)
-            if (s < P) {
-                if (s == seg) yout = Y;
-                Y = fma(co[nbp + s], z[s], fma(co[2 * nbp + s], Y, v[s].y));
-            }
+        for (int b = LEN - 1; b >= 0; --b) {
+            const int t = s0 + b - first;
+            if (t >= 0 && t < count) zx[t * S + li] = mk2<T>(z[b], Y);
+            if (b > 0) Y = fma(ps[b], Y, v[b].y);
+        }
+        __syncthreads();
     }
 };
 
 // ---------------------------------------------------------------------------
-// Row pass.  A tile is n_blk blocks of one block column: up to 128 rows x S columns.
-// FIRST: j = 0 (a = v).
+// Row pass.  A tile is n_blk blocks of one block row: S rows x up to 128 columns, so that
+// its threads can share the segment recurrence of its S rows.  FIRST: j = 0 (a = v).
+// FUSED: the recurrence runs here; otherwise its own launch has left zin and yout.
 // ---------------------------------------------------------------------------
 template <typename T, int S, bool FIRST, bool FUSED>
-__global__ void __launch_bounds__(kL, sizeof(T) == 4 ? 4 : 3) row_pass_kernel(SwArgs<T> A, int j)
+__global__ void __launch_bounds__(kL, Geo<T, S>::row_ctas) row_pass_kernel(SwArgs<T> A, int j)
 {
     using G = Geo<T, S>;
     using T2 = typename Vec2<T>::type;
@@ -229,72 +289,67 @@ __global__ void __launch_bounds__(kL, sizeof(T) == 4 ? 4 : 3) row_pass_kernel(Sw
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
     T *tile = reinterpret_cast<T *>(smem + G::off_tile);
-    T *tl = tile + kL * S, *tm = tl + S, *ts = tm + S, *psi = ts + S, *chi = psi + kL, *co = chi + kL;
+    T *tl = tile + kL * S, *tm = tl + kL, *ts = tm + kL, *psi = ts + kL, *chi = psi + S;
+    T2 *zx = reinterpret_cast<T2 *>(chi + S);
+    T *part = reinterpret_cast<T *>(zx + kL);
     const int tid = threadIdx.x;
     pdl_launch();
     const SwItem<T> it = A.items[blockIdx.x];
+    const int nb = it.nb, bi = it.b0, bk0 = it.b1, nblk = it.n_blk, Mp = nb * S;
+    LineChain<T, S> chain;
+    if (FUSED && j < it.J) chain.tables(it.chR + (int64_t)j * 6 * round4(nb), nb);
     if (!pass_begin(A, it, j, bar, 1)) return;
-    const int nb = it.nb, bi0 = it.b0, bk = it.b1, nblk = it.n_blk, Mp = nb * S, nbp = round4(nb);
     T *X = A.X + it.xoff;
-    const int64_t bstride = (int64_t)nb * G::B;  // blocks of the tile are one block row apart
+    const unsigned xb = (unsigned)(nblk * G::B * sizeof(T));  // the blocks of the tile are adjacent
     if (tid == 0) {
-        const T *tR = it.tabR + (int64_t)j * (2 * kTabs) * Mp + bk * S;
-        const T *tC = it.tabC + (int64_t)j * (2 * kTabs) * Mp + bi0 * S;
-        const unsigned tb = (unsigned)(S * sizeof(T)), pb = (unsigned)(nblk * S * sizeof(T));
-        unsigned total = (unsigned)(nblk * G::B * sizeof(T)) + 3 * tb + 2 * pb;
-        if (FUSED) total += (unsigned)(3 * nbp * sizeof(T));
-        bulk::mbar_arrive_expect_tx(bar, total);
-        for (int b = 0; b < nblk; ++b)
-            bulk::g2s(tile + b * G::B, X + b * bstride, (unsigned)(G::B * sizeof(T)), bar);
+        const T *tR = it.tabR + (int64_t)j * (2 * kTabs) * Mp + bk0 * S;
+        const T *tC = it.tabC + (int64_t)j * (2 * kTabs) * Mp + bi * S;
+        const unsigned tb = (unsigned)(nblk * S * sizeof(T)), pb = (unsigned)(S * sizeof(T));
+        bulk::mbar_arrive_expect_tx(bar, xb + 3 * tb + 2 * pb);
+        bulk::g2s(tile, X, xb, bar);
         bulk::g2s(tl, tR, tb, bar);
         bulk::g2s(tm, tR + Mp, tb, bar);
         bulk::g2s(ts, tR + 2 * Mp, tb, bar);
         bulk::g2s(psi, tC + 3 * Mp, pb, bar);
         bulk::g2s(chi, tC + 4 * Mp, pb, bar);
-        if (FUSED) bulk::g2s(co, it.chR + (int64_t)j * 6 * nbp, (unsigned)(3 * nbp * sizeof(T)), bar);
     }
     const int b = tid / S, r = tid % S;
     const bool on = b < nblk;
-    const int64_t line = it.soff + bi0 * S + tid;
-    T zin = 0, yout = 0;
-    LineSums<T> sums;
-    if (on) {
-        if (FUSED) {
-            sums.load(A.sumR + line, Mp, nb);
-        } else {
-            const T2 z = A.zxR[line + (int64_t)bk * Mp];
-            zin = z.x;
-            yout = z.y;
-        }
+    T2 zy = mk2<T>(T(0), T(0));
+    if (FUSED) {
+        chain.load(A.sumR + it.soff + bi * S, Mp, nb);
+        chain.run(zx, part, bk0, nblk);
+        if (on) zy = zx[tid];
+    } else if (on) {
+        zy = A.zxR[it.soff + bi * S + r + (int64_t)(bk0 + b) * Mp];
     }
     if (!tile_ready(bar, A.err)) return;
     if (on) {
-        if (FUSED) sums.run(co, nbp, nb, bk, zin, yout);
         T *row = tile + b * G::B + r * S;
         int sw[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) sw[q] = (q ^ (r & 7)) * V;
         T w[S];
-        T z = zin;
+        T z = zy.x;
 #pragma unroll
         for (int c = 0; c < G::CH; ++c) {
             T u[V], l[V];
             ld16(row + (c / 8) * 8 * V + sw[c % 8], u);
-            ld16(tl + c * V, l);
+            ld16(tl + b * S + c * V, l);
 #pragma unroll
             for (int e = 0; e < V; ++e) {
                 z = fma(-l[e], z, u[e]);
                 w[c * V + e] = z;
             }
         }
-        T y = yout;
+        T y = zy.y;
 #pragma unroll
         for (int c = G::CH - 1; c >= 0; --c) {
             T u[V], m[V], s[V];
             T *pc = row + (c / 8) * 8 * V + sw[c % 8];
             if (!FIRST) ld16(pc, u);
-            ld16(tm + c * V, m);
-            ld16(ts + c * V, s);
+            ld16(tm + b * S + c * V, m);
+            ld16(ts + b * S + c * V, s);
 #pragma unroll
             for (int e = V - 1; e >= 0; --e) {
                 y = fma(-m[e], y, w[c * V + e]);
@@ -306,8 +361,7 @@ __global__ void __launch_bounds__(kL, sizeof(T) == 4 ? 4 : 3) row_pass_kernel(Sw
     bulk::fence_proxy_async_shared();
     __syncthreads();
     if (tid == 0) {
-        for (int q = 0; q < nblk; ++q)
-            bulk::s2g(X + q * bstride, tile + q * G::B, (unsigned)(G::B * sizeof(T)));
+        bulk::s2g(X, tile, xb);
         bulk::commit();
     }
     // summaries of the column solve: thread = (column c, block g)
@@ -322,8 +376,8 @@ __global__ void __launch_bounds__(kL, sizeof(T) == 4 ? 4 : 3) row_pass_kernel(Sw
 #pragma unroll
             for (int r0 = 0; r0 < S; r0 += V) {
                 T ps[V], ch[V];
-                ld16(psi + g * S + r0, ps);
-                ld16(chi + g * S + r0, ch);
+                ld16(psi + r0, ps);
+                ld16(chi + r0, ch);
 #pragma unroll
                 for (int e = 0; e < V; ++e) {
                     const int rr = r0 + e;
@@ -332,14 +386,14 @@ __global__ void __launch_bounds__(kL, sizeof(T) == 4 ? 4 : 3) row_pass_kernel(Sw
                     yl[e & 1] = fma(ch[e], x, yl[e & 1]);
                 }
             }
-            A.sumC[it.soff + (int64_t)(bi0 + g) * Mp + bk * S + c] = mk2<T>(wl[0] + wl[1], yl[0] + yl[1]);
+            A.sumC[it.soff + (int64_t)bi * Mp + (bk0 + g) * S + c] = mk2<T>(wl[0] + wl[1], yl[0] + yl[1]);
         }
     }
     if (tid == 0) bulk::wait_read_all();
 }
 
-// Summaries of the row solve with tables tR (psi, chi staged in shared memory for the
-// tile's columns): thread = (row r, block g).
+// Summaries of the row solve (psi, chi staged in shared memory for the tile's columns):
+// thread = (row r, block g) of a column-pass tile.
 template <typename T, int S>
 __device__ __forceinline__ void row_summaries(const SwArgs<T> &A, const SwItem<T> &it, const T *tile, const T *psi,
                                               const T *chi)
@@ -357,8 +411,8 @@ __device__ __forceinline__ void row_summaries(const SwArgs<T> &A, const SwItem<T
     for (int c = 0; c < G::CH; ++c) {
         T x[V], ps[V], ch[V];
         ld16(row + (c / 8) * 8 * V + sw[c % 8], x);
-        ld16(psi + g * S + c * V, ps);
-        ld16(chi + g * S + c * V, ch);
+        ld16(psi + c * V, ps);
+        ld16(chi + c * V, ch);
 #pragma unroll
         for (int e = 0; e < V; ++e) {
             wl[e & 1] = fma(ps[e], x[e], wl[e & 1]);
@@ -366,16 +420,16 @@ __device__ __forceinline__ void row_summaries(const SwArgs<T> &A, const SwItem<T
         }
     }
     const int Mp = it.nb * S;
-    A.sumR[it.soff + (int64_t)(it.b1 + g) * Mp + it.b0 * S + r] = mk2<T>(wl[0] + wl[1], yl[0] + yl[1]);
+    A.sumR[it.soff + (int64_t)it.b1 * Mp + (it.b0 + g) * S + r] = mk2<T>(wl[0] + wl[1], yl[0] + yl[1]);
 }
 
 // ---------------------------------------------------------------------------
-// Column pass.  A tile is n_blk blocks of one block row: S rows x up to 128 columns.
+// Column pass.  A tile is n_blk blocks of one block column: up to 128 rows x S columns.
 // FIRST: j = 0 (D written, not read).  In the last iteration of a problem u and the
 // summaries are not needed.
 // ---------------------------------------------------------------------------
 template <typename T, int S, bool FIRST, bool FUSED>
-__global__ void __launch_bounds__(kL, 3) col_pass_kernel(SwArgs<T> A, int j)
+__global__ void __launch_bounds__(kL, Geo<T, S>::col_ctas) col_pass_kernel(SwArgs<T> A, int j)
 {
     using G = Geo<T, S>;
     using T2 = typename Vec2<T>::type;
@@ -383,64 +437,64 @@ __global__ void __launch_bounds__(kL, 3) col_pass_kernel(SwArgs<T> A, int j)
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
     T *tile = reinterpret_cast<T *>(smem + G::off_tile), *dt = tile + kL * S;
-    T *tl = dt + kL * S, *tm = tl + S, *ts = tm + S, *psi = ts + S, *chi = psi + kL, *co = chi + kL;
+    T *tl = dt + kL * S, *tm = tl + kL, *ts = tm + kL, *psi = ts + kL, *chi = psi + S;
+    T2 *zx = reinterpret_cast<T2 *>(chi + S);
+    T *part = reinterpret_cast<T *>(zx + kL);
     const int tid = threadIdx.x;
     pdl_launch();
     // tiles in the reverse order of the row pass: those it wrote last are still in L2
     const SwItem<T> it = A.items[gridDim.x - 1 - blockIdx.x];
+    const int nb = it.nb, bi0 = it.b0, bk = it.b1, nblk = it.n_blk, Mp = nb * S;
+    LineChain<T, S> chain;
+    if (FUSED && j < it.J) chain.tables(it.chC + (int64_t)j * 6 * round4(nb), nb);
     if (!pass_begin(A, it, j, bar, 2)) return;
-    const int nb = it.nb, bi = it.b0, bk0 = it.b1, nblk = it.n_blk, Mp = nb * S, nbp = round4(nb);
     const bool last = j + 1 == it.J;
     T *X = A.X + it.xoff, *D = A.D + it.xoff;
-    const unsigned xb = (unsigned)(nblk * G::B * sizeof(T));  // the blocks of the tile are adjacent
+    const int64_t bstride = (int64_t)nb * G::B;  // blocks of the tile are one block row apart
+    constexpr unsigned bb = (unsigned)(G::B * sizeof(T));
     if (tid == 0) {
-        const T *tC = it.tabC + (int64_t)j * (2 * kTabs) * Mp + bi * S;
-        const unsigned tb = (unsigned)(S * sizeof(T)), pb = (unsigned)(nblk * S * sizeof(T));
-        bulk::mbar_arrive_expect_tx(bar, xb + 3 * tb + (FUSED ? (unsigned)(3 * nbp * sizeof(T)) : 0u));
-        bulk::g2s(tile, X, xb, bar);
+        const T *tC = it.tabC + (int64_t)j * (2 * kTabs) * Mp + bi0 * S;
+        const unsigned tb = (unsigned)(nblk * S * sizeof(T)), pb = (unsigned)(S * sizeof(T));
+        bulk::mbar_arrive_expect_tx(bar, nblk * bb + 3 * tb);
+        for (int q = 0; q < nblk; ++q) bulk::g2s(tile + q * G::B, X + q * bstride, bb, bar);
         bulk::g2s(tl, tC, tb, bar);
         bulk::g2s(tm, tC + Mp, tb, bar);
         bulk::g2s(ts, tC + 2 * Mp, tb, bar);
-        if (FUSED) bulk::g2s(co, it.chC + (int64_t)j * 6 * nbp, (unsigned)(3 * nbp * sizeof(T)), bar);
-        const unsigned second = (FIRST ? 0u : xb) + (last ? 0u : 2 * pb);
+        const unsigned second = (FIRST ? 0u : nblk * bb) + (last ? 0u : 2 * pb);
         if (second) bulk::mbar_arrive_expect_tx(bar + 1, second);
-        if (!FIRST) bulk::g2s(dt, D, xb, bar + 1);
+        if (!FIRST)
+            for (int q = 0; q < nblk; ++q) bulk::g2s(dt + q * G::B, D + q * bstride, bb, bar + 1);
         if (!last) {
-            const T *tR = it.tabR + (int64_t)(j + 1) * (2 * kTabs) * Mp + bk0 * S;
+            const T *tR = it.tabR + (int64_t)(j + 1) * (2 * kTabs) * Mp + bk * S;
             bulk::g2s(psi, tR + 3 * Mp, pb, bar + 1);
             bulk::g2s(chi, tR + 4 * Mp, pb, bar + 1);
         }
     }
     const int b = tid / S, c = tid % S;
     const bool on = b < nblk;
-    const int64_t line = it.soff + bk0 * S + tid;
-    T zin = 0, yout = 0;
-    LineSums<T> sums;
-    if (on) {
-        if (FUSED) {
-            sums.load(A.sumC + line, Mp, nb);
-        } else {
-            const T2 z = A.zxC[line + (int64_t)bi * Mp];
-            zin = z.x;
-            yout = z.y;
-        }
+    T2 zy = mk2<T>(T(0), T(0));
+    if (FUSED) {
+        chain.load(A.sumC + it.soff + bk * S, Mp, nb);
+        chain.run(zx, part, bi0, nblk);
+        if (on) zy = zx[tid];
+    } else if (on) {
+        zy = A.zxC[it.soff + bk * S + c + (int64_t)(bi0 + b) * Mp];
     }
     if (!tile_ready(bar, A.err)) {
         if (!FIRST || !last) bulk::mbar_wait_bounded(bar + 1, 0);
         return;
     }
-    if (FUSED && on) sums.run(co, nbp, nb, bi, zin, yout);
     int sw[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) sw[q] = ((c / V) ^ q) * V + q * S + c % V;
     T w[S];
     if (on) {
         const T *col = tile + b * G::B;
-        T z = zin;
+        T z = zy.x;
 #pragma unroll
         for (int r0 = 0; r0 < S; r0 += V) {
             T l[V];
-            ld16(tl + r0, l);
+            ld16(tl + b * S + r0, l);
 #pragma unroll
             for (int e = 0; e < V; ++e) {
                 const int r = r0 + e;
@@ -454,12 +508,12 @@ __global__ void __launch_bounds__(kL, 3) col_pass_kernel(SwArgs<T> A, int j)
     }
     if (on) {
         T *col = tile + b * G::B, *dcol = dt + b * G::B;
-        T y = yout;
+        T y = zy.y;
 #pragma unroll
         for (int r0 = S - V; r0 >= 0; r0 -= V) {
             T m[V], s[V];
-            ld16(tm + r0, m);
-            ld16(ts + r0, s);
+            ld16(tm + b * S + r0, m);
+            ld16(ts + b * S + r0, s);
 #pragma unroll
             for (int e = V - 1; e >= 0; --e) {
                 const int r = r0 + e, o = (r / 8) * 8 * S + sw[r % 8];
@@ -472,8 +526,10 @@ __global__ void __launch_bounds__(kL, 3) col_pass_kernel(SwArgs<T> A, int j)
     bulk::fence_proxy_async_shared();
     __syncthreads();
     if (tid == 0) {
-        if (!last) bulk::s2g(X, tile, xb);
-        bulk::s2g(D, dt, xb);
+        for (int q = 0; q < nblk; ++q) {
+            if (!last) bulk::s2g(X + q * bstride, tile + q * G::B, bb);
+            bulk::s2g(D + q * bstride, dt + q * G::B, bb);
+        }
         bulk::commit();
     }
     if (!last) row_summaries<T, S>(A, it, tile, psi, chi);
@@ -488,16 +544,17 @@ __global__ void __launch_bounds__(kL) row_sums_kernel(SwArgs<T> A)
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem);
     T *tile = reinterpret_cast<T *>(smem + G::off_tile);
-    T *psi = tile + kL * S, *chi = psi + kL;
+    T *psi = tile + kL * S, *chi = psi + S;
     pdl_launch();
     const SwItem<T> it = A.items[blockIdx.x];
     if (!pass_begin(A, it, 0, bar, 1)) return;
     const int Mp = it.nb * S;
     if (threadIdx.x == 0) {
         const T *tR = it.tabR + it.b1 * S;
-        const unsigned xb = (unsigned)(it.n_blk * G::B * sizeof(T)), pb = (unsigned)(it.n_blk * S * sizeof(T));
-        bulk::mbar_arrive_expect_tx(bar, xb + 2 * pb);
-        bulk::g2s(tile, A.X + it.xoff, xb, bar);
+        const unsigned bb = (unsigned)(G::B * sizeof(T)), pb = (unsigned)(S * sizeof(T));
+        bulk::mbar_arrive_expect_tx(bar, it.n_blk * bb + 2 * pb);
+        for (int q = 0; q < it.n_blk; ++q)
+            bulk::g2s(tile + q * G::B, A.X + it.xoff + (int64_t)q * it.nb * G::B, bb, bar);
         bulk::g2s(psi, tR + 3 * Mp, pb, bar);
         bulk::g2s(chi, tR + 4 * Mp, pb, bar);
     }
@@ -511,8 +568,7 @@ __global__ void __launch_bounds__(kL) row_sums_kernel(SwArgs<T> A)
 // registers, the warps' maps are composed through shared memory, and the true values
 // follow from one more walk; then the same backwards.  The summaries are read once
 // (n = 10^4, FP32: 10 us a launch; one thread walking all segments of a line took 16).
-// Lines of at most kMaxFused segments have no launch at all: every pass CTA walks its
-// lines' summaries while its tile is in flight (n = 1000: 72 + 72 launches of 7 us less).
+// Lines of few segments have no launch at all (LineChain).
 // ---------------------------------------------------------------------------
 template <typename T, int LEN>
 __global__ void chain_kernel(SwArgs<T> A, int dir, int j)
@@ -1024,6 +1080,8 @@ cudaError_t setup_S()
 }
 
 }  // namespace
+
+bool sweep_fused(bool fp64, int S, int nb) { return nb <= chain_segments(fp64) * (kL / S); }
 
 bool sweep_segment_supported(bool fp64, int seg) { return seg == 64 || (!fp64 && seg == 128); }
 

@@ -75,9 +75,8 @@ struct Vec2<double> {
     using type = double2;
 };
 
-constexpr int kPassLines = 128;  // rows of a row-pass tile, columns of a column-pass tile
+constexpr int kPassLines = 128;  // columns of a row-pass tile, rows of a column-pass tile (whole blocks)
 constexpr int kTabs = 5;         // per position and shift: l, m, solution scale, psi, chi
-constexpr int kMaxFused = 16;    // segments per line up to which a pass runs the recurrence itself
 
 // Offset of element (r, c) inside an S x S block (V elements per 16-byte chunk).
 template <typename T>
@@ -98,8 +97,8 @@ struct alignas(16) SwItem {
     const T *chR, *chC;    // [J][2][3][nbp] segment coefficients phi, Bv, Psi (nbp = nb rounded up to 4), likewise
     int prob;              // problem index (mask of active problems)
     int J;                 // iterations of the problem at this level
-    unsigned short nb, b0; // blocks per side; passes: first block along the lines (row pass: block row)
-    unsigned short b1, n_blk;  // passes: block along the solve; blocks of the tile.  Chains: first line / 32, -
+    unsigned short nb, b0; // blocks per side; passes: block row of the tile's first block
+    unsigned short b1, n_blk;  // passes: its block column; blocks of the tile.  Chains: first line / 32, -
 };
 static_assert(sizeof(SwItem<float>) == 64, "one 64-byte record per item");
 
@@ -115,7 +114,7 @@ struct SwArgs {
     T2 *zxR, *zxC;         // recurrence results {zin, yout}, same layout (plans that run it in its own kernel)
     int *err;              // device error word: bit 0 = a bounded wait gave up
     int S;                 // block and segment size of every problem (sweep_segment_supported(., 2 S))
-    int fused;             // passes run the segment recurrence themselves (nb <= kMaxFused)
+    int fused;             // passes run the segment recurrence themselves (sweep_fused)
     int chain_len;         // chain kernel: segments per thread
     int max_nb;
 };
@@ -152,6 +151,13 @@ struct FacJob {
 };
 
 cudaError_t sweep_setup_kernels();
+// Whether the passes run the segment recurrences of lines of up to nb segments of S
+// themselves, while their tiles are in flight (otherwise launch_chain does).  A thread group
+// of a tile takes 8 segments in FP32 (n <= 2048 with both block sizes: each chain launch took
+// 5.7 us of about 20 per pass; Dirichlet solve and adjoint at n = 2048 4.43 -> 4.21 ms, 3.95
+// with fuller waves) and 4 in FP64 (n <= 1024), where the operations come on top of a bound
+// FP64 pipe.
+bool sweep_fused(bool fp64, int S, int nb);
 // Segment lengths (unknowns of both parities) with compiled pass kernels: 64 (FP32, FP64)
 // and 128 (FP32), i.e. blocks of 32 and 64.
 bool sweep_segment_supported(bool fp64, int seg);

@@ -329,7 +329,7 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
         }
         totB64 += 7 * n;
     }
-    fused_ = max_nb_ <= kMaxFused;
+    fused_ = sweep_fused(kFP64, S, max_nb_);
     npairs_ = np * nrhs;
 
     ENG_CK(sweep_setup_kernels());
@@ -619,19 +619,19 @@ int SweepEngine<T>::build_tables(Level &L, int level, const std::vector<double> 
                 x.prob = p;
                 x.J = L.J[p];
                 x.nb = (unsigned short)nb;
-                for (int b0 = 0; b0 < nb; b0 += R)
-                    for (int b1 = 0; b1 < nb; ++b1) {
-                        x.b0 = (unsigned short)b0;
-                        x.b1 = (unsigned short)b1;
-                        x.n_blk = (unsigned short)std::min(R, nb - b0);
-                        x.xoff = x0 + ((int64_t)b0 * nb + b1) * S * S;
-                        it[0].push_back(x);
-                    }
                 for (int b0 = 0; b0 < nb; ++b0)
                     for (int b1 = 0; b1 < nb; b1 += R) {
                         x.b0 = (unsigned short)b0;
                         x.b1 = (unsigned short)b1;
                         x.n_blk = (unsigned short)std::min(R, nb - b1);
+                        x.xoff = x0 + ((int64_t)b0 * nb + b1) * S * S;
+                        it[0].push_back(x);
+                    }
+                for (int b0 = 0; b0 < nb; b0 += R)
+                    for (int b1 = 0; b1 < nb; ++b1) {
+                        x.b0 = (unsigned short)b0;
+                        x.b1 = (unsigned short)b1;
+                        x.n_blk = (unsigned short)std::min(R, nb - b0);
                         x.xoff = x0 + ((int64_t)b0 * nb + b1) * S * S;
                         it[1].push_back(x);
                     }

@@ -3,9 +3,9 @@ the CPU oracle through the C ABI.
 
 One launch (resident kernel): quarters of m = ceil(n/2) <= 16 S unknowns for the compiled
 segment lengths S, FP64 up to n = 512, FP32 up to n = 1024.  Streamed: blocks of 32 (FP64,
-FP32 segment length 64) or 64 (FP32 segment length 128) unknowns, tiles of 128 lines; up
-to 16 segments per line the passes run the segment recurrence themselves, beyond that the
-chain kernel does (FP64: n > 1024; FP32: n > 1024 or n > 2048).  Bars: the FP64 and
+FP32 segment length 64) or 64 (FP32 segment length 128) unknowns, tiles of 128 x one block;
+the passes run the segment recurrence themselves up to n = 1024 (FP64) and 2048 (FP32), the
+chain kernel does beyond.  Bars: the FP64 and
 refinement bars of the workload definition."""
 import numpy as np
 import pytest
@@ -89,6 +89,24 @@ def test_refine_segment_counts(api, tmp_path, monkeypatch, seg, chain):
     for n, f in zip(ns, rhs):
         assert _relmax(X[o:o + n * n].reshape(n, n), oracle.poisson_square(f, 1e-13)) <= TOL_REFINE, n
         o += n * n
+
+
+# lines of 17, 32 and 33 segments of 32 and of 9, 16 and 17 segments of 64: the passes run the
+# segment recurrence up to 32 and 16, the chain kernel beyond
+@pytest.mark.parametrize("seg", [64, 128])
+@pytest.mark.parametrize("n", [1025, 2047, 2048, 2049])
+def test_refine_recurrence_edges(api, tmp_path, monkeypatch, seg, n):
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("FPS_AUTOTUNE_CACHE", str(cache))
+    monkeypatch.delenv("FPS_AUTOTUNE", raising=False)
+    api.plan_destroy(api.plan_create(n, 2, 1e-10, "fp32_refine"))
+    cache.write_text(f"{cache.read_text().split()[0]} {seg} 1\n")
+    F = inputs.square_rhs(n, 70 + n)
+    plan = api.plan_create(n, 2, 1e-10, "fp32_refine")
+    X = api.poisson_square_solve(plan, torch.from_numpy(F).cuda()).cpu().numpy()
+    assert api.plan_info(plan)["seg_len"] == seg
+    api.plan_destroy(plan)
+    assert _relmax(X, oracle.poisson_square(F, 1e-13)) <= TOL_REFINE
 
 
 @pytest.mark.parametrize("n", [101, 601])
