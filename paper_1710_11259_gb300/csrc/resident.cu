@@ -32,7 +32,11 @@ template <typename T, int S>
 struct ResGeo {
     static constexpr int A = 16 / (int)sizeof(T);
     __host__ __device__ static constexpr int up(int n) { return (n + A - 1) / A * A; }
-    static constexpr int kThreads = (kG * S + 31) / 32 * 32;
+    // Lines (rows, then columns) per thread.  FP32 is bound by shared memory, half of it table
+    // entries that serve every line: with two lines a thread reads them once for both.  FP64
+    // wants all its warps.
+    static constexpr int kR = sizeof(T) == 4 && S >= 20 ? 2 : 1;
+    static constexpr int kThreads = (kG * S / kR + 31) / 32 * 32;
     // a segment takes an odd number of elements and a row 16 of them, so that the 32 lanes
     // of the row solve (16 segments of two rows) hit different banks
     static constexpr int SS = S | 1, pitch = kG * SS;
@@ -91,14 +95,14 @@ __device__ __forceinline__ void scan_segments(T wl, T yl, const T *k, int g, T &
 }
 
 template <typename T, int S>
-__global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResArgs<T> a)
+__global__ void __launch_bounds__(ResGeo<T, S>::kThreads) resident_kernel(ResArgs<T> a)
 {
     using G = ResGeo<T, S>;
     using T2 = typename Vec2<T>::type;
-    constexpr int M = kG * S;
+    constexpr int M = kG * S, kR = G::kR;
     // partial sums of a summary: an FP64 instruction of a warp occupies its issue for as long as
-    // its latency, so a second chain only costs its addition
-    constexpr int kAcc = sizeof(T) == 8 ? 1 : 2;
+    // its latency, so a second chain only costs its addition; two lines are two chains
+    constexpr int kAcc = sizeof(T) == 8 || kR == 2 ? 1 : 2;
     auto total = [](const T(&x)[kAcc]) { return kAcc == 1 ? x[0] : x[0] + x[kAcc - 1]; };
     extern __shared__ __align__(16) unsigned char smem[];
     cg::cluster_group cl = cg::this_cluster();
@@ -144,28 +148,40 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
         X[r * G::pitch + (k / S) * G::SS + k % S] = v;
     }
     for (int q = tid; q < S * G::cpitch; q += G::kThreads) cs[q] = pair_of<T>(T(0), T(0));
-    T D[S];
+    T D[kR][S];
 #pragma unroll
-    for (int i = 0; i < S; ++i) D[i] = 0;
+    for (int i = 0; i < S; ++i)
+#pragma unroll
+        for (int h = 0; h < kR; ++h) D[h][i] = 0;
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     cl.sync();  // the slab is complete and every CTA of the cluster runs
 
-    // row solve: row r0, segment g; column solve: column tid = segment gc, place cc.  Threads
-    // beyond the last row or column (16 S is no multiple of 32, or fewer segments in use)
-    // compute on zeros that nobody reads.
-    const int g = tid & (kG - 1), r0 = min(tid >> 4, S - 1);
-    const bool row_on = (tid >> 4) < S;
-    const int col = min(tid, M - 1), gc = col / S, cc = col % S;
-    const bool col_on = tid < M && gc < C;
+    // row solve: rows r0 and r0 + S / 2, segment g; column solve: columns col and col + M / 2.
+    // Threads beyond the last row or column (16 S is no multiple of 32, or fewer segments in
+    // use) compute on zeros that nobody reads.
+    const int g = tid & (kG - 1), r0 = min(tid >> 4, S / kR - 1);
+    const bool row_on = (tid >> 4) < S / kR;
     T *xr = X + r0 * G::pitch + g * G::SS;
-    T *xc = X + gc * G::SS + cc;
+    constexpr int rstep = S / kR, cstep = M / kR;
     // Exchange: each of the C S pairs of a step is an asynchronous store that the receiver's
     // barrier counts.  A CTA sends a step's pairs only after it has received all of the step
     // before, which its peers send after reading what the new pairs overwrite.
     const unsigned bytes = (unsigned)(C * S * sizeof(T2));
-    const int pc = min(gc, C - 1), pr = min(g, C - 1);  // peers that own the column, that want its segment
-    const unsigned to_cs = bulk::peer_smem(cs + cc * G::cpitch + rank, pc), bar_cs = bulk::peer_smem(bar, pc);
+    const int pr = min(g, C - 1);  // peer that wants its segment of the owned columns
     const unsigned to_bd = bulk::peer_smem(bd + i0 + r0, pr), bar_bd = bulk::peer_smem(bar + 1, pr);
+    int col[kR];
+    bool col_on[kR];
+    T *xc[kR];
+    unsigned to_cs[kR], bar_cs[kR];  // at the peer that owns the column
+#pragma unroll
+    for (int h = 0; h < kR; ++h) {
+        col[h] = min(tid + h * cstep, M - 1);
+        const int gc = col[h] / S, cc = col[h] % S;
+        col_on[h] = tid + h * cstep < M && gc < C;
+        xc[h] = X + gc * G::SS + cc;
+        to_cs[h] = bulk::peer_smem(cs + cc * G::cpitch + rank, min(gc, C - 1));
+        bar_cs[h] = bulk::peer_smem(bar, min(gc, C - 1));
+    }
     bool ok = true;  // false: a wait gave up; the thread runs on without waiting or sending
     auto wait = [&](uint64_t *b, int j) {
         if (ok && !bulk::mbar_wait_cluster(b, j & 1)) {
@@ -183,76 +199,101 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
             bulk::mbar_arrive_expect_tx(bar + 1, bytes);
         }
         if (j + 1 < J) load_tables(j + 1);
-        T v[S], w[S];
+        T v[kR][S], w[kR][S];
         {
-            T wl[kAcc] = {}, yl[kAcc] = {};
+            T wl[kR][kAcc] = {}, yl[kR][kAcc] = {};
 #pragma unroll
             for (int i = 0; i < S; ++i) {
                 const T2 p = sums[i * kG];
-                v[i] = xr[i];
-                wl[i % kAcc] = fma(p.x, v[i], wl[i % kAcc]);
-                yl[i % kAcc] = fma(p.y, v[i], yl[i % kAcc]);
+#pragma unroll
+                for (int h = 0; h < kR; ++h) {
+                    v[h][i] = xr[h * rstep * G::pitch + i];
+                    wl[h][i % kAcc] = fma(p.x, v[h][i], wl[h][i % kAcc]);
+                    yl[h][i % kAcc] = fma(p.y, v[h][i], yl[h][i % kAcc]);
+                }
             }
-            T z, y;
-            scan_segments<T>(total(wl), total(yl), kr, g, z, y);
+            T z[kR], y[kR];
+#pragma unroll
+            for (int h = 0; h < kR; ++h) scan_segments<T>(total(wl[h]), total(yl[h]), kr, g, z[h], y[h]);
 #pragma unroll
             for (int i = 0; i < S; i += 2) {
                 const T2 l = fwd[i / 2 * kG];
-                z = fma(-l.x, z, v[i]);
-                w[i] = z;
-                if (i + 1 < S) {
-                    z = fma(-l.y, z, v[i + 1]);
-                    w[i + 1] = z;
+#pragma unroll
+                for (int h = 0; h < kR; ++h) {
+                    z[h] = fma(-l.x, z[h], v[h][i]);
+                    w[h][i] = z[h];
+                    if (i + 1 < S) {
+                        z[h] = fma(-l.y, z[h], v[h][i + 1]);
+                        w[h][i + 1] = z[h];
+                    }
                 }
             }
             const bool first = j == 0;
 #pragma unroll
             for (int i = S - 1; i >= 0; --i) {
                 const T2 p = back[i * kG];
-                y = fma(-p.x, y, w[i]);
-                v[i] = fma(p.y, y, first ? T(0) : v[i]);
+#pragma unroll
+                for (int h = 0; h < kR; ++h) {
+                    y[h] = fma(-p.x, y[h], w[h][i]);
+                    v[h][i] = fma(p.y, y[h], first ? T(0) : v[h][i]);
+                }
             }
             if (row_on)
 #pragma unroll
-                for (int i = 0; i < S; ++i) xr[i] = v[i];
+                for (int i = 0; i < S; ++i)
+#pragma unroll
+                    for (int h = 0; h < kR; ++h) xr[h * rstep * G::pitch + i] = v[h][i];
         }
         __syncthreads();
         {
-            T wl[kAcc] = {}, yl[kAcc] = {};
+            T wl[kR][kAcc] = {}, yl[kR][kAcc] = {};
 #pragma unroll
             for (int c = 0; c < S; c += G::A) {
                 T psi[G::A], chi[G::A];
                 read16(psi, tc + 3 * G::SP + c);
                 read16(chi, tc + 4 * G::SP + c);
 #pragma unroll
-                for (int i = c; i < min(c + G::A, S); ++i) {
-                    v[i] = xc[i * G::pitch];
-                    wl[i % kAcc] = fma(psi[i - c], v[i], wl[i % kAcc]);
-                    yl[i % kAcc] = fma(chi[i - c], v[i], yl[i % kAcc]);
-                }
+                for (int i = c; i < min(c + G::A, S); ++i)
+#pragma unroll
+                    for (int h = 0; h < kR; ++h) {
+                        v[h][i] = xc[h][i * G::pitch];
+                        wl[h][i % kAcc] = fma(psi[i - c], v[h][i], wl[h][i % kAcc]);
+                        yl[h][i % kAcc] = fma(chi[i - c], v[h][i], yl[h][i % kAcc]);
+                    }
             }
-            if (col_on && ok) bulk::send_pair(to_cs, bar_cs, pair_of<T>(total(wl), total(yl)));
+#pragma unroll
+            for (int h = 0; h < kR; ++h)
+                if (col_on[h] && ok) bulk::send_pair(to_cs[h], bar_cs[h], pair_of<T>(total(wl[h]), total(yl[h])));
         }
         wait(bar, j);
-        {  // the columns this CTA owns, rank * S + r0, all their segments
-            const T2 s = cs[r0 * G::cpitch + g];
+#pragma unroll
+        for (int h = 0; h < kR; ++h) {  // the columns this CTA owns, rank * S + r0 (+ S / 2), all their segments
+            const T2 s = cs[(r0 + h * rstep) * G::cpitch + g];
             T z, y;
             scan_segments<T>(s.x, s.y, kc, g, z, y);
-            if (row_on && g < C && ok) bulk::send_pair(to_bd, bar_bd, pair_of<T>(z, y));
+            if (row_on && g < C && ok)
+                bulk::send_pair(to_bd + h * rstep * (unsigned)sizeof(T2), bar_bd, pair_of<T>(z, y));
         }
         wait(bar + 1, j);
-        if (col_on) {
-            const T2 b = bd[col];
-            T z = b.x, y = b.y;
+        if (col_on[0]) {
+            T z[kR], y[kR];
+#pragma unroll
+            for (int h = 0; h < kR; ++h) {
+                const T2 b = bd[col[h]];
+                z[h] = b.x;
+                y[h] = b.y;
+            }
 #pragma unroll
             for (int c = 0; c < S; c += G::A) {
                 T l[G::A];
                 read16(l, tc + c);
 #pragma unroll
-                for (int i = c; i < min(c + G::A, S); ++i) {
-                    z = fma(-l[i - c], z, v[i]);
-                    w[i] = z;
-                }
+                for (int i = c; i < min(c + G::A, S); ++i)
+#pragma unroll
+                    for (int h = 0; h < kR; ++h) {
+                        z[h] = fma(-l[i - c], z[h], v[h][i]);
+                        w[h][i] = z[h];
+                    }
             }
 #pragma unroll
             for (int c = G::SP - G::A; c >= 0; c -= G::A) {
@@ -260,11 +301,13 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
                 read16(mm, tc + G::SP + c);
                 read16(gg, tc + 2 * G::SP + c);
 #pragma unroll
-                for (int i = min(c + G::A, S) - 1; i >= c; --i) {
-                    y = fma(-mm[i - c], y, w[i]);
-                    xc[i * G::pitch] = fma(gg[i - c], y, v[i]);
-                    D[i] = fma(gg[i - c], y, D[i]);
-                }
+                for (int i = min(c + G::A, S) - 1; i >= c; --i)
+#pragma unroll
+                    for (int h = 0; h < kR; ++h) {
+                        y[h] = fma(-mm[i - c], y[h], w[h][i]);
+                        if (col_on[h]) xc[h][i * G::pitch] = fma(gg[i - c], y[h], v[h][i]);
+                        D[h][i] = fma(gg[i - c], y[h], D[h][i]);
+                    }
             }
         }
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
@@ -272,14 +315,16 @@ __global__ void __launch_bounds__((kG * S + 31) / 32 * 32) resident_kernel(ResAr
     }
     // no CTA leaves while a peer whose wait gave up may still have stores under way to it
     asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
-    if (col_on && col < mc) {
+#pragma unroll
+    for (int h = 0; h < kR; ++h) {
+        if (!col_on[h] || col[h] >= mc) continue;
 #pragma unroll
         for (int r = 0; r < S; ++r) {
-            const int i = i0 + r;
-            if (!ok) D[r] = (T)NAN;
+            const int i = i0 + r, k = col[h];
+            const T d = ok ? D[h][r] : (T)NAN;
             if (i < mr) {
-                if (a.F) a.out[npos(i, col)] = it.out_scale * (double)D[r] * it.s[2 * i + it.rp] * it.s[2 * col + it.cp];
-                else a.D[qpos(i, col)] = D[r];
+                if (a.F) a.out[npos(i, k)] = it.out_scale * (double)d * it.s[2 * i + it.rp] * it.s[2 * k + it.cp];
+                else a.D[qpos(i, k)] = d;
             }
         }
     }

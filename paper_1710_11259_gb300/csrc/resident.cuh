@@ -6,7 +6,8 @@
 // line is cut into 16 segments of S.  An iteration is
 //   row solve     thread (row, segment), the 16 segments of a row on neighbouring lanes:
 //                 two summaries per thread, the recurrence over the segments as warp
-//                 scans, then the sweeps of the segment in registers;
+//                 scans, then the sweeps of the segment in registers (long FP32 segments:
+//                 two rows, then two columns, per thread);
 //   column solve  thread = column, the CTA's S rows are one segment: its summaries go to
 //                 the CTA that owns the column, which runs the same scans and returns zin
 //                 and yout to every CTA, then the sweeps.  Both ways each pair is an
@@ -22,8 +23,8 @@
 // cluster of 8 CTAs per right-hand side solving every line by cyclic reduction and
 // exchanging whole iterates; 250 us with remote stores between cluster barriers, whose
 // fences alone were a fifth of the time), n = 301 FP64 0.60 ms (2.5 ms streamed by the
-// passes, 0.69 with cluster barriers), n = 1000 FP32+refine 0.53 ms (1.18 streamed, 0.56
-// with cluster barriers).
+// passes, 0.69 with cluster barriers), n = 1000 FP32+refine 0.50 ms (1.18 streamed, 0.56
+// with cluster barriers, 0.53 with one line per thread).
 #pragma once
 #include <cuda_runtime.h>
 
