@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(ResGeo<T, S>::kThreads) resident_kernel(ResArg
     for (int h = 0; h < kR; ++h) {
         col[h] = min(tid + h * cstep, M - 1);
         const int gc = col[h] / S, cc = col[h] % S;
-        col_on[h] = tid + h * cstep < M && gc < C;
+        col_on[h] = tid < cstep && gc < C;  // a column has one thread: its summaries are counted once
         xc[h] = X + gc * G::SS + cc;
         to_cs[h] = bulk::peer_smem(cs + cc * G::cpitch + rank, min(gc, C - 1));
         bar_cs[h] = bulk::peer_smem(bar, min(gc, C - 1));
