@@ -68,6 +68,13 @@ void SweepEngine<T>::release()
     levels_.clear();
     for (void *p : allocs_) cudaFree(p);
     allocs_.clear();
+    for (Side &x : side_) {
+        if (x.st) cudaStreamDestroy(x.st);
+        cudaEventDestroy(x.done);
+    }
+    side_.clear();
+    if (fork_) cudaEventDestroy(fork_);
+    fork_ = nullptr;
     void *hp[] = {h_active_, h_pair_active_, h_stat_};
     for (void *p : hp)
         if (p) cudaFreeHost(p);
@@ -443,10 +450,15 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     if (kFP64) tols.push_back(tol);
     else tols.assign(std::begin(kLevelTols), std::end(kLevelTols));
     shifts.assign(np, {});
+    TableJobs jobs;
     for (size_t li = 0; li < tols.size(); ++li) {
         levels_.emplace_back();
         levels_.back().tol = tols[li];
-        const int st = build_tables(levels_.back(), (int)li, lo, hi, err);
+        const int st = build_tables(levels_.back(), (int)li, lo, hi, jobs, err);
+        if (st != FPS_OK) return st;
+    }
+    {
+        const int st = run_table_jobs(jobs, err);
         if (st != FPS_OK) return st;
     }
     {
@@ -462,10 +474,45 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     return FPS_OK;
 }
 
-// Shifts, tables and work items of one tolerance level.
+// The tables of all levels: a thread walks a whole line, so one launch of every level's jobs
+// takes as long as the longest line, where a launch per level took that six times over
+// (n = 1000 3.5 ms of the plan, n = 2048 6 ms).
+template <typename T>
+int SweepEngine<T>::run_table_jobs(const TableJobs &jobs, std::string &err)
+{
+    struct Scratch {  // device copies of the job lists
+        void *p[2] = {nullptr, nullptr};
+        ~Scratch()
+        {
+            for (void *q : p)
+                if (q) cudaFree(q);
+        }
+    } scratch;
+    cudaError_t e1 = cudaSuccess;
+    auto upload = [&](int slot, const void *src, size_t bytes) -> void * {
+        if (e1 == cudaSuccess) e1 = cudaMalloc(&scratch.p[slot], bytes);
+        if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(scratch.p[slot], src, bytes, cudaMemcpyHostToDevice, cap_);
+        return scratch.p[slot];
+    };
+    if (!jobs.fac.empty()) {
+        const FacJob<T> *d = (const FacJob<T> *)upload(0, jobs.fac.data(), sizeof(FacJob<T>) * jobs.fac.size());
+        if (e1 == cudaSuccess) e1 = launch_fac_tables<T>(d, (int)jobs.fac.size(), cap_);
+    }
+    if (!jobs.res.empty()) {
+        const ResTabJob<T> *d = (const ResTabJob<T> *)upload(1, jobs.res.data(), sizeof(ResTabJob<T>) * jobs.res.size());
+        if (e1 == cudaSuccess) e1 = launch_resident_tables<T>(d, (int)jobs.res.size(), cap_);
+    }
+    // the scratch must outlive the asynchronous work
+    const cudaError_t e2 = cudaStreamSynchronize(cap_);
+    ENG_CK(e1);
+    ENG_CK(e2);
+    return FPS_OK;
+}
+
+// Shifts and work items of one tolerance level; its tables go on the job lists.
 template <typename T>
 int SweepEngine<T>::build_tables(Level &L, int level, const std::vector<double> &lo, const std::vector<double> &hi,
-                                 std::string &err)
+                                 TableJobs &tables, std::string &err)
 {
     const int np = (int)ns_.size(), S = seg_len / 2;
     // intervals of kx A~ (row side) and -ky A~ (column side): [a, b] = -kx [hi, lo],
@@ -491,18 +538,10 @@ int SweepEngine<T>::build_tables(Level &L, int level, const std::vector<double> 
     ENG_CK(dalloc(&L.tab, (size_t)(2 * nfac)));
     ENG_CK(dalloc(&L.ch, (size_t)(2 * nch)));
     ENG_CK(dalloc(&L.res_tab, (size_t)(2 * nres)));
-    struct Scratch {  // device copies of the job lists
-        void *p[2] = {nullptr, nullptr};
-        ~Scratch()
-        {
-            for (void *q : p)
-                if (q) cudaFree(q);
-        }
-    } scratch;
-    std::vector<FacJob<T>> jobs;
-    std::vector<ResTabJob<T>> rjobs;
-    jobs.reserve((size_t)nq * 2);
-    rjobs.reserve((size_t)nq_res * 2);
+    std::vector<FacJob<T>> &jobs = tables.fac;
+    std::vector<ResTabJob<T>> &rjobs = tables.res;
+    jobs.reserve(jobs.size() + (size_t)nq * 2);
+    rjobs.reserve(rjobs.size() + (size_t)nq_res * 2);
     std::vector<int64_t> otab(np), och(np);  // offsets of a problem's tables (records) and coefficients
     int64_t of = 0, oc = 0, ores = 0;
     std::vector<double> q, pp;
@@ -659,20 +698,7 @@ int SweepEngine<T>::build_tables(Level &L, int level, const std::vector<double> 
             e1 = cudaMemcpyAsync(L.res[c].items, rit[c].data(), sizeof(ResItem<T>) * rit[c].size(), cudaMemcpyHostToDevice,
                                  cap_);
     }
-    auto upload = [&](int slot, const void *src, size_t bytes) -> void * {
-        if (e1 == cudaSuccess) e1 = cudaMalloc(&scratch.p[slot], bytes);
-        if (e1 == cudaSuccess) e1 = cudaMemcpyAsync(scratch.p[slot], src, bytes, cudaMemcpyHostToDevice, cap_);
-        return scratch.p[slot];
-    };
-    if (!jobs.empty()) {
-        const FacJob<T> *d = (const FacJob<T> *)upload(0, jobs.data(), sizeof(FacJob<T>) * jobs.size());
-        if (e1 == cudaSuccess) e1 = launch_fac_tables<T>(d, (int)jobs.size(), cap_);
-    }
-    if (!rjobs.empty()) {
-        const ResTabJob<T> *d = (const ResTabJob<T> *)upload(1, rjobs.data(), sizeof(ResTabJob<T>) * rjobs.size());
-        if (e1 == cudaSuccess) e1 = launch_resident_tables<T>(d, (int)rjobs.size(), cap_);
-    }
-    // the host vectors and the scratch must outlive the asynchronous work
+    // the host vectors must outlive the asynchronous work
     const cudaError_t e2 = cudaStreamSynchronize(cap_);
     ENG_CK(e1);
     ENG_CK(e2);
@@ -720,6 +746,42 @@ SwArgs<T> SweepEngine<T>::args(const Level &L, int which) const
     return a;
 }
 
+// The resident launches of a level, one per class, side by side: a launch of a few clusters
+// is bound by the latency of its iterations and leaves most of the GPU idle.  Branches of at
+// most kSide streams from `st`; the first class stays on `st` unless other work follows there.
+// join_resident() makes `st` wait for the branches.  One after the other a batch of 8 problems
+// in as many classes took 1.2 times as long as the passes over all of them; side by side
+// 0.59 ms against 1.70 (8 problems of n = 38 .. 457, two right-hand sides each).
+template <typename T>
+cudaError_t SweepEngine<T>::run_resident(const Level &L, const double *F, double *X, cudaStream_t st, bool busy,
+                                         int64_t &launches)
+{
+    cudaError_t e = cudaSuccess;
+    const int n = (int)L.res.size(), here = busy ? 0 : 1, nside = std::min((int)side_.size(), n - here);
+    side_used_ = std::max(nside, 0);
+    if (nside > 0) {
+        e = cudaEventRecord(fork_, st);
+        for (int k = 0; k < nside && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(side_[k].st, fork_, 0);
+    }
+    for (int c = 0; c < n && e == cudaSuccess; ++c) {
+        e = launch_resident<T>(res_args(L.res[c], F, X), c < here || nside <= 0 ? st : side_[(c - here) % nside].st);
+        ++launches;
+    }
+    return e;
+}
+
+template <typename T>
+cudaError_t SweepEngine<T>::join_resident(cudaStream_t st)
+{
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < side_used_ && e == cudaSuccess; ++k) {
+        e = cudaEventRecord(side_[k].done, side_[k].st);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, side_[k].done, 0);
+    }
+    side_used_ = 0;
+    return e;
+}
+
 template <typename T>
 int SweepEngine<T>::build_graph(Level &L, std::string &err)
 {
@@ -728,6 +790,14 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
         L.graph = nullptr;
     }
     const SwArgs<T> ar = args(L, 0), ac = args(L, 1), ach = args(L, 2);
+    // created outside the capture
+    for (int k = (int)side_.size(), want = std::min<int>(kSide, (int)L.res.size() - (streams_ ? 0 : 1)); k < want; ++k) {
+        Side x;
+        ENG_CK(cudaEventCreateWithFlags(&x.done, cudaEventDisableTiming));
+        side_.push_back(x);
+        ENG_CK(cudaStreamCreateWithFlags(&side_.back().st, cudaStreamNonBlocking));
+    }
+    if (!side_.empty() && !fork_) ENG_CK(cudaEventCreateWithFlags(&fork_, cudaEventDisableTiming));
     ENG_CK(cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     const bool ins = instrument_ && (int)L.ev.size() == 4 * L.Jstream + 2;
@@ -740,7 +810,9 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
         ++L.launches;
     };
     rec(4 * L.Jstream);
-    for (const ResClass &c : L.res) run(launch_resident<T>(res_args(c, nullptr, nullptr), cap_));
+    if (ins)
+        for (const ResClass &c : L.res) run(launch_resident<T>(res_args(c, nullptr, nullptr), cap_));
+    else if (e == cudaSuccess) e = run_resident(L, nullptr, nullptr, cap_, streams_, L.launches);
     rec(4 * L.Jstream + 1);
     if (streams_) run(launch_row_sums<T>(ac, cap_));
     for (int j = 0; j < L.Jstream && e == cudaSuccess; ++j) {
@@ -753,6 +825,7 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
         run(launch_col_pass<T>(ac, j, cap_));
         rec(4 * j + 3);
     }
+    if (!ins && e == cudaSuccess) e = join_resident(cap_);
     cudaGraph_t g = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(cap_, &g);
     if (e != cudaSuccess) {
@@ -780,10 +853,8 @@ int SweepEngine<T>::solve_plain(const double *F, double *X, cudaStream_t st, std
 {
     if constexpr (sizeof(T) == 8) {
         if (!streams_ && !instrument_) {  // scale-in, all iterations and scale-out in one launch per class
-            for (const ResClass &c : levels_[0].res) {
-                ENG_CK(launch_resident<T>(res_args(c, F, X), st));
-                ++launches_last;
-            }
+            ENG_CK(run_resident(levels_[0], F, X, st, false, launches_last));
+            ENG_CK(join_resident(st));
             levels_used_.push_back(0);
             rounds_last = 1;
             return FPS_OK;

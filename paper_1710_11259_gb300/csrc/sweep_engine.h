@@ -81,8 +81,24 @@ private:
     int time_chain(int mode, float &ms, std::string &err);
     SwArgs<T> args(const Level &L, int which) const;
     ResArgs<T> res_args(const ResClass &c, const double *F, double *X) const;
+    struct TableJobs {
+        std::vector<FacJob<T>> fac;
+        std::vector<ResTabJob<T>> res;
+    };
     int build_tables(Level &L, int level, const std::vector<double> &lo, const std::vector<double> &hi,
-                     std::string &err);
+                     TableJobs &tables, std::string &err);
+    int run_table_jobs(const TableJobs &jobs, std::string &err);
+    cudaError_t run_resident(const Level &L, const double *F, double *X, cudaStream_t st, bool busy, int64_t &launches);
+    cudaError_t join_resident(cudaStream_t st);
+    // branches of the resident launches (streams of this engine, joined by every solve)
+    static constexpr int kSide = 8;
+    struct Side {
+        cudaStream_t st = nullptr;
+        cudaEvent_t done = nullptr;
+    };
+    std::vector<Side> side_;
+    cudaEvent_t fork_ = nullptr;
+    int side_used_ = 0;
     enum { kLive, kPadded, kResidual };  // tile lists (sweep.cuh)
     TileArgs tiles(int which) const;
     void set_active();
