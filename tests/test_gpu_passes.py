@@ -179,7 +179,7 @@ def _along(T, B):  # B on all three modes
 
 
 # the slice kernel's line lengths (2 H unknowns per parity), full and with unused places
-@pytest.mark.parametrize("n", [3, 4, 7, 9, 12, 13, 16, 24, 25, 33, 40, 41, 49, 65, 81, 97, 113, 129, 145])
+@pytest.mark.parametrize("n", [3, 4, 7, 9, 12, 13, 16, 24, 25, 33, 40, 41, 49, 65, 81, 97, 113, 129, 145, 161, 193, 257, 289])
 def test_cube_refine_line_lengths(api, n):
     """Against the exact solution by diagonalisation, at the cube's refinement bar."""
     F = inputs.cube_rhs(n, n)
