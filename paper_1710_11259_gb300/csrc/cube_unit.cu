@@ -268,7 +268,8 @@ __global__ void __launch_bounds__(64) unit_tables_kernel(const UnitEntry *__rest
                                                          int n, int H, float *__restrict__ tabs)
 {
     const int raw = blockIdx.x * blockDim.x + threadIdx.x;
-    const int id = min(raw, 8 * shifts - 1), h = id & 1, LS = unit_half_pitch(H);  // threads past the end repeat the last pair
+    const int id = unit_table_thread(raw, shifts), h = id & 1, LS = unit_half_pitch(H);
+    const bool live = raw < 8 * shifts;
     const int x = (id >> 1) & 3, sh = id >> 3, tab = unit_table(H);
     int lo = 0, hi = count - 1;  // the entry of shift sh
     while (lo < hi) {
@@ -292,14 +293,17 @@ __global__ void __launch_bounds__(64) unit_tables_kernel(const UnitEntry *__rest
         const double eo = B.outer(h, s), c = alpha * eo, ip = 1.0 / prev, lv = c * ip;
         const double own = i < m ? alpha * B.diag(i) + beta : 1.0, piv = own - lv * c;
         const double iv = 1.0 / piv;
-        l[h * LS + s] = (float)lv;
-        if (s) mg[2 * (h * LS + s - 1)] = (float)(c * iv);
-        mg[2 * (h * LS + s) + 1] = (float)(i < m ? scale * iv : 0.0);
+        if (live) {
+            l[h * LS + s] = (float)lv;
+            if (s) mg[2 * (h * LS + s - 1)] = (float)(c * iv);
+            mg[2 * (h * LS + s) + 1] = (float)(i < m ? scale * iv : 0.0);
+        }
         prev = piv;
     }
-    mg[2 * (h * LS + H - 1)] = 0.0f;
     const double other = __shfl_xor_sync(0xffffffffu, prev, 1), em = B.off(H - 1), c = alpha * em;
     const double det = prev * other - c * c;
+    if (!live) return;
+    mg[2 * (h * LS + H - 1)] = 0.0f;
     mid[2 * h] = (float)(prev * other / det);
     mid[2 * h + 1] = (float)(-c * prev / det);
 }

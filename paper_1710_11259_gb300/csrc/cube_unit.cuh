@@ -70,6 +70,15 @@ struct UnitEntry {
     int first, J;
 };
 
+// Thread `raw` of the table kernel over `shifts` shifts computes half (id & 1) of the line
+// id >> 1 of (shift, direction, parity), id as returned; the halves of a line are a lane pair.
+// Threads past the end repeat the last pair (each its own half: they take part in the
+// exchange of the pivots) and store nothing.
+__host__ __device__ constexpr int unit_table_thread(int raw, int shifts)
+{
+    return raw < 8 * shifts ? raw : 8 * shifts - 2 + (raw & 1);
+}
+
 int unit_half(int64_t n);  // H of the compiled kernel (n <= 320; 0 beyond)
 cudaError_t unit_setup(int H);
 // Tables of `count` entries (device list, ascending `first`) with `shifts` shifts {p, q}
