@@ -109,8 +109,9 @@ typedef struct {
  * Every shift list is validated on the host before any kernel runs (finite, inside
  * the spectral interval).  Environment: FPS_MAX_REFINE_ROUNDS caps the refinement
  * rounds of FP32_REFINE plans (default 8 for squares, 12 for cubes);
- * FPS_INJECT_SHIFT_FAULT=nan|neg corrupts the first shift before validation (host-side
- * fault injection for tests).
+ * FPS_INJECT_SHIFT_FAULT=nan|neg corrupts the first shift before validation and
+ * FPS_INJECT_WAIT_FAULT=1 makes a bounded device wait of the plan's solves give up
+ * (fault injection for tests).
  * Errors: INVALID_ARG (n < 1, dim not 2/3, tol outside (0,1), nrhs < 1, out NULL, a
  * shift list that fails validation), CUDA (allocation or launch failure).  *out is
  * NULL on error.

@@ -221,4 +221,10 @@ void inject_shift_fault(std::vector<double> &q)
     else if (std::string(f) == "neg") q[0] = -q[0];
 }
 
+bool inject_wait_fault()
+{
+    const char *f = std::getenv("FPS_INJECT_WAIT_FAULT");
+    return f && std::string(f) == "1";
+}
+
 }  // namespace fps

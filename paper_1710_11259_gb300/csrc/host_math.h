@@ -42,4 +42,8 @@ bool shifts_valid(const std::vector<double> &q, double lo, double hi);
 // or =neg in the environment the first shift of the list is corrupted.
 void inject_shift_fault(std::vector<double> &q);
 
+// Likewise FPS_INJECT_WAIT_FAULT=1: a bounded device wait of the plan's kernels gives up
+// although what it waits for arrives.
+bool inject_wait_fault();
+
 }  // namespace fps

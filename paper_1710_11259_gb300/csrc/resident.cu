@@ -182,9 +182,10 @@ __global__ void __launch_bounds__(ResGeo<T, S>::kThreads) resident_kernel(ResArg
         to_cs[h] = bulk::peer_smem(cs + cc * G::cpitch + rank, min(gc, C - 1));
         bar_cs[h] = bulk::peer_smem(bar, min(gc, C - 1));
     }
-    bool ok = true;  // false: a wait gave up; the thread runs on without waiting or sending
+    bool ok = true;  // false: a wait gave up; the thread runs on without waiting, sending or arming
+    const int give_up = rank == 0 ? a.give_up : -1;
     auto wait = [&](uint64_t *b, int j) {
-        if (ok && !bulk::mbar_wait_cluster(b, j & 1)) {
+        if (ok && (j == give_up || !bulk::mbar_wait_cluster(b, j & 1))) {
             ok = false;
             *(volatile int *)a.err = 1;
         }
@@ -194,7 +195,9 @@ __global__ void __launch_bounds__(ResGeo<T, S>::kThreads) resident_kernel(ResArg
         const T2 *sums = reinterpret_cast<const T2 *>(tr) + g, *back = reinterpret_cast<const T2 *>(tr + 2 * M) + g;
         const T2 *fwd = reinterpret_cast<const T2 *>(tr + 4 * M) + g;
         const T *kr = tr + res_scan_row(S), *kc = tr + res_record(S), *tc = kc + kScan;
-        if (tid == 0) {
+        // while its waits succeed thread 0 knows that both phases before are complete; a phase
+        // that is not has had its one arrival
+        if (tid == 0 && ok) {
             bulk::mbar_arrive_expect_tx(bar, bytes);
             bulk::mbar_arrive_expect_tx(bar + 1, bytes);
         }
@@ -313,7 +316,8 @@ __global__ void __launch_bounds__(ResGeo<T, S>::kThreads) resident_kernel(ResArg
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
     }
-    // no CTA leaves while a peer whose wait gave up may still have stores under way to it
+    // no CTA leaves while a peer may still have stores under way to it: a CTA whose waits
+    // succeeded has received all of its own
     asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
 #pragma unroll
     for (int h = 0; h < kR; ++h) {
@@ -329,6 +333,9 @@ __global__ void __launch_bounds__(ResGeo<T, S>::kThreads) resident_kernel(ResArg
         }
     }
     asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");
+    // every store is issued by now, but one whose wait gave up has not seen the last ones arrive
+    if (!ok)
+        for (int t = 0; t < 1000; ++t) __nanosleep(1000);
 }
 
 // One thread per (job, parity), FP64 arithmetic; the recurrences of fac_tables_kernel.

@@ -65,6 +65,7 @@ struct ResArgs {
     const double *F;         // caller's right-hand sides and solution: scale-in and -out in the launch
     double *out;
     int *err;                // set if a bounded wait gave up (device or pinned host memory)
+    int give_up;             // fault injection: iteration in which the waits of CTA 0 give up (-1: none)
 };
 
 template <typename T>

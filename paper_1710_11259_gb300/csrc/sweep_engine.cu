@@ -289,6 +289,7 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
         const int v = std::atoi(mr);
         if (v >= 1) max_rounds = v;
     }
+    wait_fault_ = inject_wait_fault();
     res_s_.assign(np, 0);
     streams_ = false;
     for (int p = 0; p < np; ++p) {
@@ -721,6 +722,7 @@ ResArgs<T> SweepEngine<T>::res_args(const ResClass &c, const double *F, double *
     a.out = X;
     // a launch outside the solve that copies err_ back reports to the host's copy itself
     a.err = F ? (int *)(h_stat_ + 2 * npairs_) : err_;
+    a.give_up = wait_fault_ ? 0 : -1;
     return a;
 }
 

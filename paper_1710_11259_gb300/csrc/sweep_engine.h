@@ -134,6 +134,7 @@ private:
     std::vector<int> order_;     // problems, largest first
     std::vector<int> levels_used_;
     bool instrument_ = false;
+    bool wait_fault_ = false;  // fault injection (host_math.h)
     std::vector<void *> allocs_;
 
     template <typename U>
