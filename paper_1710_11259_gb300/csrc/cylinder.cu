@@ -397,16 +397,17 @@ __global__ void __launch_bounds__(CylGeo<H>::kThreads) cyl_resident_kernel(CylRe
 }
 
 // G = F D^{-1} of every unit, [unit][N][N] in the order of place_of, zero beyond the quarter.
+// Units are on grid.x: there are four per (mode, rhs) pair, up to 262140, and grid.y ends at 65535.
 __global__ void __launch_bounds__(256) cyl_quarter_kernel(const double *__restrict__ F, double *__restrict__ G,
                                                           const CylUnit *__restrict__ units, int n, int N)
 {
-    const CylUnit un = units[blockIdx.y];
+    const CylUnit un = units[blockIdx.x];
     const int64_t total = (int64_t)N * N;
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t q = blockIdx.y * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.y * blockDim.x) {
         const int i = 2 * place_of((int)(q / N), N / 2) + un.rp, k = 2 * place_of((int)(q % N), N / 2) + un.cp;
         double v = 0.0;
         if (i < n && k < n) v = -F[un.off + (int64_t)i * n + k] / (((double)k + 1.0) * ((double)k + 2.0));
-        G[blockIdx.y * total + q] = v;
+        G[blockIdx.x * total + q] = v;
     }
 }
 
@@ -964,8 +965,8 @@ int CylinderEngine::solve(const double *F, double *Y, cudaStream_t st, std::stri
     launches_last = 0;
     if (half_) {
         const int N = 2 * half_;
-        const unsigned bx = (unsigned)std::max(1, std::min(N * N / 1024, 16));
-        cyl_quarter_kernel<<<dim3(bx, (unsigned)nunits_), 256, 0, st>>>(F, G_, (const CylUnit *)units_, (int)n, N);
+        const unsigned by = (unsigned)std::max(1, std::min(N * N / 1024, 16));
+        cyl_quarter_kernel<<<dim3((unsigned)nunits_, by), 256, 0, st>>>(F, G_, (const CylUnit *)units_, (int)n, N);
         CYL_CK(cudaGetLastError());
         const CylResArgs a{(int)n, (const CylUnit *)units_, zfac_, rfac_, G_, Y};
         switch (half_) {

@@ -195,3 +195,25 @@ def test_cube_refine_line_lengths(api, n):
         lam[None, :, None] * lam[None, None, :]
     Xd = _along(_along(-F * S, V.T) / L, V) * S
     assert _relmax(X, Xd) <= TOL_REFINE
+
+
+# more than 65535 / 4 (mode, right-hand side) pairs, and the most a plan takes (65535)
+@pytest.mark.parametrize("n,modes,nrhs", [(5, 65, 256), (4, 255, 257)])
+def test_cylinder_many_pairs(api, n, modes, nrhs):
+    """Every pair of a large plan equals the same right-hand side alone in its mode's plan, and
+    the first and the last agree with the dense solve (bar of the small cylinder tests)."""
+    from oracle import cylinder as cyl
+
+    F = inputs.gaussian(n, (modes, nrhs, n, n))
+    plan = api.plan_create_cylinder(n, 2, modes + 1, 1e-13, nrhs)
+    Y = api.poisson_cylinder_solve(plan, torch.from_numpy(F).cuda()).cpu().numpy()
+    api.plan_destroy(plan)
+    one = api.plan_create_cylinder(n, 2, modes + 1, 1e-13, 1)
+    for r in (0, 1, nrhs // 2, nrhs - 1):
+        Fr = torch.from_numpy(np.ascontiguousarray(F[:, r:r + 1])).cuda()
+        assert np.array_equal(api.poisson_cylinder_solve(one, Fr).cpu().numpy()[:, 0], Y[:, r]), r
+    api.plan_destroy(one)
+    for m, r in ((0, 0), (modes - 1, nrhs - 1)):
+        P, Q, _, _ = cyl.mode_operators(n, m + 2)
+        kappa = np.linalg.cond(np.linalg.eig(np.linalg.solve(P, Q))[1])
+        assert _relmax(Y[m, r], cyl.mode_solve_dense(F[m, r], m + 2)) <= 10 * 1e-13 * kappa
