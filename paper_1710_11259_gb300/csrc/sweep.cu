@@ -638,6 +638,98 @@ __global__ void chain_kernel(SwArgs<T> A, int dir, int j)
         }
 }
 
+// The same for lines of more segments than a CTA's registers hold: kWalkWarps warps, each
+// walking its share of the line in steps of kC segments, whose operands are read together.  The summaries
+// are read once more than by chain_kernel, and {zin, y from zin} is left in the results'
+// place between the walk forwards, which also composes the maps of the walk backwards, and
+// that one.  Latency bound as chain_kernel; a solve of n = 16500 in FP64 takes 736 ms and of
+// n = 40000 4.58 s (2.76 times n = 10^4 of chain_kernel for 2.72 times the unknowns, and
+// 17.2 times for 16), FP32 with refinement n = 33000 0.49 s (12.0 times for 10.9).
+template <typename T>
+__global__ void __launch_bounds__(32 * kWalkWarps) chain_walk_kernel(SwArgs<T> A, int dir, int j)
+{
+    using T2 = typename Vec2<T>::type;
+    constexpr int kWarps = kWalkWarps, kC = sizeof(T) == 8 ? 4 : 8;
+    __shared__ T beta[2][kWarps][32];
+    __shared__ T alpha[2][kWarps];
+    pdl_launch();
+    const SwItem<T> it = A.items[blockIdx.x];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int P = it.nb, nbp = round4(P), Mp = P * A.S, run = (P + kWarps - 1) / kWarps;
+    const bool in_range = j < it.J;
+    pdl_wait();
+    if (!in_range || (*A.masked && !A.active[it.prob])) return;
+    const T *co = (dir == 0 ? it.chR : it.chC) + (int64_t)j * 6 * nbp;
+    const int64_t line = it.soff + it.b1 * 32 + lane;
+    const T2 *__restrict__ sum = (dir == 0 ? A.sumR : A.sumC) + line;
+    T2 *zx = (dir == 0 ? A.zxR : A.zxC) + line;
+    const int s0 = min(g * run, P), s1 = min(s0 + run, P);
+    T al = 1, be = 0;
+    for (int s = s0; s < s1; s += kC) {
+        T phi[kC], w[kC];
+#pragma unroll
+        for (int b = 0; b < kC; ++b) {
+            const bool ok = s + b < s1;
+            phi[b] = ok ? co[s + b] : T(1);
+            w[b] = ok ? sum[(int64_t)(s + b) * Mp].x : T(0);
+        }
+#pragma unroll
+        for (int b = 0; b < kC; ++b) {
+            be = fma(phi[b], be, w[b]);
+            al *= phi[b];
+        }
+    }
+    beta[0][g][lane] = be;
+    if (lane == 0) alpha[0][g] = al;
+    __syncthreads();
+    T W = 0;
+    for (int h = 0; h < g; ++h) W = fma(alpha[0][h], W, beta[0][h][lane]);
+    al = 1;
+    be = 0;
+    for (int s = s0; s < s1; s += kC) {
+        T phi[kC], bv[kC], ps[kC];
+        T2 v[kC];
+#pragma unroll
+        for (int b = 0; b < kC; ++b)
+            if (s + b < s1) {
+                phi[b] = co[s + b];
+                bv[b] = co[nbp + s + b];
+                ps[b] = co[2 * nbp + s + b];
+                v[b] = sum[(int64_t)(s + b) * Mp];
+            }
+#pragma unroll
+        for (int b = 0; b < kC; ++b)
+            if (s + b < s1) {
+                const T y = fma(bv[b], W, v[b].y);
+                zx[(int64_t)(s + b) * Mp] = mk2<T>(W, y);
+                be = fma(al, y, be);
+                al *= ps[b];
+                W = fma(phi[b], W, v[b].x);
+            }
+    }
+    beta[1][g][lane] = be;
+    if (lane == 0) alpha[1][g] = al;
+    __syncthreads();
+    T Y = 0;
+    for (int h = kWarps - 1; h > g; --h) Y = fma(alpha[1][h], Y, beta[1][h][lane]);
+    for (int s = s1 - 1; s >= s0; s -= kC) {
+        T ps[kC];
+        T2 v[kC];
+#pragma unroll
+        for (int b = 0; b < kC; ++b)
+            if (s - b >= s0) {
+                ps[b] = co[2 * nbp + s - b];
+                v[b] = zx[(int64_t)(s - b) * Mp];
+            }
+#pragma unroll
+        for (int b = 0; b < kC; ++b)
+            if (s - b >= s0) {
+                zx[(int64_t)(s - b) * Mp] = mk2<T>(v[b].x, Y);
+                Y = fma(ps[b], Y, v[b].y);
+            }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Elementwise kernels.  GB300's FP64 pipe takes 64 cycles of an SM quadrant per warp
 // instruction, conversions and comparisons included (and 64-bit integer comparisons
@@ -1090,6 +1182,15 @@ cudaError_t sweep_setup_kernels()
     cudaError_t e = setup_S<float, 32>();
     if (e == cudaSuccess) e = setup_S<float, 64>();
     if (e == cudaSuccess) e = setup_S<double, 32>();
+    // the registers of the chain kernels admit the launches of chain_length
+    auto admits = [&](auto *k, int warps) {
+        cudaFuncAttributes at;
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, k);
+        if (e == cudaSuccess && at.maxThreadsPerBlock < 32 * warps) e = cudaErrorInvalidConfiguration;
+    };
+    admits(chain_kernel<float, 8>, chain_warps(false, 8));
+    admits(chain_kernel<float, 16>, chain_warps(false, 16));
+    admits(chain_kernel<double, 8>, chain_warps(true, 8));
     return e;
 }
 
@@ -1139,11 +1240,15 @@ cudaError_t launch_col_pass(const SwArgs<T> &a, int j, cudaStream_t st)
 template <typename T>
 cudaError_t launch_chain(const SwArgs<T> &a, int dir, int j, cudaStream_t st)
 {
-    const unsigned warps = (unsigned)((a.max_nb + a.chain_len - 1) / a.chain_len), grid = (unsigned)a.nitems;
-    if (warps > 32) return cudaErrorInvalidValue;
+    constexpr bool kFP64 = sizeof(T) == 8;
+    const unsigned grid = (unsigned)a.nitems;
+    if (a.chain_len == 0) return launch_pdl(chain_walk_kernel<T>, grid, 32 * kWalkWarps, 0, st, a, dir, j);
+    const int warps = (a.max_nb + a.chain_len - 1) / a.chain_len;
+    if (warps > chain_warps(kFP64, a.chain_len)) return cudaErrorInvalidValue;
     if (a.chain_len == 8) return launch_pdl(chain_kernel<T, 8>, grid, 32 * warps, 0, st, a, dir, j);
-    if (a.chain_len == 16) return launch_pdl(chain_kernel<T, 16>, grid, 32 * warps, 0, st, a, dir, j);
-    if (a.chain_len == 24) return launch_pdl(chain_kernel<T, 24>, grid, 32 * warps, 0, st, a, dir, j);
+    if constexpr (!kFP64) {
+        if (a.chain_len == 16) return launch_pdl(chain_kernel<T, 16>, grid, 32 * warps, 0, st, a, dir, j);
+    }
     return cudaErrorInvalidValue;
 }
 

@@ -115,7 +115,7 @@ struct SwArgs {
     int *err;              // device error word: bit 0 = a bounded wait gave up
     int S;                 // block and segment size of every problem (sweep_segment_supported(., 2 S))
     int fused;             // passes run the segment recurrence themselves (sweep_fused)
-    int chain_len;         // chain kernel: segments per thread
+    int chain_len;         // chain kernel: segments per thread (chain_length)
     int max_nb;
 };
 
@@ -158,6 +158,23 @@ cudaError_t sweep_setup_kernels();
 // with fuller waves) and 4 in FP64 (n <= 1024), where the operations come on top of a bound
 // FP64 pipe.
 bool sweep_fused(bool fp64, int S, int nb);
+// Warps that a chain launch with `len` segments per thread can have: the segments are in
+// registers, 64 a thread (len 8) and 96 (len 16) in FP32, 96 (len 8) in FP64
+// (sweep_setup_kernels checks it).
+constexpr int chain_warps(bool fp64, int len)
+{
+    return fp64 ? (len == 8 ? 20 : 0) : (len == 8 ? 32 : (len == 16 ? 20 : 0));
+}
+// Segments per thread of the chain launches over lines of up to `nb` segments, in registers:
+// 8, or 16 where FP32 prefers it (mode 2) or needs it; 0 where no such launch covers a line
+// (FP64 n > 10240, FP32 n > 20480 in blocks of 32): its threads walk over as many as it takes.
+constexpr int chain_length(bool fp64, int mode, int nb)
+{
+    if (mode != 2 && nb <= 8 * chain_warps(fp64, 8)) return 8;
+    if (nb <= 16 * chain_warps(fp64, 16)) return 16;
+    return nb <= 8 * chain_warps(fp64, 8) ? 8 : 0;
+}
+constexpr int kWalkWarps = 16;
 // Segment lengths (unknowns of both parities) with compiled pass kernels: 64 (FP32, FP64)
 // and 128 (FP32), i.e. blocks of 32 and 64.
 bool sweep_segment_supported(bool fp64, int seg);

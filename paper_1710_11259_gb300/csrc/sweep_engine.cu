@@ -133,15 +133,6 @@ std::string tune_cache_path()
 // Entries per segment-coefficient array: 16-byte multiples for the bulk copies.
 static int nbp_of(int nb) { return (nb + 3) & ~3; }
 
-// Segments per thread of the chain kernel: short or long runs (the autotuner's choice),
-// longer where a line has more segments than 32 warps of short runs cover.
-static int chain_len_of(int mode, int max_nb)
-{
-    int len = mode == 2 ? 16 : 8;
-    while (len < 24 && (max_nb + len - 1) / len > 32) len += 8;
-    return len;
-}
-
 template <typename T>
 TileArgs SweepEngine<T>::tiles(int which) const
 {
@@ -192,7 +183,7 @@ int SweepEngine<T>::time_chain(int mode, float &ms, std::string &err)
     SwArgs<T> a = args(levels_.back(), 2);
     ms = 0.f;
     if (a.fused) return FPS_OK;
-    a.chain_len = chain_len_of(mode, max_nb_);
+    a.chain_len = chain_length(sizeof(T) == 8, mode, max_nb_);
     cudaEvent_t e0, e1;
     ENG_CK(cudaEventCreate(&e0));
     ENG_CK(cudaEventCreate(&e1));
@@ -743,7 +734,7 @@ SwArgs<T> SweepEngine<T>::args(const Level &L, int which) const
     a.err = err_;
     a.S = seg_len / 2;
     a.fused = fused_ ? 1 : 0;
-    a.chain_len = chain_len_of(chain_mode, max_nb_);
+    a.chain_len = chain_length(sizeof(T) == 8, chain_mode, max_nb_);
     a.max_nb = max_nb_;
     return a;
 }
