@@ -64,7 +64,8 @@ typedef enum {
     FPS_ERR_CUDA = -3,          /* a CUDA runtime call or launch failed */
     FPS_ERR_NOT_CONVERGED = -4, /* refinement missed its target; X holds the best iterate */
     FPS_ERR_NONFINITE = -5,     /* F (or an intermediate) holds NaN/Inf */
-    FPS_ERR_TIMEOUT = -6        /* a bounded device-side wait gave up */
+    FPS_ERR_TIMEOUT = -6        /* a bounded device-side wait gave up (square plans; see
+                                   fps_poisson_square_solve) */
 } fps_status;
 
 /* Read-only facts about a plan. */
@@ -153,7 +154,12 @@ int fps_plan_set_stream(fps_plan *plan, void *stream);
  * X = D_s Y D_s (the recovery consistent with the printed right-hand side of (3.9)).
  * Errors: INVALID_ARG (plan NULL or not dim 2, F/X NULL or overlapping, F/X device
  * memory of another device), NONFINITE (FP32_REFINE: F holds NaN/Inf), NOT_CONVERGED (FP32_REFINE missed tol),
- * CUDA.
+ * TIMEOUT, CUDA.
+ * TIMEOUT: a bounded wait inside a kernel gave up, and X is not the solution.  FP32_REFINE
+ * solves and solves with a host buffer report it themselves.  An FP64 solve on device
+ * buffers has returned by then: the plan's next solve that is called after the stream has
+ * finished reports it, before it launches anything.  The state stays with the plan, whose
+ * later solves all return TIMEOUT; the device stays usable.
  */
 int fps_poisson_square_solve(fps_plan *plan, const double *F, double *X);
 

@@ -176,6 +176,8 @@ int solve_engine(fps_plan *p, E *eng, const double *F, double *X, bool fdev, boo
     } else if (!fdev) {
         FPS_CK(cudaStreamSynchronize(p->stream));  // host F must stay valid only until copied
     }
+    if (!(xdev && fdev) && eng->timed_out())
+        return fail(FPS_ERR_TIMEOUT, std::string(what) + ": a bounded device wait gave up (data not arrived)");
     if (st != FPS_OK) return fail(st, std::string(what) + ": " + err);
     FPS_CK(cudaGetLastError());
     return FPS_OK;

@@ -44,6 +44,7 @@ double bits_to_double(unsigned long long b)
     return d;
 }
 const double kLevelTols[] = {1e-7, 1e-6, 1e-5, 1e-4, 1e-3, 1e-2};
+const char kGaveUp[] = "a bounded device wait gave up (data not arrived)";
 }  // namespace
 
 template <typename T>
@@ -361,6 +362,7 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     ENG_CK(cudaMemsetAsync(sumR_, 0, sizeof(T2) * (size_t)totS_, cap_));
     ENG_CK(cudaMemsetAsync(sumC_, 0, sizeof(T2) * (size_t)totS_, cap_));
     ENG_CK(cudaMemsetAsync(d_stat_, 0, sizeof(unsigned long long) * (2 * (size_t)npairs_ + 1), cap_));
+    if (wait_fault_ && streams_) ENG_CK(cudaMemsetAsync(err_, 1, 1, cap_));  // as if a pass had given up
 
     // bands: FP64 (d, e zero-padded, 1/sqrt(E), then {-kx d, -ky d} and {-kx e, -ky e})
     std::vector<double> hb64((size_t)totB64);
@@ -838,6 +840,10 @@ int SweepEngine<T>::solve(const double *F, double *X, cudaStream_t st, std::stri
 {
     launches_last = 0;
     levels_used_.clear();
+    if (timed_out()) {  // an FP64 solve on device buffers returned before its waits ended
+        err = kGaveUp;
+        return FPS_ERR_TIMEOUT;
+    }
     return sizeof(T) == 8 ? solve_plain(F, X, st, err) : solve_refine(F, X, st, err);
 }
 
@@ -915,7 +921,7 @@ int SweepEngine<T>::solve_refine(const double *F, double *X, cudaStream_t st, st
                                    cudaMemcpyDeviceToHost, st));
             ENG_CK(cudaStreamSynchronize(st));
             if (timed_out()) {
-                err = "a bounded device wait gave up (tile copy not completed)";
+                err = kGaveUp;
                 return FPS_ERR_TIMEOUT;
             }
             if (round == 0) {
@@ -994,7 +1000,7 @@ int SweepEngine<T>::kernel_times(int *count, double *total_ms, double *alg_bytes
                                  std::string &err)
 {
     if (timed_out()) {
-        err = "a bounded device wait gave up (tile copy not completed)";
+        err = kGaveUp;
         return FPS_ERR_TIMEOUT;
     }
     int c = 0;

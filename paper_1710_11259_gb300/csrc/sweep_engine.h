@@ -34,6 +34,10 @@ public:
     // FPS_ERR_NOT_CONVERGED with the last iterate in X when the refinement misses tol.
     int solve(const double *F, double *X, cudaStream_t st, std::string &err);
 
+    // Whether a bounded device wait of a finished solve gave up.  Nothing clears it: the
+    // plan's later solves return FPS_ERR_TIMEOUT.
+    bool timed_out() const { return h_stat_ && (unsigned)*(volatile unsigned long long *)(h_stat_ + 2 * npairs_) != 0; }
+
     int set_instrument(bool on, std::string &err);
     // ADI pass kernels (row and column passes) of the last solve: launches, summed
     // duration, and the bytes they must move (6 words per element and iteration: u, a and
@@ -128,7 +132,6 @@ private:
     int *d_active_ = nullptr, *d_pair_active_ = nullptr;
     int *h_active_ = nullptr, *h_pair_active_ = nullptr;
     unsigned long long *d_stat_ = nullptr, *h_stat_ = nullptr;  // rmax, smax [npairs], error word
-    bool timed_out() const { return h_stat_ && (unsigned)h_stat_[2 * npairs_] != 0; }
     std::vector<Level> levels_;
     std::vector<int64_t> ob64_;  // offset of each problem's bands in bands64_
     std::vector<int> order_;     // problems, largest first
