@@ -212,7 +212,10 @@ int fps_plan_shifts(const fps_plan *plan, int64_t problem, double *q, int cap);
  * the plan's ADI pass kernels (the row pass and the column pass of every
  * iteration of Algorithm 2), inside the captured graphs, so that their duration
  * can be read after a solve without changing what runs.  Rebuilds the graphs.
- * Square plans only.  Errors: INVALID_ARG, UNSUPPORTED (cube plan), CUDA.
+ * Problems that are solved in one launch (FP64 n <= 512, FP32_REFINE n <= 1024) have no
+ * pass kernels: nothing of theirs is timed, and a plan of such problems alone reports
+ * zero launches, time and bytes.  Square plans only.  Errors: INVALID_ARG, UNSUPPORTED
+ * (cube plan, FP64 square with n <= 64), CUDA.
  */
 int fps_plan_set_instrument(fps_plan *plan, int on);
 
@@ -223,7 +226,9 @@ int fps_plan_set_instrument(fps_plan *plan, int on);
  * element and iteration the residual-form ADI reads and writes six n x n words --
  * the row pass reads u and writes a, the column pass reads a and D and writes u and
  * D -- five in the first and in the last iteration; 8 bytes per FP64 and 4 per FP32
- * word; no padding, segment-summary or re-read traffic).  Synchronises the plan's stream.
+ * word; no padding, segment-summary or re-read traffic).  In a batch the problems that
+ * are solved in one launch run beside the passes and count in none of the three.
+ * Synchronises the plan's stream.
  * Errors: INVALID_ARG (not instrumented), TIMEOUT (a bounded device wait gave up), CUDA.
  */
 int fps_plan_kernel_times(fps_plan *plan, int *count, double *total_ms, double *alg_bytes);

@@ -102,7 +102,8 @@ struct fps_plan {
     // square: the ADI pass engine (FP32 sweeps + FP64 refinement, or plain FP64)
     fps::SweepEngine<float> *eng32 = nullptr;
     fps::SweepEngine<double> *eng64 = nullptr;
-    // FP64 squares with n <= 64 are never streamed: no segment length, no pass timing
+    // FP64 square with n <= 64: reports no segment length and refuses pass timing, as such plans
+    // always have (like all FP64 plans with n <= 512 they run in one launch)
     bool small = false;
     // dim = 3: the nested cube ADI
     fps::CubeEngine *cube = nullptr;

@@ -795,7 +795,7 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
     if (!side_.empty() && !fork_) ENG_CK(cudaEventCreateWithFlags(&fork_, cudaEventDisableTiming));
     ENG_CK(cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    const bool ins = instrument_ && (int)L.ev.size() == 4 * L.Jstream + 2;
+    const bool ins = instrument_ && (int)L.ev.size() == 4 * L.Jstream;
     auto rec = [&](int k) {
         if (ins && e == cudaSuccess) e = cudaEventRecordWithFlags(L.ev[k], cap_, cudaEventRecordExternal);
     };
@@ -804,11 +804,7 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
         if (e == cudaSuccess) e = r;
         ++L.launches;
     };
-    rec(4 * L.Jstream);
-    if (ins)
-        for (const ResClass &c : L.res) run(launch_resident<T>(res_args(c, nullptr, nullptr), cap_));
-    else if (e == cudaSuccess) e = run_resident(L, nullptr, nullptr, cap_, streams_, L.launches);
-    rec(4 * L.Jstream + 1);
+    e = run_resident(L, nullptr, nullptr, cap_, streams_, L.launches);
     if (streams_) run(launch_row_sums<T>(ac, cap_));
     for (int j = 0; j < L.Jstream && e == cudaSuccess; ++j) {
         if (!fused_) run(launch_chain<T>(ach, 0, j, cap_));
@@ -820,7 +816,7 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
         run(launch_col_pass<T>(ac, j, cap_));
         rec(4 * j + 3);
     }
-    if (!ins && e == cudaSuccess) e = join_resident(cap_);
+    if (e == cudaSuccess) e = join_resident(cap_);
     cudaGraph_t g = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(cap_, &g);
     if (e != cudaSuccess) {
@@ -851,7 +847,7 @@ template <typename T>
 int SweepEngine<T>::solve_plain(const double *F, double *X, cudaStream_t st, std::string &err)
 {
     if constexpr (sizeof(T) == 8) {
-        if (!streams_ && !instrument_) {  // scale-in, all iterations and scale-out in one launch per class
+        if (!streams_) {  // scale-in, all iterations and scale-out in one launch per class
             ENG_CK(run_resident(levels_[0], F, X, st, false, launches_last));
             ENG_CK(join_resident(st));
             levels_used_.push_back(0);
@@ -986,7 +982,7 @@ int SweepEngine<T>::set_instrument(bool on, std::string &err)
         for (cudaEvent_t e : L.ev) cudaEventDestroy(e);
         L.ev.clear();
         if (on) {
-            L.ev.resize(4 * (size_t)L.Jstream + 2);
+            L.ev.resize(4 * (size_t)L.Jstream);
             for (auto &e : L.ev) ENG_CK(cudaEventCreate(&e));
         }
         int st = build_graph(L, err);
@@ -1010,26 +1006,18 @@ int SweepEngine<T>::kernel_times(int *count, double *total_ms, double *alg_bytes
         if (std::find(seen.begin(), seen.end(), li) != seen.end()) continue;
         seen.push_back(li);
         const Level &L = levels_[li];
-        if ((int)L.ev.size() != 4 * L.Jstream + 2) continue;
-        if (!L.res.empty()) {  // the resident launches alternate row and column solves
-            float t = 0.f;
-            ENG_CK(cudaEventElapsedTime(&t, L.ev[4 * L.Jstream], L.ev[4 * L.Jstream + 1]));
-            rms += 0.5 * t;
-            cms += 0.5 * t;
-        }
-        for (int j = 0; j < L.Jmax; ++j) {
+        if ((int)L.ev.size() != 4 * L.Jstream) continue;
+        for (int j = 0; j < L.Jstream; ++j) {
             float t0 = 0.f, t1 = 0.f;
-            if (j < L.Jstream) {
             ENG_CK(cudaEventElapsedTime(&t0, L.ev[4 * j], L.ev[4 * j + 1]));
             ENG_CK(cudaEventElapsedTime(&t1, L.ev[4 * j + 2], L.ev[4 * j + 3]));
-            }
             rms += t0;
             cms += t1;
             c += 2;
             // row pass: u read, a written; column pass: a read, u written (but for the last
             // iteration of a problem), D written and, after the first iteration, read
             for (size_t p = 0; p < ns_.size(); ++p)
-                if (j < L.J[p])
+                if (!res_s_[p] && j < L.J[p])
                     by += (4.0 + (j > 0 ? 1.0 : 0.0) + (j + 1 < L.J[p] ? 1.0 : 0.0)) * sizeof(T) * (double)nrhs_ *
                           (double)ns_[p] * (double)ns_[p];
         }

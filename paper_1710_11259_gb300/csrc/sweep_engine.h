@@ -41,7 +41,7 @@ public:
     int set_instrument(bool on, std::string &err);
     // ADI pass kernels (row and column passes) of the last solve: launches, summed
     // duration, and the bytes they must move (6 words per element and iteration: u, a and
-    // D read and written once; 5 in the first and the last).
+    // D read and written once; 5 in the first and the last).  Resident problems have none.
     int kernel_times(int *count, double *total_ms, double *alg_bytes, double *row_ms, double *col_ms,
                      std::string &err);
 
@@ -77,7 +77,7 @@ private:
         std::vector<ResClass> res;
         int64_t launches = 0;             // kernels of the graph
         cudaGraphExec_t graph = nullptr;
-        std::vector<cudaEvent_t> ev;  // when instrumented: 4 per iteration, 2 around the resident launches
+        std::vector<cudaEvent_t> ev;  // when instrumented: 4 per iteration of the passes
     };
     int build_graph(Level &L, std::string &err);
     int autotune(const std::vector<int64_t> &ns, int nrhs, double tol, bool tight, std::string &err);
