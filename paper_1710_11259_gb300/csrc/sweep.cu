@@ -756,27 +756,32 @@ struct MaxBits {
     __device__ __forceinline__ double value() const { return __hiloint2double((int)hi, (int)lo); }
 };
 
-// (double)f, subnormal floats read as zero.
+// Conversions of subnormal floats are rare and left to the FP64 pipe, out of line.
+__device__ __noinline__ double widen_subnormal(float f) { return (double)f; }
+__device__ __noinline__ float narrow_subnormal(double x, int k) { return (float)scalbn(x, -k); }
+
+// (double)f
 __device__ __forceinline__ double widen(float f)
 {
     const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+    if (a - 1u < 0x007fffffu) return widen_subnormal(f);
     unsigned hi = (a >> 3) + 0x38000000u;
     if (a >= 0x7f800000u) hi |= 0x7ff00000u;  // Inf, NaN
-    if (a < 0x00800000u) hi = 0u;
-    return __hiloint2double((int)(hi | (u & 0x80000000u)), a < 0x00800000u ? 0 : (int)(u << 29));
+    if (a == 0u) hi = 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
 
 // x 2^54 where the scale is so small that subnormal doubles count (k is raised to match);
 // kept out of line, so that the product is not executed speculatively.
 __device__ __noinline__ double lift_subnormal(double x) { return x * 18014398509481984.0; }
 
-// (float)(x 2^-k), rounded to nearest even, -896 <= k; below the normal range zero, above
-// it Inf.
+// (float)(x 2^-k), rounded to nearest even, -896 <= k; above the range Inf.
 __device__ __forceinline__ float narrow_scaled(double x, int k)
 {
     const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu, lo = (unsigned)__double2loint(x);
     const unsigned sign = (unsigned)__double2hiint(x) & 0x80000000u;
     const int e = (int)(h >> 20) - 896 - k;  // exponent field of the float
+    if (e <= 0 && (h | lo)) return narrow_subnormal(x, k);
     unsigned f = ((h - ((unsigned)(896 + k) << 20)) << 3) | (lo >> 29);
     const unsigned rest = lo << 3;
     f += rest > 0x80000000u || (rest == 0x80000000u && (f & 1u)) ? 1u : 0u;

@@ -217,3 +217,27 @@ def test_cylinder_many_pairs(api, n, modes, nrhs):
         P, Q, _, _ = cyl.mode_operators(n, m + 2)
         kappa = np.linalg.cond(np.linalg.eig(np.linalg.solve(P, Q))[1])
         assert _relmax(Y[m, r], cyl.mode_solve_dense(F[m, r], m + 2)) <= 10 * 1e-13 * kappa
+
+
+@pytest.mark.parametrize("n", [65, 1100])
+@pytest.mark.parametrize("k", [0, -1000])
+def test_refine_keeps_subnormal_quarters(api, n, k):
+    """Parity quarters do not couple, so one whose scaled right-hand side is below FP32's normal
+    range still gets its own solution: to 1e-3, from values held to 2^-149 (22 bits at the
+    largest, about 40 iterations) and one round at 1e-6 or finer."""
+    F = inputs.square_rhs(n, 3)
+    s = 1.0 / np.sqrt((np.arange(n) + 1.0) * (np.arange(n) + 2.0))
+    scaled = np.abs(F * s[:, None] * s[None])
+    own = scaled[1::2, 1::2].max()
+    scaled[1::2, 1::2] = 0.0
+    e = int(np.floor(np.log2(scaled.max())) - np.floor(np.log2(own))) - 128  # largest in [2^-128, 2^-127) units
+    small = np.zeros_like(F)
+    small[1::2, 1::2] = F[1::2, 1::2]
+    G = F - small + np.ldexp(small, e)
+    plan = api.plan_create(n, 2, 1e-10, "fp32_refine")
+    X = api.poisson_square_solve(plan, torch.from_numpy(np.ldexp(G, k)).cuda()).cpu().numpy()
+    api.plan_destroy(plan)
+    got, want = np.ldexp(X, -k), oracle.poisson_square(small, 1e-13)
+    if k == 0:
+        assert _relmax(np.ldexp(got[1::2, 1::2], -e), want[1::2, 1::2]) <= 1e-3
+    assert _relmax(got, oracle.poisson_square(G, 1e-13)) <= TOL_REFINE
