@@ -89,10 +89,12 @@ typedef struct {
                                autotuner unless FPS_AUTOTUNE=0 */
     int64_t inner_iterations; /* cube: inner (slice Stein) ADI iterations over full
                                  tensors in the last solve, all levels and rounds */
-    int chain_mode;         /* square plans: load batching of the segment-coupling kernel
-                               (1 short, 2 long batches; FP32_REFINE: picked by the autotuner
-                               with seg_len, 0 = short when it did not run; plans of at most 16
-                               segments per line launch no such kernel) */
+    int chain_mode;         /* square plans: segments per thread of the segment-coupling kernel
+                               (1 eight, 2 sixteen; FP32_REFINE: picked by the autotuner with
+                               seg_len, 0 = eight when it did not run).  Problems up to n = 1024
+                               (FP64) and 2048 (FP32_REFINE) launch no such kernel, and lines too
+                               long for its registers take one whose threads walk (FP64 from
+                               n = 10241, FP32_REFINE with seg_len 64 from n = 20481) */
 } fps_plan_info_t;
 
 /*

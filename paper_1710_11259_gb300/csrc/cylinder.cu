@@ -417,7 +417,7 @@ constexpr int kCylThreads = 256;  // threads per CTA: all move the tile, the fir
 constexpr int kZ = 3, kR = 8;  // table entries per position: z l, m, g; r l1, l2, n1, n2, a, b, c, 1/pivot
 
 struct CylArgs {
-    int n, nrhs, Jmax, j;
+    int n, nrhs, j;
     const double *zfac, *rfac;  // [sum J][n][kZ], [sum J][n][kR]
     const int *joff, *jcount;
     const double *G;       // [modes][nrhs][n][n]
@@ -983,7 +983,6 @@ int CylinderEngine::solve(const double *F, double *Y, cudaStream_t st, std::stri
     CylArgs A;
     A.n = (int)n;
     A.nrhs = nrhs;
-    A.Jmax = Jmax;
     A.zfac = zfac_;
     A.rfac = rfac_;
     A.joff = joff_;

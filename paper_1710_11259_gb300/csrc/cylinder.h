@@ -28,8 +28,6 @@ double cyl_L1(int64_t a, int64_t i);  // L1[a][i] (zero unless |a - i| in {0, 2}
 // n x n blocks, by power iteration on A_k and on A_k^{-1} per parity, widened by 3 %.
 int cyl_mode_interval(int64_t n, int64_t k, double &a, double &b);
 
-struct CylTables;
-
 class CylinderEngine {
 public:
     int create(int64_t n, int64_t kmin, int64_t kmax, double tol, int nrhs, std::string &err);

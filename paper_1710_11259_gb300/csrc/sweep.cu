@@ -83,8 +83,10 @@ struct Geo {
     static constexpr size_t col_bytes = off_tile + 2 * tile_bytes + sizeof(T) * tab_elems;
     static constexpr size_t sum_bytes = row_bytes;
     // Resident CTAs per SM that the registers are limited for.  Blocks of 32 in FP32 serve
-    // n = 1025 .. 2048, about one wave of tiles: with 6 and 5 resident CTAs (no limit) a nearly
-    // empty second wave cost n = 2048 5 % of the solve.
+    // n = 1025 .. 2048, about one wave of tiles: 7 per SM hold the 1024 tiles of n = 2048 of the
+    // row pass at once, 6 (what shared memory admits) those of the column pass up to n = 1792;
+    // above, up to 112 of its tiles are a second wave.  Without the limits (6 and 5) n = 2048
+    // took 5 % longer.
     static constexpr int row_ctas = sizeof(T) == 8 ? 3 : (S == 32 ? 7 : 4);
     static constexpr int col_ctas = sizeof(T) == 4 && S == 32 ? 6 : 3;
     static_assert(CH >= 8, "the XOR permutation needs eight chunks per row");
@@ -1149,7 +1151,8 @@ cudaError_t col_pass_S(const SwArgs<T> &a, int j, cudaStream_t st)
     return launch_pdl(col_pass_kernel<T, S, false, false>, grid, kL, sm, st, a, j);
 }
 
-// CTAs of a reduction kernel: 8 per SM (all resident), at most one per tile.
+// CTAs of a reduction kernel: 8 per SM, at most one per tile.  The registers admit 4 (maximum)
+// and 3 (residual) of them at a time.
 unsigned reduction_grid(int64_t ntiles)
 {
     const int64_t g = 8 * (int64_t)current_sm_count();

@@ -518,7 +518,6 @@ int SweepEngine<T>::build_tables(Level &L, int level, const std::vector<double> 
     int nq = 0, nq_res = 0;               // shifts of the streamed and of the resident problems
     for (int p = 0; p < np; ++p) {
         L.J[p] = adi_iterations(-kx_ * hi[p], -kx_ * lo[p], ky_ * lo[p], ky_ * hi[p], L.tol);
-        L.Jmax = std::max(L.Jmax, L.J[p]);
         if (res_s_[p]) {
             nres += (int64_t)L.J[p] * 2 * res_record(res_s_[p]);
             nq_res += L.J[p];

@@ -13,7 +13,7 @@
 namespace fps {
 
 // T = float: FP32 sweeps inside an FP64 iterative refinement (tolerance levels,
-//            residual R~ = F~ - A~Y - YA~ in FP64, Y += max|R~| D).
+//            residual R~ = F~ - A~Y - YA~ in FP64, Y -= s D / ky with s a power of two).
 // T = double: the plain FP64 method, J iterations of (2.9) at the plan's tolerance.
 template <typename T>
 class SweepEngine {
@@ -53,7 +53,7 @@ public:
     int max_rounds = 8;
     std::vector<std::vector<double>> shifts;  // level-0 shifts per problem
     int seg_len = 0;                          // segment length in use
-    int chain_mode = 0;                       // chain kernel load batching (SwArgs::chain_mode)
+    int chain_mode = 0;                       // segments per thread of the chain kernel (chain_length)
     std::vector<float> tune_ms;               // autotuner timings per candidate (ms), if it ran
     int64_t total_elems() const { return tot64_; }
 
@@ -68,7 +68,7 @@ private:
     };
     struct Level {
         double tol = 0;
-        int Jmax = 0, Jstream = 0;  // largest J of all and of the streamed problems
+        int Jstream = 0;  // largest J of the streamed problems
         std::vector<int> J;
         T *tab = nullptr, *ch = nullptr;  // solve and summary tables, segment coefficients: rows, then columns
         T *res_tab = nullptr;             // records of the resident problems, likewise
