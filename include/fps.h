@@ -214,9 +214,9 @@ int fps_plan_shifts(const fps_plan *plan, int64_t problem, double *q, int cap);
  * the plan's ADI pass kernels (the row pass and the column pass of every
  * iteration of Algorithm 2), inside the captured graphs, so that their duration
  * can be read after a solve without changing what runs.  Rebuilds the graphs.
- * Problems that are solved in one launch (FP64 n <= 512, FP32_REFINE n <= 1024) have no
- * pass kernels: nothing of theirs is timed, and a plan of such problems alone reports
- * zero launches, time and bytes.  Square plans only.  Errors: INVALID_ARG, UNSUPPORTED
+ * Problems that are solved in one launch (FP32_REFINE n <= 1024; FP64 n <= 512, n <= 768
+ * for one right-hand side) have no pass kernels: nothing of theirs is timed, and a plan
+ * of such problems alone reports zero launches, time and bytes.  Square plans only.  Errors: INVALID_ARG, UNSUPPORTED
  * (cube plan, FP64 square with n <= 64), CUDA.
  */
 int fps_plan_set_instrument(fps_plan *plan, int on);

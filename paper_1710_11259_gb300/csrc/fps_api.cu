@@ -103,7 +103,7 @@ struct fps_plan {
     fps::SweepEngine<float> *eng32 = nullptr;
     fps::SweepEngine<double> *eng64 = nullptr;
     // FP64 square with n <= 64: reports no segment length and refuses pass timing, as such plans
-    // always have (like all FP64 plans with n <= 512 they run in one launch)
+    // always have (like all FP64 plans up to n = 512 they run in one launch)
     bool small = false;
     // dim = 3: the nested cube ADI
     fps::CubeEngine *cube = nullptr;

@@ -439,19 +439,19 @@ cudaLaunchConfig_t config_of(int64_t nitems, int C, cudaLaunchAttribute *at, cud
 }
 
 template <typename T, int S>
-cudaError_t setup_S(int C, bool *fits)
+cudaError_t setup_S(int C, int *side_by_side)
 {
-    *fits = false;
+    *side_by_side = 0;
     cudaError_t e = cudaFuncSetAttribute(resident_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)ResGeo<T, S>::bytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(resident_kernel<T, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = config_of<T, S>(1, C, at, nullptr);
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, resident_kernel<T, S>, &cfg) != cudaSuccess)
+    if (cudaOccupancyMaxActiveClusters(side_by_side, resident_kernel<T, S>, &cfg) != cudaSuccess) {
         cudaGetLastError();  // no such cluster on this device: the passes stream the problem
-    *fits = clusters >= 1;
+        *side_by_side = 0;
+    }
     return cudaSuccess;
 }
 
@@ -465,24 +465,24 @@ cudaError_t launch_S(const ResArgs<T> &a, cudaStream_t st)
 
 }  // namespace
 
-// Compiled segment lengths; FP64 stops at 16 (three arrays of S doubles per thread are
-// registers, and beyond 512 unknowns the passes on all SMs are faster).
-#define RES_SIZES_64(X) X(1) X(2) X(3) X(4) X(5) X(6) X(8) X(10) X(12) X(14) X(16)
-#define RES_SIZES_32(X) RES_SIZES_64(X) X(20) X(24) X(28) X(32)
+// Compiled segment lengths; FP64 stops at 24 (three arrays of S doubles per thread are
+// registers: 168 a thread there, spills beyond).
+#define RES_SIZES_64(X) X(1) X(2) X(3) X(4) X(5) X(6) X(8) X(10) X(12) X(14) X(16) X(20) X(24)
+#define RES_SIZES_32(X) RES_SIZES_64(X) X(28) X(32)
 
 int resident_segment(bool fp64, int m)
 {
-#define TRY(s) if (m <= kG * s && !(fp64 && s > 16)) return s;
+#define TRY(s) if (m <= kG * s && !(fp64 && s > 24)) return s;
     RES_SIZES_32(TRY)
 #undef TRY
     return 0;
 }
 
-#define CASE_SETUP(s) case s: return setup_S<T, s>(C, fits);
+#define CASE_SETUP(s) case s: return setup_S<T, s>(C, side_by_side);
 #define CASE_LAUNCH(s) case s: return launch_S<T, s>(a, st);
 
 template <typename T>
-cudaError_t resident_setup(int S, int C, bool *fits)
+cudaError_t resident_setup(int S, int C, int *side_by_side)
 {
     if constexpr (sizeof(T) == 4) {
         switch (S) { RES_SIZES_32(CASE_SETUP) }
@@ -510,8 +510,13 @@ cudaError_t launch_resident_tables(const ResTabJob<T> *jobs, int njobs, cudaStre
     return cudaGetLastError();
 }
 
-template cudaError_t resident_setup<float>(int, int, bool *);
-template cudaError_t resident_setup<double>(int, int, bool *);
+template cudaError_t resident_setup<float>(int, int, int *);
+template cudaError_t resident_setup<double>(int, int, int *);
+
+bool resident_pays(bool fp64, int S, int nrhs, int side_by_side)
+{
+    return side_by_side >= 1 && (!fp64 || S <= 16 || 4 * nrhs <= side_by_side);
+}
 template cudaError_t launch_resident<float>(const ResArgs<float> &, cudaStream_t);
 template cudaError_t launch_resident<double>(const ResArgs<double> &, cudaStream_t);
 template cudaError_t launch_resident_tables<float>(const ResTabJob<float> *, int, cudaStream_t);

@@ -79,8 +79,14 @@ struct ResTabJob {
 // Segment length for quarters of m unknowns per side (0: too large for a cluster).
 int resident_segment(bool fp64, int m);
 inline int resident_cluster(int m, int S) { return (m + S - 1) / S; }
+// Prepares the kernel; *side_by_side: clusters of it that the device runs at a time.
 template <typename T>
-cudaError_t resident_setup(int S, int C, bool *fits);
+cudaError_t resident_setup(int S, int C, int *side_by_side);
+// Whether a problem of nrhs right-hand sides, four clusters each, runs in one launch rather than
+// by the passes.  FP64 beyond n = 512 (S > 16) only while its clusters run at once (7 on GB300:
+// one right-hand side): n = 513 1.93 ms (4.16 by the passes), 640 2.05 (4.58), 641 2.69 (4.57), 768
+// 2.85 (4.67), but 5.36 against 4.72 for two right-hand sides at n = 641.
+bool resident_pays(bool fp64, int S, int nrhs, int side_by_side);
 template <typename T>
 cudaError_t launch_resident_tables(const ResTabJob<T> *jobs, int njobs, cudaStream_t st);
 template <typename T>

@@ -286,9 +286,9 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     streams_ = false;
     for (int p = 0; p < np; ++p) {
         const int m = (int)((ns[p] + 1) / 2), rs = resident_segment(kFP64, m);
-        bool fits = false;
-        if (rs > 0) ENG_CK(resident_setup<T>(rs, resident_cluster(m, rs), &fits));
-        if (fits) res_s_[p] = rs;
+        int side_by_side = 0;
+        if (rs > 0) ENG_CK(resident_setup<T>(rs, resident_cluster(m, rs), &side_by_side));
+        if (resident_pays(kFP64, rs, nrhs, side_by_side)) res_s_[p] = rs;
         else streams_ = true;
     }
     if (seg <= 0) {

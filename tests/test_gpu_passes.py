@@ -241,3 +241,21 @@ def test_refine_keeps_subnormal_quarters(api, n, k):
     if k == 0:
         assert _relmax(np.ldexp(got[1::2, 1::2], -e), want[1::2, 1::2]) <= 1e-3
     assert _relmax(got, oracle.poisson_square(G, 1e-13)) <= TOL_REFINE
+
+
+# FP64 beyond n = 512: one right-hand side runs in one launch up to n = 768, more are streamed
+@pytest.mark.parametrize("n", [513, 577, 639, 640, 641, 705, 767, 768, 769])
+@pytest.mark.parametrize("nrhs", [1, 2])
+def test_fp64_one_launch_of_few_clusters(api, n, nrhs):
+    F = inputs.square_rhs(n, n) if nrhs == 1 else np.stack([inputs.square_rhs(n, n + r) for r in range(nrhs)])
+    plan = api.plan_create(n, 2, 1e-13, "fp64", nrhs=nrhs)
+    X = api.poisson_square_solve(plan, torch.from_numpy(F).cuda()).cpu().numpy()
+    launches = api.plan_info(plan)["kernel_launches"]
+    api.plan_destroy(plan)
+    assert (launches == 1) == (nrhs == 1 and n <= 768)
+    for f, x in zip(F.reshape(nrhs, n, n), X.reshape(nrhs, n, n)):
+        assert _relmax(x, oracle.poisson_square(f, 1e-13)) <= TOL_FP64
+
+
+def test_nonfinite_input_leaves_no_trace_streamed(api):
+    test_nonfinite_input_leaves_no_trace(api, 801)
