@@ -51,7 +51,9 @@ template <typename T>
 template <typename U>
 cudaError_t SweepEngine<T>::dalloc(U **p, size_t count)
 {
-    cudaError_t e = cudaMalloc((void **)p, sizeof(U) * (count ? count : 1));
+    *p = nullptr;
+    if (!count) return cudaSuccess;
+    cudaError_t e = cudaMalloc((void **)p, sizeof(U) * count);
     if (e == cudaSuccess) {
         bytes += (int64_t)(sizeof(U) * count);
         allocs_.push_back((void *)*p);
@@ -76,9 +78,7 @@ void SweepEngine<T>::release()
     side_.clear();
     if (fork_) cudaEventDestroy(fork_);
     fork_ = nullptr;
-    void *hp[] = {h_active_, h_pair_active_, h_stat_};
-    for (void *p : hp)
-        if (p) cudaFreeHost(p);
+    if (h_stat_) cudaFreeHost(h_stat_);
     h_active_ = h_pair_active_ = nullptr;
     h_stat_ = nullptr;
 }
@@ -332,15 +332,17 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     fused_ = sweep_fused(kFP64, S, max_nb_);
     npairs_ = np * nrhs;
 
-    ENG_CK(sweep_setup_kernels());
+    if (streams_) ENG_CK(sweep_setup_kernels());
     if (!kFP64) {
         ENG_CK(dalloc(&Ft_, (size_t)totT_));  // quarter blocks, as X and D
         ENG_CK(dalloc(&Y0_, (size_t)totT_));
         ENG_CK(dalloc(&Y1_, (size_t)totT_));
     }
     ENG_CK(dalloc(&bands64_, (size_t)totB64));
-    ENG_CK(dalloc(&X_, (size_t)totT_));
-    ENG_CK(dalloc(&D_, (size_t)totT_));
+    // FP64 plans that stream nothing work on the caller's arrays (solve_plain): no X, D, graph
+    const size_t elems = graphs() ? (size_t)totT_ : 0;
+    ENG_CK(dalloc(&X_, elems));
+    ENG_CK(dalloc(&D_, elems));
     ENG_CK(dalloc(&sumR_, (size_t)totS_));
     ENG_CK(dalloc(&sumC_, (size_t)totS_));
     if (!fused_) {
@@ -352,15 +354,18 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     // what a round reports, read back in one copy: rmax and smax per pair, the error word
     ENG_CK(dalloc(&d_stat_, 2 * (size_t)npairs_ + 1));
     err_ = (int *)(d_stat_ + 2 * npairs_);
-    ENG_CK(cudaMallocHost((void **)&h_active_, sizeof(int) * (np + 1)));  // last: any problem inactive
-    ENG_CK(cudaMallocHost((void **)&h_pair_active_, sizeof(int) * npairs_));
-    ENG_CK(cudaMallocHost((void **)&h_stat_, sizeof(unsigned long long) * (2 * (size_t)npairs_ + 1)));
+    // one pinned block: statistics, then the masks (of the problems: last, any problem inactive)
+    const size_t stat_words = 2 * (size_t)npairs_ + 1;
+    ENG_CK(cudaMallocHost((void **)&h_stat_, sizeof(unsigned long long) * stat_words + sizeof(int) * (np + 1 + npairs_)));
+    h_active_ = (int *)(h_stat_ + stat_words);
+    h_pair_active_ = h_active_ + np + 1;
     h_stat_[2 * npairs_] = 0;
     // unused positions must be zero and stay zero
-    ENG_CK(cudaMemsetAsync(X_, 0, sizeof(T) * (size_t)totT_, cap_));
-    ENG_CK(cudaMemsetAsync(D_, 0, sizeof(T) * (size_t)totT_, cap_));
-    ENG_CK(cudaMemsetAsync(sumR_, 0, sizeof(T2) * (size_t)totS_, cap_));
-    ENG_CK(cudaMemsetAsync(sumC_, 0, sizeof(T2) * (size_t)totS_, cap_));
+    auto zero = [&](void *p, size_t b) { return b ? cudaMemsetAsync(p, 0, b, cap_) : cudaSuccess; };
+    ENG_CK(zero(X_, sizeof(T) * elems));
+    ENG_CK(zero(D_, sizeof(T) * elems));
+    ENG_CK(zero(sumR_, sizeof(T2) * (size_t)totS_));
+    ENG_CK(zero(sumC_, sizeof(T2) * (size_t)totS_));
     ENG_CK(cudaMemsetAsync(d_stat_, 0, sizeof(unsigned long long) * (2 * (size_t)npairs_ + 1), cap_));
     if (wait_fault_ && streams_) ENG_CK(cudaMemsetAsync(err_, 1, 1, cap_));  // as if a pass had given up
 
@@ -400,7 +405,7 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
             t.inv_ky = 1.0 / ky_;
             o64 += 7 * n;
             const int m = (int)((n + 1) / 2), nt = (m + 31) / 32, ntp = (nb_[p] << t.log_s) / 32;
-            for (int r = 0; r < nrhs; ++r) {
+            for (int r = 0; r < nrhs && graphs(); ++r) {
                 const int id = p * 256 + r;
                 for (int ty = 0; ty < nt; ++ty)
                     for (int tx = 0; tx < nt; ++tx) tiles[0].push_back(make_int4(id, tx, ty, 0));
@@ -416,6 +421,7 @@ int SweepEngine<T>::create(const std::vector<int64_t> &ns, int nrhs, double tol,
     ENG_CK(dalloc(&d_tp_, (size_t)np));
     for (int w = 0; w < 3; ++w) {
         ntiles_[w] = (int64_t)tiles[w].size();
+        if (tiles[w].empty()) continue;
         ENG_CK(dalloc(&d_tiles_[w], tiles[w].size()));
         ENG_CK(cudaMemcpyAsync(d_tiles_[w], tiles[w].data(), sizeof(int4) * tiles[w].size(), cudaMemcpyHostToDevice, cap_));
     }
@@ -681,7 +687,7 @@ int SweepEngine<T>::build_tables(Level &L, int level, const std::vector<double> 
     for (int w = 0; w < 3 && e1 == cudaSuccess; ++w) {
         L.nitems[w] = (int64_t)it[w].size();
         e1 = dalloc(&L.items[w], it[w].size());
-        if (e1 == cudaSuccess)
+        if (e1 == cudaSuccess && !it[w].empty())
             e1 = cudaMemcpyAsync(L.items[w], it[w].data(), sizeof(SwItem<T>) * it[w].size(), cudaMemcpyHostToDevice, cap_);
     }
     for (size_t c = 0; c < L.res.size() && e1 == cudaSuccess; ++c) {
@@ -784,7 +790,7 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
         L.graph = nullptr;
     }
     const SwArgs<T> ar = args(L, 0), ac = args(L, 1), ach = args(L, 2);
-    // created outside the capture
+    // branches of the resident launches, created outside the capture
     for (int k = (int)side_.size(), want = std::min<int>(kSide, (int)L.res.size() - (streams_ ? 0 : 1)); k < want; ++k) {
         Side x;
         ENG_CK(cudaEventCreateWithFlags(&x.done, cudaEventDisableTiming));
@@ -792,6 +798,7 @@ int SweepEngine<T>::build_graph(Level &L, std::string &err)
         ENG_CK(cudaStreamCreateWithFlags(&side_.back().st, cudaStreamNonBlocking));
     }
     if (!side_.empty() && !fork_) ENG_CK(cudaEventCreateWithFlags(&fork_, cudaEventDisableTiming));
+    if (!graphs()) return FPS_OK;
     ENG_CK(cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     const bool ins = instrument_ && (int)L.ev.size() == 4 * L.Jstream;
@@ -846,7 +853,7 @@ template <typename T>
 int SweepEngine<T>::solve_plain(const double *F, double *X, cudaStream_t st, std::string &err)
 {
     if constexpr (sizeof(T) == 8) {
-        if (!streams_) {  // scale-in, all iterations and scale-out in one launch per class
+        if (!graphs()) {  // scale-in, all iterations and scale-out in one launch per class
             ENG_CK(run_resident(levels_[0], F, X, st, false, launches_last));
             ENG_CK(join_resident(st));
             levels_used_.push_back(0);

@@ -117,6 +117,7 @@ private:
     std::vector<int> nb_;      // blocks per side of a quarter (of 32 for resident problems)
     std::vector<int> res_s_;   // resident problems: segment length; 0: streamed by the passes
     bool streams_ = false;     // any problem is streamed
+    bool graphs() const { return sizeof(T) == 4 || streams_; }  // otherwise one launch per class, outside a graph
     int max_nb_ = 0;
     bool fused_ = false;   // the passes run the segment recurrences
     std::vector<int64_t> off64_, offT_, offS_;
