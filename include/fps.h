@@ -315,7 +315,7 @@ int fps_poisson_dirichlet_adjoint(fps_plan *plan, const double *dLdU, double *dL
  * iteration (widened by 3 %) and the tight interval of sigma(B); J of (2.9) per mode.
  * FP64.  n >= 4, nrhs right-hand sides per mode (e.g. the real and imaginary parts
  * of f_k and f_{-k}).  The line kernels hold 32 whole lines per CTA in shared memory
- * (about 352 n bytes), so n is bounded by the device's per-CTA limit: n <= 660 on
+ * (about 352 n bytes), so n is bounded by the device's per-CTA limit: n <= 659 on
  * GB300 (227 KB).  Errors: INVALID_ARG, UNSUPPORTED (n above that bound or above
  * 4096, an interval or a pivot that cannot be formed), CUDA.
  */

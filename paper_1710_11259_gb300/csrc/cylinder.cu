@@ -833,7 +833,7 @@ int CylinderEngine::create(int64_t n_, int64_t kmin_, int64_t kmax_, double tol,
     nrhs = nrhs_;
     const int modes = (int)(kmax - kmin + 1);
     // The streaming kernels hold whole lines of 32 (mode, rhs) rows or columns in shared
-    // memory: about 352 n bytes per CTA, n <= 660 at 227 KB.
+    // memory: about 352 n bytes per CTA, n <= 659 at 227 KB.
     int dev = 0, optin = 0;
     CYL_CK(cudaGetDevice(&dev));
     CYL_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
